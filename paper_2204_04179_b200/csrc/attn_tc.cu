@@ -410,6 +410,10 @@ __global__ void __launch_bounds__(ATT_THREADS, 1) attn_tc_fwd_kernel(const __gri
         ++ord;
         for (int j = 0; j < x.nk; ++j, ++n) {
           if (pend_stage[g] >= 0 && !issue_pv(g)) { failed = true; break; }
+          // An item of three or more key tiles needs the stage that the previous item's last product (the other
+          // group's) still holds: that product goes first, or the copy of the third tile would wait for a stage
+          // that only the item after this one releases.
+          if (j == 1 && x.nk >= FWD_STAGES && pend_stage[g ^ 1] >= 0 && !issue_pv(g ^ 1)) { failed = true; break; }
           const int s = (int)(n % FWD_STAGES);
           if (!mbar_wait(full_bar(s), (uint32_t)((n / FWD_STAGES) & 1), abort_flag)) { failed = true; break; }
           tc_fence_after();
