@@ -3,6 +3,7 @@
 // (per-warp registers -> ordered block sum -> ordered sum over blocks), so results are bit-stable.
 #include "gemm.h"
 #include "layers.h"
+#include "tc_common.cuh"
 
 namespace {
 
@@ -113,46 +114,82 @@ __global__ void __launch_bounds__(256) ln_fwd_kernel(const float* __restrict__ z
   }
 }
 
+// LayerNorm backward: 14 bytes per element and little arithmetic, so it is bound by HBM once enough rows are in flight.
+// Registers are not the place to keep them (a row of 768 already takes 96 for its values and the running sums): every
+// warp has a ring of LNB_STAGES rows of dy and z in shared memory, filled by bulk copies that the warp's first lane
+// issues as soon as a slot has been read, so 18 KB per warp are on their way while it computes.  One block of eight warps
+// per SM; the partial sums (dgamma, dbeta, columns of dz) stay in registers to the end.  83 000 x 768 with its reduction: 222 us with one
+// row of loads per warp and two blocks per SM, 152 us (5.9 TB/s) now.
+constexpr int LNB_WARPS = 8, LNB_STAGES = 3;
 template <typename T, int NQ>
-__global__ void __launch_bounds__(256, 2) ln_bwd_kernel(const float* __restrict__ dy, const float* __restrict__ z,
-                                                        const float* __restrict__ mean, const float* __restrict__ rstd,
-                                                        const float* __restrict__ g, float* __restrict__ dz,
-                                                        T* __restrict__ dz_b, float* __restrict__ part, int64_t rows,
-                                                        int d, int want_col) {
-  // [3][d]: dgamma, dbeta and the column sums of dz of this block; then [d]: gamma; then, when the column sums
-  // are wanted, one float4 per (warp, i, lane): each thread's running column sums (registers are all taken)
-  extern __shared__ float sacc[];
+__global__ void __launch_bounds__(32 * LNB_WARPS, 1) ln_bwd_kernel(const float* __restrict__ dy, const float* __restrict__ z,
+                                                                  const float* __restrict__ mean, const float* __restrict__ rstd,
+                                                                  const float* __restrict__ g, float* __restrict__ dz,
+                                                                  T* __restrict__ dz_b, float* __restrict__ part, int64_t rows,
+                                                                  int d, int32_t* status) {
+  // [3][d]: dgamma, dbeta and the column sums of dz of this block; [d]: gamma; then the warps' rings
+  extern __shared__ __align__(16) float sacc[];
+  __shared__ __align__(8) uint64_t bars[LNB_WARPS * LNB_STAGES];
+  __shared__ int abort_flag;
   float* sgam = sacc + 3 * d;
-  float4* scol = reinterpret_cast<float4*>(sgam + d) + (threadIdx.x >> 5) * (NQ * 32) + (threadIdx.x & 31);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
-  const int64_t w = (int64_t)blockIdx.x * nwb + warp;
-  const int64_t nw = (int64_t)gridDim.x * nwb;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float* ring = sgam + d + (size_t)warp * LNB_STAGES * 2 * d;
+  const uint32_t bar0 = tc::smem_u32(bars + warp * LNB_STAGES);
+  const int64_t w = (int64_t)blockIdx.x * LNB_WARPS + warp;
+  const int64_t nw = (int64_t)gridDim.x * LNB_WARPS;
+  const uint32_t row_bytes = (uint32_t)d * 4u;
+  auto request = [&](int64_t r, int s) {
+    const uint32_t bar = bar0 + 8u * s, dst = tc::smem_u32(ring + (size_t)s * 2 * d);
+    tc::mbar_expect_tx(bar, 2u * row_bytes);
+    tc::bulk_load(dst, dy + r * d, row_bytes, bar);
+    tc::bulk_load(dst + row_bytes, z + r * d, row_bytes, bar);
+  };
+  if (lane == 0) {
+    for (int s = 0; s < LNB_STAGES; ++s) tc::mbar_init(bar0 + 8u * s, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int s = 0; s < LNB_STAGES; ++s)
+      if (w + s * nw < rows) request(w + s * nw, s);
+  }
+  if (threadIdx.x == 0) abort_flag = 0;
   for (int i = threadIdx.x; i < d; i += blockDim.x) sgam[i] = g[i];
   for (int i = threadIdx.x; i < 3 * d; i += blockDim.x) sacc[i] = 0.f;
   __syncthreads();
-  float4 ag[NQ], ab[NQ];
+  float4 ag[NQ], ab[NQ], ac[NQ];
 #pragma unroll
-  for (int i = 0; i < NQ; ++i) {
-    ag[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    ab[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (want_col) scol[i * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+  for (int i = 0; i < NQ; ++i) ag[i] = ab[i] = ac[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  float mu_n = 0.f, rs_n = 0.f;                  // the next row's statistics
+  if (w < rows) { mu_n = mean[w]; rs_n = rstd[w]; }
+  int s = 0;
+  uint32_t parity = 0;
   for (int64_t r = w; r < rows; r += nw) {
-    const float mu = mean[r], rs = rstd[r];
+    const float mu = mu_n, rs = rs_n;
+    if (r + nw < rows) { mu_n = mean[r + nw]; rs_n = rstd[r + nw]; }
+    if (!tc::mbar_wait(bar0 + 8u * s, parity, (volatile int*)&abort_flag)) {
+      abort_flag = 1;
+      gram_device_fail(status, GRAM_ERR_TIMEOUT);
+      const uint64_t t0 = clock64();             // let the copies that were issued arrive before the block leaves
+      while (clock64() - t0 < tc::WAIT_LIMIT_CYCLES / 64) {}
+      break;
+    }
+    const float* sd = ring + (size_t)s * 2 * d;
+    const float* sz = sd + d;
     float4 xh[NQ], dd[NQ];
     float s1 = 0.f, s2 = 0.f;
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
       const int c = 4 * (lane + 32 * i);
       if (c < d) {
-        const float4 zz = ld4f(z + r * d + c);
-        dd[i] = ld4f(dy + r * d + c);
+        const float4 zz = ld4f(sz + c);
+        dd[i] = ld4f(sd + c);
         xh[i] = make_float4((zz.x - mu) * rs, (zz.y - mu) * rs, (zz.z - mu) * rs, (zz.w - mu) * rs);
       } else {
         xh[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         dd[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
+    __syncwarp();                                // the slot has been read by every lane
+    if (lane == 0 && r + LNB_STAGES * nw < rows) request(r + LNB_STAGES * nw, s);
+    if (++s == LNB_STAGES) { s = 0; parity ^= 1u; }
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
       const int c = 4 * (lane + 32 * i);
@@ -173,26 +210,22 @@ __global__ void __launch_bounds__(256, 2) ln_bwd_kernel(const float* __restrict_
                                      rs * (dd[i].z - s1 - xh[i].z * s2), rs * (dd[i].w - s1 - xh[i].w * s2));
         st4t(dz + r * d + c, o);
         if (dz_b) st4t(dz_b + r * d + c, o);
-        if (want_col) {
-          float4 t = scol[i * 32];
-          t.x += o.x; t.y += o.y; t.z += o.z; t.w += o.w;
-          scol[i * 32] = t;
-        }
+        ac[i].x += o.x; ac[i].y += o.y; ac[i].z += o.z; ac[i].w += o.w;
       }
     }
   }
-  for (int ww = 0; ww < nwb; ++ww) {       // warps add in ascending order
+  for (int ww = 0; ww < LNB_WARPS; ++ww) {       // warps add in ascending order
     if (warp == ww) {
 #pragma unroll
       for (int i = 0; i < NQ; ++i) {
         const int c = 4 * (lane + 32 * i);
         if (c < d) {
-          sacc[c] += ag[i].x; sacc[c + 1] += ag[i].y; sacc[c + 2] += ag[i].z; sacc[c + 3] += ag[i].w;
-          sacc[d + c] += ab[i].x; sacc[d + c + 1] += ab[i].y; sacc[d + c + 2] += ab[i].z; sacc[d + c + 3] += ab[i].w;
-          if (want_col) {
-            const float4 t = scol[i * 32];
-            sacc[2 * d + c] += t.x; sacc[2 * d + c + 1] += t.y; sacc[2 * d + c + 2] += t.z; sacc[2 * d + c + 3] += t.w;
-          }
+          float4* p0 = reinterpret_cast<float4*>(sacc + c);
+          float4* p1 = reinterpret_cast<float4*>(sacc + d + c);
+          float4* p2 = reinterpret_cast<float4*>(sacc + 2 * d + c);
+          float4 t = *p0; t.x += ag[i].x; t.y += ag[i].y; t.z += ag[i].z; t.w += ag[i].w; *p0 = t;
+          t = *p1; t.x += ab[i].x; t.y += ab[i].y; t.z += ab[i].z; t.w += ab[i].w; *p1 = t;
+          t = *p2; t.x += ac[i].x; t.y += ac[i].y; t.z += ac[i].z; t.w += ac[i].w; *p2 = t;
         }
       }
     }
@@ -201,31 +234,29 @@ __global__ void __launch_bounds__(256, 2) ln_bwd_kernel(const float* __restrict_
   for (int i = threadIdx.x; i < 3 * d; i += blockDim.x) part[(int64_t)blockIdx.x * 3 * d + i] = sacc[i];
 }
 
-// out[c] += scale * sum_b part[b*stride + c]   (two outputs when out2 != null: second half of each partial row).
-// A block owns 32 columns; its 8 warps take the partial rows b = w, w+8, ... and their sums are added in
-// ascending w, so the order of additions is fixed.
+// out[c] += scale * sum_b part[b*stride + c]; grid row y > 0 does the same with columns y * n .. of the partial rows,
+// into out2 (y = 1) and out3 (y = 2).  A block owns 32 columns; its 8 warps take the partial rows b = w, w+8, ... and
+// their sums are added in ascending w, so the order of additions is fixed.
 __global__ void __launch_bounds__(256) reduce_partials_kernel(const float* __restrict__ part, int nblocks, int64_t stride,
                                                               int n, float* __restrict__ out, float* __restrict__ out2,
-                                                              float scale) {
-  __shared__ float sa[8][32], sb[8][32];
+                                                              float* __restrict__ out3, float scale) {
+  __shared__ float sa[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
-  float a = 0.f, b = 0.f;
+  part += (int64_t)blockIdx.y * n;
+  float* o = blockIdx.y == 0 ? out : (blockIdx.y == 1 ? out2 : out3);
+  float a = 0.f;
   if (c < n) {
-    for (int k = w; k < nblocks; k += 8) {
-      a += part[(int64_t)k * stride + c];
-      if (out2) b += part[(int64_t)k * stride + n + c];
-    }
+#pragma unroll 4
+    for (int k = w; k < nblocks; k += 8) a += part[(int64_t)k * stride + c];
   }
   sa[w][lane] = a;
-  sb[w][lane] = b;
   __syncthreads();
   if (w == 0 && c < n) {
-    float ta = sa[0][lane], tb = sb[0][lane];
+    float ta = sa[0][lane];
 #pragma unroll
-    for (int k = 1; k < 8; ++k) { ta += sa[k][lane]; tb += sb[k][lane]; }
-    out[c] += ta * scale;
-    if (out2) out2[c] += tb * scale;
+    for (int k = 1; k < 8; ++k) ta += sa[k][lane];
+    o[c] += ta * scale;
   }
 }
 
@@ -1112,20 +1143,15 @@ gram_status layernorm_backward(gram_ctx* ctx, int dtype, const float* dy, const 
                                float* dbeta, float* dcol, float* scratch, int64_t rows, int d, cudaStream_t st) {
   if (rows == 0) return GRAM_OK;
   if (d > 1024 || (d & 3)) return gram_set_error(ctx, "LayerNorm: d must be a multiple of 4 and at most 1024"), GRAM_ERR_UNSUPPORTED;
-  int cap = (int)(kRedScratchBytes / ((size_t)3 * d * sizeof(float)));
-  if (cap > kNumSMs * 8) cap = kNumSMs * 8;
-  // at least sixteen rows per warp where the row count allows it: a block's fixed work (clearing and writing 3 d partial
-  // sums, which the reduction kernels then read) is otherwise most of a call on a few ten thousand rows
-  int64_t want = (rows + 127) / 128;
-  if (want < kNumSMs) want = kNumSMs;
-  if (want > cap) want = cap;
-  const int blocks = grid_for(rows * 32, 256, (int)want);
-  const int nq = d <= 128 ? 1 : d <= 256 ? 2 : d <= 512 ? 4 : d <= 768 ? 6 : 8;   // float4 per lane: the kernel's NQ
-  const size_t smem = (size_t)4 * d * sizeof(float) + (dcol ? (size_t)8 * nq * 32 * sizeof(float4) : 0);
-  ProfScope prof(ctx, GRAM_K_LAYERNORM, (double)rows * d * (12.0 + (dz_b ? (dtype == GRAM_BF16 ? 2.0 : 4.0) : 0.0)), dcol ? 3 : 2, st, "ln_bwd");
-  DISPATCH_T(dtype, DISPATCH_NQ(d, ln_bwd_kernel<T, NQ><<<blocks, 256, smem, st>>>(dy, z, mean, rstd, gamma, dz, (T*)dz_b, scratch, rows, d, dcol ? 1 : 0)));
-  reduce_partials_kernel<<<ceil_div(d, 32), 256, 0, st>>>(scratch, blocks, (int64_t)3 * d, d, dgamma, dbeta, 1.f);
-  if (dcol) reduce_partials_kernel<<<ceil_div(d, 32), 256, 0, st>>>(scratch + 2 * d, blocks, (int64_t)3 * d, d, dcol, nullptr, 1.f);
+  int blocks = kNumSMs;                            // one per SM; at least one row per warp
+  if (rows < (int64_t)blocks * LNB_WARPS) blocks = (int)ceil_div64(rows, LNB_WARPS);
+  const size_t smem = (size_t)(4 + LNB_WARPS * LNB_STAGES * 2) * d * sizeof(float);
+  ProfScope prof(ctx, GRAM_K_LAYERNORM, (double)rows * d * (12.0 + (dz_b ? (dtype == GRAM_BF16 ? 2.0 : 4.0) : 0.0)), 2, st, "ln_bwd");
+  DISPATCH_T(dtype, DISPATCH_NQ(d, {
+    GRAM_TRY(set_smem(ctx, ln_bwd_kernel<T, NQ>, smem));
+    ln_bwd_kernel<T, NQ><<<blocks, 32 * LNB_WARPS, smem, st>>>(dy, z, mean, rstd, gamma, dz, (T*)dz_b, scratch, rows, d, gram_status_word(ctx));
+  }));
+  reduce_partials_kernel<<<dim3(ceil_div(d, 32), dcol ? 3 : 2), 256, 0, st>>>(scratch, blocks, (int64_t)3 * d, d, dgamma, dbeta, dcol, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1257,7 +1283,7 @@ gram_status colsum_from_partials(gram_ctx* ctx, const float* part, int64_t nrows
   if ((size_t)G * N * sizeof(float) > kRedScratchBytes) G = (int)(kRedScratchBytes / ((size_t)N * sizeof(float)));
   if (G < 1) return gram_set_error(ctx, "column sums: N too large for the reduction scratch"), GRAM_ERR_UNSUPPORTED;
   fold_partials_kernel<<<dim3((unsigned)ceil_div(N, 32), (unsigned)G), 256, 0, st>>>(part, nrows, N, scratch);
-  reduce_partials_kernel<<<ceil_div(N, 32), 256, 0, st>>>(scratch, G, (int64_t)N, N, out, nullptr, 1.f);
+  reduce_partials_kernel<<<ceil_div(N, 32), 256, 0, st>>>(scratch, G, (int64_t)N, N, out, nullptr, nullptr, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1275,7 +1301,7 @@ gram_status colsum_accumulate(gram_ctx* ctx, int dtype, const void* X, int64_t r
   dim3 grid((unsigned)ceil_div(N, 64), (unsigned)rb);
   ProfScope prof(ctx, GRAM_K_COLSUM, (double)rows * N * (dtype == GRAM_BF16 ? 2.0 : 4.0), 2, st, "colsum");
   DISPATCH_T(dtype, colsum_kernel<T><<<grid, 256, 0, st>>>((const T*)X, rows, N, per, scratch));
-  reduce_partials_kernel<<<ceil_div(N, 32), 256, 0, st>>>(scratch, (int)rb, (int64_t)N, N, out, nullptr, 1.f);
+  reduce_partials_kernel<<<ceil_div(N, 32), 256, 0, st>>>(scratch, (int)rb, (int64_t)N, N, out, nullptr, nullptr, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1294,7 +1320,7 @@ gram_status periodic_rowsum_accumulate(gram_ctx* ctx, const float* X, int64_t n_
   ProfScope prof(ctx, GRAM_K_EMBED_POOL, 4.0 * (double)n_groups * period * d, chunks > 1 ? 2 : 1, st);
   dim3 grid((unsigned)ceil_div64(n, 128), (unsigned)chunks);
   periodic_rowsum_kernel<<<grid, 128, 0, st>>>(X, n_groups, per, period, d, out, chunks > 1 ? scratch : nullptr, seq_len, seq_off);
-  if (chunks > 1) reduce_partials_kernel<<<ceil_div((int)n, 32), 256, 0, st>>>(scratch, (int)chunks, n, (int)n, out, nullptr, 1.f);
+  if (chunks > 1) reduce_partials_kernel<<<ceil_div((int)n, 32), 256, 0, st>>>(scratch, (int)chunks, n, (int)n, out, nullptr, nullptr, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1360,7 +1386,7 @@ gram_status kt_input_backward(gram_ctx* ctx, const float* dx, const int32_t* lab
   dim3 grid((unsigned)ceil_div(d, 128), (unsigned)L);
   ProfScope prof(ctx, GRAM_K_TASK_HEAD, 8.0 * (double)B * L * d, 2, st);
   kt_input_bwd_kernel<<<grid, 128, 0, st>>>(dx, labels, dE, dpos, scratch, B, L, d);
-  reduce_partials_kernel<<<ceil_div(3 * d, 32), 256, 0, st>>>(scratch, L, (int64_t)3 * d, 3 * d, dresp, nullptr, 1.f);
+  reduce_partials_kernel<<<ceil_div(3 * d, 32), 256, 0, st>>>(scratch, L, (int64_t)3 * d, 3 * d, dresp, nullptr, nullptr, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1552,7 +1578,7 @@ gram_status pool_additive_backward(gram_ctx* ctx, int dtype, const StreamRef& x,
   ProfScope prof(ctx, GRAM_K_EMBED_POOL, 4.0 * (double)n * l_t * (2 * d + 2 * pa), 2, st);
   DISPATCH_T(dtype, pool_additive_bwd_kernel<T><<<(unsigned)n, 128, 0, st>>>(x, (const T*)pre, q, alpha, G, dx, (T*)dpre, scratch, l_t, d,
                                                                             pa, seq_len, seq_off));
-  reduce_partials_kernel<<<ceil_div(pa, 32), 256, 0, st>>>(scratch, (int)n, pa, pa, dq, nullptr, 1.f);
+  reduce_partials_kernel<<<ceil_div(pa, 32), 256, 0, st>>>(scratch, (int)n, pa, pa, dq, nullptr, nullptr, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
