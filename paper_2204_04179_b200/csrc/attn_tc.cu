@@ -994,9 +994,15 @@ void plan_launch(AttnArgs& a, int64_t n_seq, int S, bool contiguous) {
 // unset: sequences of more than 64 rows.  Up to 64 rows the warp-level kernels keep several small blocks per SM resident
 // and hide memory latency by occupancy, which one persistent block per SM does not (measured on the knowledge-tracing
 // encoder: 5.9 + 16.2 ms per step against 6.9 + 19.0 ms); from 65 rows on their one-sequence tile fills an SM with a
-// single block, and beyond 128 rows they cannot hold a sequence at all.
-bool attention_tc_supported(int S, int d, int n_heads) {
+// single block, and beyond 128 rows they cannot hold a sequence at all.  Of the sequences that come here, those of 65 to
+// 96 rows (forward), 129 to 256 (forward) and 129 to 192 (backward) go on to the kernels of attn_flash.cu, which do not pad to 128-row tiles.
+static int attn_tc_mode() {
   static const int mode = []() { const char* v = getenv("GRAM_ATTN_TC"); return !v ? 2 : (v[0] == '0' ? 0 : 1); }();
+  return mode;
+}
+bool attention_tc_forced() { return attn_tc_mode() == 1; }
+bool attention_tc_supported(int S, int d, int n_heads) {
+  const int mode = attn_tc_mode();
   if (mode == 0 || !(S >= 1 && n_heads > 0 && d == n_heads * DH && get_encode_fn() != nullptr)) return false;
   return mode == 1 || S > 64;
 }

@@ -1165,13 +1165,21 @@ gram_status attention_forward(gram_ctx* ctx, int dtype, const void* qkv, void* o
   const float scale = 1.f / sqrtf((float)dh);
   ProfScope prof(ctx, GRAM_K_ATTENTION, 4.0 * (double)n_seq * n_heads * S * S * dh, 1, st, "attn_fwd");
   if (dtype == GRAM_BF16 && attention_tc_supported(S, d, n_heads)) {
+    auto flash = [&](int bound) { return !attention_tc_forced() && attention_flash_forward_supported(bound, d, n_heads); };
+    if ((!groups || !seq_off) && flash(S))
+      return attention_forward_flash(ctx, qkv, out, lse, rows, n_seq, S, d, n_heads, causal, seq_len, seq_off, nullptr, st);
     if (!groups || !seq_off) return attention_forward_tc(ctx, qkv, out, lse, rows, n_seq, S, d, n_heads, causal, seq_len, seq_off, nullptr, st);
     int32_t first = 0;
     for (int gi = 0; gi < 4; ++gi) {                 // one launch per length group, with the smallest slot that fits
       const int bound = gi < 3 ? (S < 32 * (gi + 1) ? S : 32 * (gi + 1)) : S;
-      if (groups->count[gi] > 0)
-        GRAM_TRY(attention_forward_tc(ctx, qkv, out, lse, rows, groups->count[gi], bound, d, n_heads, causal, seq_len, seq_off,
-                                      groups->list + first, st));
+      if (groups->count[gi] > 0) {
+        if (flash(bound))
+          GRAM_TRY(attention_forward_flash(ctx, qkv, out, lse, rows, groups->count[gi], bound, d, n_heads, causal, seq_len, seq_off,
+                                           groups->list + first, st));
+        else
+          GRAM_TRY(attention_forward_tc(ctx, qkv, out, lse, rows, groups->count[gi], bound, d, n_heads, causal, seq_len, seq_off,
+                                        groups->list + first, st));
+      }
       first += groups->count[gi];
     }
     return GRAM_OK;
@@ -1210,20 +1218,28 @@ gram_status attention_backward(gram_ctx* ctx, int dtype, const void* qkv, const 
   const bool grouped = groups && seq_off;
   if (dtype == GRAM_BF16 && attention_tc_supported(S, d, n_heads)) {
     auto bound = [&](int gi) { return gi < 3 ? (S < 32 * (gi + 1) ? S : 32 * (gi + 1)) : S; };
+    auto flash = [&](int b) { return !attention_tc_forced() && attention_flash_backward_supported(b, d, n_heads); };
+    auto part_rows = [&](int64_t n, int b) { return flash(b) ? n : attention_tc_colpart_rows(n, b); };
     int64_t need = 0;
-    if (!grouped) need = attention_tc_colpart_rows(n_seq, S);
-    else for (int gi = 0; gi < 4; ++gi) need += groups->count[gi] > 0 ? attention_tc_colpart_rows(groups->count[gi], bound(gi)) : 0;
+    if (!grouped) need = part_rows(n_seq, S);
+    else for (int gi = 0; gi < 4; ++gi) need += groups->count[gi] > 0 ? part_rows(groups->count[gi], bound(gi)) : 0;
     float* cp = (colpart && need <= colpart_cap_rows) ? colpart : nullptr;      // partial column sums only when they fit
     if (cp && colpart_rows_used) *colpart_rows_used = need;
+    if (!grouped && flash(S))
+      return attention_backward_flash(ctx, qkv, dctx, octx, lse, dqkv, cp, rows, n_seq, S, d, n_heads, causal, seq_len, seq_off, nullptr, st);
     if (!grouped)
       return attention_backward_tc(ctx, qkv, dctx, octx, lse, delta, dqkv, cp, 0, rows, n_seq, S, d, n_heads, causal, seq_len, seq_off, nullptr, st);
     int32_t first = 0;
     int64_t row0 = 0;
     for (int gi = 0; gi < 4; ++gi) {
       if (groups->count[gi] > 0) {
-        GRAM_TRY(attention_backward_tc(ctx, qkv, dctx, octx, lse, delta, dqkv, cp, row0, rows, groups->count[gi], bound(gi), d, n_heads,
-                                       causal, seq_len, seq_off, groups->list + first, st));
-        row0 += attention_tc_colpart_rows(groups->count[gi], bound(gi));
+        if (flash(bound(gi)))
+          GRAM_TRY(attention_backward_flash(ctx, qkv, dctx, octx, lse, dqkv, cp ? cp + row0 * 3 * d : nullptr, rows, groups->count[gi],
+                                            bound(gi), d, n_heads, causal, seq_len, seq_off, groups->list + first, st));
+        else
+          GRAM_TRY(attention_backward_tc(ctx, qkv, dctx, octx, lse, delta, dqkv, cp, row0, rows, groups->count[gi], bound(gi), d, n_heads,
+                                         causal, seq_len, seq_off, groups->list + first, st));
+        row0 += part_rows(groups->count[gi], bound(gi));
       }
       first += groups->count[gi];
     }

@@ -73,8 +73,19 @@ gram_status attention_backward(gram_ctx* ctx, int dtype, const void* qkv, const 
                                int64_t rows, int64_t n_seq, int S, int d, int n_heads, int causal, const int32_t* seq_len,
                                const int32_t* seq_off, const SeqGroups* groups, cudaStream_t st);
 
+// warp-level kernels for sequences of up to 256 (backward: 192) rows (attn_flash.cu); colpart: one row per sequence of the launch
+bool attention_flash_forward_supported(int S, int d, int n_heads);
+bool attention_flash_backward_supported(int S, int d, int n_heads);
+gram_status attention_forward_flash(gram_ctx* ctx, const void* qkv, void* out, float* lse, int64_t rows, int64_t n_seq, int S, int d,
+                                    int n_heads, int causal, const int32_t* seq_len, const int32_t* seq_off, const int32_t* seq_list,
+                                    cudaStream_t st);
+gram_status attention_backward_flash(gram_ctx* ctx, const void* qkv, const void* dctx, const void* octx, const float* lse, void* dqkv,
+                                     float* colpart, int64_t rows, int64_t n_seq, int S, int d, int n_heads, int causal,
+                                     const int32_t* seq_len, const int32_t* seq_off, const int32_t* seq_list, cudaStream_t st);
+
 // the tcgen05 kernels behind the two calls above (bf16, head width 64, sequences of any length)
 bool attention_tc_supported(int S, int d, int n_heads);
+bool attention_tc_forced();        // GRAM_ATTN_TC=1: no other kernel is to be chosen
 gram_status attention_forward_tc(gram_ctx* ctx, const void* qkv, void* out, float* lse, int64_t rows, int64_t n_seq, int S, int d,
                                  int n_heads, int causal, const int32_t* seq_len, const int32_t* seq_off, const int32_t* seq_list,
                                  cudaStream_t st);
