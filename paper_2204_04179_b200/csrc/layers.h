@@ -73,6 +73,18 @@ gram_status attention_backward(gram_ctx* ctx, int dtype, const void* qkv, const 
                                int64_t rows, int64_t n_seq, int S, int d, int n_heads, int causal, const int32_t* seq_len,
                                const int32_t* seq_off, const SeqGroups* groups, cudaStream_t st);
 
+// one query row per sequence (attn_cls.cu): q, out, dctx, dq [n, d]; kv, dkv [rows, 2d] (keys, then values); bf16.
+// part [part_cap_rows, 3d] receives *part_rows rows of column sums of dq, dK, dV
+bool attention_cls_supported(int l_t, int d, int n_heads);
+gram_status attention_cls_forward(gram_ctx* ctx, const void* q, const void* kv, void* out, int n, int l_t, int d, int n_heads,
+                                  const int32_t* seq_len, const int32_t* seq_off, cudaStream_t st);
+gram_status attention_cls_backward(gram_ctx* ctx, const void* q, const void* kv, const void* dctx, void* dq, void* dkv, float* part,
+                                   int64_t part_cap_rows, int64_t* part_rows, int n, int l_t, int d, int n_heads,
+                                   const int32_t* seq_len, const int32_t* seq_off, cudaStream_t st);
+// X[row(u), :] += r[u, :] for u < n, fp32; row(u) as in take_strided_rows
+gram_status add_strided_rows(gram_ctx* ctx, const float* r, int64_t n, int64_t stride, const int32_t* rows, int d, float* X,
+                             cudaStream_t st);
+
 // warp-level kernels for sequences of up to 256 (backward: 192) rows (attn_flash.cu); colpart: one row per sequence of the launch
 bool attention_flash_forward_supported(int S, int d, int n_heads);
 bool attention_flash_backward_supported(int S, int d, int n_heads);

@@ -102,6 +102,9 @@ struct Model {
   // last layer (output projection, feed-forward, both LayerNorms) runs on those rows alone: `tail` holds their
   // activations and scratch (one row per item), tail_* the layer's input stream at those rows.
   bool cls_tail = false;
+  // and its attention has one query row per item (bf16, heads of width 64): keys and values of every token, [T, 2d] in the
+  // layer's qkv buffer; queries [mb, d] and the layer's input at row 0 [mb, d] in the tail's qkv buffer
+  bool cls_query = false;
   Stack tail;
   float *tail_z = nullptr, *tail_mean = nullptr, *tail_rstd = nullptr;
   float* z0 = nullptr;               // token + position embedding, fp32
@@ -394,9 +397,10 @@ gram_status layer_rest_forward(Model* m, Module& mod, const LayerOff& o, LayerAc
 
 // x_in: the fp32 input stream; x_in_b: its operand-typed copy.  *out / *out_b: the same pair for the output of
 // layer n_full - 1.  Layers [0, n_full) run completely; when n_full < n_layers, layer n_full runs its attention
-// part only (its ctx is left in s.acts[n_full].ctx) and *out / *out_b describe that layer's input.
+// part only (its ctx is left in s.acts[n_full].ctx; not even that without top_attention) and *out / *out_b describe that
+// layer's input.
 gram_status stack_forward(Model* m, Module& mod, Stack& s, const StreamRef& x_in, const void* x_in_b, int64_t n_seq, int S,
-                          cudaStream_t st, StreamRef* out, const void** out_b, int n_full = -1) {
+                          cudaStream_t st, StreamRef* out, const void** out_b, int n_full = -1, bool top_attention = true) {
   const int64_t T = s.packed_rows ? s.packed_rows : n_seq * S;
   if (n_full < 0) n_full = s.n_layers;
   StreamRef x = x_in;
@@ -405,7 +409,7 @@ gram_status stack_forward(Model* m, Module& mod, Stack& s, const StreamRef& x_in
     GRAM_TRY(layer_attention_forward(m, mod, s, l, xb, n_seq, S, st));
     GRAM_TRY(layer_rest_forward(m, mod, s.off[l], s.acts[l], s.d, s.d_ff, s.attn_only, x, s.acts[l].ctx, T, st, &x, &xb));
   }
-  if (n_full < s.n_layers) GRAM_TRY(layer_attention_forward(m, mod, s, n_full, xb, n_seq, S, st));
+  if (n_full < s.n_layers && top_attention) GRAM_TRY(layer_attention_forward(m, mod, s, n_full, xb, n_seq, S, st));
   *out = x;
   *out_b = xb;
   return GRAM_OK;
@@ -485,14 +489,14 @@ gram_status layer_attention_backward(Model* m, Module& mod, Stack& s, int l, con
 // On entry s.curf holds the gradient with respect to the stack's output (fp32; for a stack of
 // attention-only layers s.dzb holds its operand-typed copy as well).  With top_attention_only the rows part of
 // the top layer has been done by the caller: s.dctx and s.othf hold what layer_rest_backward leaves, and the
-// top layer runs its attention part only.  On return *d_in points at the fp32 gradient with respect to the input
+// top layer runs its attention part only.  n_layers >= 0: layers 0 .. n_layers-1 only.  On return *d_in points at the fp32 gradient with respect to the input
 // stream.
 gram_status stack_backward(Model* m, Module& mod, Stack& s, const void* x_in_b, int64_t n_seq, int S, cudaStream_t st,
-                           float** d_in, bool top_attention_only = false) {
+                           float** d_in, bool top_attention_only = false, int n_layers = -1) {
   const int64_t T = s.packed_rows ? s.packed_rows : n_seq * S;
   float* cur = s.curf;
   float* oth = s.othf;
-  for (int l = s.n_layers - 1; l >= 0; --l) {
+  for (int l = (n_layers < 0 ? s.n_layers : n_layers) - 1; l >= 0; --l) {
     const void* xb_l = (l == 0) ? x_in_b : s.acts[l - 1].out;
     if (!(top_attention_only && l == s.n_layers - 1))
       GRAM_TRY(layer_rest_backward(m, mod, s.off[l], s, s.acts[l], T, &cur, &oth, st));
@@ -503,6 +507,37 @@ gram_status stack_backward(Model* m, Module& mod, Stack& s, const void* x_in_b, 
 }
 
 gram_status read_i32(Model* m, const int32_t* d_ptr, int32_t* out, cudaStream_t st);
+
+// the last layer's input at row 0 of every item, operand-typed [mb, d]: behind the queries in the tail's qkv buffer
+void* cls_input_rows(Model* m) { return at(m, m->tail.acts[0].qkv, (size_t)m->mb * m->cfg.d); }
+
+// Attention part of the last layer, backward, with one query row per item.  The tail's dctx holds the gradient of the
+// attention output, *oth the residual part of the gradient of the layer's input at row 0; *cur is free.  Leaves the gradient
+// with respect to the layer's input (all T rows) in enc.curf.
+gram_status cls_attention_backward(Model* m, int32_t n, int64_t T, const int32_t* seq_len, const int32_t* seq_off, float** cur,
+                                   float** oth, cudaStream_t st) {
+  const gram_config& c = m->cfg;
+  gram_ctx* ctx = m->ctx;
+  Stack& s = m->enc;
+  Stack& tl = m->tail;
+  const int last = c.n_layers - 1, d = c.d;
+  const LayerOff& o = s.off[last];
+  const size_t kv_off = (size_t)d * d;                       // rows d .. 3d of wqkv: keys, values
+  const void* xb = last == 0 ? m->x0 : s.acts[last - 1].out;
+  int64_t part_rows = 0;
+  GRAM_TRY(attention_cls_backward(ctx, tl.acts[0].qkv, s.acts[last].qkv, tl.dctx, tl.dqkv, s.dqkv, s.cpart,
+                                  (int64_t)(s.cpart_elems / ((size_t)3 * d)), &part_rows, n, c.l_t, d, c.n_heads, seq_len, seq_off, st));
+  GRAM_TRY(colsum_from_partials(ctx, s.cpart, part_rows, 3 * d, m->ce.g + o.bqkv, m->red, st));
+  GRAM_TRY(mm_dw(m, s.dqkv, xb, m->ce.g + o.wqkv + kv_off, T, 2 * d, d, st, "dw_kv"));
+  GRAM_TRY(mm_dw(m, tl.dqkv, cls_input_rows(m), m->ce.g + o.wqkv, n, d, d, st, "dw_q"));
+  GemmEpilogue e;
+  e.tag = "dx_kv";
+  GRAM_TRY(mm_dx(m, s.dqkv, W(m, m->ce, o.wqkv + kv_off), s.curf, true, T, 2 * d, d, e, st));       // dkv Wkv, every row
+  e.res = *oth;
+  e.tag = "dx_q";
+  GRAM_TRY(mm_dx(m, tl.dqkv, W(m, m->ce, o.wqkv), *cur, true, n, d, d, e, st));                      // dq Wq + dz1, row 0
+  return add_strided_rows(ctx, *cur, n, c.l_t, seq_off, d, s.curf, st);
+}
 
 // encoder forward over n items (d_items, or first_item.. when null): H_out [n, d] fp32
 gram_status encoder_forward_chunk(Model* m, const int32_t* d_item_tokens, const int32_t* d_items, int32_t first_item,
@@ -564,10 +599,26 @@ gram_status encoder_forward_chunk(Model* m, const int32_t* d_item_tokens, const 
     const int last = c.n_layers - 1;
     StreamRef x;
     const void* xb = nullptr;
-    GRAM_TRY(stack_forward(m, m->ce, m->enc, x0, m->x0, n, c.l_t, st, &x, &xb, last));
+    GRAM_TRY(stack_forward(m, m->ce, m->enc, x0, m->x0, n, c.l_t, st, &x, &xb, last, !m->cls_query));
     // row 0 of every item: the attention output and the last layer's input stream (values and LayerNorm statistics)
     LayerActs& ta = m->tail.acts[0];
-    GRAM_TRY(take_strided_rows(ctx, m->enc.acts[last].ctx, n, c.l_t, seq_off, c.d, (int)m->esz, ta.ctx, st));
+    if (m->cls_query) {
+      const LayerOff& o = m->enc.off[last];
+      void* kv = m->enc.acts[last].qkv;
+      void* q = ta.qkv;
+      void* xr = cls_input_rows(m);
+      GemmEpilogue e;
+      e.bias = m->ce.w + o.bqkv + c.d;
+      e.tag = "fwd_kv";
+      GRAM_TRY(mm_fwd(m, xb, W(m, m->ce, o.wqkv + (size_t)c.d * c.d), kv, false, T, 2 * c.d, c.d, e, st));
+      GRAM_TRY(take_strided_rows(ctx, xb, n, c.l_t, seq_off, c.d, (int)m->esz, xr, st));
+      e.bias = m->ce.w + o.bqkv;
+      e.tag = "fwd_q";
+      GRAM_TRY(mm_fwd(m, xr, W(m, m->ce, o.wqkv), q, false, n, c.d, c.d, e, st));
+      GRAM_TRY(attention_cls_forward(ctx, q, kv, ta.ctx, n, c.l_t, c.d, c.n_heads, seq_len, seq_off, st));
+    } else {
+      GRAM_TRY(take_strided_rows(ctx, m->enc.acts[last].ctx, n, c.l_t, seq_off, c.d, (int)m->esz, ta.ctx, st));
+    }
     GRAM_TRY(take_strided_rows(ctx, x.z, n, c.l_t, seq_off, c.d, 4, m->tail_z, st));
     GRAM_TRY(take_strided_rows(ctx, x.mean, n, c.l_t, seq_off, 1, 4, m->tail_mean, st));
     GRAM_TRY(take_strided_rows(ctx, x.rstd, n, c.l_t, seq_off, 1, 4, m->tail_rstd, st));
@@ -609,12 +660,17 @@ gram_status encoder_backward_chunk(Model* m, const float* G, int32_t n, cudaStre
     float* cur = tl.curf;
     float* oth = tl.othf;
     GRAM_TRY(layer_rest_backward(m, m->ce, tl.off[0], tl, tl.acts[0], n, &cur, &oth, st));
+    if (m->cls_query) {
+      GRAM_TRY(cls_attention_backward(m, n, T, seq_len, seq_off, &cur, &oth, st));
+      GRAM_TRY(stack_backward(m, m->ce, m->enc, m->x0, n, c.l_t, st, &dx0, false, c.n_layers - 1));
+    } else {
     // back into whole sequences: every other row of the two gradients is zero
     GRAM_CUDA(ctx, cudaMemsetAsync(m->enc.dctx, 0, (size_t)T * c.d * m->esz, st));
     GRAM_CUDA(ctx, cudaMemsetAsync(m->enc.othf, 0, (size_t)T * c.d * 4, st));
     GRAM_TRY(put_strided_rows(ctx, tl.dctx, n, c.l_t, seq_off, c.d, (int)m->esz, m->enc.dctx, st));
     GRAM_TRY(put_strided_rows(ctx, oth, n, c.l_t, seq_off, c.d, 4, m->enc.othf, st));
     GRAM_TRY(stack_backward(m, m->ce, m->enc, m->x0, n, c.l_t, st, &dx0, true));
+    }
   }
   float* dz0 = (dx0 == m->enc.curf) ? m->enc.othf : m->enc.curf;
   GRAM_TRY(layernorm_backward(ctx, m->dtype, dx0, m->z0, m->mean0, m->rstd0, m->ce.w + m->o_elng, dz0, nullptr,
@@ -865,6 +921,7 @@ gram_status model_create(gram_ctx* ctx, const gram_config* cfg, Model** out) {
   m->enc.cap = (int64_t)m->mb * c.l_t;
   m->tk.cap = c.task == GRAM_TASK_NR ? (int64_t)c.B_max * (c.L - c.n_cand) : P;
   m->cls_tail = c.n_layers > 0 && c.pooling == GRAM_POOL_CLS && c.l_t > 1;
+  m->cls_query = m->cls_tail && c.dtype == GRAM_BF16 && attention_cls_supported(c.l_t, c.d, c.n_heads);
   if (m->cls_tail) {
     m->tail.d = c.d; m->tail.heads = c.n_heads; m->tail.d_ff = c.d_ff; m->tail.n_layers = 1;
     m->tail.attn_only = 0; m->tail.causal = 0;
