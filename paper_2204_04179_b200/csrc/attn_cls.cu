@@ -66,6 +66,7 @@ constexpr int ROWS = 4;                          // row groups a warp keeps in f
 __global__ void __launch_bounds__(512) attn_cls_fwd_kernel(const bf16* __restrict__ q, const bf16* __restrict__ kv,
                                                           bf16* __restrict__ ctx, int n, int l_t, int d, float c,
                                                           const int32_t* __restrict__ seq_len, const int32_t* __restrict__ seq_off) {
+  if (!chain_begin()) return;
   extern __shared__ float scores[];              // [heads][l_t]
   const int h = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane >> 3, p = lane & 7;
   float* sc = scores + h * l_t;
@@ -128,6 +129,7 @@ __global__ void __launch_bounds__(512) attn_cls_bwd_kernel(const bf16* __restric
                                                           bf16* __restrict__ dkv, float* __restrict__ part, int n, int l_t, int d,
                                                           float c, float scale, const int32_t* __restrict__ seq_len,
                                                           const int32_t* __restrict__ seq_off) {
+  if (!chain_begin()) return;
   extern __shared__ float scores[];              // [heads][2][l_t]: scores, later probabilities; dP, later dS
   const int h = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane >> 3, p = lane & 7;
   float* sc = scores + h * 2 * l_t;
@@ -226,6 +228,7 @@ __global__ void __launch_bounds__(512) attn_cls_bwd_kernel(const bf16* __restric
 // X[row(u), :] += r[u, :], fp32, row(u) = rows[u] or u * stride
 __global__ void add_strided_rows_kernel(const float4* __restrict__ r, float4* __restrict__ X, int64_t n, int64_t stride, int words,
                                         const int32_t* __restrict__ rows) {
+  if (!chain_begin()) return;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * words) return;
   const int64_t u = i / words;
@@ -251,7 +254,7 @@ gram_status attention_cls_forward(gram_ctx* ctx, const void* q, const void* kv, 
   const size_t smem = cls_smem(n_heads, l_t, 1);
   ProfScope prof(ctx, GRAM_K_ATTENTION, 4.0 * (double)n * l_t * d, 1, st, "attn_cls_fwd");
   if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(attn_cls_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  attn_cls_fwd_kernel<<<n, n_heads * 32, smem, st>>>((const bf16*)q, (const bf16*)kv, (bf16*)out, n, l_t, d,
+  launch_chain(attn_cls_fwd_kernel, n, n_heads * 32, smem, st, (const bf16*)q, (const bf16*)kv, (bf16*)out, n, l_t, d,
                                                      1.4426950408889634f / sqrtf((float)DH), seq_len, seq_off);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -268,7 +271,7 @@ gram_status attention_cls_backward(gram_ctx* ctx, const void* q, const void* kv,
   const size_t smem = cls_smem(n_heads, l_t, 2);
   ProfScope prof(ctx, GRAM_K_ATTENTION, 10.0 * (double)n * l_t * d, 1, st, "attn_cls_bwd");
   if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(attn_cls_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  attn_cls_bwd_kernel<<<(unsigned)blocks, n_heads * 32, smem, st>>>((const bf16*)q, (const bf16*)kv, (const bf16*)dctx, (bf16*)dq,
+  launch_chain(attn_cls_bwd_kernel, (unsigned)blocks, n_heads * 32, smem, st, (const bf16*)q, (const bf16*)kv, (const bf16*)dctx, (bf16*)dq,
                                                                     (bf16*)dkv, part, n, l_t, d, 1.4426950408889634f / sqrtf((float)DH),
                                                                     1.f / sqrtf((float)DH), seq_len, seq_off);
   GRAM_LAUNCH_CHECK(ctx);
@@ -281,7 +284,7 @@ gram_status add_strided_rows(gram_ctx* ctx, const float* r, int64_t n, int64_t s
   if (n == 0) return GRAM_OK;
   if (d % 4) return gram_set_error(ctx, "row sum: d must be a multiple of 4"), GRAM_ERR_ARG;
   ProfScope prof(ctx, GRAM_K_OTHER, 12.0 * (double)n * d, 1, st);
-  add_strided_rows_kernel<<<(unsigned)ceil_div64(n * (d / 4), 256), 256, 0, st>>>((const float4*)r, (float4*)X, n, stride, d / 4, rows);
+  launch_chain(add_strided_rows_kernel, (unsigned)ceil_div64(n * (d / 4), 256), 256, 0, st, (const float4*)r, (float4*)X, n, stride, d / 4, rows);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }

@@ -99,6 +99,7 @@ __device__ __forceinline__ void flash_colsum(const bf16* stage, int rows, int la
 
 template <bool CAUSAL>
 __global__ void __launch_bounds__(FL_MAX_WARPS * 32, 2) attn_flash_fwd_kernel(FlashArgs a) {
+  if (!chain_begin()) return;
   extern __shared__ __align__(16) uint8_t smem_raw[];
   bf16* Ks = reinterpret_cast<bf16*>(smem_raw);
   bf16* Vs = Ks + a.rows_cap * LD;
@@ -209,6 +210,7 @@ __global__ void __launch_bounds__(FL_MAX_WARPS * 32, 2) attn_flash_fwd_kernel(Fl
 // NWMAX: most warps a launch of this form has.  5: two blocks per SM; 12: one.
 template <bool CAUSAL, int NWMAX>
 __global__ void __launch_bounds__(NWMAX * 32, NWMAX <= 5 ? 2 : 1) attn_flash_bwd_kernel(FlashArgs a) {
+  if (!chain_begin()) return;
   extern __shared__ __align__(16) uint8_t smem_raw[];
   bf16* Qs = reinterpret_cast<bf16*>(smem_raw);
   bf16* Ks = Qs + a.rows_cap * LD;
@@ -455,7 +457,7 @@ gram_status attention_forward_flash(gram_ctx* ctx, const void* qkv, void* out, f
   const size_t smem = flash_fwd_smem(a.rows_cap, warps);
   auto kern = causal ? attn_flash_fwd_kernel<true> : attn_flash_fwd_kernel<false>;
   GRAM_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)flash_fwd_smem(256, FL_MAX_WARPS)));
-  kern<<<(unsigned)(n_seq * n_heads), warps * 32, smem, st>>>(a);
+  launch_chain(kern, (unsigned)(n_seq * n_heads), warps * 32, smem, st, a);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -480,7 +482,7 @@ gram_status attention_backward_flash(gram_ctx* ctx, const void* qkv, const void*
   auto kern = two ? (causal ? attn_flash_bwd_kernel<true, 5> : attn_flash_bwd_kernel<false, 5>)
                   : (causal ? attn_flash_bwd_kernel<true, FL_BWD_WARPS> : attn_flash_bwd_kernel<false, FL_BWD_WARPS>);
   GRAM_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)flash_bwd_smem(192, FL_BWD_WARPS)));
-  kern<<<(unsigned)(n_seq * n_heads), warps * 32, smem, st>>>(a);
+  launch_chain(kern, (unsigned)(n_seq * n_heads), warps * 32, smem, st, a);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }

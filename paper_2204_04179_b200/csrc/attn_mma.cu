@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(NW * 32) attn_fwd_mma_kernel(const bf16* __res
                                                            const int32_t* __restrict__ seq_len,
                                                            const int32_t* __restrict__ seq_off,
                                                            const int32_t* __restrict__ seq_list) {
+  if (!chain_begin()) return;
   constexpr int LD = DH + 8;
   extern __shared__ __align__(16) uint8_t smem_raw[];
   bf16* Qs = reinterpret_cast<bf16*>(smem_raw);
@@ -189,6 +190,7 @@ __global__ void __launch_bounds__(NW * 32) attn_bwd_mma_kernel(const bf16* __res
                                                            const int32_t* __restrict__ seq_len,
                                                            const int32_t* __restrict__ seq_off,
                                                            const int32_t* __restrict__ seq_list) {
+  if (!chain_begin()) return;
   constexpr int LD = DH + 8, LP = SP + 8;
   extern __shared__ __align__(16) uint8_t smem_raw[];
   bf16* Qs = reinterpret_cast<bf16*>(smem_raw);   // [SP][DH+8]
@@ -336,7 +338,7 @@ gram_status launch_fwd(gram_ctx* ctx, const bf16* qkv, bf16* out, int64_t n_seq,
   constexpr int NW = SP >= 96 ? 8 : 4;                // one 16-row query tile per warp up to 128 rows
   auto kern = causal ? attn_fwd_mma_kernel<SP, DH, NW, true> : attn_fwd_mma_kernel<SP, DH, NW, false>;
   if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<(unsigned)(n_seq * n_heads), NW * 32, smem, st>>>(qkv, out, S, d, n_heads, causal, 1.f / sqrtf((float)DH), seq_len, seq_off, seq_list);
+  launch_chain(kern, (unsigned)(n_seq * n_heads), NW * 32, smem, st, qkv, out, S, d, n_heads, causal, 1.f / sqrtf((float)DH), seq_len, seq_off, seq_list);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -349,7 +351,7 @@ gram_status launch_bwd(gram_ctx* ctx, const bf16* qkv, const bf16* dctx, bf16* d
   constexpr int NW = SP >= 96 ? 8 : 4;
   auto kern = causal ? attn_bwd_mma_kernel<SP, DH, NW, true> : attn_bwd_mma_kernel<SP, DH, NW, false>;
   if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<(unsigned)(n_seq * n_heads), NW * 32, smem, st>>>(qkv, dctx, dqkv, colpart, S, d, n_heads, causal, 1.f / sqrtf((float)DH), seq_len, seq_off, seq_list);
+  launch_chain(kern, (unsigned)(n_seq * n_heads), NW * 32, smem, st, qkv, dctx, dqkv, colpart, S, d, n_heads, causal, 1.f / sqrtf((float)DH), seq_len, seq_off, seq_list);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }

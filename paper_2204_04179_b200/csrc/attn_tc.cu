@@ -366,6 +366,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 1) attn_tc_fwd_kernel(const __gri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (!chain_begin()) return;              // barriers and tensor memory are set up before the wait
   bool failed = false;
 
   if (warp == 0) {
@@ -674,6 +675,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 1) attn_tc_bwd_kernel(const __gri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (!chain_begin()) return;              // barriers and tensor memory are set up before the wait
   bool failed = false;
   const bool want_kv = b.mode != 2, want_q = b.mode != 1;
 
@@ -956,6 +958,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 1) attn_tc_bwd_kernel(const __gri
 // long sequences (one warp per row, two columns per lane and head)
 __global__ void __launch_bounds__(256) attn_delta_kernel(const bf16* __restrict__ dO, const bf16* __restrict__ O, float* __restrict__ delta,
                                                          int64_t T, int d, int H) {
+  if (!chain_begin()) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t row = warp; row < T; row += nw) {
@@ -1029,9 +1032,9 @@ gram_status attention_forward_tc(gram_ctx* ctx, const void* qkv, void* out, floa
     attr_set = true;
   }
   const int grid = (int)(a.n_items < kNumSMs ? a.n_items : kNumSMs);
-  if (!a.long_mode && a.slot <= 32) attn_tc_fwd_kernel<32><<<grid, ATT_THREADS, FWD_SMEM, st>>>(tm, a);
-  else if (!a.long_mode && a.slot == 64) attn_tc_fwd_kernel<64><<<grid, ATT_THREADS, FWD_SMEM, st>>>(tm, a);
-  else attn_tc_fwd_kernel<128><<<grid, ATT_THREADS, FWD_SMEM, st>>>(tm, a);
+  if (!a.long_mode && a.slot <= 32) launch_chain(attn_tc_fwd_kernel<32>, grid, ATT_THREADS, FWD_SMEM, st, tm, a);
+  else if (!a.long_mode && a.slot == 64) launch_chain(attn_tc_fwd_kernel<64>, grid, ATT_THREADS, FWD_SMEM, st, tm, a);
+  else launch_chain(attn_tc_fwd_kernel<128>, grid, ATT_THREADS, FWD_SMEM, st, tm, a);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1074,20 +1077,20 @@ gram_status attention_backward_tc(gram_ctx* ctx, const void* qkv, const void* dc
   const int grid = (int)(a.n_items < kNumSMs ? a.n_items : kNumSMs);
   if (!a.long_mode) {
     b.mode = 0;
-    if (a.slot <= 32) attn_tc_bwd_kernel<32><<<grid, ATT_THREADS, BWD_SMEM, st>>>(tq, td, b);
-    else if (a.slot == 64) attn_tc_bwd_kernel<64><<<grid, ATT_THREADS, BWD_SMEM, st>>>(tq, td, b);
-    else attn_tc_bwd_kernel<128><<<grid, ATT_THREADS, BWD_SMEM, st>>>(tq, td, b);
+    if (a.slot <= 32) launch_chain(attn_tc_bwd_kernel<32>, grid, ATT_THREADS, BWD_SMEM, st, tq, td, b);
+    else if (a.slot == 64) launch_chain(attn_tc_bwd_kernel<64>, grid, ATT_THREADS, BWD_SMEM, st, tq, td, b);
+    else launch_chain(attn_tc_bwd_kernel<128>, grid, ATT_THREADS, BWD_SMEM, st, tq, td, b);
   } else {
     if (!delta || !octx) return gram_set_error(ctx, "attention backward: long sequences need the forward output and a scratch row vector"), GRAM_ERR_ARG;
     int blocks = (int)((rows + 7) / 8);
     if (blocks > kNumSMs * 8) blocks = kNumSMs * 8;
-    attn_delta_kernel<<<blocks, 256, 0, st>>>((const bf16*)dctx, (const bf16*)octx, delta, rows, d, n_heads);
+    launch_chain(attn_delta_kernel, blocks, 256, 0, st, (const bf16*)dctx, (const bf16*)octx, delta, rows, d, n_heads);
     if (colpart)      // tiles a sequence does not have leave their rows unwritten
       GRAM_CUDA(ctx, cudaMemsetAsync(colpart + colpart_row0 * 3 * (int64_t)d, 0, (size_t)(n_seq * a.nq_max) * 3 * d * sizeof(float), st));
     b.mode = 1;
-    attn_tc_bwd_kernel<128><<<grid, ATT_THREADS, BWD_SMEM, st>>>(tq, td, b);
+    launch_chain(attn_tc_bwd_kernel<128>, grid, ATT_THREADS, BWD_SMEM, st, tq, td, b);
     b.mode = 2;
-    attn_tc_bwd_kernel<128><<<grid, ATT_THREADS, BWD_SMEM, st>>>(tq, td, b);
+    launch_chain(attn_tc_bwd_kernel<128>, grid, ATT_THREADS, BWD_SMEM, st, tq, td, b);
   }
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;

@@ -144,6 +144,7 @@ constexpr int TOT_COPIES = 8;
 __global__ void __launch_bounds__(TOT_THREADS) digit_totals_kernel(const int32_t* __restrict__ keys, int64_t P, int passes,
                                                                    int32_t n_items, uint32_t* __restrict__ totals,
                                                                    int32_t* status) {
+  if (!chain_begin()) return;
   __shared__ uint32_t sh[kMaxPasses * RADIX * TOT_COPIES];
   for (int i = threadIdx.x; i < passes * RADIX * TOT_COPIES; i += TOT_THREADS) sh[i] = 0;
   __syncthreads();
@@ -216,6 +217,7 @@ __global__ void __launch_bounds__(RS_THREADS, 2) radix_pass_kernel(const int32_t
                                                                    const uint32_t* __restrict__ totals, uint32_t* lb,
                                                                    int32_t* ticket, int32_t* __restrict__ keys_out,
                                                                    int32_t* __restrict__ vals_out, int32_t* status) {
+  if (!chain_begin()) return;
   extern __shared__ __align__(16) unsigned char pass_smem_raw[];
   PassSmem& s = *reinterpret_cast<PassSmem*>(pass_smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -361,6 +363,7 @@ __global__ void __launch_bounds__(RLE_THREADS) rle_kernel(const int32_t* __restr
                                                           uint32_t* lb, int32_t* ticket, int32_t* __restrict__ unique,
                                                           int32_t* __restrict__ seg_off, int32_t* __restrict__ rank_table,
                                                           int32_t* __restrict__ n_unique, int32_t* status) {
+  if (!chain_begin()) return;
   __shared__ int32_t sw[33];
   __shared__ int32_t s_tile, s_excl, s_abort;
   if (threadIdx.x == 0) {
@@ -416,6 +419,7 @@ __global__ void __launch_bounds__(RLE_THREADS) rle_kernel(const int32_t* __restr
 
 __global__ void __launch_bounds__(256) inverse_kernel(const int32_t* __restrict__ ids, int64_t P, int32_t n_items,
                                                       const int32_t* __restrict__ rank_table, int32_t* __restrict__ inverse) {
+  if (!chain_begin()) return;
   constexpr int UNROLL = 4;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x * UNROLL;
   for (int64_t p0 = (int64_t)blockIdx.x * blockDim.x * UNROLL + threadIdx.x; p0 < P; p0 += stride) {
@@ -475,6 +479,7 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
                                                                   int32_t* __restrict__ inverse, int32_t* __restrict__ perm,
                                                                   int32_t* __restrict__ seg_off, int32_t* __restrict__ n_unique,
                                                                   int32_t* status) {
+  if (!chain_begin()) return;
   constexpr int TILE = CD_THREADS * ROUNDS;
   extern __shared__ __align__(16) unsigned char cd_smem_raw[];
   ClusterSmem<ROUNDS>& s = *reinterpret_cast<ClusterSmem<ROUNDS>*>(cd_smem_raw);
@@ -620,6 +625,7 @@ ClusterDedup cluster_dedup_form(int i) {
 }
 
 __global__ void dedup_empty_kernel(int32_t* seg_off, int32_t* n_unique) {
+  if (!chain_begin()) return;
   seg_off[0] = 0;
   *n_unique = 0;
 }
@@ -692,7 +698,7 @@ gram_status dedup_launch(gram_ctx* ctx, IndexWorkspace* ws, const int32_t* d_ids
   if (P > (int64_t)LB_MASK)
     return gram_set_error(ctx, "gram_dedup: P=%lld is above the limit of 2^30 - 1 positions per call", (long long)P), GRAM_ERR_UNSUPPORTED;
   if (P == 0) {
-    dedup_empty_kernel<<<1, 1, 0, st>>>(d_seg_off, d_n_unique);
+    launch_chain(dedup_empty_kernel, 1, 1, 0, st, d_seg_off, d_n_unique);
     GRAM_LAUNCH_CHECK(ctx);
     return GRAM_OK;
   }
@@ -714,13 +720,14 @@ gram_status dedup_launch(gram_ctx* ctx, IndexWorkspace* ws, const int32_t* d_ids
     cfg.blockDim = dim3(CD_THREADS);
     cfg.dynamicSmemBytes = f.smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)blocks;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1] = chain_attribute();
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     GRAM_CUDA(ctx, cudaLaunchKernelEx(&cfg, f.fn, d_ids, (int32_t)P, n_items, key_bits, d_unique, d_inverse, d_perm, d_seg_off, d_n_unique,
                                       gram_status_word(ctx)));
     return GRAM_OK;
@@ -736,7 +743,7 @@ gram_status dedup_launch(gram_ctx* ctx, IndexWorkspace* ws, const int32_t* d_ids
   uint32_t* lb = ctl + CTL_WORDS;
   int tb = (int)ceil_div64(P, (int64_t)TOT_THREADS * 16);
   if (tb > kNumSMs * 4) tb = kNumSMs * 4;
-  digit_totals_kernel<<<tb, TOT_THREADS, 0, st>>>(d_ids, P, passes, n_items, totals, status);
+  launch_chain(digit_totals_kernel, tb, TOT_THREADS, 0, st, d_ids, P, passes, n_items, totals, status);
 
   const int32_t* kin = d_ids;
   const int32_t* vin = nullptr;
@@ -746,7 +753,7 @@ gram_status dedup_launch(gram_ctx* ctx, IndexWorkspace* ws, const int32_t* d_ids
     int32_t* kout = kbuf[p & 1];
     int32_t* vout = (p == passes - 1) ? d_perm : vbuf[p & 1];
     const int pass_bits = (key_bits - 8 * p) < 8 ? (key_bits - 8 * p < 1 ? 1 : key_bits - 8 * p) : 8;   // digit bits that can be set
-    radix_pass_fn(pass_bits)<<<ntiles, RS_THREADS, sizeof(PassSmem), st>>>(kin, vin, P, 8 * p, n_items, p == 0, totals + p * RADIX,
+    launch_chain(radix_pass_fn(pass_bits), ntiles, RS_THREADS, sizeof(PassSmem), st, kin, vin, P, 8 * p, n_items, p == 0, totals + p * RADIX,
                                                                           lb + (size_t)p * ntiles * RADIX,
                                                                           reinterpret_cast<int32_t*>(ctl) + CTL_TICKET + p,
                                                                           kout, vout, status);
@@ -755,12 +762,12 @@ gram_status dedup_launch(gram_ctx* ctx, IndexWorkspace* ws, const int32_t* d_ids
   }
   GRAM_LAUNCH_CHECK(ctx);
   const int32_t cap = (int32_t)(P < (int64_t)n_items ? P : (int64_t)n_items);
-  rle_kernel<<<rtiles, RLE_THREADS, 0, st>>>(kin, P, rtiles, cap, n_items, lb + (size_t)passes * ntiles * RADIX,
+  launch_chain(rle_kernel, rtiles, RLE_THREADS, 0, st, kin, P, rtiles, cap, n_items, lb + (size_t)passes * ntiles * RADIX,
                                              reinterpret_cast<int32_t*>(ctl) + CTL_RLE_TICKET, d_unique, d_seg_off,
                                              ws->rank_table, d_n_unique, status);
   int ib = (int)ceil_div64(P, 256 * 4);
   if (ib > kNumSMs * 16) ib = kNumSMs * 16;
-  inverse_kernel<<<ib, 256, 0, st>>>(d_ids, P, n_items, ws->rank_table, d_inverse);
+  launch_chain(inverse_kernel, ib, 256, 0, st, d_ids, P, n_items, ws->rank_table, d_inverse);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }

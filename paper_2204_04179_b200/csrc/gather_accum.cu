@@ -13,6 +13,7 @@ template <int ROWS>   // rows a warp keeps in flight
 __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restrict__ src, int64_t n_src_rows,
                                                           const int32_t* __restrict__ index, int64_t P, int nvec,
                                                           uint4* __restrict__ dst, int32_t* status) {
+  if (!chain_begin()) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -43,6 +44,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restric
 template <typename T>
 __global__ void gather_scalar_kernel(const T* __restrict__ src, int64_t n_src_rows, const int32_t* __restrict__ index,
                                      int64_t P, int d, T* __restrict__ dst, int32_t* status) {
+  if (!chain_begin()) return;
   const int64_t n = P * d;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
     int64_t p = k / d;
@@ -62,6 +64,7 @@ template <int ROWS>
 __global__ void __launch_bounds__(256) gather_widen_kernel(const uint4* __restrict__ src, int64_t n_src_rows,
                                                            const int32_t* __restrict__ index, int64_t P, int nvec,
                                                            float4* __restrict__ dst, int32_t* status) {
+  if (!chain_begin()) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -102,6 +105,7 @@ __global__ void __launch_bounds__(256) gather_diff_kernel(const float* __restric
                                                           int64_t n_src_rows, const int32_t* __restrict__ index, int64_t n,
                                                           int d, const float* __restrict__ x, float* __restrict__ out,
                                                           int32_t* status) {
+  if (!chain_begin()) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -205,6 +209,7 @@ __global__ void __launch_bounds__(256) segsum_chunks_kernel(const InT* __restric
                                                             int2* __restrict__ span, int32_t* status,
                                                             const int32_t* __restrict__ d_U,
                                                             const int32_t* __restrict__ gate) {
+  if (!chain_begin()) return;
   if (d_U) U = *d_U;            // the number of items may live on the device
   if (U <= 0) return;
   if (gate && *gate) return;    // an earlier kernel of the step reported an error: leave the accumulated rows alone
@@ -284,6 +289,7 @@ __global__ void __launch_bounds__(256) segsum_fixup_kernel(const int32_t* __rest
                                                            float* __restrict__ out, const float* __restrict__ partial,
                                                            const int2* __restrict__ span, const int32_t* __restrict__ d_U,
                                                            const int32_t* __restrict__ gate) {
+  if (!chain_begin()) return;
   __shared__ float4 red[8][VPL][32];
   if (d_U) U = *d_U;
   if (U <= 0) return;
@@ -348,6 +354,7 @@ __global__ void __launch_bounds__(256) segsum_fixup_kernel(const int32_t* __rest
 __global__ void touched_mark_kernel(const int32_t* __restrict__ unique, int32_t U, const int32_t* __restrict__ d_U,
                                     int32_t n_items, uint32_t* __restrict__ bits, int32_t* __restrict__ count,
                                     int32_t* status, int gated) {
+  if (!chain_begin()) return;
   if (d_U) U = *d_U;
   if (gated && *status) return;
   for (int32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < U; u += gridDim.x * blockDim.x) {
@@ -365,6 +372,7 @@ __global__ void touched_mark_kernel(const int32_t* __restrict__ unique, int32_t 
 // ascending list of set bits, one block
 __global__ void __launch_bounds__(1024) touched_list_kernel(const uint32_t* __restrict__ bits, int32_t n_items,
                                                             int32_t* __restrict__ list, int32_t* __restrict__ count) {
+  if (!chain_begin()) return;
   __shared__ int32_t sw[33];
   const int nwords = (n_items + 31) >> 5;
   const int per = (nwords + 1023) / 1024;
@@ -427,16 +435,16 @@ gram_status gather_launch(gram_ctx* ctx, const void* d_src, int64_t n_src_rows, 
     int blocks = (int)ceil_div64(warps, 8);
     const int cap = kNumSMs * 8;
     if (blocks > cap) blocks = cap;
-    gather_rows_kernel<ROWS><<<blocks, 256, 0, st>>>((const uint4*)d_src, n_src_rows, d_index, P, nvec, (uint4*)d_E,
+    launch_chain(gather_rows_kernel<ROWS>, blocks, 256, 0, st, (const uint4*)d_src, n_src_rows, d_index, P, nvec, (uint4*)d_E,
                                                      status);
   } else {
     int64_t n = P * d;
     int blocks = (int)ceil_div64(n, 256);
     if (blocks > kNumSMs * 16) blocks = kNumSMs * 16;
     if (elem_bytes == 4)
-      gather_scalar_kernel<float><<<blocks, 256, 0, st>>>((const float*)d_src, n_src_rows, d_index, P, d, (float*)d_E, status);
+      launch_chain(gather_scalar_kernel<float>, blocks, 256, 0, st, (const float*)d_src, n_src_rows, d_index, P, d, (float*)d_E, status);
     else
-      gather_scalar_kernel<bf16><<<blocks, 256, 0, st>>>((const bf16*)d_src, n_src_rows, d_index, P, d, (bf16*)d_E, status);
+      launch_chain(gather_scalar_kernel<bf16>, blocks, 256, 0, st, (const bf16*)d_src, n_src_rows, d_index, P, d, (bf16*)d_E, status);
   }
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -452,7 +460,7 @@ gram_status gather_widen_launch(gram_ctx* ctx, const void* d_src_bf16, int64_t n
   constexpr int ROWS = 4;
   int blocks = (int)ceil_div64(ceil_div64(P, ROWS), 8);
   if (blocks > kNumSMs * 8) blocks = kNumSMs * 8;
-  gather_widen_kernel<ROWS><<<blocks, 256, 0, st>>>((const uint4*)d_src_bf16, n_src_rows, d_index, P, d / 8, (float4*)d_E,
+  launch_chain(gather_widen_kernel<ROWS>, blocks, 256, 0, st, (const uint4*)d_src_bf16, n_src_rows, d_index, P, d / 8, (float4*)d_E,
                                                     gram_status_word(ctx));
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -466,7 +474,7 @@ gram_status gather_diff_launch(gram_ctx* ctx, const float* d_a, const float* d_b
   ProfScope prof(ctx, GRAM_K_GATHER, (double)n * d * 4.0 * (d_x ? 4.0 : 3.0) + 4.0 * (double)n, 1, st);
   int blocks = (int)ceil_div64(n, 8);
   if (blocks > kNumSMs * 8) blocks = kNumSMs * 8;
-  gather_diff_kernel<<<blocks, 256, 0, st>>>(d_a, d_b, n_src_rows, d_index, n, d, d_x, d_out, gram_status_word(ctx));
+  launch_chain(gather_diff_kernel, blocks, 256, 0, st, d_a, d_b, n_src_rows, d_index, n, d, d_x, d_out, gram_status_word(ctx));
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -478,10 +486,10 @@ static void segsum_run(const void* d_in, const int32_t* d_perm, const int32_t* d
   const int nslabs = ceil_div(d, VPL * 128);
   const int64_t warps = (int64_t)nchunks * nslabs;
   const int blocks = (int)ceil_div64(warps, 8);
-  segsum_chunks_kernel<InT, VPL, 8><<<blocks, 256, 0, st>>>((const InT*)d_in, d_perm, d_seg_off, P, U, d, R, nchunks, nslabs,
+  launch_chain(segsum_chunks_kernel<InT, VPL, 8>, blocks, 256, 0, st, (const InT*)d_in, d_perm, d_seg_off, P, U, d, R, nchunks, nslabs,
                                                             d_rows, add, d_out, partial, span, status, d_U, gate);
   if (nchunks > 1)
-    segsum_fixup_kernel<VPL><<<(unsigned)warps, 256, 0, st>>>(d_seg_off, P, U, d, R, nchunks, nslabs, d_rows, add, d_out, partial, span, d_U, gate);
+    launch_chain(segsum_fixup_kernel<VPL>, (unsigned)warps, 256, 0, st, d_seg_off, P, U, d, R, nchunks, nslabs, d_rows, add, d_out, partial, span, d_U, gate);
 }
 
 gram_status accumulate_launch(gram_ctx* ctx, IndexWorkspace* ws, const void* d_in, int in_bf16, const int32_t* d_perm,
@@ -521,7 +529,7 @@ gram_status touched_mark_launch(gram_ctx* ctx, const int32_t* d_unique, int32_t 
   ProfScope prof(ctx, GRAM_K_OTHER, 8.0 * U, 1, st);
   int blocks = ceil_div(U, 256);
   if (blocks > kNumSMs * 4) blocks = kNumSMs * 4;
-  touched_mark_kernel<<<blocks, 256, 0, st>>>(d_unique, U, d_U, n_items, d_bits, d_count, gram_status_word(ctx), gated);
+  launch_chain(touched_mark_kernel, blocks, 256, 0, st, d_unique, U, d_U, n_items, d_bits, d_count, gram_status_word(ctx), gated);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -530,7 +538,7 @@ gram_status touched_list_launch(gram_ctx* ctx, const uint32_t* d_bits, int32_t n
                                 int32_t* d_count, cudaStream_t st) {
   if (n_items <= 0 || !d_bits || !d_list || !d_count) return gram_set_error(ctx, "gram_touched_list: bad argument"), GRAM_ERR_ARG;
   ProfScope prof(ctx, GRAM_K_OTHER, (double)n_items / 8.0, 1, st);
-  touched_list_kernel<<<1, 1024, 0, st>>>(d_bits, n_items, d_list, d_count);
+  launch_chain(touched_list_kernel, 1, 1024, 0, st, d_bits, n_items, d_list, d_count);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }

@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
                                                                         const float* __restrict__ B, int64_t ldb, float* C,
                                                                         int64_t ldc, int64_t M, int N, int64_t K,
                                                                         int64_t k_per_split, int vec_a, int vec_b, EpiDev e) {
+  if (!chain_begin()) return;
   using Cfg = F32Cfg<TILE>;
   constexpr int LD = Cfg::LD, NV = Cfg::NV, T = Cfg::THREADS;
   __shared__ __align__(16) float sm[2][2][SK * LD];        // [buffer][operand]; later the block's partial tile
@@ -333,13 +334,14 @@ cudaError_t launch_f32(const float* A, int64_t lda, const float* B, int64_t ldb,
   cfg.gridDim = dim3((unsigned)ceil_div(N, TILE), (unsigned)ceil_div64(M, TILE), (unsigned)splits);
   cfg.blockDim = dim3(F32Cfg<TILE>::THREADS);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 1;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = (unsigned)splits;
+  attr[1] = chain_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   const int vec_a = (lda % 4 == 0) && ((uintptr_t)A % 16 == 0), vec_b = (ldb % 4 == 0) && ((uintptr_t)B % 16 == 0);
   return cudaLaunchKernelEx(&cfg, kern, A, lda, B, ldb, C, ldc, M, N, K, k_per_split, vec_a, vec_b, e);
 }
@@ -688,6 +690,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gemm_tc_kernel(const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (!chain_begin()) return;              // barriers and tensor memory are set up before the wait
 
   const int64_t total = (int64_t)a.n_tiles_m * a.n_tiles_n * a.splits;
   bool failed = false;
@@ -1165,6 +1168,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
   cluster_sync_all();                           // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (!chain_begin()) return;              // barriers and tensor memory are set up before the wait
 
   const int64_t total = (int64_t)a.n_tiles_m * a.n_tiles_n * a.splits;
   const int64_t cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
@@ -1329,6 +1333,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
 template <typename CT>
 __global__ void splitk_reduce_kernel(const float* __restrict__ part, int splits, int64_t split_stride, int64_t M, int N,
                                      CT* __restrict__ C, int64_t ldc, EpiDev e) {
+  if (!chain_begin()) return;
   const int64_t n_el = M * N;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_el; i += (int64_t)gridDim.x * blockDim.x) {
     float acc = 0.f;
@@ -1349,7 +1354,7 @@ cudaError_t launch_tc(const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  kern<<<grid, TC_THREADS, TcCfg<BN>::SMEM_BYTES, st>>>(ma, mb, args);
+  launch_chain(kern, grid, TC_THREADS, TcCfg<BN>::SMEM_BYTES, st, ma, mb, args);
   return cudaGetLastError();
 }
 
@@ -1378,13 +1383,14 @@ cudaError_t launch_tc2(const CUtensorMap& ma, const CUtensorMap& mb, const TcArg
   cfg.blockDim = dim3(Tc2::THREADS);
   cfg.dynamicSmemBytes = Tc2::SMEM_BYTES;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1] = chain_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, ma, mb, mc ? *mc : ma, mp ? *mp : (mc ? *mc : ma), args);
 }
 template <typename CT>
@@ -1514,8 +1520,8 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     if (err != cudaSuccess) return gram_set_error(ctx, "gemm launch failed: %s", cudaGetErrorString(err)), GRAM_ERR_CUDA;
     int rb = (int)ceil_div64(M * N, 256);
     if (rb > kNumSMs * 8) rb = kNumSMs * 8;
-    if (c_f32) splitk_reduce_kernel<float><<<rb, 256, 0, st>>>(ws->splitk, splits, (int64_t)M * N, M, N, (float*)C, ldc, e);
-    else splitk_reduce_kernel<bf16><<<rb, 256, 0, st>>>(ws->splitk, splits, (int64_t)M * N, M, N, (bf16*)C, ldc, e);
+    if (c_f32) launch_chain(splitk_reduce_kernel<float>, rb, 256, 0, st, ws->splitk, splits, (int64_t)M * N, M, N, (float*)C, ldc, e);
+    else launch_chain(splitk_reduce_kernel<bf16>, rb, 256, 0, st, ws->splitk, splits, (int64_t)M * N, M, N, (bf16*)C, ldc, e);
     GRAM_LAUNCH_CHECK(ctx);
     return GRAM_OK;
   }

@@ -33,6 +33,42 @@ void gram_set_error(gram_ctx* ctx, const char* fmt, ...);
 
 #define GRAM_LAUNCH_CHECK(ctx) GRAM_CUDA(ctx, cudaGetLastError())
 
+// ---------------------------------------------------------------------------
+// Launches.  A step is a chain of some hundred short kernels on one stream; with ordinary launches each waits for the one
+// before it to drain, flush and retire and then pays its own start.  Every kernel here is launched with programmatic stream
+// serialisation instead: its blocks are placed as soon as all blocks of the kernel before have ended, they set up what needs
+// no memory of others, and chain_begin() then waits until that kernel's writes are visible.  (Ordinary launches -> this ->
+// with an early trigger that lets blocks in while the kernel before still runs: the check's step 686 -> 532 -> 554 us, the
+// task module at 25 600 rows 3.49 -> 3.40 -> 3.39 ms, encodings of 2048 ragged texts 2.86 -> 2.85 -> 2.92 ms: the blocks that
+// wait on the SMs cost the large kernels more than they save, so there is no early trigger.)
+// A kernel launched with launch_chain (or chain_attribute) must call chain_begin() before it touches global memory.
+// It returns true; that the compiler cannot know it keeps loads that it takes to be of constant memory behind the wait.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ bool chain_begin() {
+  uint32_t n;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, %%nctaid.x;" : "=r"(n)::"memory");
+  return n != 0u;
+}
+static inline cudaLaunchAttribute chain_attribute() {
+  cudaLaunchAttribute a = {};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
+// errors are left for the caller's GRAM_LAUNCH_CHECK
+template <typename... P, typename... A>
+static inline void launch_chain(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = chain_attribute();
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 static inline int64_t ceil_div64(int64_t a, int64_t b) { return (a + b - 1) / b; }
 static inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 

@@ -36,6 +36,7 @@ __global__ void embed_fwd_kernel(const int32_t* __restrict__ item_tokens, const 
                                  const float* __restrict__ tok_emb, const float* __restrict__ pos_emb,
                                  float* __restrict__ z0, int32_t* __restrict__ tok_ids,
                                  const int32_t* __restrict__ seq_len, const int32_t* __restrict__ seq_off, int32_t* status) {
+  if (!chain_begin()) return;
   const int lane = threadIdx.x & 31;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -75,6 +76,7 @@ __global__ void __launch_bounds__(256) ln_fwd_kernel(const float* __restrict__ z
                                                      const float* __restrict__ b, T* __restrict__ y,
                                                      float* __restrict__ mean, float* __restrict__ rstd, int64_t rows,
                                                      int d) {
+  if (!chain_begin()) return;
   const int lane = threadIdx.x & 31;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -127,6 +129,7 @@ __global__ void __launch_bounds__(32 * LNB_WARPS, 1) ln_bwd_kernel(const float* 
                                                                   const float* __restrict__ g, float* __restrict__ dz,
                                                                   T* __restrict__ dz_b, float* __restrict__ part, int64_t rows,
                                                                   int d, int32_t* status) {
+  if (!chain_begin()) return;
   // [3][d]: dgamma, dbeta and the column sums of dz of this block; [d]: gamma; then the warps' rings
   extern __shared__ __align__(16) float sacc[];
   __shared__ __align__(8) uint64_t bars[LNB_WARPS * LNB_STAGES];
@@ -240,6 +243,7 @@ __global__ void __launch_bounds__(32 * LNB_WARPS, 1) ln_bwd_kernel(const float* 
 __global__ void __launch_bounds__(256) reduce_partials_kernel(const float* __restrict__ part, int nblocks, int64_t stride,
                                                               int n, float* __restrict__ out, float* __restrict__ out2,
                                                               float* __restrict__ out3, float scale) {
+  if (!chain_begin()) return;
   __shared__ float sa[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
@@ -268,6 +272,7 @@ __global__ void __launch_bounds__(128) attn_fwd_kernel(const T* __restrict__ qkv
                                                        int n_heads, int causal, float scale,
                                                        const int32_t* __restrict__ seq_len,
                                                        const int32_t* __restrict__ seq_off) {
+  if (!chain_begin()) return;
   extern __shared__ float sm[];
   const int dh = d / n_heads, ld = dh + 1;
   int64_t row0 = (int64_t)(blockIdx.x / n_heads) * S;
@@ -338,6 +343,7 @@ __global__ void __launch_bounds__(128) attn_bwd_kernel(const T* __restrict__ qkv
                                                        T* __restrict__ dqkv, int S, int d, int n_heads, int causal,
                                                        float scale, const int32_t* __restrict__ seq_len,
                                                        const int32_t* __restrict__ seq_off) {
+  if (!chain_begin()) return;
   extern __shared__ float sm[];
   int64_t row0 = (int64_t)(blockIdx.x / n_heads) * S;
   if (seq_off) {
@@ -450,6 +456,7 @@ __global__ void __launch_bounds__(128) attn_bwd_kernel(const T* __restrict__ qkv
 template <typename T>
 __global__ void __launch_bounds__(256) colsum_kernel(const T* __restrict__ X, int64_t rows, int N, int64_t rows_per_block,
                                                      float* __restrict__ part) {
+  if (!chain_begin()) return;
   __shared__ float2 sw[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = blockIdx.x * 64 + 2 * lane;
@@ -478,6 +485,7 @@ __global__ void __launch_bounds__(256) colsum_kernel(const T* __restrict__ X, in
 __global__ void periodic_rowsum_kernel(const float* __restrict__ X, int64_t n_groups, int64_t per, int period, int d,
                                        float* __restrict__ out, float* __restrict__ part,
                                        const int32_t* __restrict__ seq_len, const int32_t* __restrict__ seq_off) {
+  if (!chain_begin()) return;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (int64_t)period * d) return;
   const int s = (int)(i / d), c = (int)(i - (int64_t)s * d);
@@ -501,6 +509,7 @@ __device__ __forceinline__ float stream_at(const StreamRef& x, int64_t row, int 
 }
 __global__ void pool_fwd_kernel(StreamRef x, float* __restrict__ H, int64_t n, int l_t, int d, int pooling,
                                 const int32_t* __restrict__ seq_len, const int32_t* __restrict__ seq_off) {
+  if (!chain_begin()) return;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * d) return;
   const int64_t u = i / d;
@@ -517,6 +526,7 @@ __global__ void pool_fwd_kernel(StreamRef x, float* __restrict__ H, int64_t n, i
 }
 __global__ void pool_bwd_kernel(const float* __restrict__ G, float* __restrict__ dx, int64_t n, int l_t, int d, int pooling,
                                 const int32_t* __restrict__ seq_len, const int32_t* __restrict__ seq_off) {
+  if (!chain_begin()) return;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * l_t * d) return;
   const int64_t t = i / d;
@@ -543,6 +553,7 @@ __global__ void __launch_bounds__(128) pool_additive_fwd_kernel(StreamRef x, con
                                                                 float* __restrict__ H, float* __restrict__ alpha, int l_t, int d,
                                                                 int pa, const int32_t* __restrict__ seq_len,
                                                                 const int32_t* __restrict__ seq_off) {
+  if (!chain_begin()) return;
   __shared__ float sa[128];
   const int64_t u = blockIdx.x;
   const int64_t row0 = seq_off ? (int64_t)seq_off[u] : u * l_t;
@@ -583,6 +594,7 @@ __global__ void __launch_bounds__(128) pool_additive_bwd_kernel(StreamRef x, con
                                                                 float* __restrict__ qpart, int l_t, int d, int pa,
                                                                 const int32_t* __restrict__ seq_len,
                                                                 const int32_t* __restrict__ seq_off) {
+  if (!chain_begin()) return;
   __shared__ float sda[128], sal[128];
   __shared__ float sdelta;
   const int64_t u = blockIdx.x;
@@ -629,6 +641,7 @@ __global__ void kt_input_fwd_kernel(const ET* __restrict__ E, const int32_t* __r
                                     const float* __restrict__ pos, const float* __restrict__ resp,
                                     const int32_t* __restrict__ labels, float* __restrict__ x, T* __restrict__ x_b, int64_t P,
                                     int L, int d, int32_t* status) {
+  if (!chain_begin()) return;
   const int64_t p = blockIdx.x;                  // one block per position
   const int n = (int)(p % L);
   int prev = (n == 0) ? 2 : labels[p - 1];
@@ -653,6 +666,7 @@ __global__ void kt_input_fwd_kernel(const ET* __restrict__ E, const int32_t* __r
 // one thread per column: dE = dx (when dE is not null); dpos[n, c] += sum_b; dresp[r, c] += sum over positions with prev == r
 __global__ void kt_input_bwd_kernel(const float* __restrict__ dx, const int32_t* __restrict__ labels, float* __restrict__ dE,
                                     float* __restrict__ dpos, float* __restrict__ dresp, int B, int L, int d) {
+  if (!chain_begin()) return;
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = blockIdx.y;
   if (c >= d) return;
@@ -692,6 +706,7 @@ __global__ void __launch_bounds__(256) kt_head_kernel(StreamRef y, const float* 
                                                       float* __restrict__ dy, T* __restrict__ dy_b,
                                                       float* __restrict__ part, int64_t P, int d, int64_t pstride,
                                                       const int32_t* __restrict__ n_real) {
+  if (!chain_begin()) return;
   extern __shared__ float sacc[];            // [warps][d + 2]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
   const float b0 = bias[0], invP = 1.f / (float)max(*n_real, 1);   // the mean runs over the real predictions
@@ -754,6 +769,7 @@ __global__ void __launch_bounds__(256) kt_head_kernel(StreamRef y, const float* 
 __global__ void kt_head_reduce_kernel(const float* __restrict__ part, int nblocks, int64_t pstride, int d,
                                       const int32_t* __restrict__ n_real, float* __restrict__ dw, float* __restrict__ db,
                                       float* __restrict__ loss) {
+  if (!chain_begin()) return;
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= d + 2) return;
   const float invP = 1.f / (float)max(*n_real, 1);
@@ -766,6 +782,7 @@ __global__ void kt_head_reduce_kernel(const float* __restrict__ part, int nblock
 
 // positions with a label >= 0 (integer adds: the count does not depend on their order); *n_real must start at zero
 __global__ void count_real_kernel(const int32_t* __restrict__ labels, int64_t P, int32_t* __restrict__ n_real) {
+  if (!chain_begin()) return;
   int32_t c = 0;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x) c += labels[p] >= 0;
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
@@ -779,6 +796,7 @@ __global__ void __launch_bounds__(256) nr_user_kernel(const float* __restrict__ 
                                                       const float* __restrict__ qa, float* __restrict__ dE,
                                                       T* __restrict__ dpre, float* __restrict__ part, int L, int n_cand,
                                                       int d, int d_a, float invB, const int32_t* __restrict__ labels) {
+  if (!chain_begin()) return;
   extern __shared__ float sm[];
   const int n_hist = L - n_cand;
   float* a = sm;                 // [L] scores / alpha
@@ -876,6 +894,7 @@ __global__ void __launch_bounds__(256) nr_user_kernel(const float* __restrict__ 
 
 __global__ void nr_reduce_kernel(const float* __restrict__ part, int B, int d_a, float invB, float* __restrict__ dqa,
                                  float* __restrict__ loss) {
+  if (!chain_begin()) return;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k > d_a) return;
   float a = 0.f;
@@ -891,6 +910,7 @@ __global__ void nr_reduce_kernel(const float* __restrict__ part, int B, int d_a,
 __global__ void __launch_bounds__(1024) nr_layout_kernel(const int32_t* __restrict__ labels, int B, int L, int n_hist,
                                                          int32_t* __restrict__ seq_len, int32_t* __restrict__ seq_off,
                                                          int32_t* __restrict__ rows, int32_t* __restrict__ pos2row) {
+  if (!chain_begin()) return;
   __shared__ int32_t total;
   if (threadIdx.x == 0) total = 0;
   __syncthreads();
@@ -933,6 +953,7 @@ __global__ void __launch_bounds__(1024) nr_layout_kernel(const int32_t* __restri
 template <typename T>
 __global__ void nr_pack_kernel(const float* __restrict__ src, const int32_t* __restrict__ rows, int64_t n, int d,
                                float* __restrict__ out, T* __restrict__ out_b) {
+  if (!chain_begin()) return;
   const int64_t r = blockIdx.x;
   const int32_t p = rows[r];
   for (int c = threadIdx.x; c < d; c += blockDim.x) {
@@ -945,6 +966,7 @@ __global__ void nr_pack_kernel(const float* __restrict__ src, const int32_t* __r
 // out[p, :] = y(pos2row[p], :) where the position has a packed row, else other[p, :]; y is a view of the residual stream
 __global__ void nr_select_kernel(StreamRef y, const int32_t* __restrict__ pos2row, const float* __restrict__ other, int64_t P, int d,
                                  float* __restrict__ out) {
+  if (!chain_begin()) return;
   const int64_t p = blockIdx.x;
   const int32_t r = pos2row[p];
   if (r < 0) {
@@ -961,15 +983,18 @@ __global__ void nr_select_kernel(StreamRef y, const int32_t* __restrict__ pos2ro
 
 // ---------------------------------------------------------------------------- element-wise
 __global__ void f32_to_bf16_kernel(const float* __restrict__ in, bf16* __restrict__ out, size_t n) {
+  if (!chain_begin()) return;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     out[i] = __float2bfloat16(in[i]);
 }
 __global__ void bf16_to_f32_kernel(const bf16* __restrict__ in, float* __restrict__ out, size_t n) {
+  if (!chain_begin()) return;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     out[i] = __bfloat162float(in[i]);
 }
 // gate (may be null): a device word; nothing is updated when it is not zero (an error met earlier in the step)
 __global__ void sgd_kernel(float* __restrict__ w, const float* __restrict__ g, float lr, size_t n, const int32_t* __restrict__ gate) {
+  if (!chain_begin()) return;
   if (gate && *gate) return;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     w[i] -= lr * g[i];
@@ -977,6 +1002,7 @@ __global__ void sgd_kernel(float* __restrict__ w, const float* __restrict__ g, f
 template <typename T>
 __global__ void scatter_rows_kernel(const float* __restrict__ src, const int32_t* __restrict__ index, int64_t n, int d,
                                     int64_t n_dst_rows, T* __restrict__ dst, int32_t* status) {
+  if (!chain_begin()) return;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * d) return;
   const int64_t u = i / d;
@@ -991,6 +1017,7 @@ __global__ void scatter_rows_kernel(const float* __restrict__ src, const int32_t
 __global__ void strided_rows_kernel(const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n, int64_t in_stride,
                                     int64_t out_stride, int words, const int32_t* __restrict__ in_rows,
                                     const int32_t* __restrict__ out_rows) {
+  if (!chain_begin()) return;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * words) return;
   const int64_t r = i / words;
@@ -1006,6 +1033,7 @@ __global__ void __launch_bounds__(1024) seq_layout_kernel(const int32_t* __restr
                                                           int32_t* __restrict__ seq_len, int32_t* __restrict__ seq_off,
                                                           int32_t* __restrict__ group_list, int32_t* __restrict__ info,
                                                           int32_t* status) {
+  if (!chain_begin()) return;
   __shared__ int32_t sw[33];
   __shared__ int32_t carry_s;
   if (threadIdx.x == 0) carry_s = 0;
@@ -1121,7 +1149,7 @@ gram_status embed_forward(gram_ctx* ctx, const int32_t* item_tokens, const int32
   if (n_tok == 0) return GRAM_OK;
   const int blocks = grid_for(n_tok * 32, 256, kNumSMs * 8);
   ProfScope prof(ctx, GRAM_K_EMBED_POOL, 8.0 * (double)n_tok * d, 1, st);
-  embed_fwd_kernel<<<blocks, 256, 0, st>>>(item_tokens, items, first_item, n_tok, n_items_total, l_t, vocab, d, tok_emb,
+  launch_chain(embed_fwd_kernel, blocks, 256, 0, st, item_tokens, items, first_item, n_tok, n_items_total, l_t, vocab, d, tok_emb,
                                            pos_emb, z0, tok_ids, seq_len, seq_off, gram_status_word(ctx));
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -1133,7 +1161,7 @@ gram_status layernorm_forward(gram_ctx* ctx, int dtype, const float* z, const fl
   if (d > 1024 || (d & 3)) return gram_set_error(ctx, "LayerNorm: d must be a multiple of 4 and at most 1024"), GRAM_ERR_UNSUPPORTED;
   const int blocks = grid_for(rows * 32, 256, kNumSMs * 8);
   ProfScope prof(ctx, GRAM_K_LAYERNORM, (double)rows * d * (4.0 + (dtype == GRAM_BF16 ? 2.0 : 4.0)), 1, st, "ln_fwd");
-  DISPATCH_T(dtype, DISPATCH_NQ(d, ln_fwd_kernel<T, NQ><<<blocks, 256, 0, st>>>(z, gamma, beta, (T*)y, mean, rstd, rows, d)));
+  DISPATCH_T(dtype, DISPATCH_NQ(d, launch_chain(ln_fwd_kernel<T, NQ>, blocks, 256, 0, st, z, gamma, beta, (T*)y, mean, rstd, rows, d)));
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1149,9 +1177,9 @@ gram_status layernorm_backward(gram_ctx* ctx, int dtype, const float* dy, const 
   ProfScope prof(ctx, GRAM_K_LAYERNORM, (double)rows * d * (12.0 + (dz_b ? (dtype == GRAM_BF16 ? 2.0 : 4.0) : 0.0)), 2, st, "ln_bwd");
   DISPATCH_T(dtype, DISPATCH_NQ(d, {
     GRAM_TRY(set_smem(ctx, ln_bwd_kernel<T, NQ>, smem));
-    ln_bwd_kernel<T, NQ><<<blocks, 32 * LNB_WARPS, smem, st>>>(dy, z, mean, rstd, gamma, dz, (T*)dz_b, scratch, rows, d, gram_status_word(ctx));
+    launch_chain(ln_bwd_kernel<T, NQ>, blocks, 32 * LNB_WARPS, smem, st, dy, z, mean, rstd, gamma, dz, (T*)dz_b, scratch, rows, d, gram_status_word(ctx));
   }));
-  reduce_partials_kernel<<<dim3(ceil_div(d, 32), dcol ? 3 : 2), 256, 0, st>>>(scratch, blocks, (int64_t)3 * d, d, dgamma, dbeta, dcol, 1.f);
+  launch_chain(reduce_partials_kernel, dim3(ceil_div(d, 32), dcol ? 3 : 2), 256, 0, st, scratch, blocks, (int64_t)3 * d, d, dgamma, dbeta, dcol, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1199,7 +1227,7 @@ gram_status attention_forward(gram_ctx* ctx, int dtype, const void* qkv, void* o
   }
   DISPATCH_T(dtype, {
     GRAM_TRY(set_smem(ctx, attn_fwd_kernel<T>, smem));
-    attn_fwd_kernel<T><<<(unsigned)(n_seq * n_heads), 128, smem, st>>>((const T*)qkv, (T*)out, S, d, n_heads, causal, scale, seq_len, seq_off);
+    launch_chain(attn_fwd_kernel<T>, (unsigned)(n_seq * n_heads), 128, smem, st, (const T*)qkv, (T*)out, S, d, n_heads, causal, scale, seq_len, seq_off);
   });
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -1263,7 +1291,7 @@ gram_status attention_backward(gram_ctx* ctx, int dtype, const void* qkv, const 
   }
   DISPATCH_T(dtype, {
     GRAM_TRY(set_smem(ctx, attn_bwd_kernel<T>, smem));
-    attn_bwd_kernel<T><<<(unsigned)(n_seq * n_heads), 128, smem, st>>>((const T*)qkv, (const T*)dctx, (T*)dqkv, S, d, n_heads, causal, scale, seq_len, seq_off);
+    launch_chain(attn_bwd_kernel<T>, (unsigned)(n_seq * n_heads), 128, smem, st, (const T*)qkv, (const T*)dctx, (T*)dqkv, S, d, n_heads, causal, scale, seq_len, seq_off);
   });
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -1273,6 +1301,7 @@ gram_status attention_backward(gram_ctx* ctx, int dtype, const void* qkv, const 
 // eighth of them and adding their sums in ascending order
 __global__ void __launch_bounds__(256) fold_partials_kernel(const float* __restrict__ part, int64_t nrows, int n,
                                                             float* __restrict__ fold) {
+  if (!chain_begin()) return;
   __shared__ float sa[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
@@ -1298,8 +1327,8 @@ gram_status colsum_from_partials(gram_ctx* ctx, const float* part, int64_t nrows
   int G = 32;                                             // rows of the folded matrix (fixed: the order of additions depends on it)
   if ((size_t)G * N * sizeof(float) > kRedScratchBytes) G = (int)(kRedScratchBytes / ((size_t)N * sizeof(float)));
   if (G < 1) return gram_set_error(ctx, "column sums: N too large for the reduction scratch"), GRAM_ERR_UNSUPPORTED;
-  fold_partials_kernel<<<dim3((unsigned)ceil_div(N, 32), (unsigned)G), 256, 0, st>>>(part, nrows, N, scratch);
-  reduce_partials_kernel<<<ceil_div(N, 32), 256, 0, st>>>(scratch, G, (int64_t)N, N, out, nullptr, nullptr, 1.f);
+  launch_chain(fold_partials_kernel, dim3((unsigned)ceil_div(N, 32), (unsigned)G), 256, 0, st, part, nrows, N, scratch);
+  launch_chain(reduce_partials_kernel, ceil_div(N, 32), 256, 0, st, scratch, G, (int64_t)N, N, out, nullptr, nullptr, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1316,8 +1345,8 @@ gram_status colsum_accumulate(gram_ctx* ctx, int dtype, const void* X, int64_t r
   rb = ceil_div64(rows, per);
   dim3 grid((unsigned)ceil_div(N, 64), (unsigned)rb);
   ProfScope prof(ctx, GRAM_K_COLSUM, (double)rows * N * (dtype == GRAM_BF16 ? 2.0 : 4.0), 2, st, "colsum");
-  DISPATCH_T(dtype, colsum_kernel<T><<<grid, 256, 0, st>>>((const T*)X, rows, N, per, scratch));
-  reduce_partials_kernel<<<ceil_div(N, 32), 256, 0, st>>>(scratch, (int)rb, (int64_t)N, N, out, nullptr, nullptr, 1.f);
+  DISPATCH_T(dtype, launch_chain(colsum_kernel<T>, grid, 256, 0, st, (const T*)X, rows, N, per, scratch));
+  launch_chain(reduce_partials_kernel, ceil_div(N, 32), 256, 0, st, scratch, (int)rb, (int64_t)N, N, out, nullptr, nullptr, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1335,8 +1364,8 @@ gram_status periodic_rowsum_accumulate(gram_ctx* ctx, const float* X, int64_t n_
   const int64_t per = ceil_div64(n_groups, chunks);
   ProfScope prof(ctx, GRAM_K_EMBED_POOL, 4.0 * (double)n_groups * period * d, chunks > 1 ? 2 : 1, st);
   dim3 grid((unsigned)ceil_div64(n, 128), (unsigned)chunks);
-  periodic_rowsum_kernel<<<grid, 128, 0, st>>>(X, n_groups, per, period, d, out, chunks > 1 ? scratch : nullptr, seq_len, seq_off);
-  if (chunks > 1) reduce_partials_kernel<<<ceil_div((int)n, 32), 256, 0, st>>>(scratch, (int)chunks, n, (int)n, out, nullptr, nullptr, 1.f);
+  launch_chain(periodic_rowsum_kernel, grid, 128, 0, st, X, n_groups, per, period, d, out, chunks > 1 ? scratch : nullptr, seq_len, seq_off);
+  if (chunks > 1) launch_chain(reduce_partials_kernel, ceil_div((int)n, 32), 256, 0, st, scratch, (int)chunks, n, (int)n, out, nullptr, nullptr, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1345,7 +1374,7 @@ gram_status pool_forward(gram_ctx* ctx, const StreamRef& x, float* H, int64_t n,
                          const int32_t* seq_len, const int32_t* seq_off, cudaStream_t st) {
   if (n == 0) return GRAM_OK;
   ProfScope prof(ctx, GRAM_K_EMBED_POOL, 4.0 * (double)n * d * (pooling == GRAM_POOL_CLS ? 2 : l_t + 1), 1, st);
-  pool_fwd_kernel<<<(unsigned)ceil_div64(n * d, 256), 256, 0, st>>>(x, H, n, l_t, d, pooling, seq_len, seq_off);
+  launch_chain(pool_fwd_kernel, (unsigned)ceil_div64(n * d, 256), 256, 0, st, x, H, n, l_t, d, pooling, seq_len, seq_off);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1354,7 +1383,7 @@ gram_status pool_backward(gram_ctx* ctx, const float* G, float* dx, int64_t n, i
                           const int32_t* seq_len, const int32_t* seq_off, cudaStream_t st) {
   if (n == 0) return GRAM_OK;
   ProfScope prof(ctx, GRAM_K_EMBED_POOL, 4.0 * (double)n * d * (l_t + 1), 1, st);
-  pool_bwd_kernel<<<(unsigned)ceil_div64(n * l_t * d, 256), 256, 0, st>>>(G, dx, n, l_t, d, pooling, seq_len, seq_off);
+  launch_chain(pool_bwd_kernel, (unsigned)ceil_div64(n * l_t * d, 256), 256, 0, st, G, dx, n, l_t, d, pooling, seq_len, seq_off);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1368,9 +1397,9 @@ gram_status kt_input_forward(gram_ctx* ctx, int dtype, const void* E, int e_bf16
   const int threads = d >= 256 ? 256 : 64;
   int32_t* sw = gram_status_word(ctx);
   if (e_bf16) {
-    DISPATCH_T(dtype, kt_input_fwd_kernel<T, bf16><<<(unsigned)P, threads, 0, st>>>((const bf16*)E, index, n_rows, pos, resp, labels, x, (T*)x_b, P, L, d, sw));
+    DISPATCH_T(dtype, launch_chain(kt_input_fwd_kernel<T, bf16>, (unsigned)P, threads, 0, st, (const bf16*)E, index, n_rows, pos, resp, labels, x, (T*)x_b, P, L, d, sw));
   } else {
-    DISPATCH_T(dtype, kt_input_fwd_kernel<T, float><<<(unsigned)P, threads, 0, st>>>((const float*)E, index, n_rows, pos, resp, labels, x, (T*)x_b, P, L, d, sw));
+    DISPATCH_T(dtype, launch_chain(kt_input_fwd_kernel<T, float>, (unsigned)P, threads, 0, st, (const float*)E, index, n_rows, pos, resp, labels, x, (T*)x_b, P, L, d, sw));
   }
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -1387,9 +1416,9 @@ gram_status kt_head(gram_ctx* ctx, int dtype, const StreamRef& y, const float* w
   const size_t smem = (size_t)8 * (d + 2) * sizeof(float);
   ProfScope prof(ctx, GRAM_K_TASK_HEAD, 12.0 * (double)P * d, 3, st);
   GRAM_CUDA(ctx, cudaMemsetAsync(n_real, 0, sizeof(int32_t), st));
-  count_real_kernel<<<grid_for(P, 256, kNumSMs), 256, 0, st>>>(labels, P, n_real);
-  DISPATCH_T(dtype, kt_head_kernel<T><<<blocks, 256, smem, st>>>(y, w, b, labels, dy, (T*)dy_b, scratch, P, d, pstride, n_real));
-  kt_head_reduce_kernel<<<ceil_div(d + 2, 256), 256, 0, st>>>(scratch, blocks, pstride, d, n_real, dw, db, loss);
+  launch_chain(count_real_kernel, grid_for(P, 256, kNumSMs), 256, 0, st, labels, P, n_real);
+  DISPATCH_T(dtype, launch_chain(kt_head_kernel<T>, blocks, 256, smem, st, y, w, b, labels, dy, (T*)dy_b, scratch, P, d, pstride, n_real));
+  launch_chain(kt_head_reduce_kernel, ceil_div(d + 2, 256), 256, 0, st, scratch, blocks, pstride, d, n_real, dw, db, loss);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1401,8 +1430,8 @@ gram_status kt_input_backward(gram_ctx* ctx, const float* dx, const int32_t* lab
   if ((size_t)L * 3 * d * sizeof(float) > kRedScratchBytes) return gram_set_error(ctx, "kt task: L*d too large for the reduction scratch"), GRAM_ERR_UNSUPPORTED;
   dim3 grid((unsigned)ceil_div(d, 128), (unsigned)L);
   ProfScope prof(ctx, GRAM_K_TASK_HEAD, 8.0 * (double)B * L * d, 2, st);
-  kt_input_bwd_kernel<<<grid, 128, 0, st>>>(dx, labels, dE, dpos, scratch, B, L, d);
-  reduce_partials_kernel<<<ceil_div(3 * d, 32), 256, 0, st>>>(scratch, L, (int64_t)3 * d, 3 * d, dresp, nullptr, nullptr, 1.f);
+  launch_chain(kt_input_bwd_kernel, grid, 128, 0, st, dx, labels, dE, dpos, scratch, B, L, d);
+  launch_chain(reduce_partials_kernel, ceil_div(3 * d, 32), 256, 0, st, scratch, L, (int64_t)3 * d, 3 * d, dresp, nullptr, nullptr, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1416,9 +1445,9 @@ gram_status nr_user(gram_ctx* ctx, int dtype, const float* E, const void* pre, c
   ProfScope prof(ctx, GRAM_K_TASK_HEAD, (double)B * L * (8.0 * d + 4.0 * d_a), 2, st);
   DISPATCH_T(dtype, {
     GRAM_TRY(set_smem(ctx, nr_user_kernel<T>, smem));
-    nr_user_kernel<T><<<B, 256, smem, st>>>(E, (const T*)pre, qa, dE, (T*)dpre, scratch, L, n_cand, d, d_a, 1.f / (float)B, labels);
+    launch_chain(nr_user_kernel<T>, B, 256, smem, st, E, (const T*)pre, qa, dE, (T*)dpre, scratch, L, n_cand, d, d_a, 1.f / (float)B, labels);
   });
-  nr_reduce_kernel<<<ceil_div(d_a + 1, 256), 256, 0, st>>>(scratch, B, d_a, 1.f / (float)B, dqa, loss);
+  launch_chain(nr_reduce_kernel, ceil_div(d_a + 1, 256), 256, 0, st, scratch, B, d_a, 1.f / (float)B, dqa, loss);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1427,7 +1456,7 @@ gram_status nr_layout(gram_ctx* ctx, const int32_t* labels, int B, int L, int n_
                       int32_t* rows, int32_t* pos2row, cudaStream_t st) {
   if (B == 0) return GRAM_OK;
   ProfScope prof(ctx, GRAM_K_TASK_HEAD, 12.0 * (double)B * L, 1, st);
-  nr_layout_kernel<<<1, 1024, 0, st>>>(labels, B, L, n_hist, seq_len, seq_off, rows, pos2row);
+  launch_chain(nr_layout_kernel, 1, 1024, 0, st, labels, B, L, n_hist, seq_len, seq_off, rows, pos2row);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1435,7 +1464,7 @@ gram_status nr_pack(gram_ctx* ctx, int dtype, const float* src, const int32_t* r
                     cudaStream_t st) {
   if (n == 0) return GRAM_OK;
   ProfScope prof(ctx, GRAM_K_TASK_HEAD, (double)n * d * (8.0 + (out_b ? (dtype == GRAM_BF16 ? 2.0 : 4.0) : 0.0)), 1, st);
-  DISPATCH_T(dtype, nr_pack_kernel<T><<<(unsigned)n, d >= 256 ? 256 : 64, 0, st>>>(src, rows, n, d, out, (T*)out_b));
+  DISPATCH_T(dtype, launch_chain(nr_pack_kernel<T>, (unsigned)n, d >= 256 ? 256 : 64, 0, st, src, rows, n, d, out, (T*)out_b));
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1443,7 +1472,7 @@ gram_status nr_select(gram_ctx* ctx, const StreamRef& y, const int32_t* pos2row,
                       cudaStream_t st) {
   if (P == 0) return GRAM_OK;
   ProfScope prof(ctx, GRAM_K_TASK_HEAD, 8.0 * (double)P * d, 1, st);
-  nr_select_kernel<<<(unsigned)P, d >= 256 ? 256 : 64, 0, st>>>(y, pos2row, other, P, d, out);
+  launch_chain(nr_select_kernel, (unsigned)P, d >= 256 ? 256 : 64, 0, st, y, pos2row, other, P, d, out);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1451,7 +1480,7 @@ gram_status nr_select(gram_ctx* ctx, const StreamRef& y, const int32_t* pos2row,
 gram_status convert_f32_to_bf16(gram_ctx* ctx, const float* in, bf16* out, size_t n, cudaStream_t st) {
   if (n == 0) return GRAM_OK;
   ProfScope prof(ctx, GRAM_K_OTHER, 6.0 * (double)n, 1, st);
-  f32_to_bf16_kernel<<<grid_for((int64_t)n, 256, kNumSMs * 16), 256, 0, st>>>(in, out, n);
+  launch_chain(f32_to_bf16_kernel, grid_for((int64_t)n, 256, kNumSMs * 16), 256, 0, st, in, out, n);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1460,7 +1489,7 @@ gram_status convert_to_f32(gram_ctx* ctx, int dtype, const void* in, float* out,
   if (dtype == GRAM_F32) GRAM_CUDA(ctx, cudaMemcpyAsync(out, in, n * sizeof(float), cudaMemcpyDeviceToDevice, st));
   else {
     ProfScope prof(ctx, GRAM_K_OTHER, 6.0 * (double)n, 1, st);
-    bf16_to_f32_kernel<<<grid_for((int64_t)n, 256, kNumSMs * 16), 256, 0, st>>>((const bf16*)in, out, n);
+    launch_chain(bf16_to_f32_kernel, grid_for((int64_t)n, 256, kNumSMs * 16), 256, 0, st, (const bf16*)in, out, n);
   }
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -1471,6 +1500,7 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ w, const 
                                                    float* __restrict__ v, bf16* __restrict__ wb, size_t n, float rate,
                                                    float beta1, float beta2, float eps, float c1, float c2,
                                                    const int32_t* __restrict__ gate) {
+  if (!chain_begin()) return;
   if (gate && *gate) return;                    // an error met earlier in the step: no update
   const size_t n4 = n >> 2;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -1517,8 +1547,8 @@ gram_status adam_update(gram_ctx* ctx, float* w, const float* g, float* m, float
   const float c2 = (float)(1.0 / (1.0 - pow((double)beta2, (double)t)));
   ProfScope prof(ctx, GRAM_K_OPTIMIZER, (double)n * (28.0 + (wb ? 2.0 : 0.0)), 1, st, "adam");
   const int grid = grid_for((int64_t)((n + 3) / 4), 256, kNumSMs * 8);
-  if (wb) adam_kernel<true><<<grid, 256, 0, st>>>(w, g, m, v, (bf16*)wb, n, rate, beta1, beta2, eps, c1, c2, gate);
-  else adam_kernel<false><<<grid, 256, 0, st>>>(w, g, m, v, nullptr, n, rate, beta1, beta2, eps, c1, c2, gate);
+  if (wb) launch_chain(adam_kernel<true>, grid, 256, 0, st, w, g, m, v, (bf16*)wb, n, rate, beta1, beta2, eps, c1, c2, gate);
+  else launch_chain(adam_kernel<false>, grid, 256, 0, st, w, g, m, v, nullptr, n, rate, beta1, beta2, eps, c1, c2, gate);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1526,7 +1556,7 @@ gram_status adam_update(gram_ctx* ctx, float* w, const float* g, float* m, float
 gram_status sgd_update(gram_ctx* ctx, float* w, const float* g, float lr, size_t n, cudaStream_t st, const int32_t* gate) {
   if (n == 0 || lr == 0.f) return GRAM_OK;
   ProfScope prof(ctx, GRAM_K_OPTIMIZER, 12.0 * (double)n, 1, st, "sgd");
-  sgd_kernel<<<grid_for((int64_t)n, 256, kNumSMs * 16), 256, 0, st>>>(w, g, lr, n, gate);
+  launch_chain(sgd_kernel, grid_for((int64_t)n, 256, kNumSMs * 16), 256, 0, st, w, g, lr, n, gate);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1534,7 +1564,7 @@ gram_status scatter_rows(gram_ctx* ctx, int dtype, const float* src, const int32
                          int64_t n_dst_rows, void* dst, cudaStream_t st) {
   if (n == 0) return GRAM_OK;
   ProfScope prof(ctx, GRAM_K_OTHER, (double)n * d * (4.0 + (dtype == GRAM_BF16 ? 2.0 : 4.0)), 1, st);
-  DISPATCH_T(dtype, scatter_rows_kernel<T><<<(unsigned)ceil_div64(n * d, 256), 256, 0, st>>>(src, index, n, d, n_dst_rows, (T*)dst, gram_status_word(ctx)));
+  DISPATCH_T(dtype, launch_chain(scatter_rows_kernel<T>, (unsigned)ceil_div64(n * d, 256), 256, 0, st, src, index, n, d, n_dst_rows, (T*)dst, gram_status_word(ctx)));
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1545,7 +1575,7 @@ gram_status take_strided_rows(gram_ctx* ctx, const void* in, int64_t n, int64_t 
   if ((d * elem_bytes) % 4) return gram_set_error(ctx, "row copy: rows must be whole 32-bit words"), GRAM_ERR_ARG;
   const int words = d * elem_bytes / 4;
   ProfScope prof(ctx, GRAM_K_OTHER, 2.0 * (double)n * d * elem_bytes, 1, st);
-  strided_rows_kernel<<<(unsigned)ceil_div64(n * words, 256), 256, 0, st>>>((const uint32_t*)in, (uint32_t*)out, n,
+  launch_chain(strided_rows_kernel, (unsigned)ceil_div64(n * words, 256), 256, 0, st, (const uint32_t*)in, (uint32_t*)out, n,
                                                                           rows ? words : stride * words, words, words, rows,
                                                                           nullptr);
   GRAM_LAUNCH_CHECK(ctx);
@@ -1557,7 +1587,7 @@ gram_status put_strided_rows(gram_ctx* ctx, const void* in, int64_t n, int64_t s
   if ((d * elem_bytes) % 4) return gram_set_error(ctx, "row copy: rows must be whole 32-bit words"), GRAM_ERR_ARG;
   const int words = d * elem_bytes / 4;
   ProfScope prof(ctx, GRAM_K_OTHER, 2.0 * (double)n * d * elem_bytes, 1, st);
-  strided_rows_kernel<<<(unsigned)ceil_div64(n * words, 256), 256, 0, st>>>((const uint32_t*)in, (uint32_t*)out, n, words,
+  launch_chain(strided_rows_kernel, (unsigned)ceil_div64(n * words, 256), 256, 0, st, (const uint32_t*)in, (uint32_t*)out, n, words,
                                                                           rows ? words : stride * words, words, nullptr, rows);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -1568,7 +1598,7 @@ gram_status sequence_layout(gram_ctx* ctx, const int32_t* item_len, const int32_
                             int32_t* info, cudaStream_t st) {
   if (n <= 0) return GRAM_OK;
   ProfScope prof(ctx, GRAM_K_EMBED_POOL, 12.0 * (double)n, 1, st);
-  seq_layout_kernel<<<1, 1024, 0, st>>>(item_len, items, first_item, n, n_items_total, l_t, seq_len, seq_off, group_list, info,
+  launch_chain(seq_layout_kernel, 1, 1024, 0, st, item_len, items, first_item, n, n_items_total, l_t, seq_len, seq_off, group_list, info,
                                         gram_status_word(ctx));
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -1580,7 +1610,7 @@ gram_status pool_additive_forward(gram_ctx* ctx, int dtype, const StreamRef& x, 
   if (n == 0) return GRAM_OK;
   if (l_t > 128) return gram_set_error(ctx, "additive pooling: at most 128 tokens per item"), GRAM_ERR_UNSUPPORTED;
   ProfScope prof(ctx, GRAM_K_EMBED_POOL, 4.0 * (double)n * l_t * (d + pa), 1, st);
-  DISPATCH_T(dtype, pool_additive_fwd_kernel<T><<<(unsigned)n, 128, 0, st>>>(x, (const T*)pre, q, H, alpha, l_t, d, pa, seq_len, seq_off));
+  DISPATCH_T(dtype, launch_chain(pool_additive_fwd_kernel<T>, (unsigned)n, 128, 0, st, x, (const T*)pre, q, H, alpha, l_t, d, pa, seq_len, seq_off));
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -1592,9 +1622,9 @@ gram_status pool_additive_backward(gram_ctx* ctx, int dtype, const StreamRef& x,
   if ((size_t)n * pa * sizeof(float) > kRedScratchBytes)
     return gram_set_error(ctx, "additive pooling: %lld items x %d exceed the reduction scratch", (long long)n, pa), GRAM_ERR_WORKSPACE;
   ProfScope prof(ctx, GRAM_K_EMBED_POOL, 4.0 * (double)n * l_t * (2 * d + 2 * pa), 2, st);
-  DISPATCH_T(dtype, pool_additive_bwd_kernel<T><<<(unsigned)n, 128, 0, st>>>(x, (const T*)pre, q, alpha, G, dx, (T*)dpre, scratch, l_t, d,
+  DISPATCH_T(dtype, launch_chain(pool_additive_bwd_kernel<T>, (unsigned)n, 128, 0, st, x, (const T*)pre, q, alpha, G, dx, (T*)dpre, scratch, l_t, d,
                                                                             pa, seq_len, seq_off));
-  reduce_partials_kernel<<<ceil_div(pa, 32), 256, 0, st>>>(scratch, (int)n, pa, pa, dq, nullptr, nullptr, 1.f);
+  launch_chain(reduce_partials_kernel, ceil_div(pa, 32), 256, 0, st, scratch, (int)n, pa, pa, dq, nullptr, nullptr, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
