@@ -194,7 +194,7 @@ gram_status gram_encode_unique(gram_ctx* ctx, const int32_t* d_item_tokens, cons
 /* Failure detection: every wait of one thread block on another (the tile look-back of gram_dedup, the pipeline
  * barriers of the matrix products) has a poll limit, after which the kernel records GRAM_ERR_TIMEOUT in the context,
  * writes nothing more and returns, so that a stuck wait costs about a second instead of the device.  This call shows
- * it: it launches the dedup's run-length kernel with a predecessor tile that never runs.  It returns GRAM_OK once the
+ * it: it launches a sort pass of the dedup with a predecessor tile that never runs.  It returns GRAM_OK once the
  * launch is queued; the next gram_sync takes about a second and returns GRAM_ERR_TIMEOUT; the context stays usable.
  * (No counterpart in the paper.) */
 gram_status gram_selftest_bounded_wait(gram_ctx* ctx, gram_stream stream);

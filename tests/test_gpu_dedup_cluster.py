@@ -1,4 +1,5 @@
-"""gram_dedup at the edges of its one-launch form: the tiles of one thread block, full clusters, one position more."""
+"""gram_dedup at the edges of its one-launch form (the tiles of one thread block, full clusters, one position more) and of the
+chain of launches: one, two and three passes, the last tile full, one key short, one key long."""
 import numpy as np
 import pytest
 
@@ -21,4 +22,32 @@ def test_dedup_at_tile_and_cluster_edges(P, kind):
     assert U == len(want[0])
     for x, w in zip(got, want):                          # whole numbers: one correct answer
         assert np.array_equal(x, w)
+    g.close()
+
+
+@pytest.mark.parametrize("n_items", [1, 2, 300, 1024, 1025, 65_536, 1_048_576, 1_048_577, 20_000_000])
+@pytest.mark.parametrize("P", [65_537, 73_728, 73_729, 524_288 + 8191])
+def test_dedup_chain_of_launches(P, n_items):
+    ids = synth.zipf_ids(6, n_items, 0.9, P)
+    ids[: min(P, 50)] = n_items - 1                      # the largest key that the passes must place
+    g = index_ctx(P, n_items, 4)
+    U, *got = run_dedup(g, ids, n_items)
+    want = orc.unique_inverse(ids)
+    assert U == len(want[0])
+    for x, w in zip(got, want):
+        assert np.array_equal(x, w)
+    g.close()
+
+
+def test_dedup_of_fewer_items_than_the_context_holds():
+    """A context for many items serves calls with any number of them: the widths of the passes differ from call to call."""
+    P = 200_000
+    g = index_ctx(P, 20_000_000, 4)
+    for n_items in (20_000_000, 900_000, 5000, 700, 3, 1_100_000):
+        ids = synth.zipf_ids(7, n_items, 1.0, P)
+        U, *got = run_dedup(g, ids, n_items)
+        want = orc.unique_inverse(ids)
+        assert U == len(want[0])
+        for x, w in zip(got, want):
+            assert np.array_equal(x, w)
     g.close()
