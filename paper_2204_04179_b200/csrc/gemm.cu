@@ -195,18 +195,19 @@ __device__ __forceinline__ void epilogue_store4(const EpiDev& e, CT* C, int64_t 
   if (e.copy_out) st4(reinterpret_cast<bf16*>(e.copy_out) + o, v);
 }
 
-// A tile of TILE x TILE results per block, TILE^2 / 16 threads with 4 x 4 results each; 16 k at a time through two
-// shared-memory buffers, the next 16 fetched into registers (16-byte loads where the rows allow them) while the current
+// A tile of TILE x TILE results per block, TILE^2 / 16 threads with 4 x 4 results each; a k-block at a time through two
+// shared-memory buffers, the next one fetched into registers (16-byte loads where the rows allow them) while the current
 // ones are multiplied.  The configurations that run in fp32 are small, so what bounds these products is the chain of
 // k-blocks of one block and the number of blocks, not the FMA rate: the K range is therefore cut over a cluster of up
 // to 16 blocks, whose partial tiles are added through distributed shared memory in ascending order of the block's rank
 // (the order depends on the sizes alone), each block finishing its share of the tile's rows.  One launch, no
 // workspace.  Weight gradients of the check's model (64 x 64 to 256 x 64 over about 900 rows): 130 to 185 us each with
-// one 64 x 64 block per tile and a synchronous load per k-block, 11 us now (timed with an event on either side); the
-// model's whole training step 2.49 -> 0.73 ms.
-constexpr int SK = 16;
+// one 64 x 64 block per tile and a synchronous load per k-block, 6 to 7 us now; the
+// model's whole training step 2.49 -> 0.48 ms with the chain of launches below.
+// What a k-block waits for is its loads: 32 k at a time in the small tiles (two rounds of loads for K = 64 instead of four).
 constexpr int F32_MAX_SPLIT = 16;
 template <int TILE> struct F32Cfg {
+  static constexpr int SK = TILE == 32 ? 32 : 16;          // k of one k-block
   static constexpr int THREADS = TILE * TILE / 16;
   static constexpr int LD = TILE + 4;                      // keeps rows 16-byte aligned
   static constexpr int NV = TILE * SK / 4 / THREADS;       // 16-byte pieces per thread, operand and k-block
@@ -217,7 +218,8 @@ template <int TILE, bool KMAJOR>
 __device__ __forceinline__ float4 f32_fetch(const float* __restrict__ X, int64_t ld, int64_t r0, int64_t rows, int64_t k0,
                                             int64_t kend, int idx, bool vec) {
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int64_t r = r0 + (KMAJOR ? idx / 4 : 4 * (idx % (TILE / 4))), k = k0 + (KMAJOR ? 4 * (idx % 4) : idx / (TILE / 4));
+  constexpr int KQ = F32Cfg<TILE>::SK / 4;                 // pieces of one row's k-block
+  const int64_t r = r0 + (KMAJOR ? idx / KQ : 4 * (idx % (TILE / 4))), k = k0 + (KMAJOR ? 4 * (idx % KQ) : idx / (TILE / 4));
   if (r >= rows || k >= kend) return v;
   const float* p = KMAJOR ? X + r * ld + k : X + k * ld + r;
   const int64_t left = KMAJOR ? kend - k : rows - r;       // elements of the piece that exist
@@ -232,21 +234,62 @@ template <int TILE, bool KMAJOR>
 __device__ __forceinline__ void f32_stage(float* s, int idx, float4 v) {
   constexpr int LD = F32Cfg<TILE>::LD;
   if (KMAJOR) {
-    float* q = s + 4 * (idx % 4) * LD + idx / 4;
+    constexpr int KQ = F32Cfg<TILE>::SK / 4;
+    float* q = s + 4 * (idx % KQ) * LD + idx / KQ;
     q[0] = v.x; q[LD] = v.y; q[2 * LD] = v.z; q[3 * LD] = v.w;
   } else {
     *reinterpret_cast<float4*>(s + (idx / (TILE / 4)) * LD + 4 * (idx % (TILE / 4))) = v;
   }
 }
 
+// The epilogue for four columns of a row at a time (vec_e launches: every matrix and vector it touches allows 16-byte
+// accesses, and at most one of residual, GELU derivative and accumulation is asked for).  What it reads per element is
+// fetched ahead (f32_aux), for all of a thread's rows before the first of them is stored: element by element, every load
+// waits for the store before it.
+__device__ __forceinline__ float4 f32_ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 f32_aux(const EpiDev& e, const float* C, int64_t o) {
+  if (e.res) return f32_ld4(e.res + o);
+  if (e.dgelu_pre) return f32_ld4(reinterpret_cast<const float*>(e.dgelu_pre) + o);
+  if (e.accumulate) return f32_ld4(C + o);
+  return make_float4(0.f, 0.f, 0.f, 0.f);
+}
+struct F32Cols { float4 bias, gamma, beta; };           // of the thread's four columns
+__device__ __forceinline__ F32Cols f32_cols(const EpiDev& e, int n) {
+  F32Cols c;
+  c.bias = e.bias ? f32_ld4(e.bias + n) : make_float4(0.f, 0.f, 0.f, 0.f);
+  c.gamma = e.res_mean ? f32_ld4(e.res_gamma + n) : make_float4(0.f, 0.f, 0.f, 0.f);
+  c.beta = e.res_mean ? f32_ld4(e.res_beta + n) : make_float4(0.f, 0.f, 0.f, 0.f);
+  return c;
+}
+__device__ __forceinline__ void f32_finish(const EpiDev& e, float* C, int64_t o, const float (&acc)[4], const float4& aux4,
+                                           const F32Cols& c, float mu, float rs) {
+  const float bias[4] = {c.bias.x, c.bias.y, c.bias.z, c.bias.w}, gam[4] = {c.gamma.x, c.gamma.y, c.gamma.z, c.gamma.w};
+  const float bet[4] = {c.beta.x, c.beta.y, c.beta.z, c.beta.w}, aux[4] = {aux4.x, aux4.y, aux4.z, aux4.w};
+  float v[4], dg[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    v[i] = acc[i] + bias[i];
+    if (e.gelu) {
+      dg[i] = gelu_grad_f(v[i]);
+      v[i] = gelu_f(v[i]);
+    }
+    if (e.res) v[i] += e.res_mean ? (aux[i] - mu) * rs * gam[i] + bet[i] : aux[i];
+    else if (e.dgelu_pre) v[i] *= aux[i];
+    else if (e.accumulate) v[i] += aux[i];
+  }
+  if (e.gelu && e.pre) st4(reinterpret_cast<float*>(e.pre) + o, dg);
+  st4(C + o, v);
+  if (e.copy_out) st4(reinterpret_cast<float*>(e.copy_out) + o, v);
+}
+
 template <int TILE, bool A_K, bool B_K>
 __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const float* __restrict__ A, int64_t lda,
                                                                         const float* __restrict__ B, int64_t ldb, float* C,
                                                                         int64_t ldc, int64_t M, int N, int64_t K,
-                                                                        int64_t k_per_split, int vec_a, int vec_b, EpiDev e) {
+                                                                        int64_t k_per_split, int vec_a, int vec_b, int vec_e, EpiDev e) {
   if (!chain_begin()) return;
   using Cfg = F32Cfg<TILE>;
-  constexpr int LD = Cfg::LD, NV = Cfg::NV, T = Cfg::THREADS;
+  constexpr int LD = Cfg::LD, NV = Cfg::NV, T = Cfg::THREADS, SK = Cfg::SK;
   __shared__ __align__(16) float sm[2][2][SK * LD];        // [buffer][operand]; later the block's partial tile
   static_assert(sizeof(sm) >= sizeof(float) * TILE * LD, "the partial tile reuses the operand buffers");
   const int tid = threadIdx.x, tx = tid % (TILE / 4), ty = tid / (TILE / 4);
@@ -288,6 +331,27 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
   }
   const int splits = gridDim.z;
   if (splits == 1) {
+    if (vec_e) {
+      const int64_t n = n0 + 4 * tx;
+      if (n >= N) return;                        // N is a multiple of 4
+      const F32Cols cols = f32_cols(e, (int)n);
+      float4 aux[4];
+      float mu[4], rs[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int64_t m = m0 + 4 * ty + i;
+        const bool ok = m < M;
+        aux[i] = ok ? f32_aux(e, C, m * ldc + n) : make_float4(0.f, 0.f, 0.f, 0.f);
+        mu[i] = ok && e.res_mean ? e.res_mean[m] : 0.f;
+        rs[i] = ok && e.res_mean ? e.res_rstd[m] : 1.f;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int64_t m = m0 + 4 * ty + i;
+        if (m < M) f32_finish(e, C, m * ldc + n, acc[i], aux[i], cols, mu[i], rs[i]);
+      }
+      return;
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -302,21 +366,47 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
 #pragma unroll
   for (int i = 0; i < 4; ++i)
     *reinterpret_cast<float4*>(part + (4 * ty + i) * LD + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   const int rows = TILE / splits, r0 = blockIdx.z * rows;          // this block's share of the tile's rows
-  for (int idx = tid; idx < rows * TILE; idx += T) {
-    const int r = r0 + idx / TILE, c = idx % TILE;
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  for (int idx = tid; idx < rows * (TILE / 4); idx += T) {         // four columns of a row each
+    const int r = r0 + idx / (TILE / 4), c = 4 * (idx % (TILE / 4));
     const int64_t m = m0 + r, n = n0 + c;
     const uint32_t at = smem_u32(part + r * LD + c);
-    float v = 0.f;
-    for (int s = 0; s < splits; ++s) {
-      uint32_t ra;
-      float x;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(at), "r"(s));
-      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(ra) : "memory");
-      v += x;
+    const bool ok = m < M && n < N;
+    float4 aux = make_float4(0.f, 0.f, 0.f, 0.f);
+    F32Cols cols = {aux, aux, aux};
+    float mu = 0.f, rs = 1.f;
+    if (vec_e && ok) {
+      aux = f32_aux(e, C, m * ldc + n);
+      cols = f32_cols(e, (int)n);
+      if (e.res_mean) { mu = e.res_mean[m]; rs = e.res_rstd[m]; }
     }
-    if (m < M && n < N) epilogue_store<float, float>(e, C, ldc, m, (int)n, v);
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int s0 = 0; s0 < F32_MAX_SPLIT; s0 += 8) {                // eight parts on their way at once, added in order
+      if (s0 >= splits) break;
+      float4 x[8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        uint32_t ra;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(at), "r"(min(s0 + s, splits - 1)));
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(x[s].x), "=f"(x[s].y), "=f"(x[s].z), "=f"(x[s].w)
+                     : "r"(ra)
+                     : "memory");
+      }
+#pragma unroll
+      for (int s = 0; s < 8; ++s)
+        if (s0 + s < splits) { v[0] += x[s].x; v[1] += x[s].y; v[2] += x[s].z; v[3] += x[s].w; }
+    }
+    if (!ok) continue;
+    if (vec_e) {
+      f32_finish(e, C, m * ldc + n, v, aux, cols, mu, rs);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (n + j < N) epilogue_store<float, float>(e, C, ldc, m, (int)n + j, v[j]);
+    }
   }
   // no block may leave while another still reads its partial tile
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -343,7 +433,11 @@ cudaError_t launch_f32(const float* A, int64_t lda, const float* B, int64_t ldb,
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   const int vec_a = (lda % 4 == 0) && ((uintptr_t)A % 16 == 0), vec_b = (ldb % 4 == 0) && ((uintptr_t)B % 16 == 0);
-  return cudaLaunchKernelEx(&cfg, kern, A, lda, B, ldb, C, ldc, M, N, K, k_per_split, vec_a, vec_b, e);
+  auto al = [](const void* p) { return (uintptr_t)p % 16 == 0; };
+  const int one_aux = (e.res != nullptr) + (e.dgelu_pre != nullptr) + (e.accumulate != 0) <= 1;
+  const int vec_e = one_aux && N % 4 == 0 && ldc % 4 == 0 && al(C) && al(e.bias) && al(e.res) && al(e.res_gamma) && al(e.res_beta) && al(e.pre) &&
+                    al(e.dgelu_pre) && al(e.copy_out);
+  return cudaLaunchKernelEx(&cfg, kern, A, lda, B, ldb, C, ldc, M, N, K, k_per_split, vec_a, vec_b, vec_e, e);
 }
 template <int TILE>
 cudaError_t launch_f32_major(bool a_k, bool b_k, const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc,
@@ -1468,8 +1562,9 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     const bool big = b64 >= kNumSMs;
     const int64_t blocks = big ? b64 : b32, enough = big ? kNumSMs : 4 * kNumSMs;
     int parts = 1;
-    while (parts < F32_MAX_SPLIT && blocks * parts * 2 <= enough && K >= 4 * SK * parts) parts *= 2;
-    const int64_t per = ceil_div64(ceil_div64(K, parts), SK) * SK;
+    const int sk = big ? F32Cfg<64>::SK : F32Cfg<32>::SK;
+    while (parts < F32_MAX_SPLIT && blocks * parts * 2 <= enough && K >= 64 * parts) parts *= 2;
+    const int64_t per = ceil_div64(ceil_div64(K, parts), sk) * sk;
     if (ceil_div64(M, big ? 64 : 32) > 65535)
       return gram_set_error(ctx, "gemm: %lld rows are more than an fp32 product takes", (long long)M), GRAM_ERR_UNSUPPORTED;
     const cudaError_t ferr = big ? launch_f32_major<64>(a_kmajor, b_kmajor, (const float*)A, lda, (const float*)B, ldb, (float*)C, ldc, M, N, K, parts, per, e, st)
