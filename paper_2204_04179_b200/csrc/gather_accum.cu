@@ -2,6 +2,7 @@
 // gradients of each item, Eq. 6; Multi-step: add them into the per-item table, Section 4.2).
 // Both are HBM-bound: 128-bit accesses, a warp per row, several rows in flight per warp.
 #include "gram_internal.h"
+#include "tc_common.cuh"
 
 namespace {
 
@@ -279,6 +280,121 @@ __global__ void __launch_bounds__(256) segsum_chunks_kernel(const InT* __restric
   if (slab == 0 && lane == 0) span[chunk] = sp;   // (item, last chunk it reaches), or -1: nothing to fix up from here
 }
 
+// The same walk for fp32 rows of 516 to 1024 columns with one warp per chunk (all columns): the rows arrive as bulk copies
+// in a ring of `stages` slots per warp, so a warp has that many rows on their way while it adds, instead of none between
+// two batches of register loads.  Sums, partial sums and spans as above, bit for bit (a chunk's rows are added in the same
+// order).  Through registers / this way, us: 25 600 rows of 768 36 / 32, 150 000 107 / 104, 10^6 606 / 586; of 1024 41 / 41,
+// 138 / 130.  Narrower rows (512: 75 / 80 at 150 000; 256: 45 / 50) and short calls (3000 rows: 12 / 15) stay with registers:
+// a bulk copy of 2 KB or less costs its issue.
+constexpr int SEG_WARPS = 8, SEG_STAGES_MAX = 8;
+constexpr int kSegRingMin = 512;                 // columns, more than
+constexpr int64_t kSegRingRows = 20000;          // positions, at least
+constexpr int64_t kSegRingBytes = 110 * 1024;    // shared memory of a block: two per SM
+template <int NQ>
+__global__ void __launch_bounds__(32 * SEG_WARPS) segsum_ring_kernel(const float* __restrict__ in, const int32_t* __restrict__ perm,
+                                                                    const int32_t* __restrict__ seg_off, int64_t P, int32_t U, int d,
+                                                                    int64_t R, int nchunks, int stages, const int32_t* __restrict__ rows,
+                                                                    int add, float* __restrict__ out, float* __restrict__ partial,
+                                                                    int2* __restrict__ span, int32_t* status,
+                                                                    const int32_t* __restrict__ d_U, const int32_t* __restrict__ gate) {
+  if (!chain_begin()) return;
+  extern __shared__ __align__(16) float seg_ring[];
+  __shared__ __align__(8) uint64_t bars[SEG_WARPS * SEG_STAGES_MAX];
+  __shared__ int abort_flag;
+  if (d_U) U = *d_U;
+  if (U <= 0) return;
+  if (gate && *gate) return;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int chunk = blockIdx.x * SEG_WARPS + wib;
+  float* ring = seg_ring + (size_t)wib * stages * d;
+  const uint32_t bar0 = tc::smem_u32(bars + wib * SEG_STAGES_MAX), ring0 = tc::smem_u32(ring), row_bytes = (uint32_t)d * 4u;
+  if (threadIdx.x == 0) abort_flag = 0;
+  if (lane == 0) {
+    for (int s = 0; s < stages; ++s) tc::mbar_init(bar0 + 8u * s, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  const int64_t c0 = (int64_t)chunk * R, c1 = min(c0 + R, P);
+  if (chunk >= nchunks || c0 >= c1) return;
+  auto fetch_perm = [&](int64_t j0) -> int32_t {             // positions j0 + lane of the sorted order
+    int32_t p = 0;
+    if (j0 + lane < c1) {
+      p = perm[j0 + lane];
+      if ((uint32_t)p >= (uint32_t)P) {                      // a position outside the batch: record it, read row 0 instead
+        gram_device_fail(status, GRAM_ERR_ID_RANGE);
+        p = 0;
+      }
+    }
+    return p;
+  };
+  auto request = [&](int32_t p, int s) {
+    tc::mbar_expect_tx(bar0 + 8u * s, row_bytes);
+    tc::bulk_load(ring0 + (uint32_t)s * row_bytes, in + (int64_t)p * d, row_bytes, bar0 + 8u * s);
+  };
+  int32_t cur = fetch_perm(c0), nxt = fetch_perm(c0 + 32);
+  for (int k = 0; k < stages; ++k) {                          // stages <= 8: inside the first window
+    const int32_t p = __shfl_sync(0xffffffffu, cur, k);
+    if (lane == 0 && c0 + k < c1) request(p, k);
+  }
+  int32_t u = find_segment(seg_off, U, c0, lane);
+  int64_t seg_begin = seg_off[u], seg_end = seg_off[u + 1];
+  float4 acc[NQ];
+#pragma unroll
+  for (int v = 0; v < NQ; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+  int s = 0;
+  uint32_t parity = 0;
+  bool failed = false;
+  for (int64_t j = c0; j < c1; ++j) {
+    if (!__all_sync(0xffffffffu, tc::mbar_wait(bar0 + 8u * s, parity, (volatile int*)&abort_flag))) { failed = true; break; }
+    float4 x[NQ];
+    const float* row = ring + (size_t)s * d;
+#pragma unroll
+    for (int v = 0; v < NQ; ++v) {
+      const int c = (v * 32 + lane) * 4;
+      x[v] = c < d ? *reinterpret_cast<const float4*>(row + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    const int at = (int)((j - c0) & 31) + stages;             // the row `stages` places on, in this window or the next
+    const int32_t pa = __shfl_sync(0xffffffffu, cur, at & 31), pb = __shfl_sync(0xffffffffu, nxt, at & 31);
+    __syncwarp();                                              // every lane has read the slot
+    if (lane == 0 && j + stages < c1) request(at < 32 ? pa : pb, s);
+    if (((j - c0) & 31) == 31) {
+      cur = nxt;
+      nxt = fetch_perm(j + 33);
+    }
+    if (++s == stages) { s = 0; parity ^= 1u; }
+    while (j == seg_end && u + 1 < U) {                        // item u is complete (its end lies inside this chunk)
+      if (seg_begin >= c0) store_row<NQ>(out, rows ? rows[u] : u, d, 0, lane, acc, add != 0);
+      else store_row<NQ>(partial, (int64_t)chunk * 2 + 0, d, 0, lane, acc, false);
+      ++u;
+      seg_begin = seg_end;
+      seg_end = seg_off[u + 1];
+#pragma unroll
+      for (int v = 0; v < NQ; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int v = 0; v < NQ; ++v) { acc[v].x += x[v].x; acc[v].y += x[v].y; acc[v].z += x[v].z; acc[v].w += x[v].w; }
+  }
+  if (failed) {
+    if (lane == 0) {
+      abort_flag = 1;
+      gram_device_fail(status, GRAM_ERR_TIMEOUT);
+      const uint64_t t0 = clock64();                           // let the copies that were issued end (bounded)
+      while (clock64() - t0 < tc::WAIT_LIMIT_CYCLES / 64) {}
+    }
+    __syncwarp();
+    return;
+  }
+  int2 sp = make_int2(-1, 0);
+  if (seg_end <= c1) {             // the item still open ends exactly at the chunk end
+    if (seg_begin >= c0) store_row<NQ>(out, rows ? rows[u] : u, d, 0, lane, acc, add != 0);
+    else store_row<NQ>(partial, (int64_t)chunk * 2 + 0, d, 0, lane, acc, false);
+  } else {                         // it continues to the right
+    store_row<NQ>(partial, (int64_t)chunk * 2 + (seg_begin >= c0 ? 1 : 0), d, 0, lane, acc, false);
+    if (seg_begin >= c0) sp = make_int2(u, (int)((seg_end - 1) / R));
+  }
+  if (lane == 0) span[chunk] = sp;
+}
+
 // one block per (chunk, slab): if an item starts in this chunk and runs past its end, add its parts.  Warp w adds
 // the following chunks' parts number w, w+8, ... (ascending), warp 0 starts from this chunk's own part, and the
 // eight warp sums are added in ascending w: a fixed association, whatever the schedule.
@@ -486,7 +602,19 @@ static void segsum_run(const void* d_in, const int32_t* d_perm, const int32_t* d
   const int nslabs = ceil_div(d, VPL * 128);
   const int64_t warps = (int64_t)nchunks * nslabs;
   const int blocks = (int)ceil_div64(warps, 8);
-  launch_chain(segsum_chunks_kernel<InT, VPL, 8>, blocks, 256, 0, st, (const InT*)d_in, d_perm, d_seg_off, P, U, d, R, nchunks, nslabs,
+  bool ring = false;
+  if constexpr (sizeof(InT) == 4) {
+    if (d > kSegRingMin && d <= 1024 && P >= kSegRingRows) {
+      ring = true;
+      auto kern = d <= 768 ? segsum_ring_kernel<6> : segsum_ring_kernel<8>;
+      int stages = (int)(kSegRingBytes / ((int64_t)SEG_WARPS * d * 4));
+      if (stages > SEG_STAGES_MAX) stages = SEG_STAGES_MAX;
+      (void)cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegRingBytes);
+      launch_chain(kern, ceil_div(nchunks, SEG_WARPS), 32 * SEG_WARPS, (size_t)SEG_WARPS * stages * d * 4, st, (const float*)d_in, d_perm,
+                   d_seg_off, P, U, d, R, nchunks, stages, d_rows, add, d_out, partial, span, status, d_U, gate);
+    }
+  }
+  if (!ring) launch_chain(segsum_chunks_kernel<InT, VPL, 8>, blocks, 256, 0, st, (const InT*)d_in, d_perm, d_seg_off, P, U, d, R, nchunks, nslabs,
                                                             d_rows, add, d_out, partial, span, status, d_U, gate);
   if (nchunks > 1)
     launch_chain(segsum_fixup_kernel<VPL>, (unsigned)warps, 256, 0, st, d_seg_off, P, U, d, R, nchunks, nslabs, d_rows, add, d_out, partial, span, d_U, gate);
