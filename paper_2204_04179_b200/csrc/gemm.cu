@@ -1425,8 +1425,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
 
 // C(m, n) = sum over splits of part[s](m, n), in ascending s; then the epilogue.  Four columns per thread (N is a multiple of
 // 8), four splits' loads on their way at once; PLAIN: the only epilogue is "add to fp32 C" or none (weight gradients).
-// 3072 x 768: 21 us from six parts with a column per thread and split after split; 6.6 now, from the two parts that the
-// dispatch takes there since partial sums have a price.
+// 3072 x 768 from six parts: 21 us with a column per thread and split after split.
 template <typename CT, bool PLAIN>
 __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restrict__ part, int splits, int64_t split_stride, int64_t M,
                                                            int N, CT* C, int64_t ldc, EpiDev e) {
@@ -1603,19 +1602,24 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
   const int units = pair ? kNumSMs / 2 : kNumSMs;        // CTAs, or CTA pairs, that run at once
   int splits = 1;
   if (allow_splitk && tiles < units && args.num_kb >= 16 && ws && ws->splitk) {
-    // the count that is cheapest in microseconds: whole waves of units of num_kb / splits k-blocks (0.3 each on a 256 x 256
-    // pair tile; a smaller tile scales every count alike), the last unit's epilogue (3), and the partial sums written and
-    // read again (5 MB a microsecond).  A count must leave at least eight k-blocks per part.
+    // between 2 and 4 work units per CTA (pair), each of at least eight k-blocks; among those, the count that leaves the last
+    // wave fullest.  Fewer parts can be faster (25 600 rows: 768 x 768 40 us from 24 parts, 31 from 8; 3072 x 768 103 from 6,
+    // 94 from 2) but cost precision: the tensor core adds into its fp32 accumulator by cutting off, so the error of a part
+    // grows with the length of its chain of additions, while the parts themselves are added with rounding (65 536 rows,
+    // 3072 x 768, against 64 bits: 1.2e-5 from 6 parts, 3.8e-5 from 2).
     const int64_t per = (int64_t)M * N * (int64_t)sizeof(float);
+    int lo = (int)((2 * units + tiles - 1) / tiles), hi = (int)((4 * units + tiles - 1) / tiles);
     int cap = args.num_kb / 8;
     if ((int64_t)cap * per > (int64_t)ws->splitk_bytes) cap = (int)(ws->splitk_bytes / per);
-    const int64_t most = ceil_div64(4 * units, tiles);
-    if (cap > most) cap = (int)most;
-    double best = 0.0;
-    for (int sp = 1; sp <= cap; ++sp) {
-      const double cost = (double)ceil_div64(tiles * sp, units) * ceil_div(args.num_kb, sp) * 0.3 + 3.0 + (sp > 1 ? (double)per * 2e-7 * sp : 0.0);
-      if (sp == 1 || cost < best) { best = cost; splits = sp; }
+    if (hi > cap) hi = cap;
+    if (lo > hi) lo = hi;
+    double best = -1.0;
+    for (int sp = lo; sp <= hi && sp >= 1; ++sp) {
+      const int64_t total = tiles * sp;
+      const double fill = (double)total / (double)(ceil_div64(total, units) * units);
+      if (fill > best + 1e-9) { best = fill; splits = sp; }
     }
+    if (splits < 1) splits = 1;
   }
   args.kb_per_split = ceil_div(args.num_kb, splits);
   splits = ceil_div(args.num_kb, args.kb_per_split);

@@ -134,3 +134,25 @@ def test_gemm_epilogues_against_float64(M, N, K, kind):
     g.sync()
     assert torch.equal(Cd, Ce)
     g.close()
+
+
+@pytest.mark.parametrize("M,N,K,parts", [(3072, 768, 65_536, 5), (768, 3072, 40_000, 5), (2304, 768, 65_536, 6), (768, 768, 65_536, 17)])
+def test_long_sums_keep_their_precision(M, N, K, parts):
+    """Weight gradients of many rows.  The tensor core cuts each of a chain of additions off to 24 bits, so a chain of n
+    16-term steps over values of one sign loses about n * 2^-24 of the sum; `parts`: how many chains at least two work units
+    per pair of SMs make of the K range (256 x 256 tiles)."""
+    cfg = binding.GramConfig()
+    cfg.n_items = cfg.P_max = 8
+    cfg.d, cfg.d_ff = 768, 3072                                 # the workspace of partial products is sized by these
+    g = binding.Gram(cfg)
+    gen = torch.Generator(device=DEV).manual_seed(5)
+    A = (torch.randn(K, M, generator=gen, device=DEV) + 1).to(torch.bfloat16)
+    B = (torch.randn(K, N, generator=gen, device=DEV) + 1).to(torch.bfloat16)
+    C = torch.zeros(M, N, device=DEV)
+    g.gemm_bf16(A, 0, B, 0, C, None, 1, M, N, K)
+    g.sync()
+    g.close()
+    want = torch.zeros(M, N, dtype=torch.float64, device=DEV)
+    for o in range(0, K, 8192):
+        want += A[o:o + 8192].double().T @ B[o:o + 8192].double()
+    assert ((C - want).norm() / want.norm()).item() <= K / 16 / parts * 2.0 ** -24
