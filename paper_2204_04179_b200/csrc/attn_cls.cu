@@ -240,12 +240,13 @@ __global__ void add_strided_rows_kernel(const float4* __restrict__ r, float4* __
   *x = b;
 }
 
+constexpr size_t kClsSmemMost = 96 * 1024;       // the kernels' limit is set to this, whatever a call needs: other threads launch them too
 size_t cls_smem(int heads, int l_t, int arrays) { return (size_t)heads * l_t * arrays * sizeof(float); }
 
 }  // namespace
 
 bool attention_cls_supported(int l_t, int d, int n_heads) {
-  return n_heads > 0 && n_heads <= 16 && d == n_heads * DH && cls_smem(n_heads, l_t, 2) <= 96 * 1024;
+  return n_heads > 0 && n_heads <= 16 && d == n_heads * DH && cls_smem(n_heads, l_t, 2) <= kClsSmemMost;
 }
 
 gram_status attention_cls_forward(gram_ctx* ctx, const void* q, const void* kv, void* out, int n, int l_t, int d, int n_heads,
@@ -253,7 +254,7 @@ gram_status attention_cls_forward(gram_ctx* ctx, const void* q, const void* kv, 
   if (n == 0) return GRAM_OK;
   const size_t smem = cls_smem(n_heads, l_t, 1);
   ProfScope prof(ctx, GRAM_K_ATTENTION, 4.0 * (double)n * l_t * d, 1, st, "attn_cls_fwd");
-  if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(attn_cls_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(attn_cls_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClsSmemMost));
   launch_chain(attn_cls_fwd_kernel, n, n_heads * 32, smem, st, (const bf16*)q, (const bf16*)kv, (bf16*)out, n, l_t, d,
                                                      1.4426950408889634f / sqrtf((float)DH), seq_len, seq_off);
   GRAM_LAUNCH_CHECK(ctx);
@@ -270,7 +271,7 @@ gram_status attention_cls_backward(gram_ctx* ctx, const void* q, const void* kv,
   if (blocks < 1) return gram_set_error(ctx, "attention backward: no room for the column sums"), GRAM_ERR_WORKSPACE;
   const size_t smem = cls_smem(n_heads, l_t, 2);
   ProfScope prof(ctx, GRAM_K_ATTENTION, 10.0 * (double)n * l_t * d, 1, st, "attn_cls_bwd");
-  if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(attn_cls_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(attn_cls_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClsSmemMost));
   launch_chain(attn_cls_bwd_kernel, (unsigned)blocks, n_heads * 32, smem, st, (const bf16*)q, (const bf16*)kv, (const bf16*)dctx, (bf16*)dq,
                                                                     (bf16*)dkv, part, n, l_t, d, 1.4426950408889634f / sqrtf((float)DH),
                                                                     1.f / sqrtf((float)DH), seq_len, seq_off);

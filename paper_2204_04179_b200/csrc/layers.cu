@@ -1311,9 +1311,13 @@ inline int grid_for(int64_t n, int threads, int cap) {
   return (int)b;
 }
 
-template <typename F> gram_status set_smem(gram_ctx* ctx, F kern, size_t bytes) {
-  if (bytes > 227 * 1024) return gram_set_error(ctx, "a sequence is too long for the attention kernel's shared memory"), GRAM_ERR_UNSUPPORTED;
-  if (bytes > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+constexpr size_t kSmemMost = 227 * 1024;
+// Lets a kernel be launched with `bytes` of dynamic shared memory.  The limit belongs to the kernel and not to the context,
+// and another thread may be between its own call of this and its launch: it is set to the most that the kernel can ever ask
+// for, the same value from every caller.
+template <typename F> gram_status set_smem(gram_ctx* ctx, F kern, size_t bytes, size_t most = kSmemMost) {
+  if (bytes > most) return gram_set_error(ctx, "a sequence is too long for the attention kernel's shared memory"), GRAM_ERR_UNSUPPORTED;
+  if (bytes > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
   return GRAM_OK;
 }
 
@@ -1372,10 +1376,11 @@ gram_status layernorm_backward(gram_ctx* ctx, int dtype, const float* dy, const 
   if (d > 1024 || (d & 3)) return gram_set_error(ctx, "LayerNorm: d must be a multiple of 4 and at most 1024"), GRAM_ERR_UNSUPPORTED;
   int blocks = kNumSMs;                            // one per SM; at least one row per warp
   if (rows < (int64_t)blocks * LNB_WARPS) blocks = (int)ceil_div64(rows, LNB_WARPS);
-  const size_t smem = (size_t)(4 + LNB_WARPS * LNB_STAGES * 2) * d * sizeof(float);
+  auto smem_of = [](int cols) { return (size_t)(4 + LNB_WARPS * LNB_STAGES * 2) * cols * sizeof(float); };
+  const size_t smem = smem_of(d);
   ProfScope prof(ctx, GRAM_K_LAYERNORM, (double)rows * d * (12.0 + (dz_b ? (dtype == GRAM_BF16 ? 2.0 : 4.0) : 0.0)), 2, st, "ln_bwd");
   DISPATCH_T(dtype, DISPATCH_NQ(d, {
-    GRAM_TRY(set_smem(ctx, ln_bwd_kernel<T, NQ>, smem));
+    GRAM_TRY(set_smem(ctx, ln_bwd_kernel<T, NQ>, smem, smem_of(128 * NQ)));
     launch_chain(ln_bwd_kernel<T, NQ>, blocks, 32 * LNB_WARPS, smem, st, dy, z, mean, rstd, gamma, dz, (T*)dz_b, scratch, rows, d, gram_status_word(ctx));
   }));
   launch_chain(reduce_partials_kernel, dim3(ceil_div(d, 32), dcol ? 3 : 2), 256, 0, st, scratch, blocks, (int64_t)3 * d, d, dgamma, dbeta, dcol, 1.f);
