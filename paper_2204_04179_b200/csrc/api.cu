@@ -37,6 +37,7 @@ struct gram_ctx {
   int prof_ntags = 0;
   char err[512];
   int32_t* d_status = nullptr;      // device status word (first device-side error)
+  int32_t ring_rows = INT32_MAX;    // gram_selftest_ring_rows
   IndexWorkspace iws;
   GemmWorkspace gws;
   Model* model = nullptr;           // encoder + task module state (null for an index-only context)
@@ -51,6 +52,7 @@ void gram_set_error(gram_ctx* ctx, const char* fmt, ...) {
 }
 
 int32_t* gram_status_word(gram_ctx* ctx) { return ctx->d_status; }
+int32_t gram_ring_rows(const gram_ctx* ctx) { return ctx->ring_rows; }
 
 void gram_prof_open(gram_ctx* ctx, int kind, const char* tag, double work, int launches, cudaStream_t st, int* slot) {
   *slot = -1;
@@ -241,6 +243,11 @@ gram_status gram_dedup(gram_ctx* ctx, const int32_t* d_ids, int64_t P, int32_t n
 gram_status gram_selftest_bounded_wait(gram_ctx* ctx, gram_stream stream) {
   if (!ctx) return GRAM_ERR_ARG;
   return dedup_wait_selftest(ctx, &ctx->iws, S(stream));
+}
+gram_status gram_selftest_ring_rows(gram_ctx* ctx, int32_t rows) {
+  if (!ctx) return GRAM_ERR_ARG;
+  ctx->ring_rows = rows < 0 ? INT32_MAX : rows;
+  return GRAM_OK;
 }
 gram_status gram_gather(gram_ctx* ctx, const void* d_src, int64_t n_src_rows, const int32_t* d_index, int64_t P,
                         int32_t d, int dtype, void* d_E, gram_stream stream) {

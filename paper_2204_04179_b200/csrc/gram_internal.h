@@ -146,3 +146,4 @@ struct ProfScope {
 // the device status word: kernels record the first error kind they meet
 __device__ __forceinline__ void gram_device_fail(int32_t* status, int32_t code) { atomicCAS(status, 0, code); }
 int32_t* gram_status_word(gram_ctx* ctx);
+int32_t gram_ring_rows(const gram_ctx* ctx);   // rows a warp may take from a ring of bulk copies before it gives up; see gram_selftest_ring_rows

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(32 * LNB_WARPS, 1) ln_bwd_kernel(const float* 
                                                                   const float* __restrict__ mean, const float* __restrict__ rstd,
                                                                   const float* __restrict__ g, float* __restrict__ dz,
                                                                   T* __restrict__ dz_b, float* __restrict__ part, int64_t rows,
-                                                                  int d, int32_t* status) {
+                                                                  int d, int32_t ring_rows, int32_t* status) {
   if (!chain_begin()) return;
   // [3][d]: dgamma, dbeta and the column sums of dz of this block; [d]: gamma; then the warps' rings
   extern __shared__ __align__(16) float sacc[];
@@ -169,7 +169,8 @@ __global__ void __launch_bounds__(32 * LNB_WARPS, 1) ln_bwd_kernel(const float* 
   for (int64_t r = w; r < rows; r += nw) {
     const float mu = mu_n, rs = rs_n;
     if (r + nw < rows) { mu_n = mean[r + nw]; rs_n = rstd[r + nw]; }
-    if (!tc::mbar_wait(bar0 + 8u * s, parity, (volatile int*)&abort_flag)) {
+    // a vote: lanes that disagreed would part at the shuffles below
+    if (!__all_sync(0xffffffffu, ring_rows-- > 0 && tc::mbar_wait(bar0 + 8u * s, parity, (volatile int*)&abort_flag))) {
       abort_flag = 1;
       gram_device_fail(status, GRAM_ERR_TIMEOUT);
       const uint64_t t0 = clock64();             // let the copies that were issued arrive before the block leaves
@@ -236,7 +237,8 @@ __global__ void __launch_bounds__(32 * LNB_WARPS, 1) ln_bwd_kernel(const float* 
     }
     __syncthreads();
   }
-  for (int i = threadIdx.x; i < 3 * d; i += blockDim.x) part[(int64_t)blockIdx.x * 3 * d + i] = sacc[i];
+  const bool failed = *(volatile int*)&abort_flag != 0;          // then the block adds nothing to the gradients
+  for (int i = threadIdx.x; i < 3 * d; i += blockDim.x) part[(int64_t)blockIdx.x * 3 * d + i] = failed ? 0.f : sacc[i];
 }
 
 // out[c] += scale * sum_b part[b*stride + c]; grid row y > 0 does the same with columns y * n .. of the partial rows,
@@ -1381,7 +1383,7 @@ gram_status layernorm_backward(gram_ctx* ctx, int dtype, const float* dy, const 
   ProfScope prof(ctx, GRAM_K_LAYERNORM, (double)rows * d * (12.0 + (dz_b ? (dtype == GRAM_BF16 ? 2.0 : 4.0) : 0.0)), 2, st, "ln_bwd");
   DISPATCH_T(dtype, DISPATCH_NQ(d, {
     GRAM_TRY(set_smem(ctx, ln_bwd_kernel<T, NQ>, smem, smem_of(128 * NQ)));
-    launch_chain(ln_bwd_kernel<T, NQ>, blocks, 32 * LNB_WARPS, smem, st, dy, z, mean, rstd, gamma, dz, (T*)dz_b, scratch, rows, d, gram_status_word(ctx));
+    launch_chain(ln_bwd_kernel<T, NQ>, blocks, 32 * LNB_WARPS, smem, st, dy, z, mean, rstd, gamma, dz, (T*)dz_b, scratch, rows, d, gram_ring_rows(ctx), gram_status_word(ctx));
   }));
   launch_chain(reduce_partials_kernel, dim3(ceil_div(d, 32), dcol ? 3 : 2), 256, 0, st, scratch, blocks, (int64_t)3 * d, d, dgamma, dbeta, dcol, 1.f);
   GRAM_LAUNCH_CHECK(ctx);
