@@ -198,7 +198,8 @@ gram_status gram_encode_unique(gram_ctx* ctx, const int32_t* d_item_tokens, cons
  * launch is queued; the next gram_sync takes about a second and returns GRAM_ERR_TIMEOUT; the context stays usable.
  * (No counterpart in the paper.) */
 gram_status gram_selftest_bounded_wait(gram_ctx* ctx, gram_stream stream);
-/* The same for the kernels whose warps read rows through a ring of bulk copies (LayerNorm backward): in the context's later
+/* The same for the kernels whose warps read rows through a ring of bulk copies (LayerNorm backward, the
+ * segment sums of many wide rows): in the context's later
  * calls a warp gives up on its wait for row number `rows` (from 0) of those it has to read, as if the copy never arrived.
  * The calls return GRAM_OK, what the kernels add to is left without the rows' sums, and the next gram_sync returns
  * GRAM_ERR_TIMEOUT.  rows < 0: no such limit (as created). */

@@ -293,7 +293,8 @@ constexpr int64_t kSegRingBytes = 110 * 1024;    // shared memory of a block: tw
 template <int NQ>
 __global__ void __launch_bounds__(32 * SEG_WARPS) segsum_ring_kernel(const float* __restrict__ in, const int32_t* __restrict__ perm,
                                                                     const int32_t* __restrict__ seg_off, int64_t P, int32_t U, int d,
-                                                                    int64_t R, int nchunks, int stages, const int32_t* __restrict__ rows,
+                                                                    int64_t R, int nchunks, int stages, int32_t ring_rows,
+                                                                    const int32_t* __restrict__ rows,
                                                                     int add, float* __restrict__ out, float* __restrict__ partial,
                                                                     int2* __restrict__ span, int32_t* status,
                                                                     const int32_t* __restrict__ d_U, const int32_t* __restrict__ gate) {
@@ -345,7 +346,7 @@ __global__ void __launch_bounds__(32 * SEG_WARPS) segsum_ring_kernel(const float
   uint32_t parity = 0;
   bool failed = false;
   for (int64_t j = c0; j < c1; ++j) {
-    if (!__all_sync(0xffffffffu, tc::mbar_wait(bar0 + 8u * s, parity, (volatile int*)&abort_flag))) { failed = true; break; }
+    if (!__all_sync(0xffffffffu, ring_rows-- > 0 && tc::mbar_wait(bar0 + 8u * s, parity, (volatile int*)&abort_flag))) { failed = true; break; }
     float4 x[NQ];
     const float* row = ring + (size_t)s * d;
 #pragma unroll
@@ -377,6 +378,7 @@ __global__ void __launch_bounds__(32 * SEG_WARPS) segsum_ring_kernel(const float
   if (failed) {
     if (lane == 0) {
       abort_flag = 1;
+      span[chunk] = make_int2(-1, 0);                          // not what an earlier call left there: the fix-up reads it
       gram_device_fail(status, GRAM_ERR_TIMEOUT);
       const uint64_t t0 = clock64();                           // let the copies that were issued end (bounded)
       while (clock64() - t0 < tc::WAIT_LIMIT_CYCLES / 64) {}
@@ -416,7 +418,7 @@ __global__ void __launch_bounds__(256) segsum_fixup_kernel(const int32_t* __rest
   const int64_t c0 = (int64_t)chunk * R, c1 = min(c0 + R, P);
   if (c0 >= c1 || c1 >= P) return;
   const int2 sp = span[chunk];                       // left by the first launch
-  if (sp.x < 0) return;                              // no item starts here and runs on (same for the whole block)
+  if (sp.x < 0 || sp.x >= U) return;                 // no item starts here and runs on (same for the whole block)
   const int32_t u = sp.x;
   const int last = min(sp.y, nchunks - 1);
   float4 acc[VPL];
@@ -598,7 +600,7 @@ gram_status gather_diff_launch(gram_ctx* ctx, const float* d_a, const float* d_b
 template <typename InT, int VPL>
 static void segsum_run(const void* d_in, const int32_t* d_perm, const int32_t* d_seg_off, int64_t P, int32_t U, int32_t d,
                        int64_t R, int nchunks, const int32_t* d_rows, int add, float* d_out, float* partial, int2* span,
-                       int32_t* status, const int32_t* d_U, cudaStream_t st, const int32_t* gate = nullptr) {
+                       int32_t* status, const int32_t* d_U, cudaStream_t st, const int32_t* gate, int32_t ring_rows) {
   const int nslabs = ceil_div(d, VPL * 128);
   const int64_t warps = (int64_t)nchunks * nslabs;
   const int blocks = (int)ceil_div64(warps, 8);
@@ -611,7 +613,7 @@ static void segsum_run(const void* d_in, const int32_t* d_perm, const int32_t* d
       if (stages > SEG_STAGES_MAX) stages = SEG_STAGES_MAX;
       (void)cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegRingBytes);
       launch_chain(kern, ceil_div(nchunks, SEG_WARPS), 32 * SEG_WARPS, (size_t)SEG_WARPS * stages * d * 4, st, (const float*)d_in, d_perm,
-                   d_seg_off, P, U, d, R, nchunks, stages, d_rows, add, d_out, partial, span, status, d_U, gate);
+                   d_seg_off, P, U, d, R, nchunks, stages, ring_rows, d_rows, add, d_out, partial, span, status, d_U, gate);
     }
   }
   if (!ring) launch_chain(segsum_chunks_kernel<InT, VPL, 8>, blocks, 256, 0, st, (const InT*)d_in, d_perm, d_seg_off, P, U, d, R, nchunks, nslabs,
@@ -639,12 +641,13 @@ gram_status accumulate_launch(gram_ctx* ctx, IndexWorkspace* ws, const void* d_i
                  nchunks > 1 ? 2 : 1, st);
   int32_t* sw = gram_status_word(ctx);
   const int32_t* gate = gated ? sw : nullptr;
+  const int32_t ring_rows = gram_ring_rows(ctx);
   if (d >= 256) {
-    if (in_bf16) segsum_run<bf16, 2>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate);
-    else segsum_run<float, 2>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate);
+    if (in_bf16) segsum_run<bf16, 2>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate, ring_rows);
+    else segsum_run<float, 2>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate, ring_rows);
   } else {
-    if (in_bf16) segsum_run<bf16, 1>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate);
-    else segsum_run<float, 1>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate);
+    if (in_bf16) segsum_run<bf16, 1>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate, ring_rows);
+    else segsum_run<float, 1>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate, ring_rows);
   }
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
@@ -730,8 +733,8 @@ extern "C" gram_status gram_accumulate_static(const float* d_dE, const int32_t* 
   if (nchunks > kStaticChunks) nchunks = kStaticChunks;
   const int64_t R = ceil_div64(P, nchunks);
   nchunks = ceil_div64(P, R);
-  if (d >= 256) segsum_run<float, 2>(d_dE, d_perm, d_seg_off, P, U, d, R, (int)nchunks, nullptr, 0, d_G, partial, span, status, nullptr, st);
-  else segsum_run<float, 1>(d_dE, d_perm, d_seg_off, P, U, d, R, (int)nchunks, nullptr, 0, d_G, partial, span, status, nullptr, st);
+  if (d >= 256) segsum_run<float, 2>(d_dE, d_perm, d_seg_off, P, U, d, R, (int)nchunks, nullptr, 0, d_G, partial, span, status, nullptr, st, nullptr, INT32_MAX);
+  else segsum_run<float, 1>(d_dE, d_perm, d_seg_off, P, U, d, R, (int)nchunks, nullptr, 0, d_G, partial, span, status, nullptr, st, nullptr, INT32_MAX);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     if (h_err && err_len) snprintf(h_err, err_len, "gram_accumulate_static: launch failed: %s", cudaGetErrorString(e));

@@ -4,7 +4,9 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import gram_oracle as orc
 from paper_2204_04179_b200 import binding, synth
+from tests.test_gpu_index import index_ctx
 
 pytestmark = pytest.mark.gpu
 
@@ -40,4 +42,36 @@ def test_layernorm_backward_gives_up(dtype, rows):
     again = grads()
     for name, w in want.items():
         assert np.array_equal(again[name], w), name
+    g.close()
+
+
+@pytest.mark.parametrize("rows", [0, 7])
+def test_segment_sums_give_up(rows):
+    """A call over few items after one over many: what the first left in the workspace (its items that run over the end of a
+    chunk) names rows that the second does not have.  The rows after its own are the test's, and stay as they are."""
+    P, d, many = 40_000, 768, 5000
+    g = index_ctx(P, many, d)
+    dE = torch.rand(P, d, generator=torch.Generator().manual_seed(2)).cuda()
+
+    def index(n):
+        ids = np.sort(np.arange(P, dtype=np.int32) % n)
+        unique, _, perm, seg = orc.unique_inverse(ids)
+        return len(unique), torch.from_numpy(perm.astype(np.int32)).cuda(), torch.from_numpy(seg.astype(np.int32)).cuda()
+
+    G = torch.zeros(many, d, device="cuda")
+    U, perm, seg = index(many)
+    g.accumulate(dE, perm, seg, U, G)
+    g.sync()
+    U, perm, seg = index(3)
+    G.fill_(-7.0)
+    g.selftest_ring_rows(rows)
+    g.accumulate(dE, perm, seg, U, G)
+    with pytest.raises(binding.GramError, match="GRAM_ERR_TIMEOUT"):
+        g.sync()
+    assert (G[U:] == -7.0).all()
+    g.selftest_ring_rows(-1)
+    g.accumulate(dE, perm, seg, U, G)
+    g.sync()
+    want = torch.stack([dE[perm[seg[u]:seg[u + 1]].long()].double().sum(0) for u in range(U)])
+    assert ((G[:U] - want).abs() <= 1e-5 * want.abs()).all()        # sums of 13 000 positive terms over chunks of 17
     g.close()
