@@ -38,6 +38,7 @@ struct gram_ctx {
   char err[512];
   int32_t* d_status = nullptr;      // device status word (first device-side error)
   int32_t ring_rows = INT32_MAX;    // gram_selftest_ring_rows
+  int32_t cluster_blocks = 1;       // what the device can place, or gram_selftest_cluster_blocks
   IndexWorkspace iws;
   GemmWorkspace gws;
   Model* model = nullptr;           // encoder + task module state (null for an index-only context)
@@ -52,6 +53,7 @@ void gram_set_error(gram_ctx* ctx, const char* fmt, ...) {
 }
 
 int32_t* gram_status_word(gram_ctx* ctx) { return ctx->d_status; }
+int32_t gram_cluster_blocks(const gram_ctx* ctx) { return ctx->cluster_blocks; }
 int32_t gram_ring_rows(const gram_ctx* ctx) { return ctx->ring_rows; }
 
 void gram_prof_open(gram_ctx* ctx, int kind, const char* tag, double work, int launches, cudaStream_t st, int* slot) {
@@ -139,6 +141,7 @@ gram_status gram_create(const gram_config* cfg, gram_ctx** out) {
     int32_t n_keys = cfg->n_items > cfg->vocab ? cfg->n_items : cfg->vocab;
     s = index_ws_alloc(ctx, &ctx->iws, P_max, n_keys, d_max);
     if (s != GRAM_OK) break;
+    ctx->cluster_blocks = index_cluster_blocks();
     {  // split-K partial products: up to 16 parts of the largest weight matrix, within 32..256 MB
       size_t w = (size_t)(cfg->d_ff > cfg->task_d_ff ? cfg->d_ff : cfg->task_d_ff) * (size_t)cfg->d * sizeof(float) * 16;
       if (w < ((size_t)32 << 20)) w = (size_t)32 << 20;
@@ -243,6 +246,13 @@ gram_status gram_dedup(gram_ctx* ctx, const int32_t* d_ids, int64_t P, int32_t n
 gram_status gram_selftest_bounded_wait(gram_ctx* ctx, gram_stream stream) {
   if (!ctx) return GRAM_ERR_ARG;
   return dedup_wait_selftest(ctx, &ctx->iws, S(stream));
+}
+gram_status gram_selftest_cluster_blocks(gram_ctx* ctx, int32_t blocks) {
+  if (!ctx) return GRAM_ERR_ARG;
+  const int32_t placed = index_cluster_blocks();
+  ctx->cluster_blocks = placed;
+  while (blocks > 0 && ctx->cluster_blocks > blocks) ctx->cluster_blocks /= 2;
+  return GRAM_OK;
 }
 gram_status gram_selftest_ring_rows(gram_ctx* ctx, int32_t rows) {
   if (!ctx) return GRAM_ERR_ARG;

@@ -548,7 +548,6 @@ __global__ void __launch_bounds__(256) inverse_kernel(const int32_t* __restrict_
 constexpr int CD_THREADS = 512;
 constexpr int CD_WARPS = CD_THREADS / 32;
 constexpr int kClusterMaxBlocks = 16;     // an opt-in above 8
-constexpr int64_t kClusterMaxKeys = (int64_t)kClusterMaxBlocks * CD_THREADS * 8;
 
 __device__ __forceinline__ void cd_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -743,8 +742,8 @@ size_t ctl_words(int64_t P, int max_key_bits) {
     const size_t w = (size_t)d.passes * d.bins;
     if (w > per_tile) per_tile = w;
   }
-  if (p <= kClusterMaxKeys) return (size_t)CTL_WORDS + 2 * RADIX;    // the one-launch form; the self-test
-  return (size_t)CTL_WORDS + per_tile * (size_t)ceil_div64(p, RS_TILE) + rle_words(p);
+  const size_t words = per_tile * (size_t)ceil_div64(p, RS_TILE) + rle_words(p);
+  return (size_t)CTL_WORDS + (words > 2 * RADIX ? words : 2 * RADIX);         // the self-test: two tiles of 256 bins
 }
 size_t totals_smem(const DigitPlan& d, int copies) { return (size_t)d.passes * (1 << d.bits) * copies * sizeof(uint32_t); }
 int totals_copies(const DigitPlan& d) { return d.bins == 256 ? 8 : 4; }
@@ -778,6 +777,29 @@ gram_status index_ws_alloc(gram_ctx* ctx, IndexWorkspace* ws, int64_t P_max, int
     if (dev < 64) attributes_set[dev] = true;
   }
   return GRAM_OK;
+}
+
+// The largest cluster of the widest one-launch form that can be placed now (a process may be limited to a part of the
+// GPU's multiprocessors); the other kernels with clusters ask for less shared memory and fewer threads.
+int32_t index_cluster_blocks() {
+  const ClusterDedup f = cluster_dedup_form(kClusterForms - 1);
+  for (int b = kClusterMaxBlocks; b > 1; b /= 2) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)b);
+    cfg.blockDim = dim3(CD_THREADS);
+    cfg.dynamicSmemBytes = f.smem;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)b;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, f.fn, &cfg) == cudaSuccess && n > 0) return b;
+    (void)cudaGetLastError();
+  }
+  return 1;
 }
 
 void index_ws_free(IndexWorkspace* ws) {
@@ -822,11 +844,11 @@ gram_status dedup_launch(gram_ctx* ctx, IndexWorkspace* ws, const int32_t* d_ids
   const int passes = plan.passes;
   // Up to 65 536 positions: the single launch, with the fewest positions per block.  Against the chain of launches, 10 000
   // items: 16 against 30 us at 25 600 positions, 25 / 33 at 65 536; with twice the positions per block it took 42 us at
-  // 131 072 where the chain takes 35: 16 SMs are then too few.
-  if (P <= kClusterMaxKeys) {
-    int i = 0;
-    while (P > (int64_t)kClusterMaxBlocks * cluster_dedup_form(i).tile) ++i;
-    const ClusterDedup f = cluster_dedup_form(i);
+  // 131 072 where the chain takes 35: 16 SMs are then too few.  Where only smaller clusters can be placed, the line is lower.
+  int form = 0;
+  while (form < kClusterForms && P > (int64_t)gram_cluster_blocks(ctx) * cluster_dedup_form(form).tile) ++form;
+  if (form < kClusterForms) {
+    const ClusterDedup f = cluster_dedup_form(form);
     int blocks = 1;
     while ((int64_t)blocks * f.tile < P) blocks *= 2;
     ProfScope prof(ctx, GRAM_K_DEDUP, (16.0 * passes + 20.0) * (double)P, 1, st);

@@ -1562,7 +1562,8 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     const int64_t blocks = big ? b64 : b32, enough = big ? kNumSMs : 4 * kNumSMs;
     int parts = 1;
     const int sk = big ? F32Cfg<64>::SK : F32Cfg<32>::SK;
-    while (parts < F32_MAX_SPLIT && blocks * parts * 2 <= enough && K >= 64 * parts) parts *= 2;
+    const int most = F32_MAX_SPLIT < gram_cluster_blocks(ctx) ? F32_MAX_SPLIT : gram_cluster_blocks(ctx);
+    while (parts < most && blocks * parts * 2 <= enough && K >= 64 * parts) parts *= 2;
     const int64_t per = ceil_div64(ceil_div64(K, parts), sk) * sk;
     if (ceil_div64(M, big ? 64 : 32) > 65535)
       return gram_set_error(ctx, "gemm: %lld rows are more than an fp32 product takes", (long long)M), GRAM_ERR_UNSUPPORTED;

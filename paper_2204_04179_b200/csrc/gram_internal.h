@@ -90,6 +90,7 @@ struct IndexWorkspace {
 
 gram_status index_ws_alloc(gram_ctx* ctx, IndexWorkspace* ws, int64_t P_max, int32_t n_items_max, int32_t d_max);
 void index_ws_free(IndexWorkspace* ws);
+int32_t index_cluster_blocks();                      // asks the device; after index_ws_alloc
 
 gram_status dedup_launch(gram_ctx* ctx, IndexWorkspace* ws, const int32_t* d_ids, int64_t P, int32_t n_items,
                          int32_t* d_unique, int32_t* d_inverse, int32_t* d_perm, int32_t* d_seg_off,
@@ -146,4 +147,5 @@ struct ProfScope {
 // the device status word: kernels record the first error kind they meet
 __device__ __forceinline__ void gram_device_fail(int32_t* status, int32_t code) { atomicCAS(status, 0, code); }
 int32_t* gram_status_word(gram_ctx* ctx);
+int32_t gram_cluster_blocks(const gram_ctx* ctx);   // blocks of the largest cluster that can be placed: 16, 8, 4, 2 or 1
 int32_t gram_ring_rows(const gram_ctx* ctx);   // rows a warp may take from a ring of bulk copies before it gives up; see gram_selftest_ring_rows

@@ -51,3 +51,19 @@ def test_dedup_of_fewer_items_than_the_context_holds():
         for x, w in zip(got, want):
             assert np.array_equal(x, w)
     g.close()
+
+
+@pytest.mark.parametrize("blocks", [8, 4, 2, 1])
+def test_dedup_where_smaller_clusters_are_placed(blocks):
+    """A process limited to part of the multiprocessors: the one-launch form up to 4096 positions per block that can be placed,
+    the chain of launches beyond, also for contexts of few positions."""
+    for P in (3, 4096, 4097, 8192, 25_600, 32_768, 32_769, 65_536):
+        ids = synth.zipf_ids(8, 10_000, 1.0, P)
+        g = index_ctx(P, 10_000, 4)
+        g.selftest_cluster_blocks(blocks)
+        U, *got = run_dedup(g, ids, 10_000)
+        want = orc.unique_inverse(ids)
+        assert U == len(want[0])
+        for x, w in zip(got, want):
+            assert np.array_equal(x, w)
+        g.close()

@@ -1,6 +1,7 @@
 """fp32 contexts at sizes that reach every form of the fp32 matrix product: 32- and 64-wide tiles, the K range in one
 piece and over clusters of up to 16 blocks, rows that allow 16-byte loads and rows that do not."""
 import pytest
+import torch
 
 from oracle import gram_oracle as orc
 from paper_2204_04179_b200 import synth
@@ -26,6 +27,22 @@ def test_f32_step(name):
     want = orc.gram_single_step(shape, ce, tk, toks, ids, lab)
     rep, gce, gtk = gh.gpu_single_step(shape, ce, tk, toks, ids, lab)
     # fp32 sums against 64 bits: 2e-6 is what such models show on their worst tensor; an order of magnitude above it
+    assert abs(rep.loss - want["loss"]) <= 2e-5 * abs(want["loss"])
+    assert gh.worst_rel_err(gce, want["grad_ce"])[0] <= 2e-5
+    assert gh.worst_rel_err(gtk, want["grad_task"])[0] <= 2e-5
+
+
+@pytest.mark.parametrize("blocks", [8, 1])
+def test_f32_step_where_smaller_clusters_are_placed(blocks):
+    shape = synth.GramShape(**dict(dict(name="c", dtype="f32", vocab=50, pooling="mean", task="kt", task_layers=1, task_attn_only=False,
+                                        zipf_s=0.5), **SHAPES["odd_rows"]))
+    ce, tk, toks, ids, lab = gh.make_inputs(shape, seed=4)
+    want = orc.gram_single_step(shape, ce, tk, toks, ids, lab)
+    g = gh.make_ctx(shape, ce, tk, toks)
+    g.selftest_cluster_blocks(blocks)
+    rep = g.step(torch.from_numpy(ids).cuda(), torch.from_numpy(lab).cuda(), ids.shape[0])
+    gce, gtk = gh.gpu_grads(g, shape)
+    g.close()
     assert abs(rep.loss - want["loss"]) <= 2e-5 * abs(want["loss"])
     assert gh.worst_rel_err(gce, want["grad_ce"])[0] <= 2e-5
     assert gh.worst_rel_err(gtk, want["grad_task"])[0] <= 2e-5
