@@ -980,7 +980,17 @@ __global__ void count_real_kernel(const int32_t* __restrict__ labels, int64_t P,
 }
 
 // ---------------------------------------------------------------------------- NR task (per user)
-// pre[b, n, :] = E[b, n, :] wa^T + ba is given.  One block per user.
+// pre[b, n, :] = E[b, n, :] wa^T + ba is given.  One block per user.  What bounds it is the latency of the loads in its chains
+// of additions, so NR_AHEAD of them are fetched before the first is added; left to the compiler, they were after the wait of
+// chain_begin() no longer (the whole module at 64 users x 55 positions 115 us before that wait, 120 with it, 100 this way; at
+// 512 x 55 334, 359 and 313; 4 ahead 102 and 317, 16 ahead 99 and 310).
+constexpr int NR_AHEAD = 8;                      // loads of a chain of additions that are on their way at once
+// x[i] = p[(j + i * by) * stride] for those below `end`, zero for the others
+template <typename T>
+__device__ __forceinline__ void nr_fetch(float (&x)[NR_AHEAD], const T* __restrict__ p, int j, int by, int end, int64_t stride) {
+#pragma unroll
+  for (int i = 0; i < NR_AHEAD; ++i) x[i] = j + i * by < end ? ldf(p + (j + i * by) * stride) : 0.f;
+}
 template <typename T>
 __global__ void __launch_bounds__(256) nr_user_kernel(const float* __restrict__ E, const T* __restrict__ pre,
                                                       const float* __restrict__ qa, float* __restrict__ dE,
@@ -1000,7 +1010,13 @@ __global__ void __launch_bounds__(256) nr_user_kernel(const float* __restrict__ 
   const T* pb = pre + (int64_t)b * L * d_a;
   for (int n = warp; n < n_hist; n += nwb) {
     float acc = 0.f;
-    for (int k = lane; k < d_a; k += 32) acc += qa[k] * tanhf(ldf(pb + (int64_t)n * d_a + k));
+    for (int k0 = lane; k0 < d_a; k0 += 32 * NR_AHEAD) {
+      float x[NR_AHEAD];
+      nr_fetch(x, pb + (int64_t)n * d_a, k0, 32, d_a, 1);
+#pragma unroll
+      for (int i = 0; i < NR_AHEAD; ++i)
+        if (k0 + 32 * i < d_a) acc += qa[k0 + 32 * i] * tanhf(x[i]);
+    }
     acc = warp_sum(acc);
     if (labels && labels[(int64_t)b * L + n] < 0) acc = -INFINITY;       // a slot without a click takes no part
     if (lane == 0) a[n] = acc;
@@ -1020,7 +1036,13 @@ __global__ void __launch_bounds__(256) nr_user_kernel(const float* __restrict__ 
   __syncthreads();
   for (int c = threadIdx.x; c < d; c += blockDim.x) {
     float acc = 0.f;
-    for (int n = 0; n < n_hist; ++n) acc += a[n] * ldf(Eb + (int64_t)n * d + c);
+    for (int n0 = 0; n0 < n_hist; n0 += NR_AHEAD) {
+      float x[NR_AHEAD];
+      nr_fetch(x, Eb + c, n0, 1, n_hist, d);
+#pragma unroll
+      for (int i = 0; i < NR_AHEAD; ++i)
+        if (n0 + i < n_hist) acc += a[n0 + i] * x[i];
+    }
     u[c] = acc;
   }
   __syncthreads();
@@ -1051,7 +1073,13 @@ __global__ void __launch_bounds__(256) nr_user_kernel(const float* __restrict__ 
   __syncthreads();
   for (int n = warp; n < n_hist; n += nwb) {     // d alpha_n = du . h_n
     float acc = 0.f;
-    for (int c = lane; c < d; c += 32) acc += du[c] * ldf(Eb + (int64_t)n * d + c);
+    for (int c0 = lane; c0 < d; c0 += 32 * NR_AHEAD) {
+      float x[NR_AHEAD];
+      nr_fetch(x, Eb + (int64_t)n * d, c0, 32, d, 1);
+#pragma unroll
+      for (int i = 0; i < NR_AHEAD; ++i)
+        if (c0 + 32 * i < d) acc += du[c0 + 32 * i] * x[i];
+    }
     acc = warp_sum(acc);
     if (lane == 0) da[n] = acc;
   }
@@ -1069,14 +1097,21 @@ __global__ void __launch_bounds__(256) nr_user_kernel(const float* __restrict__ 
   }
   for (int k = threadIdx.x; k < d_a; k += blockDim.x) {
     float gq = 0.f;
-    for (int n = 0; n < L; ++n) {
-      float v = 0.f;
-      if (n < n_hist) {
-        const float t = tanhf(ldf(pb + (int64_t)n * d_a + k));
-        gq += da[n] * t;
-        v = da[n] * qa[k] * (1.f - t * t);
+    for (int n0 = 0; n0 < L; n0 += NR_AHEAD) {
+      float x[NR_AHEAD];
+      nr_fetch(x, pb + k, n0, 1, n_hist, d_a);
+#pragma unroll
+      for (int i = 0; i < NR_AHEAD; ++i) {
+        const int n = n0 + i;
+        if (n >= L) break;
+        float v = 0.f;
+        if (n < n_hist) {
+          const float t = tanhf(x[i]);
+          gq += da[n] * t;
+          v = da[n] * qa[k] * (1.f - t * t);
+        }
+        stf(dpre + ((int64_t)b * L + n) * d_a + k, v);
       }
-      stf(dpre + ((int64_t)b * L + n) * d_a + k, v);
     }
     part[(int64_t)b * (d_a + 1) + k] = gq;
   }
