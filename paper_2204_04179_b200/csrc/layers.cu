@@ -980,10 +980,7 @@ __global__ void count_real_kernel(const int32_t* __restrict__ labels, int64_t P,
 }
 
 // ---------------------------------------------------------------------------- NR task (per user)
-// pre[b, n, :] = E[b, n, :] wa^T + ba is given.  One block per user.  What bounds it is the latency of the loads in its chains
-// of additions, so NR_AHEAD of them are fetched before the first is added; left to the compiler, they were after the wait of
-// chain_begin() no longer (the whole module at 64 users x 55 positions 115 us before that wait, 120 with it, 100 this way; at
-// 512 x 55 334, 359 and 313; 4 ahead 102 and 317, 16 ahead 99 and 310).
+// pre[b, n, :] = E[b, n, :] wa^T + ba is given.  One block per user.
 constexpr int NR_AHEAD = 8;                      // loads of a chain of additions that are on their way at once
 // x[i] = p[(j + i * by) * stride] for those below `end`, zero for the others
 template <typename T>

@@ -921,7 +921,7 @@ gram_status model_create(gram_ctx* ctx, const gram_config* cfg, Model** out) {
   m->enc.cap = (int64_t)m->mb * c.l_t;
   m->tk.cap = c.task == GRAM_TASK_NR ? (int64_t)c.B_max * (c.L - c.n_cand) : P;
   m->cls_tail = c.n_layers > 0 && c.pooling == GRAM_POOL_CLS && c.l_t > 1;
-  m->cls_query = m->cls_tail && c.dtype == GRAM_BF16 && attention_cls_supported(c.l_t, c.d, c.n_heads);
+  m->cls_query = m->cls_tail && c.dtype == GRAM_BF16 && !attention_tc_forced() && attention_cls_supported(c.l_t, c.d, c.n_heads);
   if (m->cls_tail) {
     m->tail.d = c.d; m->tail.heads = c.n_heads; m->tail.d_ff = c.d_ff; m->tail.n_layers = 1;
     m->tail.attn_only = 0; m->tail.causal = 0;

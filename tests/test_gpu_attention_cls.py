@@ -1,4 +1,8 @@
 """Token-0 pooling with heads of width 64: the last layer's attention runs with one query row per item."""
+import os
+import subprocess
+import sys
+
 import pytest
 
 from paper_2204_04179_b200 import synth
@@ -25,3 +29,30 @@ def test_many_lengths(l_t):
 
 def test_more_items_than_blocks():
     check_encoder(shape(3, 1, n_items=1300))
+
+
+CHILD = """
+import torch
+from paper_2204_04179_b200 import synth
+from tests import gram_helpers as gh
+from tests.test_gpu_attention_cls import shape
+s = shape(20, 1)
+ce, tk, toks, _, _ = gh.make_inputs(s, seed=6)
+g = gh.make_ctx(s, ce, tk, toks)
+g.profile(True)
+g.encode_unique(None, torch.arange(s.n_items, dtype=torch.int32, device="cuda"), s.n_items, torch.empty(s.n_items, s.d, device="cuda"))
+g.sync()
+print(" ".join(sorted(g.profile_dump())))
+"""
+
+
+@pytest.mark.parametrize("forced", [False, True])
+def test_the_switch_that_forces_the_tcgen05_kernels(forced):
+    """GRAM_ATTN_TC=1 (read once per process) leaves no attention to other kernels, the last layer's included."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = {k: v for k, v in os.environ.items() if k != "GRAM_ATTN_TC"}
+    out = subprocess.run([sys.executable, "-c", CHILD], cwd=root, env=dict(env, GRAM_ATTN_TC="1") if forced else env, capture_output=True,
+                         text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-1000:]
+    tags = out.stdout.split()
+    assert ("attn_cls_fwd" in tags, "attn_fwd" in tags) == (not forced, forced)
