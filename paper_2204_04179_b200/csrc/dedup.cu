@@ -705,6 +705,13 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
     seg_off[U] = P;
   }
   cd_cluster_sync();                                     // nobody leaves while its counts may still be read
+  if (bad) {                                             // an ID out of range belongs to no item, as in inverse_kernel
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+      const int i = lbase + r * 32;
+      if (i < n_valid && (uint32_t)ids[base + i] >= (uint32_t)n_items) inverse[base + i] = -1;
+    }
+  }
 }
 
 typedef void (*ClusterDedupFn)(const int32_t*, int32_t, int32_t, int, int32_t*, int32_t*, int32_t*, int32_t*, int32_t*, int32_t*);

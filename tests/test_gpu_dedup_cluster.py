@@ -2,9 +2,10 @@
 chain of launches: one, two and three passes, the last tile full, one key short, one key long."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import gram_oracle as orc
-from paper_2204_04179_b200 import synth
+from paper_2204_04179_b200 import binding, synth
 from tests.test_gpu_index import index_ctx, run_dedup
 
 pytestmark = pytest.mark.gpu
@@ -67,3 +68,24 @@ def test_dedup_where_smaller_clusters_are_placed(blocks):
         for x, w in zip(got, want):
             assert np.array_equal(x, w)
         g.close()
+
+
+@pytest.mark.parametrize("P", [700, 9000, 40_000, 65_537])
+def test_ids_out_of_range(P):
+    """Both forms report the error, sort such an ID as item 0 and give its positions the index -1."""
+    n = 500
+    ids = synth.zipf_ids(9, n, 1.0, P)
+    ids[::97] = n
+    ids[5::131] = -3
+    bad = (ids < 0) | (ids >= n)
+    unique, inverse, perm, seg = orc.unique_inverse(np.where(bad, 0, ids).astype(np.int32))
+    g = index_ctx(P, n, 4)
+    out = [torch.zeros(k, dtype=torch.int32, device="cuda") for k in (n, P, P, n + 1, 1)]
+    g.dedup(torch.from_numpy(ids).cuda(), n, *out)
+    with pytest.raises(binding.GramError, match="GRAM_ERR_ID_RANGE"):
+        g.sync()
+    U = int(out[4].item())
+    assert U == len(unique) and np.array_equal(out[0][:U].cpu().numpy(), unique)
+    assert np.array_equal(out[1].cpu().numpy(), np.where(bad, -1, inverse))
+    assert np.array_equal(out[2].cpu().numpy(), perm) and np.array_equal(out[3][:U + 1].cpu().numpy(), seg)
+    g.close()
