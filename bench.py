@@ -158,13 +158,21 @@ def stack_flops(tokens, n_layers, d, d_ff, seq, attn_only=False):
     return tokens * n_layers * per_layer
 
 
+def dedup_bytes(P, U, n_items):
+    """Bytes that gram_dedup moves.  Up to 65 536 positions one launch sorts in shared memory: the IDs in, inverse, perm,
+    unique and seg_off out.  Beyond: 16 P per radix pass (10 bits of the key at most), 20 P around them."""
+    if P <= 65_536:
+        return 12 * P + 8 * U
+    passes = (max(1, (n_items - 1).bit_length()) + 9) // 10
+    return (16 * passes + 20) * P + 8 * U
+
+
 def stage_fractions(shape, stage_ms, U, peaks):
     """Algorithmic work of each stage of a Single-step step (fixed-length texts) over its device time, against the
     roofline that bounds it: HBM bytes for dedup, gather and accumulate, bf16 tensor flops for the three model stages.
     With token-0 pooling the row-wise part of the last encoder layer is needed for one row per item only; the flops
     counted are those the method needs, not the ones a plain implementation would spend."""
-    P, d, N = shape.B * shape.L, shape.d, shape.n_items
-    passes = (max(1, (N - 1).bit_length()) + 7) // 8
+    P, d = shape.B * shape.L, shape.d
     T = U * shape.l_t
     enc = stack_flops(T, shape.n_layers, d, shape.d_ff, shape.l_t)
     if shape.pooling == "cls" and shape.n_layers > 0:          # output projection + feed-forward of the last layer: U rows, not T
@@ -173,7 +181,7 @@ def stage_fractions(shape, stage_ms, U, peaks):
         task = 3.0 * stack_flops(P, shape.task_layers, d, shape.task_d_ff, shape.L / 2.0, shape.task_attn_only)   # causal: half the scores
     else:
         task = 3.0 * 2.0 * P * d * shape.d_a
-    work = {"ms_dedup": ((16 * passes + 20) * P + 8 * U, "hbm"),
+    work = {"ms_dedup": (dedup_bytes(P, U, shape.n_items), "hbm"),
             "ms_encode": (enc, "tensor"),
             "ms_gather": (4.0 * P * d + 4.0 * U * d + 4 * P, "hbm"),
             "ms_task": (task, "tensor"),
@@ -227,11 +235,10 @@ def index_cell(binding, synth, torch, dev, P, N, s, d, iters=20, seed=1, peaks=N
             a = torch.cuda.Event(enable_timing=True); b = torch.cuda.Event(enable_timing=True)
             a.record(); fn(); b.record(); torch.cuda.synchronize(); ts.append(a.elapsed_time(b))
         return statistics.median(ts)
-    passes = (max(1, (N - 1).bit_length()) + 7) // 8
     out = {"cell": {"P": P, "n_items": N, "zipf_s": s, "d": d, "U": U, "working_set_MB": (4.0 * P * d + 4.0 * U * d) / 1e6,
                     "l2": "flushed between timed iterations"}}
     for name, fn, nbytes in (
-            ("dedup", lambda: g.dedup(ids, N, unique, inverse, perm, seg, nu), (16 * passes + 20) * P + 8 * U),
+            ("dedup", lambda: g.dedup(ids, N, unique, inverse, perm, seg, nu), dedup_bytes(P, U, N)),
             ("gather_f32", lambda: g.gather(H, inverse, E), 4 * P * d + 4 * U * d + 4 * P),
             ("accumulate", lambda: g.accumulate(dE, perm, seg, U, G), 4 * P * d + 4 * U * d + 4 * P + 4 * (U + 1))):
         ms = timeit(fn)

@@ -858,7 +858,7 @@ gram_status dedup_launch(gram_ctx* ctx, IndexWorkspace* ws, const int32_t* d_ids
     const ClusterDedup f = cluster_dedup_form(form);
     int blocks = 1;
     while ((int64_t)blocks * f.tile < P) blocks *= 2;
-    ProfScope prof(ctx, GRAM_K_DEDUP, (16.0 * passes + 20.0) * (double)P, 1, st);
+    ProfScope prof(ctx, GRAM_K_DEDUP, 12.0 * (double)P, 1, st);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(CD_THREADS);

@@ -21,6 +21,15 @@ def test_reference_arm_prints_one_json_line():
     assert d["e2e"]["h2d_bytes_per_step"] == 0 and d["vs_baseline"] is None and "workload" in d["config"]
 
 
+def test_dedup_bytes_follow_the_passes_of_the_sort():
+    """One launch up to 65 536 positions; then as many passes as digits of up to 10 bits make of the largest key."""
+    from bench import dedup_bytes
+    assert dedup_bytes(65_536, 100, 10_000) == 12 * 65_536 + 800
+    P = 1_000_000
+    for n_items, passes in ((1, 1), (1024, 1), (1025, 2), (100_000, 2), (1 << 20, 2), ((1 << 20) + 1, 3)):
+        assert dedup_bytes(P, 7, n_items) == (16 * passes + 20) * P + 56
+
+
 def test_other_ranks_of_the_reference_arm_do_no_work():
     env = dict(os.environ, RANK="1", WORLD_SIZE="2")
     out = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--workload", "tiny",
