@@ -29,8 +29,12 @@ def test_segment_sums_of_wide_rows(P, d, kind):
     g.close()
     assert torch.equal(out[0], out[1])                        # bit-identical from call to call
     want = torch.zeros(U, d, dtype=torch.float64, device="cuda")
-    n = torch.diff(s.long())
-    want.index_add_(0, torch.repeat_interleave(torch.arange(U, device="cuda"), n), x[p.long()].double())
-    # n terms of at most 1 in fp32: below n * 2^-24 * n, and a unit roundoff of the result
-    tol = (n.double() ** 2 * 2.0 ** -24 + 1e-6)[:, None]
-    assert ((out[0].double() - want).abs() <= tol).all()
+    size = torch.zeros_like(want)
+    item = torch.repeat_interleave(torch.arange(U, device="cuda"), torch.diff(s.long()))
+    want.index_add_(0, item, x[p.long()].double())
+    size.index_add_(0, item, x[p.long()].double().abs())
+    # a sum is a chain of at most one chunk's rows, then of an eighth of the chunks' parts, then of eight: 2^-24 of what has
+    # been added for each link (for one item of 50 003 rows 0.5, where a chunk's part is about 3)
+    chunks = min(-(-P // 16), 148 * 16)
+    links = -(-P // chunks) + -(-chunks // 8) + 8
+    assert ((out[0].double() - want).abs() <= links * 2.0 ** -24 * size + 1e-6).all()

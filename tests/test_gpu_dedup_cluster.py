@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("kind", ["zipf", "same", "descending"])
-@pytest.mark.parametrize("P", [2, 511, 513, 8192, 8193, 16_385, 65_537, 131_071, 131_072, 131_073])
+@pytest.mark.parametrize("P", [2, 511, 513, 8192, 8193, 16_385, 32_768, 32_769, 40_001, 65_535, 65_536, 65_537, 131_072, 131_073])
 def test_dedup_at_tile_and_cluster_edges(P, kind):
     n = {"zipf": 70_001, "same": 300, "descending": P}[kind]
     ids = {"zipf": lambda: synth.zipf_ids(5, n, 1.0, P), "same": lambda: np.full(P, n - 1, np.int32),

@@ -239,7 +239,7 @@ def test_largest_sweep_cell(s):
 
 
 def test_a_wait_that_nothing_satisfies_ends_with_a_status():
-    """The look-back of the dedup's run-length kernel, started as a tile whose predecessor never runs, gives up after its
+    """The look-back of a sort pass of the dedup, started as a tile whose predecessor never runs, gives up after its
     poll limit: the host reads GRAM_ERR_TIMEOUT, nothing faults, and the context keeps working."""
     import time
     g = index_ctx(4096, 100)
