@@ -10,7 +10,7 @@
 // The second walk computes S and dP again (14 S^2 dh flops instead of 10), which costs less than passing P and dS
 // between warps would: no tile leaves a warp, there is one barrier after the loads, and several blocks fit an SM.
 // Chunks stop at the sequence's last 16 rows (and at the diagonal of causal launches), so a text of 147 tokens costs
-// 147 rows where 128-row tensor-memory tiles cost 256: 364 -> 152 us forward, 936 -> 516 us backward per layer of 54 000
+// 160 rows where 128-row tensor-memory tiles cost 256: 364 -> 152 us forward, 936 -> 516 us backward per layer of 54 000
 // such rows.  What bounds them now is the shared-memory traffic of the fragments (two B fragments per 16 x 16 x 16 product).
 #include "layers.h"
 #include "warp_mma.cuh"

@@ -980,7 +980,10 @@ __global__ void count_real_kernel(const int32_t* __restrict__ labels, int64_t P,
 }
 
 // ---------------------------------------------------------------------------- NR task (per user)
-// pre[b, n, :] = E[b, n, :] wa^T + ba is given.  One block per user.
+// pre[b, n, :] = E[b, n, :] wa^T + ba is given.  One block per user.  What bounds it is the latency of the loads in its chains
+// of additions, so NR_AHEAD of them are fetched before the first is added.  The compiler did some of that by itself until
+// the kernel began with chain_begin()'s wait: the whole task module at 64 users x 55 positions took 115 us, then 120, and
+// 100 this way; at 512 x 55 334, 359 and 313 (4 ahead: 102 and 317; 16: 99 and 310).
 constexpr int NR_AHEAD = 8;                      // loads of a chain of additions that are on their way at once
 // x[i] = p[(j + i * by) * stride] for those below `end`, zero for the others
 template <typename T>
