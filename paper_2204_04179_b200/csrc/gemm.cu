@@ -1425,7 +1425,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
 
 // C(m, n) = sum over splits of part[s](m, n), in ascending s; then the epilogue.  Four columns per thread (N is a multiple of
 // 8), four splits' loads on their way at once; PLAIN: the only epilogue is "add to fp32 C" or none (weight gradients).
-// 3072 x 768 from six parts: 21 us with a column per thread and split after split.
+// 3072 x 768 from six parts: 21 us with a column per thread and split after split, 13 this way (from a cold L2).
 template <typename CT, bool PLAIN>
 __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restrict__ part, int splits, int64_t split_stride, int64_t M,
                                                            int N, CT* C, int64_t ldc, EpiDev e) {
