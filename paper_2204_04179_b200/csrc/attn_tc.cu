@@ -371,36 +371,40 @@ __global__ void __launch_bounds__(ATT_THREADS, 1) attn_tc_fwd_kernel(const __gri
 
   if (warp == 0) {
     // ------------------------------ bulk tensor copies ------------------------------
-    if (lane == 0) {
-      int64_t n = 0;
-      for (int64_t it = blockIdx.x; it < a.n_items && !failed; it += gridDim.x) {
-        const Item x = item_of(a, it);
-        for (int j = 0; j < x.nk; ++j, ++n) {
-          const int s = (int)(n % FWD_STAGES);
-          if (!mbar_wait(empty_bar(s), (uint32_t)((n / FWD_STAGES) & 1) ^ 1u, abort_flag)) { failed = true; break; }
+    int64_t n = 0;
+    for (int64_t it = blockIdx.x; it < a.n_items && !failed; it += gridDim.x) {
+      const Item x = item_of(a, it);
+      for (int j = 0; j < x.nk; ++j, ++n) {
+        const int s = (int)(n % FWD_STAGES);
+        if (!mbar_wait_warp(empty_bar(s), (uint32_t)((n / FWD_STAGES) & 1) ^ 1u, abort_flag)) { failed = true; break; }
+        const uint32_t st = tiles + s * FWD_STAGE_BYTES;
+        if (elect_one()) {
           mbar_expect_tx(full_bar(s), FWD_STAGE_BYTES);
-          const uint32_t st = tiles + s * FWD_STAGE_BYTES;
           load_tile(a, &tm_qkv, st, x.h * DH, x, x.qt, full_bar(s));
           load_tile(a, &tm_qkv, st + TILE_BYTES, a.d + x.h * DH, x, j, full_bar(s));
           load_tile(a, &tm_qkv, st + 2 * TILE_BYTES, 2 * a.d + x.h * DH, x, j, full_bar(s));
         }
+        __syncwarp();
       }
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issue ------------------------------
-    if (lane == 0) {
+    {
       int64_t n = 0, ord = 0;
       int pend_stage[2] = {-1, -1};
       bool pend_acc[2] = {false, false};
       uint32_t pcount[2] = {0, 0};
       auto issue_pv = [&](int g) -> bool {
-        if (!mbar_wait(pfull_bar(g), pcount[g] & 1u, abort_flag)) return false;
+        if (!mbar_wait_warp(pfull_bar(g), pcount[g] & 1u, abort_flag)) return false;
         ++pcount[g];
         tc_fence_after();
         const uint32_t st = tiles + pend_stage[g] * FWD_STAGE_BYTES;
-        mma_k_mn(tmem_base + 256u + 64u * g, pbuf + g * P_BYTES, st + 2 * TILE_BYTES, pend_acc[g]);
-        tc_commit(pvdone_bar(g));
-        tc_commit(empty_bar(pend_stage[g]));
+        if (elect_one()) {
+          mma_k_mn(tmem_base + 256u + 64u * g, pbuf + g * P_BYTES, st + 2 * TILE_BYTES, pend_acc[g]);
+          tc_commit(pvdone_bar(g));
+          tc_commit(empty_bar(pend_stage[g]));
+        }
+        __syncwarp();
         pend_stage[g] = -1;
         return true;
       };
@@ -416,11 +420,14 @@ __global__ void __launch_bounds__(ATT_THREADS, 1) attn_tc_fwd_kernel(const __gri
           // that only the item after this one releases.
           if (j == 1 && x.nk >= FWD_STAGES && pend_stage[g ^ 1] >= 0 && !issue_pv(g ^ 1)) { failed = true; break; }
           const int s = (int)(n % FWD_STAGES);
-          if (!mbar_wait(full_bar(s), (uint32_t)((n / FWD_STAGES) & 1), abort_flag)) { failed = true; break; }
+          if (!mbar_wait_warp(full_bar(s), (uint32_t)((n / FWD_STAGES) & 1), abort_flag)) { failed = true; break; }
           tc_fence_after();
           const uint32_t st = tiles + s * FWD_STAGE_BYTES;
-          mma_kk(tmem_base + 128u * g, st, st + TILE_BYTES, 128, 4, false);          // S = Q K^T
-          tc_commit(sfull_bar(g));
+          if (elect_one()) {
+            mma_kk(tmem_base + 128u * g, st, st + TILE_BYTES, 128, 4, false);          // S = Q K^T
+            tc_commit(sfull_bar(g));
+          }
+          __syncwarp();
           pend_stage[g] = s;
           pend_acc[g] = j > 0;
         }
@@ -681,26 +688,27 @@ __global__ void __launch_bounds__(ATT_THREADS, 1) attn_tc_bwd_kernel(const __gri
 
   if (warp == 0) {
     // ------------------------------ bulk tensor copies ------------------------------
-    if (lane == 0) {
-      int64_t n = 0;
-      for (int64_t it = blockIdx.x; it < a.n_items && !failed; it += gridDim.x) {
-        const BwdItem y = bwd_item_of(b, it);
-        for (int t = 0; t < y.n; ++t, ++n) {
-          const int qi = b.mode == 1 ? y.first + t : y.x.qt, kj = b.mode == 2 ? t : y.x.qt;
-          const int s = (int)(n % BWD_STAGES);
-          if (!mbar_wait(empty_bar(s), (uint32_t)((n / BWD_STAGES) & 1) ^ 1u, abort_flag)) { failed = true; break; }
+    int64_t n = 0;
+    for (int64_t it = blockIdx.x; it < a.n_items && !failed; it += gridDim.x) {
+      const BwdItem y = bwd_item_of(b, it);
+      for (int t = 0; t < y.n; ++t, ++n) {
+        const int qi = b.mode == 1 ? y.first + t : y.x.qt, kj = b.mode == 2 ? t : y.x.qt;
+        const int s = (int)(n % BWD_STAGES);
+        if (!mbar_wait_warp(empty_bar(s), (uint32_t)((n / BWD_STAGES) & 1) ^ 1u, abort_flag)) { failed = true; break; }
+        const uint32_t st = tiles + s * BWD_STAGE_BYTES;
+        if (elect_one()) {
           mbar_expect_tx(full_bar(s), BWD_STAGE_BYTES);
-          const uint32_t st = tiles + s * BWD_STAGE_BYTES;
           load_tile(a, &tm_qkv, st, y.x.h * DH, y.x, qi, full_bar(s));
           load_tile(a, &tm_qkv, st + TILE_BYTES, a.d + y.x.h * DH, y.x, kj, full_bar(s));
           load_tile(a, &tm_qkv, st + 2 * TILE_BYTES, 2 * a.d + y.x.h * DH, y.x, kj, full_bar(s));
           load_tile(a, &tm_do, st + 3 * TILE_BYTES, y.x.h * DH, y.x, qi, full_bar(s));
         }
+        __syncwarp();
       }
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issue ------------------------------
-    if (lane == 0) {
+    {
       int64_t n = 0, ord = 0;
       uint32_t steps[2] = {0, 0}, items[2] = {0, 0};
       int prev_g = -1;
@@ -711,27 +719,36 @@ __global__ void __launch_bounds__(ATT_THREADS, 1) attn_tc_bwd_kernel(const __gri
         ++ord;
         for (int t = 0; t < y.n; ++t, ++n) {
           const int s = (int)(n % BWD_STAGES);
-          if (!mbar_wait(full_bar(s), (uint32_t)((n / BWD_STAGES) & 1), abort_flag)) { failed = true; break; }
+          if (!mbar_wait_warp(full_bar(s), (uint32_t)((n / BWD_STAGES) & 1), abort_flag)) { failed = true; break; }
           tc_fence_after();
           const uint32_t st = tiles + s * BWD_STAGE_BYTES;
-          mma_kk(tmem_base, st, st + TILE_BYTES, 128, 4, false);                                   // S = Q K^T
-          mma_kk(tmem_base + 128u, st + 3 * TILE_BYTES, st + 2 * TILE_BYTES, 128, 4, false);      // dP = dO V^T
-          tc_commit(sdp_bar(g));
-          if (!mbar_wait(pds_bar(g), steps[g] & 1u, abort_flag)) { failed = true; break; }
+          if (elect_one()) {
+            mma_kk(tmem_base, st, st + TILE_BYTES, 128, 4, false);                                   // S = Q K^T
+            mma_kk(tmem_base + 128u, st + 3 * TILE_BYTES, st + 2 * TILE_BYTES, 128, 4, false);      // dP = dO V^T
+            tc_commit(sdp_bar(g));
+          }
+          __syncwarp();
+          if (!mbar_wait_warp(pds_bar(g), steps[g] & 1u, abort_flag)) { failed = true; break; }
           ++steps[g];
           if (t == 0 && prev_g >= 0) {             // the previous item's results have been read out of tensor memory
-            if (!mbar_wait(outfree_bar(prev_g), (items[prev_g] - 1) & 1u, abort_flag)) { failed = true; break; }
+            if (!mbar_wait_warp(outfree_bar(prev_g), (items[prev_g] - 1) & 1u, abort_flag)) { failed = true; break; }
           }
           tc_fence_after();
-          if (want_kv) {
-            mma_mn_mn(tmem_base + 256u, pbuf, st + 3 * TILE_BYTES, t > 0);                        // dV += P^T dO
-            mma_mn_mn(tmem_base + 320u, dsbuf, st, t > 0);                                        // dK += dS^T Q
+          const bool last = t + 1 == y.n;
+          if (elect_one()) {
+            if (want_kv) {
+              mma_mn_mn(tmem_base + 256u, pbuf, st + 3 * TILE_BYTES, t > 0);                      // dV += P^T dO
+              mma_mn_mn(tmem_base + 320u, dsbuf, st, t > 0);                                      // dK += dS^T Q
+            }
+            if (want_q) mma_k_mn(tmem_base + 384u, dsbuf, st + TILE_BYTES, t > 0);                // dQ += dS K
+            if (last) {
+              tc_commit(outfull_bar(g));
+            } else {
+              for (int k4 = 0; k4 < 4; ++k4) tc_commit(empty_bar(s));   // the stage is free once these products are done
+            }
           }
-          if (want_q) mma_k_mn(tmem_base + 384u, dsbuf, st + TILE_BYTES, t > 0);                  // dQ += dS K
-          if (t + 1 < y.n) {
-            for (int k4 = 0; k4 < 4; ++k4) tc_commit(empty_bar(s));   // the stage is free once these products are done
-          } else {
-            tc_commit(outfull_bar(g));
+          __syncwarp();
+          if (last) {
             ++items[g];
             prev_g = g;
           }

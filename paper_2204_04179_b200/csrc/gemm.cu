@@ -791,18 +791,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gemm_tc_kernel(const __grid_con
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
-    if (lane == 0) {
-      int s = 0;
-      uint32_t ph = 0;
-      for (int64_t t = blockIdx.x; t < total && !failed; t += gridDim.x) {
-        const int split = (int)(t / ((int64_t)a.n_tiles_m * a.n_tiles_n));
-        const int64_t r = t - (int64_t)split * a.n_tiles_m * a.n_tiles_n;
-        const int tm = (int)(r / a.n_tiles_n), tn = (int)(r % a.n_tiles_n);
-        const int kb0 = split * a.kb_per_split, kb1 = min(kb0 + a.kb_per_split, a.num_kb);
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { failed = true; break; }
+    int s = 0;
+    uint32_t ph = 0;
+    for (int64_t t = blockIdx.x; t < total && !failed; t += gridDim.x) {
+      const int split = (int)(t / ((int64_t)a.n_tiles_m * a.n_tiles_n));
+      const int64_t r = t - (int64_t)split * a.n_tiles_m * a.n_tiles_n;
+      const int tm = (int)(r / a.n_tiles_n), tn = (int)(r % a.n_tiles_n);
+      const int kb0 = split * a.kb_per_split, kb1 = min(kb0 + a.kb_per_split, a.num_kb);
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag)) { failed = true; break; }
+        const uint32_t sa = tiles + s * Cfg::STAGE_BYTES, sb = sa + Cfg::A_BYTES;
+        if (elect_one()) {
           mbar_expect_tx(full_bar(s), Cfg::STAGE_BYTES);
-          const uint32_t sa = tiles + s * Cfg::STAGE_BYTES, sb = sa + Cfg::A_BYTES;
           if (A_K) {
             tma_load_2d(sa, &tmA, kb * BK, tm * BM, full_bar(s));
           } else {
@@ -815,33 +815,34 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gemm_tc_kernel(const __grid_con
 #pragma unroll
             for (int i = 0; i < BN / 64; ++i) tma_load_2d(sb + i * 8192, &tmB, tn * BN + i * 64, kb * BK, full_bar(s));
           }
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
+        __syncwarp();
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
-      if (failed) {
-        *abort_flag = 1;
-        gram_device_fail(a.status, GRAM_ERR_TIMEOUT);
-      }
+    }
+    if (failed && lane == 0) {
+      *abort_flag = 1;
+      gram_device_fail(a.status, GRAM_ERR_TIMEOUT);
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer --------------------------------
-    if (lane == 0) {
-      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_K ? 0u : 1u) << 15) |
-                                 ((B_K ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-      int s = 0;
-      uint32_t ph = 0;
-      int64_t it = 0;
-      for (int64_t t = blockIdx.x; t < total && !failed; t += gridDim.x, ++it) {
-        const int split = (int)(t / ((int64_t)a.n_tiles_m * a.n_tiles_n));
-        const int kb0 = split * a.kb_per_split, kb1 = min(kb0 + a.kb_per_split, a.num_kb);
-        const int buf = (int)(it & 1);
-        if (!mbar_wait(tempty_bar(buf), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag)) { failed = true; break; }
+    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_K ? 0u : 1u) << 15) |
+                               ((B_K ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+    int s = 0;
+    uint32_t ph = 0;
+    int64_t it = 0;
+    for (int64_t t = blockIdx.x; t < total && !failed; t += gridDim.x, ++it) {
+      const int split = (int)(t / ((int64_t)a.n_tiles_m * a.n_tiles_n));
+      const int kb0 = split * a.kb_per_split, kb1 = min(kb0 + a.kb_per_split, a.num_kb);
+      const int buf = (int)(it & 1);
+      if (!mbar_wait_warp(tempty_bar(buf), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag)) { failed = true; break; }
+      tc_fence_after();
+      const uint32_t tmem_d = tmem_base + (uint32_t)(buf * BN);
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait_warp(full_bar(s), ph, abort_flag)) { failed = true; break; }
         tc_fence_after();
-        const uint32_t tmem_d = tmem_base + (uint32_t)(buf * BN);
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(full_bar(s), ph, abort_flag)) { failed = true; break; }
-          tc_fence_after();
-          const uint32_t sa = tiles + s * Cfg::STAGE_BYTES, sb = sa + Cfg::A_BYTES;
+        const uint32_t sa = tiles + s * Cfg::STAGE_BYTES, sb = sa + Cfg::A_BYTES;
+        if (elect_one()) {
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) {
             const uint64_t da = A_K ? make_desc(sa + k * 32, 16, 1024) : make_desc(sa + k * 2048, 8192, 1024);
@@ -849,15 +850,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gemm_tc_kernel(const __grid_con
             tc_mma(tmem_d, da, db, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
           }
           tc_commit(empty_bar(s));            // the stage is free once these MMAs have read it
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
+          if (kb == kb1 - 1) tc_commit(tfull_bar(buf));      // accumulator complete
         }
-        if (failed) break;
-        tc_commit(tfull_bar(buf));            // accumulator complete
+        __syncwarp();
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
-      if (failed) {
-        *abort_flag = 1;
-        gram_device_fail(a.status, GRAM_ERR_TIMEOUT);
-      }
+    }
+    if (failed && lane == 0) {
+      *abort_flag = 1;
+      gram_device_fail(a.status, GRAM_ERR_TIMEOUT);
     }
   } else {
     // ------------------------------ epilogue warps ----------------------------
@@ -920,7 +921,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gemm_tc_kernel(const __grid_con
 // moves 32 KB through shared memory instead of 48 KB, which is what bounds the single-CTA kernel.
 // Protocol: each CTA's TMA loads signal the leader's "full" barrier (two arrivals with their byte
 // counts); the leader's commits arrive on the "empty" and "accumulator full" barriers of both CTAs
-// (one plain commit per CTA); the epilogue warps of both CTAs arrive on the leader's
+// (one commit for the two); the epilogue warps of both CTAs arrive on the leader's
 // "accumulator empty" barrier.  Every wait is bounded as in the single-CTA kernel; the CTAs meet at a
 // cluster barrier before they exit so that neither releases shared or tensor memory the other may
 // still touch.
@@ -951,8 +952,11 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
       "l"(map), "r"(cluster_bar), "r"(c0), "r"(c1)
       : "memory");
 }
-__device__ __forceinline__ void tc_commit_pair(uint32_t cluster_bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(cluster_bar) : "memory");
+// arrives on the barrier at this shared-memory offset in both CTAs of the pair
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+               "h"((uint16_t)3)
+               : "memory");
 }
 __device__ __forceinline__ void tc_mma_pair(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accum) {
   asm volatile(
@@ -1270,22 +1274,22 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
 
   if (warp == 0) {
     // ------------------------------ TMA producer (both CTAs) ------------------------------
-    if (lane == 0) {
-      int s = 0;
-      uint32_t ph = 0;
-      const uint32_t lead_bar0 = map_to_cta(bar0, 0);          // the leader's barrier block, as seen from this CTA
-      for (int64_t t = cluster_id; t < total && !failed; t += n_clusters) {
-        const int split = (int)(t / ((int64_t)a.n_tiles_m * a.n_tiles_n));
-        const int64_t r = t - (int64_t)split * a.n_tiles_m * a.n_tiles_n;
-        const int tm = (int)(r / a.n_tiles_n), tn = (int)(r % a.n_tiles_n);
-        const int kb0 = split * a.kb_per_split, kb1 = min(kb0 + a.kb_per_split, a.num_kb);
-        const int m0 = tm * 2 * BM + (int)rank * BM;            // this CTA's rows of A
-        const int n0 = tn * BN + (int)rank * (BN / 2);          // this CTA's columns of B
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { failed = true; break; }
-          const uint32_t lead_full = lead_bar0 + 8u * s;           // the leader's full_bar(s)
+    int s = 0;
+    uint32_t ph = 0;
+    const uint32_t lead_bar0 = map_to_cta(bar0, 0);          // the leader's barrier block, as seen from this CTA
+    for (int64_t t = cluster_id; t < total && !failed; t += n_clusters) {
+      const int split = (int)(t / ((int64_t)a.n_tiles_m * a.n_tiles_n));
+      const int64_t r = t - (int64_t)split * a.n_tiles_m * a.n_tiles_n;
+      const int tm = (int)(r / a.n_tiles_n), tn = (int)(r % a.n_tiles_n);
+      const int kb0 = split * a.kb_per_split, kb1 = min(kb0 + a.kb_per_split, a.num_kb);
+      const int m0 = tm * 2 * BM + (int)rank * BM;            // this CTA's rows of A
+      const int n0 = tn * BN + (int)rank * (BN / 2);          // this CTA's columns of B
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag)) { failed = true; break; }
+        const uint32_t lead_full = lead_bar0 + 8u * s;           // the leader's full_bar(s)
+        const uint32_t sa = tiles + s * Cfg::STAGE_BYTES, sb = sa + Cfg::A_BYTES;
+        if (elect_one()) {
           mbar_arrive_expect_tx_remote(lead_full, Cfg::STAGE_BYTES);
-          const uint32_t sa = tiles + s * Cfg::STAGE_BYTES, sb = sa + Cfg::A_BYTES;
           if (A_K) {
             tma_load_2d_pair(sa, &tmA, kb * BK, m0, lead_full);
           } else {
@@ -1298,58 +1302,56 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
 #pragma unroll
             for (int i = 0; i < BN / 128; ++i) tma_load_2d_pair(sb + i * 8192, &tmB, n0 + i * 64, kb * BK, lead_full);
           }
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
+        __syncwarp();
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
-      if (failed) {
-        *abort_flag = 1;
-        gram_device_fail(a.status, GRAM_ERR_TIMEOUT);
-      }
+    }
+    if (failed && lane == 0) {
+      *abort_flag = 1;
+      gram_device_fail(a.status, GRAM_ERR_TIMEOUT);
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer (leader CTA only) ----------------------------
-    if (leader && lane == 0) {
+    // What bounded the main loop was this warp's own time per k-block, not its operands: with the copies left out, 643 of 647
+    // cycles per k-block stayed (512 is what the MMAs take), and the wait for the operands was the barrier's latency.  With
+    // the loop run by one lane and a commit per CTA: 65 536 x 2304 x 768 171 us, with all lanes and one commit 150 us
+    // (1540 TFLOP/s); 65 536 x 768 x 3072 with the fp32 residual 242 -> 215 us.
+    // The descriptors of stage 0 are built once: a later stage or k-step only adds to the 14-bit address field, which
+    // cannot overflow inside shared memory.
+    if (leader) {
       constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_K ? 0u : 1u) << 15) |
                                  ((B_K ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
       int s = 0;
       uint32_t ph = 0;
       int64_t it = 0;
-      // This thread shares its scheduler with four busy epilogue warps, so the loop is kept to a few instructions
-      // per k-block: the descriptors of stage 0 are built once (a later stage or k-step only adds to the 14-bit
-      // address field, which cannot overflow inside shared memory), and so are the barrier addresses of both CTAs.
       const uint64_t da0 = A_K ? make_desc(tiles, 16, 1024) : make_desc(tiles, 8192, 1024);
       const uint64_t db0 = B_K ? make_desc(tiles + Cfg::A_BYTES, 16, 1024) : make_desc(tiles + Cfg::A_BYTES, 8192, 1024);
       constexpr uint32_t ka = (A_K ? 32 : 2048) >> 4, kbs = (B_K ? 32 : 2048) >> 4;
-      const uint32_t rbar0 = map_to_cta(bar0, 0), rbar1 = map_to_cta(bar0, 1);
       for (int64_t t = cluster_id; t < total && !failed; t += n_clusters, ++it) {
         const int split = (int)(t / ((int64_t)a.n_tiles_m * a.n_tiles_n));
         const int kb0 = split * a.kb_per_split, kb1 = min(kb0 + a.kb_per_split, a.num_kb);
         const int buf = (int)(it & 1);
-        if (!mbar_wait(tempty_bar(buf), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag)) { failed = true; break; }
+        if (!mbar_wait_warp(tempty_bar(buf), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag)) { failed = true; break; }
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)(buf * BN);
-        uint32_t acc = 0u;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(full_bar(s), ph, abort_flag)) { failed = true; break; }
+          if (!mbar_wait_warp(full_bar(s), ph, abort_flag)) { failed = true; break; }
           tc_fence_after();
           const uint32_t soff = (uint32_t)(s * (Cfg::STAGE_BYTES >> 4));
           const uint64_t da = da0 + soff, db = db0 + soff;
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            tc_mma_pair(tmem_d, da + (uint64_t)(k * ka), db + (uint64_t)(k * kbs), idesc, acc);
-            acc = 1u;
+            for (int k = 0; k < BK / 16; ++k)
+              tc_mma_pair(tmem_d, da + (uint64_t)(k * ka), db + (uint64_t)(k * kbs), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+            tc_commit_pair(empty_bar(s));                      // the stage is free in both CTAs once these MMAs are done
+            if (kb == kb1 - 1) tc_commit_pair(tfull_bar(buf));   // accumulator complete in both CTAs
           }
-          const uint32_t eb = 8u * (uint32_t)(STAGES + s);  // empty_bar(s): the stage is free in both CTAs once these MMAs are done
-          tc_commit_pair(rbar0 + eb);
-          tc_commit_pair(rbar1 + eb);
+          __syncwarp();
           if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
-        if (failed) break;
-        const uint32_t fb = 8u * (uint32_t)(2 * STAGES + buf);   // tfull_bar(buf): accumulator complete in both CTAs
-        tc_commit_pair(rbar0 + fb);
-        tc_commit_pair(rbar1 + fb);
       }
-      if (failed) {
+      if (failed && lane == 0) {
         *abort_flag = 1;
         gram_device_fail(a.status, GRAM_ERR_TIMEOUT);
       }

@@ -48,6 +48,27 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// The same for a whole warp, which leaves as one: every lane gets the same answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  uint64_t t0 = 0;
+  for (uint32_t it = 1;; ++it) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    if ((it & 0xFFF) == 0) {
+      const uint64_t now = clock64();
+      if (t0 == 0) t0 = now;
+      if (__any_sync(0xffffffffu, *abort_flag != 0 || now - t0 > WAIT_LIMIT_CYCLES)) return false;
+    }
+  }
+}
+// One lane of a converged warp.  The warps that issue copies and MMAs run their loops with all lanes and elect one for the
+// issue alone: descriptors, barrier addresses and loop counters are then uniform values, which those instructions take
+// directly, where a loop inside "if (lane == 0)" has to move each of them over first.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int32_t c0, int32_t c1, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
