@@ -966,6 +966,20 @@ __device__ __forceinline__ void tc_mma_pair(uint32_t tmem_d, uint64_t da, uint64
       : "memory");
 }
 
+// 32 columns of a per-column vector from column n (zeros at and past N, or without a vector).  The tests are made once per
+// block of columns, so that the arithmetic on it is one straight line: with a test per four columns a warp had two pairs of
+// values to interleave and waited for their chains.
+__device__ __forceinline__ void load_cols32(const float* __restrict__ p, int n, int N, float4 (&x)[8]) {
+  if (p && n + 32 <= N) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = __ldg(reinterpret_cast<const float4*>(p + n + 4 * j));
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      x[j] = p && n + 4 * j < N ? __ldg(reinterpret_cast<const float4*>(p + n + 4 * j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+
 // Epilogue of the pair kernel for bf16 results (EPI_BIAS, EPI_GELU, EPI_DG): one warp owns rows row0 .. row0+31
 // and NB blocks of 32 columns from global column col0 (tile column c_local).  A thread keeps its own row: 32
 // accumulators from tensor memory per block, the arithmetic, 64 bytes of bf16 written into a 32-row x 64-column
@@ -1003,6 +1017,8 @@ __device__ __forceinline__ bool epilogue_tile_ts(const TcArgs& a, const CUtensor
   for (int b = 0; b < NB; ++b) {
     uint32_t v[32];
     tc_ld32_issue(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + c_local + b * 32), v);
+    float4 bias[MODE == EPI_DG ? 1 : 8];
+    if constexpr (MODE != EPI_DG) load_cols32(a.epi.bias, col0 + b * 32, a.N, bias);
     tc_ld32_wait(v);
     if (b == NB - 1) {                                     // every value of this tile is in registers now
       tc_fence_before();
@@ -1010,7 +1026,6 @@ __device__ __forceinline__ bool epilogue_tile_ts(const TcArgs& a, const CUtensor
       if (lane == 0) mbar_arrive_remote(tempty_remote);
     }
     const int nbx = col0 + (b >> 1) * 64;                  // first column of the box
-    const int n = col0 + b * 32;
     if (nbx >= a.N || !rows_ok) continue;
     const uint32_t p0 = (uint32_t)(b & 1) * 4u;            // this block's first 16-byte piece of the row
     uint32_t oc[16];
@@ -1032,8 +1047,7 @@ __device__ __forceinline__ bool epilogue_tile_ts(const TcArgs& a, const CUtensor
       uint32_t op[MODE == EPI_GELU ? 16 : 1];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (a.epi.bias && n + 4 * j < a.N) b4 = __ldg(reinterpret_cast<const float4*>(a.epi.bias + n + 4 * j));
+        const float4 b4 = bias[j];
         if constexpr (MODE == EPI_GELU) {
           uint64_t g0, g1, d0, d1;
           gelu_pair(f2_add(f2_pack(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1])), f2_pack(b4.x, b4.y)), g0, d0);
@@ -1141,8 +1155,15 @@ __device__ __forceinline__ bool epilogue_tile_res(const TcArgs& a, const CUtenso
   for (int b = 0; b < nv; ++b) {
     const uint32_t k = nb + (uint32_t)b;
     const uint32_t box = sbuf + (k % 3u) * 4096u, srow = box + (uint32_t)lane * 128u;
+    const int n = col0 + b * 32;
     uint32_t v[32];
     tc_ld32_issue(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + c_local + b * 32), v);
+    float4 bias[8], gam[8], bet[8];
+    load_cols32(a.epi.bias, n, a.N, bias);
+    if (ln) {
+      load_cols32(a.epi.res_gamma, n, a.N, gam);
+      load_cols32(a.epi.res_beta, n, a.N, bet);
+    }
     tc_ld32_wait(v);
     if (b == nv - 1) {                                      // every value of this tile is in registers now
       tc_fence_before();
@@ -1150,30 +1171,26 @@ __device__ __forceinline__ bool epilogue_tile_res(const TcArgs& a, const CUtenso
       if (lane == 0) mbar_arrive_remote(tempty_remote);
     }
     if (!mbar_wait(ld_bar0 + 8u * (k % 3u), (k / 3u) & 1u, abort_flag)) return false;
-    const int n = col0 + b * 32;
+    if (ln) {                                               // columns past N: zeros in, and the store clips them
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const uint32_t addr = srow + ((((uint32_t)c) ^ swz) << 4);
-      const uint4 ru = lds128(addr);
-      float x[4] = {__uint_as_float(v[4 * c]), __uint_as_float(v[4 * c + 1]), __uint_as_float(v[4 * c + 2]), __uint_as_float(v[4 * c + 3])};
-      const float r[4] = {__uint_as_float(ru.x), __uint_as_float(ru.y), __uint_as_float(ru.z), __uint_as_float(ru.w)};
-      if (n + 4 * c < a.N) {                                // N is a multiple of 8: a piece of four columns is in or out
-        if (a.epi.bias) {
-          const float4 b4 = __ldg(reinterpret_cast<const float4*>(a.epi.bias + n + 4 * c));
-          x[0] += b4.x; x[1] += b4.y; x[2] += b4.z; x[3] += b4.w;
-        }
-        if (ln) {
-          const float4 g4 = __ldg(reinterpret_cast<const float4*>(a.epi.res_gamma + n + 4 * c));
-          const float4 e4 = __ldg(reinterpret_cast<const float4*>(a.epi.res_beta + n + 4 * c));
-          x[0] += (r[0] - mu) * rs * g4.x + e4.x;
-          x[1] += (r[1] - mu) * rs * g4.y + e4.y;
-          x[2] += (r[2] - mu) * rs * g4.z + e4.z;
-          x[3] += (r[3] - mu) * rs * g4.w + e4.w;
-        } else {
-          x[0] += r[0]; x[1] += r[1]; x[2] += r[2]; x[3] += r[3];
-        }
+      for (int c = 0; c < 8; ++c) {
+        const uint32_t addr = srow + ((((uint32_t)c) ^ swz) << 4);
+        const uint4 r = lds128(addr);
+        sts128(addr, __float_as_uint(__uint_as_float(v[4 * c]) + bias[c].x + ((__uint_as_float(r.x) - mu) * rs * gam[c].x + bet[c].x)),
+               __float_as_uint(__uint_as_float(v[4 * c + 1]) + bias[c].y + ((__uint_as_float(r.y) - mu) * rs * gam[c].y + bet[c].y)),
+               __float_as_uint(__uint_as_float(v[4 * c + 2]) + bias[c].z + ((__uint_as_float(r.z) - mu) * rs * gam[c].z + bet[c].z)),
+               __float_as_uint(__uint_as_float(v[4 * c + 3]) + bias[c].w + ((__uint_as_float(r.w) - mu) * rs * gam[c].w + bet[c].w)));
       }
-      sts128(addr, __float_as_uint(x[0]), __float_as_uint(x[1]), __float_as_uint(x[2]), __float_as_uint(x[3]));
+    } else {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const uint32_t addr = srow + ((((uint32_t)c) ^ swz) << 4);
+        const uint4 r = lds128(addr);
+        sts128(addr, __float_as_uint(__uint_as_float(v[4 * c]) + bias[c].x + __uint_as_float(r.x)),
+               __float_as_uint(__uint_as_float(v[4 * c + 1]) + bias[c].y + __uint_as_float(r.y)),
+               __float_as_uint(__uint_as_float(v[4 * c + 2]) + bias[c].z + __uint_as_float(r.z)),
+               __float_as_uint(__uint_as_float(v[4 * c + 3]) + bias[c].w + __uint_as_float(r.w)));
+      }
     }
     fence_proxy_async_smem();
     __syncwarp();
