@@ -199,15 +199,28 @@ __device__ __forceinline__ int2 scan_pair(int a, int b, int32_t (*sw)[16]) {
   return make_int2(pa + ia - a, pb + ib - b);
 }
 
+// How the lanes of a round with equal digits find each other.  One vote per digit bit costs about three instructions a bit; an
+// OR of the lane's bit into the digit's word of the warp's own table costs the same for any width, but the lanes of one
+// digit follow each other, so it is for passes of MATCH_BITS bits and more.  10^7 positions of 20-bit keys, both passes:
+// 204 us with ten votes a key, 181 this way.
+constexpr int MATCH_BITS = 8;
+
 template <int BINS> struct PassSmem {
   uint16_t cnt[RS_WARPS][BINS];    // keys of (warp, digit); later the warp's base inside the tile's digit run
   int32_t tile_excl[BINS];         // start of a digit's run inside the reordered tile
   int32_t gbase[BINS];             // global position of reordered element i of digit g is gbase[g] + i
   int32_t scan_w[2][16];
   int32_t tile, abort;
-  int32_t keys[RS_TILE];
-  int32_t vals[RS_TILE];
+  union alignas(16) {              // cleared by 16-byte stores
+    struct {
+      int32_t keys[RS_TILE];
+      int32_t vals[RS_TILE];
+    };
+    uint32_t match[RS_WARPS][BINS];  // before the reordering: lanes of the current round per (warp, digit); zeros between rounds
+  };
 };
+static_assert(alignof(PassSmem<256>) == 16 && alignof(PassSmem<RADIX_MAX>) == 16, "the match tables start on 16 bytes");
+static_assert(sizeof(uint32_t) * RS_WARPS * RADIX_MAX <= 2 * sizeof(int32_t) * RS_TILE, "the match tables fit the reordered tile");
 
 // ---- one stable radix pass ------------------------------------------------------------------
 // Warp w of a tile owns 32*RS_ITEMS consecutive keys and visits them 32 at a time, so that
@@ -242,21 +255,30 @@ __device__ __forceinline__ void radix_tile(PassSmem<(NBITS <= 8 ? 256 : 1024)>& 
   for (int r = 0; r < RS_ITEMS; ++r) {
     const bool valid = FULL || lbase + r * 32 < n_valid;
     const uint32_t dig = ((uint32_t)key[r] >> shift) & MASK;
-    // lanes of this round with the same digit: one vote per digit bit that can be set in this pass (a fixed cost,
-    // unlike a hardware match, whose latency grows with the number of distinct values)
-    uint32_t peers = FULL ? 0xffffffffu : __ballot_sync(0xffffffffu, valid);
-#pragma unroll
-    for (int b = 0; b < NBITS; ++b) {
-      const bool bit = (dig >> b) & 1u;
-      const uint32_t vote = __ballot_sync(0xffffffffu, bit);
-      peers &= vote ^ (bit ? 0u : 0xffffffffu);
-    }
+    // lanes of this round with the same digit (a hardware match's latency grows with the number of distinct values)
+    uint32_t peers;
     int32_t before = 0;
+    if constexpr (NBITS >= MATCH_BITS) {
+      if (valid) atomicOr(&s.match[warp][dig], 1u << lane);
+      __syncwarp();
+      peers = s.match[warp][dig];
+    } else {
+      peers = FULL ? 0xffffffffu : __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+      for (int b = 0; b < NBITS; ++b) {
+        const bool bit = (dig >> b) & 1u;
+        const uint32_t vote = __ballot_sync(0xffffffffu, bit);
+        peers &= vote ^ (bit ? 0u : 0xffffffffu);
+      }
+    }
     if (valid) before = my_cnt[dig];
     __syncwarp();
     const uint32_t earlier = peers & lt;
     pos[r] = before + __popc(earlier);
-    if (valid && earlier == 0u) my_cnt[dig] = (uint16_t)(before + __popc(peers));
+    if (valid && earlier == 0u) {
+      my_cnt[dig] = (uint16_t)(before + __popc(peers));
+      if constexpr (NBITS >= MATCH_BITS) s.match[warp][dig] = 0u;
+    }
     __syncwarp();
   }
   __syncthreads();
@@ -353,6 +375,9 @@ __global__ void __launch_bounds__(RS_THREADS, 2) radix_pass_kernel(const int32_t
     s.abort = 0;
   }
   for (int i = threadIdx.x; i < RS_WARPS * BINS / 2; i += RS_THREADS) reinterpret_cast<uint32_t*>(&s.cnt[0][0])[i] = 0u;
+  if constexpr (NBITS >= MATCH_BITS) {
+    for (int i = threadIdx.x; i < RS_WARPS * BINS / 4; i += RS_THREADS) reinterpret_cast<uint4*>(&s.match[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+  }
   __syncthreads();
   const int tile = s.tile;
   const int64_t tbase = (int64_t)tile * RS_TILE, left = P - tbase;
@@ -385,7 +410,7 @@ RadixPassFn radix_pass_fn(int nbits) {
 size_t radix_pass_smem(int nbits) { return nbits <= 8 ? sizeof(PassSmem<256>) : sizeof(PassSmem<1024>); }
 
 // Passes of the sort over keys of `key_bits` bits: as few as 10-bit digits allow, the bits spread evenly.  Two passes over
-// 1024 bins take 107 + 102 us at 10^7 positions of 20-bit keys, where three over 256 bins took 95 + 89 + 73.
+// 1024 bins took 107 + 102 us at 10^7 positions of 20-bit keys (with votes), where three over 256 bins took 95 + 89 + 73.
 struct DigitPlan {
   int passes, bits, bins;
 };
