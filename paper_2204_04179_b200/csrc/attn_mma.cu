@@ -331,11 +331,15 @@ __global__ void __launch_bounds__(NW * 32) attn_bwd_mma_kernel(const bf16* __res
   }
 }
 
+// Warps per block: one 16-row tile each.  Up to 32 rows that is two; with four, half of them only copied, while their registers
+// kept other blocks off the SM (42 500 rows of 32-token texts, width 768: backward 185 -> 113 us, forward 57 -> 48).
+constexpr int attn_warps(int SP) { return SP >= 96 ? 8 : SP / 16; }
+
 template <int SP, int DH>
 gram_status launch_fwd(gram_ctx* ctx, const bf16* qkv, bf16* out, int64_t n_seq, int S, int d, int n_heads, int causal,
                        const int32_t* seq_len, const int32_t* seq_off, const int32_t* seq_list, cudaStream_t st) {
   constexpr size_t smem = (size_t)3 * SP * (DH + 8) * 2;
-  constexpr int NW = SP >= 96 ? 8 : 4;                // one 16-row query tile per warp up to 128 rows
+  constexpr int NW = attn_warps(SP);
   auto kern = causal ? attn_fwd_mma_kernel<SP, DH, NW, true> : attn_fwd_mma_kernel<SP, DH, NW, false>;
   if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   launch_chain(kern, (unsigned)(n_seq * n_heads), NW * 32, smem, st, qkv, out, S, d, n_heads, causal, 1.f / sqrtf((float)DH), seq_len, seq_off, seq_list);
@@ -348,7 +352,7 @@ gram_status launch_bwd(gram_ctx* ctx, const bf16* qkv, const bf16* dctx, bf16* d
                        cudaStream_t st) {
   constexpr size_t smem = ((size_t)4 * SP * (DH + 8) + (size_t)2 * SP * (SP + 8)) * 2;
   static_assert(smem <= 227 * 1024, "attention backward tile exceeds shared memory");
-  constexpr int NW = SP >= 96 ? 8 : 4;
+  constexpr int NW = attn_warps(SP);
   auto kern = causal ? attn_bwd_mma_kernel<SP, DH, NW, true> : attn_bwd_mma_kernel<SP, DH, NW, false>;
   if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   launch_chain(kern, (unsigned)(n_seq * n_heads), NW * 32, smem, st, qkv, dctx, dqkv, colpart, S, d, n_heads, causal, 1.f / sqrtf((float)DH), seq_len, seq_off, seq_list);
