@@ -30,10 +30,11 @@ struct StreamRef {
 // tok_ids[t] = token(t).  items == null means items[u] = first_item + u.  seq_len / seq_off (both or neither): packed
 // rows for texts of different lengths: item u's tokens 0 .. seq_len[u]-1 go to rows seq_off[u] .. and its padding
 // slots get no row at all.
-gram_status embed_forward(gram_ctx* ctx, const int32_t* item_tokens, const int32_t* items, int32_t first_item,
-                          int32_t n_items_chunk, int32_t n_items_total, int l_t, int vocab, int d, const float* tok_emb,
-                          const float* pos_emb, float* z0, int32_t* tok_ids, const int32_t* seq_len, const int32_t* seq_off,
-                          cudaStream_t st);
+gram_status embed_layernorm_forward(gram_ctx* ctx, int dtype, const int32_t* item_tokens, const int32_t* items, int32_t first_item,
+                                    int32_t n_chunk, int32_t n_items_total, int l_t, int vocab, int d, const float* tok_emb,
+                                    const float* pos_emb, const float* gamma, const float* beta, float* z0, int32_t* tok_ids,
+                                    void* x0, float* mean, float* rstd, const int32_t* seq_len, const int32_t* seq_off,
+                                    cudaStream_t st);
 // seq_len[u] = item_len[item(u)] for the n items of an encoder pass and seq_off = its exclusive prefix sum
 // (seq_off[n] = rows in total)
 // Also: group_list [n] = the sequence numbers grouped by length (SeqGroups), info[0..3] = the size of each group,

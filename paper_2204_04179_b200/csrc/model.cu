@@ -573,10 +573,9 @@ gram_status encoder_forward_chunk(Model* m, const int32_t* d_item_tokens, const 
   m->enc.packed_rows = seq_off ? T : 0;
   m->enc.grouped = seq_off != nullptr;
   m->saved_rows = T;
-  GRAM_TRY(embed_forward(ctx, d_item_tokens ? d_item_tokens : m->item_tokens, d_items, first_item, n, c.n_items, c.l_t,
-                         c.vocab, c.d, m->ce.w + m->o_tok, m->ce.w + m->o_pos, m->z0, m->tok_ids, seq_len, seq_off, st));
-  GRAM_TRY(layernorm_forward(ctx, m->dtype, m->z0, m->ce.w + m->o_elng, m->ce.w + m->o_elnb, m->x0, m->mean0, m->rstd0, T,
-                             c.d, st));
+  GRAM_TRY(embed_layernorm_forward(ctx, m->dtype, d_item_tokens ? d_item_tokens : m->item_tokens, d_items, first_item, n,
+                                   c.n_items, c.l_t, c.vocab, c.d, m->ce.w + m->o_tok, m->ce.w + m->o_pos, m->ce.w + m->o_elng,
+                                   m->ce.w + m->o_elnb, m->z0, m->tok_ids, m->x0, m->mean0, m->rstd0, seq_len, seq_off, st));
   StreamRef x0;
   x0.z = m->z0; x0.mean = m->mean0; x0.rstd = m->rstd0; x0.gamma = m->ce.w + m->o_elng; x0.beta = m->ce.w + m->o_elnb;
   StreamRef out;
