@@ -118,7 +118,7 @@ __device__ __forceinline__ uint64_t f2_const(float c) {
   const uint64_t u = (uint64_t)__float_as_uint(c);
   return u | (u << 32);
 }
-__device__ __forceinline__ void gelu_pair(uint64_t x, uint64_t& g, uint64_t& dg) {
+template <bool DERIVATIVE> __device__ __forceinline__ void gelu_pair(uint64_t x, uint64_t& g, uint64_t& dg) {
   float e0, e1, y0, y1;
   f2_unpack(f2_mul(f2_mul(x, x), f2_const(-0.72134752f)), e0, e1);
   asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(e0));                          // exp(-x^2 / 2)
@@ -136,7 +136,7 @@ __device__ __forceinline__ void gelu_pair(uint64_t x, uint64_t& g, uint64_t& dg)
   const uint64_t h = f2_fma(f2_mul(p, ex), f2_const(-0.5f), f2_const(0.5f));    // erf(|x| / sqrt 2) / 2
   const uint64_t cdf = f2_add(h | (x & 0x8000000080000000ull), f2_const(0.5f));   // 1/2 + sign(x) * h
   g = f2_mul(x, cdf);
-  dg = f2_fma(f2_mul(x, ex), f2_const(0.39894228f), cdf);
+  if (DERIVATIVE) dg = f2_fma(f2_mul(x, ex), f2_const(0.39894228f), cdf);
 }
 __device__ __forceinline__ uint32_t f2_to_bf16x2(uint64_t v) {
   float lo, hi;
@@ -503,9 +503,10 @@ template <int BN> struct TcCfg {
 //   EPI_DG    multiply by the saved GELU derivative, bf16 out (values prefetched during the main loop)
 //   EPI_BIAS  (+ bias), bf16 or fp32 out
 //   EPI_GELU  + bias, GELU, saved derivative, both bf16
+//   EPI_GELU_V  the same without the derivative (passes that no backward pass follows; pair kernel)
 //   EPI_RES   (+ bias) + fp32 residual (LayerNorm on the fly when res_mean is set), fp32 out (+ bf16 copy)
 //   EPI_RES_TS  the same without the bf16 copy, residual in and result out by bulk tensor copies (pair kernel)
-enum { EPI_GENERAL = 0, EPI_DG = 1, EPI_BIAS = 2, EPI_GELU = 3, EPI_RES = 4, EPI_RES_TS = 5 };
+enum { EPI_GENERAL = 0, EPI_DG = 1, EPI_BIAS = 2, EPI_GELU = 3, EPI_RES = 4, EPI_RES_TS = 5, EPI_GELU_V = 6 };
 
 template <int BN, typename CT, int MODE, int PARTS = 2>
 __device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t row0, int tn, int half, int q, int lane,
@@ -986,7 +987,8 @@ __device__ __forceinline__ void load_cols32(const float* __restrict__ p, int n, 
 // box in shared memory (128-byte rows whose 16-byte pieces are XOR-swizzled as the 128-byte swizzle of the
 // tensor map expects, which also keeps the writes free of bank conflicts).  Two blocks fill a box, and lane 0
 // hands it to a bulk tensor store, which writes whole 128-byte lines and clips the box at the matrix edges.
-// EPI_GELU fills a second box with the derivative; EPI_DG (NB = 2) first fetches the box of the saved derivative
+// EPI_GELU fills a second box with the derivative (the two results are what bounds it: 805 MB in 257 us at 65 536 x 3072, of
+// which 255 us stay without the arithmetic and 177 without the stores; one result alone EPI_GELU_V); EPI_DG (NB = 2) first fetches the box of the saved derivative
 // with a bulk tensor load (issued before the wait for the accumulator), multiplies in place and stores the same
 // box.  The accumulator buffer is handed back as soon as the last block has been read.  sbuf: 4 KB (8 KB for
 // EPI_GELU), 1024-byte aligned, private to the warp.  Returns false if a bounded wait gave up.
@@ -1044,18 +1046,21 @@ __device__ __forceinline__ bool epilogue_tile_ts(const TcArgs& a, const CUtensor
       for (int c = 0; c < 4; ++c)
         sts128(srow + (((p0 + (uint32_t)c) ^ swz) << 4), oc[4 * c], oc[4 * c + 1], oc[4 * c + 2], oc[4 * c + 3]);
     } else {
-      uint32_t op[MODE == EPI_GELU ? 16 : 1];
+      constexpr bool GELU = MODE == EPI_GELU || MODE == EPI_GELU_V, DERIVATIVE = MODE == EPI_GELU;
+      uint32_t op[DERIVATIVE ? 16 : 1];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const float4 b4 = bias[j];
-        if constexpr (MODE == EPI_GELU) {
+        if constexpr (GELU) {
           uint64_t g0, g1, d0, d1;
-          gelu_pair(f2_add(f2_pack(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1])), f2_pack(b4.x, b4.y)), g0, d0);
-          gelu_pair(f2_add(f2_pack(__uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])), f2_pack(b4.z, b4.w)), g1, d1);
+          gelu_pair<DERIVATIVE>(f2_add(f2_pack(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1])), f2_pack(b4.x, b4.y)), g0, d0);
+          gelu_pair<DERIVATIVE>(f2_add(f2_pack(__uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])), f2_pack(b4.z, b4.w)), g1, d1);
           oc[2 * j] = f2_to_bf16x2(g0);
           oc[2 * j + 1] = f2_to_bf16x2(g1);
-          op[2 * j] = f2_to_bf16x2(d0);
-          op[2 * j + 1] = f2_to_bf16x2(d1);
+          if constexpr (DERIVATIVE) {
+            op[2 * j] = f2_to_bf16x2(d0);
+            op[2 * j + 1] = f2_to_bf16x2(d1);
+          }
         } else {
           oc[2 * j] = pack_bf16x2(__uint_as_float(v[4 * j]) + b4.x, __uint_as_float(v[4 * j + 1]) + b4.y);
           oc[2 * j + 1] = pack_bf16x2(__uint_as_float(v[4 * j + 2]) + b4.z, __uint_as_float(v[4 * j + 3]) + b4.w);
@@ -1235,7 +1240,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
                                                                   const __grid_constant__ CUtensorMap tmC,
                                                                   const __grid_constant__ CUtensorMap tmP, TcArgs a) {
   constexpr bool RS = sizeof(CT) == 4 && MODE == EPI_RES_TS;       // fp32 residual epilogue through bulk tensor copies
-  constexpr bool TS = RS || (sizeof(CT) == 2 && ((EW == 16 && MODE == EPI_DG) || MODE == EPI_BIAS || MODE == EPI_GELU));
+  constexpr bool TS = RS || (sizeof(CT) == 2 && ((EW == 16 && MODE == EPI_DG) || MODE == EPI_BIAS || MODE == EPI_GELU || MODE == EPI_GELU_V));
   constexpr int WARP_BYTES = warp_bytes<CT, MODE>();
   using Cfg = Tc2Cfg<EW, WARP_BYTES>;
   constexpr int BN = Cfg::BN, STAGES = Cfg::STAGES;
@@ -1678,11 +1683,11 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
                        !b_kmajor;
   const bool others = e.gelu || e.dgelu_pre || e.res || e.accumulate || e.copy_out || e.pre;
   const bool m_bias = !others;
-  const bool m_gelu = e.gelu && e.pre && !e.dgelu_pre && !e.res && !e.accumulate && !e.copy_out && !c_f32 && a_kmajor && b_kmajor;
+  const bool m_gelu = e.gelu && !e.dgelu_pre && !e.res && !e.accumulate && !e.copy_out && !c_f32 && a_kmajor && b_kmajor;
   const bool m_res = e.res && !e.gelu && !e.dgelu_pre && !e.accumulate && !e.pre && c_f32 && a_kmajor;
   if (pair) {
     // bf16 results leave through bulk tensor stores: maps of C and of the GELU-derivative matrix (boxes of 32 rows x 64 columns)
-    const void* aux = e.gelu ? e.pre : e.dgelu_pre;
+    const void* aux = e.gelu ? e.pre : e.dgelu_pre;          // null: the value alone
     const bool ts = !c_f32 && M < (int64_t)1 << 31 && (!aux || (uintptr_t)aux % 16 == 0);
     CUtensorMap mc, mp;
     bool ts_ok = ts && make_map(&mc, C, (uint64_t)N, (uint64_t)M, (uint64_t)ldc, 64, 32);
@@ -1700,7 +1705,8 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     if (e.colsum_part && !(dg_only && ts_ok))
       return gram_set_error(ctx, "gemm: column-sum partials need the GELU-derivative variant with bulk stores"), GRAM_ERR_UNSUPPORTED;
     if (dg_only && ts_ok) err = launch_tc2<true, false, bf16, EPI_DG, 16>(ma, mb, args, grid, st, pc, pp);
-    else if (m_gelu && ts_ok) err = launch_tc2<true, true, bf16, EPI_GELU, 8>(ma, mb, args, grid, st, pc, pp);
+    else if (m_gelu && ts_ok && e.pre) err = launch_tc2<true, true, bf16, EPI_GELU, 8>(ma, mb, args, grid, st, pc, pp);
+    else if (m_gelu && ts_ok) err = launch_tc2<true, true, bf16, EPI_GELU_V, 8>(ma, mb, args, grid, st, pc, pp);
     else if (m_res && rs_ok && b_kmajor) err = launch_tc2<true, true, float, EPI_RES_TS>(ma, mb, args, grid, st, &mcf, &mrf);
     else if (m_res && rs_ok && !b_kmajor) err = launch_tc2<true, false, float, EPI_RES_TS>(ma, mb, args, grid, st, &mcf, &mrf);
     else if (m_res && b_kmajor) err = launch_tc2<true, true, float, EPI_RES>(ma, mb, args, grid, st);

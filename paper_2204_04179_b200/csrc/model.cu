@@ -357,17 +357,19 @@ gram_status layer_attention_forward(Model* m, Module& mod, Stack& s, int l, cons
 
 // the row-wise rest of the layer over T rows: output projection + residual, LayerNorm, feed-forward + residual,
 // LayerNorm.  x: the layer's input stream at those rows; ctx_in: the attention output at those rows; a: where the
-// activations of these rows are kept.  The rows need not be whole sequences.
+// activations of these rows are kept.  The rows need not be whole sequences.  keep: a backward pass may follow (else the
+// GELU derivative is not written).  want_b: someone reads the operand-typed copy of the layer's output (the next layer does;
+// the top layer's readers take the stream and its statistics), else it is not written.
 gram_status layer_rest_forward(Model* m, Module& mod, const LayerOff& o, LayerActs& a, int d, int f, int attn_only,
                                const StreamRef& x, const void* ctx_in, int64_t T, cudaStream_t st, StreamRef* x_out,
-                               const void** xb_out) {
+                               const void** xb_out, bool keep, bool want_b) {
   gram_ctx* ctx = m->ctx;
   GemmEpilogue e;
   e.bias = mod.w + o.bo;
   e.tag = "fwd_attn_out";
   set_res(e, x);
   if (attn_only) {
-    e.copy_out = a.out;
+    e.copy_out = want_b ? a.out : nullptr;
     GRAM_TRY(mm_fwd(m, ctx_in, W(m, mod, o.wo), a.outf, true, T, d, d, e, st));       // out = x + ctx Wo^T + bo
     *x_out = StreamRef();
     x_out->z = a.outf;
@@ -377,7 +379,7 @@ gram_status layer_rest_forward(Model* m, Module& mod, const LayerOff& o, LayerAc
     e = GemmEpilogue();
     e.bias = mod.w + o.b1;
     e.gelu = 1;
-    e.pre = a.u;
+    e.pre = keep ? a.u : nullptr;
     e.tag = "fwd_ffn1";
     GRAM_TRY(mm_fwd(m, a.h1, W(m, mod, o.w1), a.g, false, T, f, d, e, st));          // v = h1 W1^T + b1: g = gelu(v), u = gelu'(v)
     e = GemmEpilogue();
@@ -387,27 +389,29 @@ gram_status layer_rest_forward(Model* m, Module& mod, const LayerOff& o, LayerAc
     h1.z = a.z1; h1.mean = a.mean1; h1.rstd = a.rstd1; h1.gamma = mod.w + o.ln1g; h1.beta = mod.w + o.ln1b;
     set_res(e, h1);
     GRAM_TRY(mm_fwd(m, a.g, W(m, mod, o.w2), a.z2, true, T, d, f, e, st));           // z2 = LN1(z1) + g W2^T + b2
-    GRAM_TRY(layernorm_forward(ctx, m->dtype, a.z2, mod.w + o.ln2g, mod.w + o.ln2b, a.out, a.mean2, a.rstd2, T, d, st));
+    GRAM_TRY(layernorm_forward(ctx, m->dtype, a.z2, mod.w + o.ln2g, mod.w + o.ln2b, want_b ? a.out : nullptr, a.mean2, a.rstd2, T, d, st));
     *x_out = StreamRef();
     x_out->z = a.z2; x_out->mean = a.mean2; x_out->rstd = a.rstd2; x_out->gamma = mod.w + o.ln2g; x_out->beta = mod.w + o.ln2b;
   }
-  *xb_out = a.out;
+  *xb_out = want_b ? a.out : nullptr;
   return GRAM_OK;
 }
 
 // x_in: the fp32 input stream; x_in_b: its operand-typed copy.  *out / *out_b: the same pair for the output of
 // layer n_full - 1.  Layers [0, n_full) run completely; when n_full < n_layers, layer n_full runs its attention
 // part only (its ctx is left in s.acts[n_full].ctx; not even that without top_attention) and *out / *out_b describe that
-// layer's input.
+// layer's input.  keep, want_out_b: as above; without want_out_b *out_b is null.
 gram_status stack_forward(Model* m, Module& mod, Stack& s, const StreamRef& x_in, const void* x_in_b, int64_t n_seq, int S,
-                          cudaStream_t st, StreamRef* out, const void** out_b, int n_full = -1, bool top_attention = true) {
+                          cudaStream_t st, StreamRef* out, const void** out_b, bool keep, bool want_out_b, int n_full = -1,
+                          bool top_attention = true) {
   const int64_t T = s.packed_rows ? s.packed_rows : n_seq * S;
   if (n_full < 0) n_full = s.n_layers;
   StreamRef x = x_in;
   const void* xb = x_in_b;
   for (int l = 0; l < n_full; ++l) {
     GRAM_TRY(layer_attention_forward(m, mod, s, l, xb, n_seq, S, st));
-    GRAM_TRY(layer_rest_forward(m, mod, s.off[l], s.acts[l], s.d, s.d_ff, s.attn_only, x, s.acts[l].ctx, T, st, &x, &xb));
+    GRAM_TRY(layer_rest_forward(m, mod, s.off[l], s.acts[l], s.d, s.d_ff, s.attn_only, x, s.acts[l].ctx, T, st, &x, &xb, keep,
+                                want_out_b || l + 1 < n_full));
   }
   if (n_full < s.n_layers && top_attention) GRAM_TRY(layer_attention_forward(m, mod, s, n_full, xb, n_seq, S, st));
   *out = x;
@@ -539,12 +543,13 @@ gram_status cls_attention_backward(Model* m, int32_t n, int64_t T, const int32_t
   return add_strided_rows(ctx, *cur, n, c.l_t, seq_off, d, s.curf, st);
 }
 
-// encoder forward over n items (d_items, or first_item.. when null): H_out [n, d] fp32
+// encoder forward over n items (d_items, or first_item.. when null): H_out [n, d] fp32; keep: its backward pass may follow
 gram_status encoder_forward_chunk(Model* m, const int32_t* d_item_tokens, const int32_t* d_items, int32_t first_item,
-                                  int32_t n, float* H_out, cudaStream_t st) {
+                                  int32_t n, float* H_out, bool keep, cudaStream_t st) {
   const gram_config& c = m->cfg;
   gram_ctx* ctx = m->ctx;
   if (n > m->mb) return gram_set_error(ctx, "encoder pass over %d items exceeds the micro-batch of %d", n, m->mb), GRAM_ERR_WORKSPACE;
+  m->saved_n = -1;
   GRAM_TRY(refresh_bf16(m, m->ce, st));
   // texts of different lengths: rows are packed, item u owns rows seq_off[u] .. + seq_len[u] and padding has no rows
   const int32_t* seq_len = nullptr;
@@ -581,7 +586,7 @@ gram_status encoder_forward_chunk(Model* m, const int32_t* d_item_tokens, const 
   StreamRef out;
   const void* out_b = nullptr;
   if (!m->cls_tail) {
-    GRAM_TRY(stack_forward(m, m->ce, m->enc, x0, m->x0, n, c.l_t, st, &out, &out_b));
+    GRAM_TRY(stack_forward(m, m->ce, m->enc, x0, m->x0, n, c.l_t, st, &out, &out_b, keep, c.pooling == GRAM_POOL_ADDITIVE));
     if (c.pooling == GRAM_POOL_ADDITIVE) {
       GemmEpilogue e;
       e.bias = m->ce.w + m->o_pba;
@@ -598,7 +603,7 @@ gram_status encoder_forward_chunk(Model* m, const int32_t* d_item_tokens, const 
     const int last = c.n_layers - 1;
     StreamRef x;
     const void* xb = nullptr;
-    GRAM_TRY(stack_forward(m, m->ce, m->enc, x0, m->x0, n, c.l_t, st, &x, &xb, last, !m->cls_query));
+    GRAM_TRY(stack_forward(m, m->ce, m->enc, x0, m->x0, n, c.l_t, st, &x, &xb, keep, true, last, !m->cls_query));
     // row 0 of every item: the attention output and the last layer's input stream (values and LayerNorm statistics)
     LayerActs& ta = m->tail.acts[0];
     if (m->cls_query) {
@@ -623,10 +628,10 @@ gram_status encoder_forward_chunk(Model* m, const int32_t* d_item_tokens, const 
     GRAM_TRY(take_strided_rows(ctx, x.rstd, n, c.l_t, seq_off, 1, 4, m->tail_rstd, st));
     StreamRef xr = x;
     xr.z = m->tail_z; xr.mean = m->tail_mean; xr.rstd = m->tail_rstd;
-    GRAM_TRY(layer_rest_forward(m, m->ce, m->tail.off[0], ta, c.d, c.d_ff, 0, xr, ta.ctx, n, st, &out, &out_b));
+    GRAM_TRY(layer_rest_forward(m, m->ce, m->tail.off[0], ta, c.d, c.d_ff, 0, xr, ta.ctx, n, st, &out, &out_b, keep, false));
     GRAM_TRY(pool_forward(ctx, out, H_out, n, 1, c.d, c.pooling, nullptr, nullptr, st));       // one row per item: the pooled row itself
   }
-  m->saved_n = n;
+  if (keep) m->saved_n = n;
   return GRAM_OK;
 }
 
@@ -711,7 +716,7 @@ gram_status task_forward_backward(Model* m, const EncodingSource& src, const int
     x.z = m->tx;
     StreamRef y;
     const void* y_b = nullptr;
-    GRAM_TRY(stack_forward(m, m->task, m->tk, x, m->txb, B, c.L, st, &y, &y_b));
+    GRAM_TRY(stack_forward(m, m->task, m->tk, x, m->txb, B, c.L, st, &y, &y_b, true, false));
     void* dy_b = (m->tk.attn_only && m->tk.n_layers > 0) ? m->tk.dzb : nullptr;
     GRAM_TRY(kt_head(ctx, m->dtype, y, m->task.w + m->t_headw, m->task.w + m->t_headb, labels, m->tk.curf, dy_b,
                      m->task.g + m->t_headw, m->task.g + m->t_headb, loss, m->red, m->n_real, P, c.d, st));
@@ -739,7 +744,7 @@ gram_status task_forward_backward(Model* m, const EncodingSource& src, const int
       x.z = m->tx;
       StreamRef y;
       const void* y_b = nullptr;
-      GRAM_TRY(stack_forward(m, m->task, m->tk, x, m->txb, B, n_hist, st, &y, &y_b));
+      GRAM_TRY(stack_forward(m, m->task, m->tk, x, m->txb, B, n_hist, st, &y, &y_b, true, false));
       GRAM_TRY(nr_select(ctx, y, m->nr_pos2row, E_in, P, c.d, m->nr_E2, st));
       E = m->nr_E2;
       dE = m->nr_dE2;
@@ -810,7 +815,7 @@ template <typename GFn>
 gram_status encoder_pass(Model* m, const int32_t* d_items, int32_t n_total, bool update_cache, GFn G_of, cudaStream_t st) {
   for (int32_t u0 = 0; u0 < n_total; u0 += m->mb) {
     const int32_t n = (n_total - u0 < m->mb) ? n_total - u0 : m->mb;
-    GRAM_TRY(encoder_forward_chunk(m, nullptr, d_items + u0, 0, n, m->H, st));
+    GRAM_TRY(encoder_forward_chunk(m, nullptr, d_items + u0, 0, n, m->H, true, st));
     const float* G = nullptr;
     GRAM_TRY(G_of(u0, n, &G));                 // may read the cache rows of these items: before they are replaced
     if (update_cache) GRAM_TRY(scatter_rows(m->ctx, m->cache_dtype, m->H, d_items + u0, n, m->cfg.d, m->cfg.n_items, m->cache, st));
@@ -1025,7 +1030,7 @@ gram_status model_encode(Model* m, const int32_t* d_item_tokens, const int32_t* 
     return gram_set_error(m->ctx, "gram_encode_unique: %d items do not fit the micro-batch of %d when activations are kept", U, m->mb), GRAM_ERR_WORKSPACE;
   for (int32_t u0 = 0; u0 < U; u0 += m->mb) {
     const int32_t n = (U - u0 < m->mb) ? U - u0 : m->mb;
-    GRAM_TRY(encoder_forward_chunk(m, d_item_tokens, d_items + u0, 0, n, d_H + (size_t)u0 * m->cfg.d, st));
+    GRAM_TRY(encoder_forward_chunk(m, d_item_tokens, d_items + u0, 0, n, d_H + (size_t)u0 * m->cfg.d, save != 0, st));
   }
   if (!save || U == 0) m->saved_n = save ? 0 : -1;
   return GRAM_OK;
@@ -1066,7 +1071,7 @@ gram_status model_cache_fill(Model* m, cudaStream_t st) {
   const gram_config& c = m->cfg;
   for (int32_t u0 = 0; u0 < c.n_items; u0 += m->mb) {
     const int32_t n = (c.n_items - u0 < m->mb) ? c.n_items - u0 : m->mb;
-    GRAM_TRY(encoder_forward_chunk(m, nullptr, nullptr, u0, n, m->H, st));
+    GRAM_TRY(encoder_forward_chunk(m, nullptr, nullptr, u0, n, m->H, false, st));
     if (m->cache_dtype == GRAM_BF16) GRAM_TRY(convert_f32_to_bf16(m->ctx, m->H, (bf16*)m->cache + (size_t)u0 * c.d, (size_t)n * c.d, st));
     else GRAM_CUDA(m->ctx, cudaMemcpyAsync((float*)m->cache + (size_t)u0 * c.d, m->H, (size_t)n * c.d * 4, cudaMemcpyDeviceToDevice, st));
   }
@@ -1213,7 +1218,7 @@ gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in
     // stage 2: one encoding per unique item (Eq. 4)
     for (int32_t u0 = 0; u0 < U; u0 += m->mb) {
       const int32_t n = (U - u0 < m->mb) ? U - u0 : m->mb;
-      GRAM_TRY(encoder_forward_chunk(m, nullptr, m->unique + u0, 0, n, m->H + (size_t)u0 * c.d, st));
+      GRAM_TRY(encoder_forward_chunk(m, nullptr, m->unique + u0, 0, n, m->H + (size_t)u0 * c.d, U <= m->mb, st));
     }
     GRAM_CUDA(ctx, cudaEventRecord(ev[2], st));
     // stage 3: the KT task module gathers H[inverse[p]] in its first load; the NR module reads a materialised E
@@ -1300,7 +1305,7 @@ gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in
       if (c.refresh_after_update) {      // Eq. 4 with the updated parameters: the next window reads fresh encodings
         for (int32_t u0 = 0; u0 < n_touched; u0 += m->mb) {
           const int32_t n = (n_touched - u0 < m->mb) ? n_touched - u0 : m->mb;
-          GRAM_TRY(encoder_forward_chunk(m, nullptr, m->tlist + u0, 0, n, m->H, st));
+          GRAM_TRY(encoder_forward_chunk(m, nullptr, m->tlist + u0, 0, n, m->H, false, st));
           GRAM_TRY(scatter_rows(ctx, m->cache_dtype, m->H, m->tlist + u0, n, c.d, c.n_items, m->cache, st));
         }
         m->saved_n = -1;

@@ -10,6 +10,7 @@ from tests import gram_helpers as gh
 
 pytestmark = pytest.mark.gpu
 
+
 @pytest.mark.parametrize("d,heads,l_t,pooling,ragged,shift", [(36, 3, 1, "mean", False, 1), (36, 3, 7, "mean", True, 0), (132, 3, 33, "mean", True, 2),
                                                              (256, 4, 70, "mean", False, 0), (1024, 16, 9, "mean", True, 3),
                                                              (128, 2, 5, "cls", True, 1), (128, 2, 1, "cls", False, 3)])
@@ -30,13 +31,15 @@ def test_encodings_and_their_gradients(d, heads, l_t, pooling, ragged, shift):
     items = torch.arange(n, dtype=torch.int32, device="cuda")
     H, Gd = (torch.zeros(n * d + shift, device="cuda")[shift:] for _ in range(2))
     Gd.copy_(torch.from_numpy(G).reshape(-1))
-
+    bare = torch.zeros(n, d, device="cuda")
+    g.encode_unique(None, items, n, bare)                          # nothing kept for a backward pass: the same encodings
     g.encode_unique(None, items, n, H, save_activations=True)
     g.zero_grads(binding.GRAM_MODULE_CE)
     g.encoder_backward(Gd, items, n)
     g.sync()
     got, _ = gh.gpu_grads(g, shape)
     g.close()
+    assert torch.equal(H.view(n, d), bare)
     # fp32 sums over at most 1024 columns or 770 rows: an order of magnitude above what such models show
     assert gh.rel_err(H.cpu().numpy().reshape(n, d), want.detach().numpy()) <= 2e-5
     err, name = gh.worst_rel_err(got, {k: t.grad.numpy() for k, t in th.items()})
