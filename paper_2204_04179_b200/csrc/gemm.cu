@@ -475,6 +475,8 @@ struct TcArgs {
   int32_t N;
   int32_t num_kb;          // k-blocks of 64 over the whole K
   int32_t n_tiles_m, n_tiles_n, splits, kb_per_split;
+  int32_t chain;           // k-blocks added up in one accumulator (EPI_SUM: fewer than kb_per_split)
+  int32_t half_from;       // pair kernel: tiles from this one on are two work units of half the columns each (unit numbers go on)
   int64_t split_stride;    // elements between the partial outputs of two splits
   EpiDev epi;
   int32_t* status;
@@ -491,7 +493,8 @@ template <int BN> struct TcCfg {
 };
 
 // The epilogue of one output tile for one epilogue warp: rows row0 .. row0+31 (TMEM lanes q*32..), columns
-// [half*BN/PARTS, (half+1)*BN/PARTS) of tile column tn.  A warp may read only its quarter of the TMEM lanes; PARTS warps
+// [half*BN/PARTS, (half+1)*BN/PARTS) of the tile whose first column is n_first; columns from n_lim on (the matrix's edge, or
+// the end of a half-width unit) are not touched.  A warp may read only its quarter of the TMEM lanes; PARTS warps
 // share a quarter and split the columns.  Each 32 x 32 block is loaded one row per thread, turned through a
 // padded shared-memory buffer, and then handled four rows per instruction with eight lanes per row, so that
 // global loads and stores of a row are contiguous 128-byte pieces.  Returns false if the bounded wait for the
@@ -505,11 +508,12 @@ template <int BN> struct TcCfg {
 //   EPI_GELU  + bias, GELU, saved derivative, both bf16
 //   EPI_GELU_V  the same without the derivative (passes that no backward pass follows; pair kernel)
 //   EPI_RES   (+ bias) + fp32 residual (LayerNorm on the fly when res_mean is set), fp32 out (+ bf16 copy)
+//   EPI_SUM   fp32 out (added to C on request) of a K range that is cut into several accumulator chains (pair kernel)
 //   EPI_RES_TS  the same without the bf16 copy, residual in and result out by bulk tensor copies (pair kernel)
-enum { EPI_GENERAL = 0, EPI_DG = 1, EPI_BIAS = 2, EPI_GELU = 3, EPI_RES = 4, EPI_RES_TS = 5, EPI_GELU_V = 6 };
+enum { EPI_GENERAL = 0, EPI_DG = 1, EPI_BIAS = 2, EPI_GELU = 3, EPI_RES = 4, EPI_RES_TS = 5, EPI_GELU_V = 6, EPI_SUM = 7 };
 
 template <int BN, typename CT, int MODE, int PARTS = 2>
-__device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t row0, int tn, int half, int q, int lane,
+__device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t row0, int n_first, int n_lim, int half, int q, int lane,
                                               float* stage, uint32_t tmem_base, int buf, uint32_t tfull_addr,
                                               uint32_t parity, volatile int* abort_flag) {
   if constexpr (MODE == EPI_DG) {
@@ -517,12 +521,12 @@ __device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t r
     const int sub = lane >> 3, slot = lane & 7;
     const int64_t rows_left = a.M - (row0 + sub);
     const int64_t step = 4 * a.ldc;
-    const int ncol0 = tn * BN + half * (BN / PARTS) + slot * 4;
+    const int ncol0 = n_first + half * (BN / PARTS) + slot * 4;
     const int64_t o0 = (row0 + sub) * a.ldc + ncol0;
     const bf16* pre = reinterpret_cast<const bf16*>(a.epi.dgelu_pre) + o0;
 #pragma unroll
     for (int blk = 0; blk < BN / (32 * PARTS); ++blk) {
-      const bool col_ok = ncol0 + blk * 32 < a.N;
+      const bool col_ok = ncol0 + blk * 32 < n_lim;
 #pragma unroll
       for (int rr = 0; rr < 8; ++rr)
         pf[blk][rr] = (col_ok && rr * 4 < rows_left) ? *reinterpret_cast<const uint2*>(pre + blk * 32 + rr * step) : make_uint2(0u, 0u);
@@ -537,7 +541,7 @@ __device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t r
       tc_ld32_wait(v);
       stage_write_row(stage, lane, v);
       __syncwarp();
-      if (ncol0 + blk * 32 < a.N) {
+      if (ncol0 + blk * 32 < n_lim) {
         CT* cp = Cs + o0 + blk * 32;
 #pragma unroll
         for (int rr = 0; rr < 8; ++rr) {
@@ -564,11 +568,11 @@ __device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t r
     const int sub = lane >> 3, slot = lane & 7;
     const int64_t rows_left = a.M - (row0 + sub);         // row rr*4 + sub exists iff rr*4 < rows_left
     const int64_t step = 4 * a.ldc;
-    const int nbase = tn * BN + half * (BN / PARTS) + slot * 4;
+    const int nbase = n_first + half * (BN / PARTS) + slot * 4;
     const int64_t obase = (row0 + sub) * a.ldc + nbase;
     float4 rnext[8];
     auto load_res = [&](int blk, float4 (&dst)[8]) {
-      const bool col_ok = nbase + blk * 32 < a.N;
+      const bool col_ok = nbase + blk * 32 < n_lim;
       const float* rp = a.epi.res + obase + blk * 32;
 #pragma unroll
       for (int rr = 0; rr < 8; ++rr)
@@ -595,7 +599,7 @@ __device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t r
       stage_write_row(stage, lane, v);
       __syncwarp();
       const int n = nbase + blk * 32;
-      const bool col_ok = n < a.N;                          // lanes of a warp may differ here when N is not a multiple of 32
+      const bool col_ok = n < n_lim;                          // lanes of a warp may differ here when N is not a multiple of 32
       float b4[4] = {0.f, 0.f, 0.f, 0.f}, g4[4] = {0.f, 0.f, 0.f, 0.f}, be4[4] = {0.f, 0.f, 0.f, 0.f};
       if (col_ok) {
         if (a.epi.bias) ld4(a.epi.bias + n, b4);
@@ -644,8 +648,8 @@ __device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t r
       tc_ld32_wait(v);
       stage_write_row(stage, lane, v);
       __syncwarp();
-      const int n = tn * BN + c0 + slot * 4;
-      if (n < a.N) {                                      // N is a multiple of 8
+      const int n = n_first + c0 + slot * 4;
+      if (n < n_lim) {                                      // N is a multiple of 8
         float b4[4] = {0.f, 0.f, 0.f, 0.f};
         if (a.epi.bias) ld4(a.epi.bias + n, b4);
         const int64_t o0 = (row0 + sub) * a.ldc + n;      // element offset of this lane's first row
@@ -704,8 +708,8 @@ __device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t r
       tc_ld32_wait(v);
       stage_write_row(stage, lane, v);
       __syncwarp();
-      const int n = tn * BN + c0 + (lane & 7) * 4;
-      const bool col_ok = n < a.N;                // N is a multiple of 8
+      const int n = n_first + c0 + (lane & 7) * 4;
+      const bool col_ok = n < n_lim;                // N is a multiple of 8
       float bias4[4] = {0.f, 0.f, 0.f, 0.f}, gam4[4] = {0.f, 0.f, 0.f, 0.f}, bet4[4] = {0.f, 0.f, 0.f, 0.f};
       if (col_ok) {
         if (a.epi.bias) ld4(a.epi.bias + n, bias4);
@@ -876,7 +880,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gemm_tc_kernel(const __grid_con
       const int buf = (int)(it & 1);
       const int64_t row0 = (int64_t)tm * BM + q * 32;
       CT* Cs = C + (int64_t)split * a.split_stride;
-      if (!epilogue_tile<BN, CT, MODE>(a, Cs, row0, tn, half, q, lane, stage, tmem_base, buf, tfull_bar(buf),
+      if (!epilogue_tile<BN, CT, MODE>(a, Cs, row0, tn * BN, a.N, half, q, lane, stage, tmem_base, buf, tfull_bar(buf),
                                      (uint32_t)((it >> 1) & 1), abort_flag)) {
         failed = true;
         break;
@@ -988,13 +992,14 @@ __device__ __forceinline__ void load_cols32(const float* __restrict__ p, int n, 
 // tensor map expects, which also keeps the writes free of bank conflicts).  Two blocks fill a box, and lane 0
 // hands it to a bulk tensor store, which writes whole 128-byte lines and clips the box at the matrix edges.
 // EPI_GELU fills a second box with the derivative (the two results are what bounds it: 805 MB in 257 us at 65 536 x 3072, of
-// which 255 us stay without the arithmetic and 177 without the stores; one result alone EPI_GELU_V); EPI_DG (NB = 2) first fetches the box of the saved derivative
+// which 255 us stay without the arithmetic and 177 without the stores; one result alone, EPI_GELU_V, takes 239 us where the
+// two take 282 at 70 000 rows); EPI_DG (NB = 2) first fetches the box of the saved derivative
 // with a bulk tensor load (issued before the wait for the accumulator), multiplies in place and stores the same
 // box.  The accumulator buffer is handed back as soon as the last block has been read.  sbuf: 4 KB (8 KB for
 // EPI_GELU), 1024-byte aligned, private to the warp.  Returns false if a bounded wait gave up.
 template <int MODE, int NB>
 __device__ __forceinline__ bool epilogue_tile_ts(const TcArgs& a, const CUtensorMap* tmC, const CUtensorMap* tmP, int32_t row0,
-                                                 int32_t col0, int c_local, int q, int lane, uint32_t sbuf,
+                                                 int32_t col0, int32_t n_lim, int c_local, int q, int lane, uint32_t sbuf,
                                                  uint32_t tmem_base, int buf, uint32_t tfull_addr, uint32_t parity,
                                                  volatile int* abort_flag, uint32_t tempty_remote, uint32_t ld_bar,
                                                  uint32_t ld_parity) {
@@ -1028,7 +1033,7 @@ __device__ __forceinline__ bool epilogue_tile_ts(const TcArgs& a, const CUtensor
       if (lane == 0) mbar_arrive_remote(tempty_remote);
     }
     const int nbx = col0 + (b >> 1) * 64;                  // first column of the box
-    if (nbx >= a.N || !rows_ok) continue;
+    if (nbx >= n_lim || !rows_ok) continue;
     const uint32_t p0 = (uint32_t)(b & 1) * 4u;            // this block's first 16-byte piece of the row
     uint32_t oc[16];
     if constexpr (MODE == EPI_DG) {
@@ -1102,7 +1107,7 @@ __device__ __forceinline__ bool epilogue_tile_ts(const TcArgs& a, const CUtensor
             s1 += f.y;
           }
           const int cc = nbx + 2 * lane;
-          if (cc < a.N) *reinterpret_cast<float2*>(a.epi.colsum_part + (int64_t)(row0 >> 5) * a.N + cc) = make_float2(s0, s1);
+          if (cc < n_lim) *reinterpret_cast<float2*>(a.epi.colsum_part + (int64_t)(row0 >> 5) * a.N + cc) = make_float2(s0, s1);
           __syncwarp();                                    // every lane has read the box before it is refilled
         }
       }
@@ -1122,12 +1127,12 @@ __device__ __forceinline__ bool epilogue_tile_ts(const TcArgs& a, const CUtensor
 // accumulator, that of block b + 2 after the store of block b has been committed and the store before it has read its box.
 // sbuf: 12 KB, 1024-byte aligned, private to the warp; nb: the warp's running block count.
 __device__ __forceinline__ bool epilogue_tile_res(const TcArgs& a, const CUtensorMap* tmC, const CUtensorMap* tmR, int32_t row0,
-                                                  int32_t col0, int c_local, int q, int lane, uint32_t sbuf, uint32_t tmem_base,
+                                                  int32_t col0, int32_t n_lim, int c_local, int q, int lane, uint32_t sbuf, uint32_t tmem_base,
                                                   int buf, uint32_t tfull_addr, uint32_t parity, volatile int* abort_flag,
                                                   uint32_t tempty_remote, uint32_t ld_bar0, uint32_t& nb) {
   int nv = 0;                                               // blocks of this warp that lie inside the matrix
   if (row0 < a.M) {
-    nv = (a.N - col0 + 31) / 32;
+    nv = (n_lim - col0 + 31) / 32;
     nv = nv < 0 ? 0 : (nv > 4 ? 4 : nv);
   }
   auto request = [&](int b) {                               // residual box of block b of this tile -> box (nb + b) % 3
@@ -1232,6 +1237,94 @@ template <int EW, int WARP_BYTES = 4096> struct Tc2Cfg {
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 512;
 };
 
+// A work unit of the pair kernel: a tile, or half of its columns, over the k-blocks [kb0, kb1).  The last wave of tiles is
+// seldom full: where its tiles fit one wave as halves they are handed out as such (300 tiles over 74 pairs are 4 waves and
+// 4 tiles; the rest of the chip would wait for those).  25 600 x 768 x 3072 with the LayerNorm residual: 102 -> 94 us.
+struct Tc2Unit {
+  int32_t split, tm, n_first, width, kb0, kb1;
+};
+__device__ __forceinline__ Tc2Unit tc2_unit(const TcArgs& a, int64_t t) {
+  Tc2Unit u;
+  const int64_t per_split = (int64_t)a.n_tiles_m * a.n_tiles_n;
+  int32_t right = 0;
+  u.width = 256;
+  if (t >= a.half_from) {                              // one part of the K range only
+    right = (int32_t)((t - a.half_from) & 1);
+    t = a.half_from + ((t - a.half_from) >> 1);
+    u.width = 128;
+  }
+  u.split = (int32_t)(t / per_split);
+  const int64_t r = t - (int64_t)u.split * per_split;
+  u.tm = (int32_t)(r / a.n_tiles_n);
+  u.n_first = (int32_t)(r % a.n_tiles_n) * 256 + right * 128;
+  u.kb0 = u.split * a.kb_per_split;
+  u.kb1 = min(u.kb0 + a.kb_per_split, a.num_kb);
+  return u;
+}
+__device__ __forceinline__ int64_t tc2_units(const TcArgs& a) {
+  const int64_t tiles = (int64_t)a.n_tiles_m * a.n_tiles_n * a.splits;
+  return tiles + (tiles > a.half_from ? tiles - a.half_from : 0);
+}
+
+// Epilogue of EPI_SUM: the unit's K range arrives as several accumulators, each a chain of a.chain k-blocks, which the warp
+// adds up in its registers (128 columns a thread) in ascending order before it writes its 32 rows x 128 columns.  The tensor
+// core cuts off where this adds with rounding, so the length of a chain sets the precision; with the chains of one unit added
+// here, the parts of the K range that go through memory need no longer be as many as the chains.
+__device__ __forceinline__ bool epilogue_unit_sum(const TcArgs& a, float* Cs, int64_t row0, int n_first, int half, int q, int lane,
+                                                  float* stage, uint32_t tmem_base, int64_t it, int chains, uint32_t tfull0,
+                                                  uint32_t tempty0_remote, volatile int* abort_flag) {
+  float acc[4][32];
+#pragma unroll
+  for (int b = 0; b < 4; ++b)
+#pragma unroll
+    for (int k = 0; k < 32; ++k) acc[b][k] = 0.f;
+#pragma unroll 1
+  for (int c = 0; c < chains; ++c, ++it) {
+    const uint32_t buf = (uint32_t)(it & 1);
+    if (!mbar_wait(tfull0 + 8u * buf, (uint32_t)((it >> 1) & 1), abort_flag)) return false;
+    tc_fence_after();
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      uint32_t v[32];
+      tc_ld32_issue(tmem_base + ((uint32_t)(q * 32) << 16) + buf * 256u + (uint32_t)(half * 128 + b * 32), v);
+      tc_ld32_wait(v);
+#pragma unroll
+      for (int k = 0; k < 32; ++k) acc[b][k] += __uint_as_float(v[k]);
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive_remote(tempty0_remote + 8u * buf);
+  }
+  const int sub = lane >> 3, slot = lane & 7;
+  const int64_t rows_left = a.M - (row0 + sub);
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    uint32_t v[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) v[k] = __float_as_uint(acc[b][k]);
+    stage_write_row(stage, lane, v);
+    __syncwarp();
+    const int n = n_first + half * 128 + b * 32 + slot * 4;
+    if (n < a.N) {                                     // N is a multiple of 8
+      float* cp = Cs + (row0 + sub) * a.ldc + n;
+#pragma unroll
+      for (int rr = 0; rr < 8; ++rr) {
+        if (rr * 4 < rows_left) {
+          const float4 t = stage_read(stage, rr * 4 + sub, slot);
+          float x[4] = {t.x, t.y, t.z, t.w}, o[4] = {0.f, 0.f, 0.f, 0.f};
+          if (a.epi.accumulate) ld4(cp, o);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) x[k] += o[k];
+          st4(cp, x);
+        }
+        cp += 4 * a.ldc;
+      }
+    }
+    __syncwarp();
+  }
+  return true;
+}
+
 // n_tiles_m counts 256-row tiles here.  tmC / tmP: maps of the bf16 result and of the GELU-derivative matrix
 // (boxes of 32 rows x 64 columns, 128-byte swizzle) for the variants whose epilogue uses bulk tensor stores; unused otherwise.
 template <bool A_K, bool B_K, typename CT, int MODE = EPI_GENERAL, int EW = EPI_WARPS>
@@ -1290,7 +1383,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
   const uint32_t tmem_base = *tmem_slot;
   if (!chain_begin()) return;              // barriers and tensor memory are set up before the wait
 
-  const int64_t total = (int64_t)a.n_tiles_m * a.n_tiles_n * a.splits;
+  const int64_t total = tc2_units(a);
   const int64_t cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
   bool failed = false;
 
@@ -1300,18 +1393,16 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
     uint32_t ph = 0;
     const uint32_t lead_bar0 = map_to_cta(bar0, 0);          // the leader's barrier block, as seen from this CTA
     for (int64_t t = cluster_id; t < total && !failed; t += n_clusters) {
-      const int split = (int)(t / ((int64_t)a.n_tiles_m * a.n_tiles_n));
-      const int64_t r = t - (int64_t)split * a.n_tiles_m * a.n_tiles_n;
-      const int tm = (int)(r / a.n_tiles_n), tn = (int)(r % a.n_tiles_n);
-      const int kb0 = split * a.kb_per_split, kb1 = min(kb0 + a.kb_per_split, a.num_kb);
-      const int m0 = tm * 2 * BM + (int)rank * BM;            // this CTA's rows of A
-      const int n0 = tn * BN + (int)rank * (BN / 2);          // this CTA's columns of B
-      for (int kb = kb0; kb < kb1; ++kb) {
+      const Tc2Unit u = tc2_unit(a, t);
+      const int m0 = u.tm * 2 * BM + (int)rank * BM;             // this CTA's rows of A
+      const int n0 = u.n_first + (int)rank * (u.width / 2);      // this CTA's columns of B: one or two boxes of 64
+      const uint32_t bytes = Cfg::A_BYTES + (uint32_t)u.width * (BK * 2 / 2);
+      for (int kb = u.kb0; kb < u.kb1; ++kb) {
         if (!mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag)) { failed = true; break; }
         const uint32_t lead_full = lead_bar0 + 8u * s;           // the leader's full_bar(s)
         const uint32_t sa = tiles + s * Cfg::STAGE_BYTES, sb = sa + Cfg::A_BYTES;
         if (elect_one()) {
-          mbar_arrive_expect_tx_remote(lead_full, Cfg::STAGE_BYTES);
+          mbar_arrive_expect_tx_remote(lead_full, bytes);
           if (A_K) {
             tma_load_2d_pair(sa, &tmA, kb * BK, m0, lead_full);
           } else {
@@ -1320,9 +1411,10 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
           }
           if (B_K) {
             tma_load_2d_pair(sb, &tmB, kb * BK, n0, lead_full);
+            if (u.width == BN) tma_load_2d_pair(sb + 8192, &tmB, kb * BK, n0 + 64, lead_full);
           } else {
-#pragma unroll
-            for (int i = 0; i < BN / 128; ++i) tma_load_2d_pair(sb + i * 8192, &tmB, n0 + i * 64, kb * BK, lead_full);
+            tma_load_2d_pair(sb, &tmB, n0, kb * BK, lead_full);
+            if (u.width == BN) tma_load_2d_pair(sb + 8192, &tmB, n0 + 64, kb * BK, lead_full);
           }
         }
         __syncwarp();
@@ -1342,35 +1434,38 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
     // The descriptors of stage 0 are built once: a later stage or k-step only adds to the 14-bit address field, which
     // cannot overflow inside shared memory.
     if (leader) {
-      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_K ? 0u : 1u) << 15) |
-                                 ((B_K ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
+      constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((A_K ? 0u : 1u) << 15) | ((B_K ? 0u : 1u) << 16) |
+                                  ((uint32_t)((2 * BM) >> 4) << 24);
       int s = 0;
       uint32_t ph = 0;
       int64_t it = 0;
       const uint64_t da0 = A_K ? make_desc(tiles, 16, 1024) : make_desc(tiles, 8192, 1024);
       const uint64_t db0 = B_K ? make_desc(tiles + Cfg::A_BYTES, 16, 1024) : make_desc(tiles + Cfg::A_BYTES, 8192, 1024);
       constexpr uint32_t ka = (A_K ? 32 : 2048) >> 4, kbs = (B_K ? 32 : 2048) >> 4;
-      for (int64_t t = cluster_id; t < total && !failed; t += n_clusters, ++it) {
-        const int split = (int)(t / ((int64_t)a.n_tiles_m * a.n_tiles_n));
-        const int kb0 = split * a.kb_per_split, kb1 = min(kb0 + a.kb_per_split, a.num_kb);
-        const int buf = (int)(it & 1);
-        if (!mbar_wait_warp(tempty_bar(buf), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag)) { failed = true; break; }
-        tc_fence_after();
-        const uint32_t tmem_d = tmem_base + (uint32_t)(buf * BN);
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait_warp(full_bar(s), ph, abort_flag)) { failed = true; break; }
+      for (int64_t t = cluster_id; t < total && !failed; t += n_clusters) {
+        const Tc2Unit u = tc2_unit(a, t);
+        const uint32_t idesc = idesc0 | ((uint32_t)(u.width >> 3) << 17);
+        for (int c0 = u.kb0; c0 < u.kb1 && !failed; c0 += a.chain, ++it) {       // one accumulator each
+          const int c1 = min(c0 + a.chain, u.kb1);
+          const int buf = (int)(it & 1);
+          if (!mbar_wait_warp(tempty_bar(buf), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag)) { failed = true; break; }
           tc_fence_after();
-          const uint32_t soff = (uint32_t)(s * (Cfg::STAGE_BYTES >> 4));
-          const uint64_t da = da0 + soff, db = db0 + soff;
-          if (elect_one()) {
+          const uint32_t tmem_d = tmem_base + (uint32_t)(buf * BN);
+          for (int kb = c0; kb < c1; ++kb) {
+            if (!mbar_wait_warp(full_bar(s), ph, abort_flag)) { failed = true; break; }
+            tc_fence_after();
+            const uint32_t soff = (uint32_t)(s * (Cfg::STAGE_BYTES >> 4));
+            const uint64_t da = da0 + soff, db = db0 + soff;
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              tc_mma_pair(tmem_d, da + (uint64_t)(k * ka), db + (uint64_t)(k * kbs), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-            tc_commit_pair(empty_bar(s));                      // the stage is free in both CTAs once these MMAs are done
-            if (kb == kb1 - 1) tc_commit_pair(tfull_bar(buf));   // accumulator complete in both CTAs
+              for (int k = 0; k < BK / 16; ++k)
+                tc_mma_pair(tmem_d, da + (uint64_t)(k * ka), db + (uint64_t)(k * kbs), idesc, (kb > c0 || k > 0) ? 1u : 0u);
+              tc_commit_pair(empty_bar(s));                      // the stage is free in both CTAs once these MMAs are done
+              if (kb == c1 - 1) tc_commit_pair(tfull_bar(buf));    // accumulator complete in both CTAs
+            }
+            __syncwarp();
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
           }
-          __syncwarp();
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
       }
       if (failed && lane == 0) {
@@ -1388,13 +1483,20 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
     int64_t it = 0;
     uint32_t res_blocks = 0;                      // EPI_RES_TS: this warp's running count of 32-column blocks
     for (int64_t t = cluster_id; t < total && !failed; t += n_clusters, ++it) {
-      const int split = (int)(t / ((int64_t)a.n_tiles_m * a.n_tiles_n));
-      const int64_t r = t - (int64_t)split * a.n_tiles_m * a.n_tiles_n;
-      const int tm = (int)(r / a.n_tiles_n), tn = (int)(r % a.n_tiles_n);
+      const Tc2Unit u = tc2_unit(a, t);
+      const int n_lim = min(a.N, u.n_first + u.width);
       const int buf = (int)(it & 1);
-      const int64_t row0 = (int64_t)tm * 2 * BM + (int64_t)rank * BM + q * 32;
-      if constexpr (RS) {
-        if (!epilogue_tile_res(a, &tmC, &tmP, (int32_t)row0, tn * BN + half * 128, half * 128, q, lane,
+      const int64_t row0 = (int64_t)u.tm * 2 * BM + (int64_t)rank * BM + q * 32;
+      if constexpr (MODE == EPI_SUM) {
+        const int chains = (u.kb1 - u.kb0 + a.chain - 1) / a.chain;
+        if (!epilogue_unit_sum(a, reinterpret_cast<float*>(C) + (int64_t)u.split * a.split_stride, row0, u.n_first, half, q, lane, stage,
+                               tmem_base, it, chains, tfull_bar(0), map_to_cta(tempty_bar(0), 0), abort_flag)) {
+          failed = true;
+          break;
+        }
+        it += chains - 1;
+      } else if constexpr (RS) {
+        if (!epilogue_tile_res(a, &tmC, &tmP, (int32_t)row0, u.n_first + half * 128, n_lim, half * 128, q, lane,
                                tiles + STAGES * Cfg::STAGE_BYTES + (uint32_t)(ew * WARP_BYTES), tmem_base, buf, tfull_bar(buf),
                                (uint32_t)((it >> 1) & 1), abort_flag, map_to_cta(tempty_bar(buf), 0), ld_bar(3 * ew), res_blocks)) {
           failed = true;
@@ -1402,7 +1504,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
         }
       } else if constexpr (TS) {
         constexpr int NB = 32 / EW;               // blocks of 32 columns per warp
-        const bool ok = epilogue_tile_ts<MODE, NB>(a, &tmC, &tmP, (int32_t)row0, tn * BN + half * (NB * 32), half * (NB * 32), q, lane,
+        const bool ok = epilogue_tile_ts<MODE, NB>(a, &tmC, &tmP, (int32_t)row0, u.n_first + half * (NB * 32), n_lim, half * (NB * 32), q, lane,
                                     tiles + STAGES * Cfg::STAGE_BYTES + (uint32_t)(ew * WARP_BYTES), tmem_base, buf, tfull_bar(buf),
                                     (uint32_t)((it >> 1) & 1), abort_flag, map_to_cta(tempty_bar(buf), 0), ld_bar(ew),
                                     (uint32_t)(it & 1));
@@ -1411,8 +1513,8 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
           break;
         }
       } else {
-        CT* Cs = C + (int64_t)split * a.split_stride;
-        if (!epilogue_tile<BN, CT, MODE, EW / 4>(a, Cs, row0, tn, half, q, lane, stage, tmem_base, buf, tfull_bar(buf),
+        CT* Cs = C + (int64_t)u.split * a.split_stride;
+        if (!epilogue_tile<BN, CT, MODE, EW / 4>(a, Cs, row0, u.n_first, n_lim, half, q, lane, stage, tmem_base, buf, tfull_bar(buf),
                                                  (uint32_t)((it >> 1) & 1), abort_flag)) {
           failed = true;
           break;
@@ -1612,7 +1714,7 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
   bool ok;
   if (a_kmajor) ok = make_map(&ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM);
   else ok = make_map(&ma, A, (uint64_t)M, (uint64_t)K, (uint64_t)lda, 64, BK);
-  if (b_kmajor) ok = ok && make_map(&mb, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, BK, (uint32_t)(pair ? BNsel / 2 : BNsel));
+  if (b_kmajor) ok = ok && make_map(&mb, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, BK, (uint32_t)(pair ? 64 : BNsel));
   else ok = ok && make_map(&mb, B, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 64, BK);
   if (!ok) return gram_set_error(ctx, "gemm: cuTensorMapEncodeTiled failed"), GRAM_ERR_CUDA;
 
@@ -1626,12 +1728,13 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
   const int64_t tiles = (int64_t)args.n_tiles_m * args.n_tiles_n;
   const int units = pair ? kNumSMs / 2 : kNumSMs;        // CTAs, or CTA pairs, that run at once
   int splits = 1;
+  // weight gradients: a plain fp32 result, added to C or not
+  const bool sum_form = pair && !a_kmajor && !b_kmajor && c_f32 && !e.bias && !e.gelu && !e.dgelu_pre && !e.res && !e.copy_out && !e.pre;
   if (allow_splitk && tiles < units && args.num_kb >= 16 && ws && ws->splitk) {
-    // between 2 and 4 work units per CTA (pair), each of at least eight k-blocks; among those, the count that leaves the last
-    // wave fullest.  Fewer parts can be faster (25 600 rows: 768 x 768 40 us from 24 parts, 31 from 8; 3072 x 768 103 from 6,
-    // 94 from 2) but cost precision: the tensor core adds into its fp32 accumulator by cutting off, so the error of a part
-    // grows with the length of its chain of additions, while the parts themselves are added with rounding (65 536 rows,
-    // 3072 x 768, against 64 bits: 1.2e-5 from 6 parts, 3.8e-5 from 2).
+    // chains of additions in the accumulator: between 2 and 4 per CTA (pair), each of at least eight k-blocks; among those, the
+    // count that leaves the last wave fullest.  Longer chains cost precision: the tensor core adds into its fp32 accumulator by
+    // cutting off, so the error of a chain grows with its length, while the chains themselves are added with rounding
+    // (65 536 rows, 3072 x 768, against 64 bits: 1.2e-5 from 6 chains, 3.8e-5 from 2).
     const int64_t per = (int64_t)M * N * (int64_t)sizeof(float);
     int lo = (int)((2 * units + tiles - 1) / tiles), hi = (int)((4 * units + tiles - 1) / tiles);
     int cap = args.num_kb / 8;
@@ -1648,17 +1751,45 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
   }
   args.kb_per_split = ceil_div(args.num_kb, splits);
   splits = ceil_div(args.num_kb, args.kb_per_split);
+  args.chain = args.kb_per_split;
+  if (sum_form && splits > 1) {
+    // The chains of a unit are added in its epilogue's registers, so that the parts of the K range that go through memory are
+    // only as many as fill the chip: of those counts, from one unit per pair of SMs up, the one that leaves the last wave
+    // fullest, the smallest of equals (within two per cent: a part costs its write, its read and a place in the sum).
+    // 42 500 rows, a layer's four weight gradients on average: product 98 -> 90 us, sum of the parts 11.4 -> 7.0.
+    int best_sp = splits;
+    double best = 0.0;
+    for (int sp = splits; sp >= 1; --sp) {
+      const int per = ceil_div(splits, sp);                              // chains of a part
+      if (ceil_div(splits, per) != sp) continue;
+      const int64_t total = tiles * sp;
+      const double fill = (double)tiles * splits / ((double)ceil_div64(total, units) * units * per);
+      if (fill >= best - 0.02) { best_sp = sp; if (fill > best) best = fill; }
+    }
+    args.kb_per_split = ceil_div(splits, best_sp) * args.chain;
+    splits = ceil_div(args.num_kb, args.kb_per_split);
+  }
   args.splits = splits;
+  // The last wave's tiles as halves where twice as many still fit one wave.
+  args.half_from = INT32_MAX;
+  int64_t work = tiles * splits;
+  if (pair && splits == 1 && args.chain >= args.num_kb) {
+    const int64_t rest = tiles % units;
+    if (rest > 0 && 2 * rest <= units && tiles - rest < INT32_MAX) {
+      args.half_from = (int32_t)(tiles - rest);
+      work += rest;
+    }
+  }
   cudaError_t err;
   ProfScope prof(ctx, GRAM_K_GEMM, 2.0 * (double)M * N * (double)K, splits > 1 ? 2 : 1, st, epi.tag ? epi.tag : "gemm");
-  const int grid = pair ? 2 * (int)((tiles * splits < units) ? tiles * splits : units)
+  const int grid = pair ? 2 * (int)(work < units ? work : units)
                         : (int)((tiles * splits < kNumSMs) ? tiles * splits : kNumSMs);
   if (splits > 1) {
     args.C = ws->splitk;
     args.ldc = N;
     args.split_stride = (int64_t)M * N;
     args.epi = EpiDev{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 0};
-    if (pair && !a_kmajor && !b_kmajor) err = launch_tc2<false, false, float, EPI_BIAS>(ma, mb, args, grid, st);
+    if (sum_form) err = launch_tc2<false, false, float, EPI_SUM>(ma, mb, args, grid, st);
     else if (pair) err = launch_tc2_major<float>(a_kmajor, b_kmajor, ma, mb, args, grid, st);
     else if (BNsel == 256) err = launch_tc_major<256, float>(a_kmajor, b_kmajor, ma, mb, args, grid, st);
     else if (BNsel == 128) err = launch_tc_major<128, float>(a_kmajor, b_kmajor, ma, mb, args, grid, st);
@@ -1713,6 +1844,7 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     else if (m_res && !b_kmajor) err = launch_tc2<true, false, float, EPI_RES>(ma, mb, args, grid, st);
     else if (m_bias && a_kmajor && b_kmajor && ts_ok) err = launch_tc2<true, true, bf16, EPI_BIAS, 8>(ma, mb, args, grid, st, pc, pp);
     else if (m_bias && a_kmajor && !b_kmajor && ts_ok) err = launch_tc2<true, false, bf16, EPI_BIAS, 8>(ma, mb, args, grid, st, pc, pp);
+    else if (sum_form && args.half_from == INT32_MAX) err = launch_tc2<false, false, float, EPI_SUM>(ma, mb, args, grid, st);
     else if (m_bias && c_f32 && a_kmajor && !b_kmajor) err = launch_tc2<true, false, float, EPI_BIAS>(ma, mb, args, grid, st);
     else if (c_f32) err = launch_tc2_major<float>(a_kmajor, b_kmajor, ma, mb, args, grid, st);
     else err = launch_tc2_major<bf16>(a_kmajor, b_kmajor, ma, mb, args, grid, st);

@@ -1,4 +1,5 @@
-"""The paired matrix product's GELU epilogue without the derivative."""
+"""Work units of the paired matrix product: whole waves followed by a last one of half-width units, K ranges of several accumulator
+chains, the GELU epilogue without the derivative."""
 import numpy as np
 import pytest
 import torch
@@ -6,6 +7,14 @@ import torch
 from tests import test_gpu_gemm as base
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("kind", ["gelu", "dgelu", "res", "res_ln", "res_ln_copy", "bias_f32", "plain_bf16"])
+@pytest.mark.parametrize("M,N,K", [(19_000, 768, 72), (6400, 1096, 136), (3000, 1800, 1032)])
+def test_last_wave_of_halves(M, N, K, kind):
+    """225, 125 and 96 tiles over 74 pairs of SMs: whole units, then halves of 3, 51 (too many: whole) and 22 tiles, ragged at the
+    lower and right edges (a half that lies outside the matrix among them)."""
+    base.test_gemm_epilogues_against_float64(M, N, K, kind)
 
 
 @pytest.mark.parametrize("M,N,K", [(512, 768, 768), (1000, 768, 136), (520, 1032, 128), (136, 200, 72), (19_000, 768, 72)])
@@ -23,3 +32,19 @@ def test_gelu_without_its_derivative(M, N, K):
     scale = want.abs().max().item()
     # the bound of the epilogue with the derivative: sums of K products, the rational erf, the result's rounding
     assert (C.double().cpu() - want).abs().max().item() <= 1e-4 * np.sqrt(K) + 2.0 ** -8 * scale + 2e-6 * scale + 4e-7 * scale + 2e-6
+
+
+@pytest.mark.parametrize("M,N,K", [(768, 768, 9000), (3072, 768, 4104), (1536, 768, 2056), (2048, 2048, 136), (2304, 2304, 1104), (264, 520, 3000)])
+def test_chains_of_a_weight_gradient(M, N, K):
+    """C += A^T B over K rows: several chains per unit and parts, one part alone, fewer k-blocks than chains would take."""
+    g = base.ctx()
+    gen = torch.Generator(device=base.DEV).manual_seed(M + N + K)
+    A = (torch.randn(K, M, generator=gen, device=base.DEV) * 0.5).to(torch.bfloat16)
+    B = (torch.randn(K, N, generator=gen, device=base.DEV) * 0.5).to(torch.bfloat16)
+    C = torch.full((M, N), 2.0, device=base.DEV)
+    g.gemm_bf16(A, 0, B, 0, C, None, 1, M, N, K)
+    g.sync()
+    g.close()
+    want = A.double().T @ B.double() + 2.0
+    # as in the products' own test: sums of K products of bf16 values
+    assert (C.double() - want).abs().max().item() <= 1e-4 * np.sqrt(K)
