@@ -204,13 +204,18 @@ __device__ __forceinline__ void epilogue_store4(const EpiDev& e, CT* C, int64_t 
 // workspace.  Weight gradients of the check's model (64 x 64 to 256 x 64 over about 900 rows): 130 to 185 us each with
 // one 64 x 64 block per tile and a synchronous load per k-block, 6 to 7 us now; the
 // model's whole training step 2.49 -> 0.48 ms with the chain of launches below.
-// What a k-block waits for is its loads: 32 k at a time in the small tiles (two rounds of loads for K = 64 instead of four).
+// What a k-block waits for is its loads: 32 k at a time in the small tiles, and four groups of 64 threads with a k-block each, so
+// that K = 128 takes one round of loads and no cluster; the groups' tiles are added in ascending order in shared memory (the 30
+// products of that step 204 -> 164 us, the step 0.47 -> 0.43 ms).
 constexpr int F32_MAX_SPLIT = 16;
 template <int TILE> struct F32Cfg {
   static constexpr int SK = TILE == 32 ? 32 : 16;          // k of one k-block
-  static constexpr int THREADS = TILE * TILE / 16;
+  static constexpr int GROUP = TILE * TILE / 16;           // threads that hold one copy of the tile
+  static constexpr int GROUPS = TILE == 32 ? 4 : 1;        // copies, each over its own k-blocks
+  static constexpr int THREADS = GROUP * GROUPS;
+  static constexpr int BUFS = GROUPS == 1 ? 2 : 1;         // operand buffers per group
   static constexpr int LD = TILE + 4;                      // keeps rows 16-byte aligned
-  static constexpr int NV = TILE * SK / 4 / THREADS;       // 16-byte pieces per thread, operand and k-block
+  static constexpr int NV = TILE * SK / 4 / GROUP;         // 16-byte pieces per thread, operand and k-block
 };
 
 // piece `idx` of an operand's k-block: rows r0 .. of a matrix with leading dimension ld, k from k0; zeros outside
@@ -289,45 +294,80 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
                                                                         int64_t k_per_split, int vec_a, int vec_b, int vec_e, EpiDev e) {
   if (!chain_begin()) return;
   using Cfg = F32Cfg<TILE>;
-  constexpr int LD = Cfg::LD, NV = Cfg::NV, T = Cfg::THREADS, SK = Cfg::SK;
-  __shared__ __align__(16) float sm[2][2][SK * LD];        // [buffer][operand]; later the block's partial tile
-  static_assert(sizeof(sm) >= sizeof(float) * TILE * LD, "the partial tile reuses the operand buffers");
-  const int tid = threadIdx.x, tx = tid % (TILE / 4), ty = tid / (TILE / 4);
+  constexpr int LD = Cfg::LD, NV = Cfg::NV, T = Cfg::GROUP, G = Cfg::GROUPS, SK = Cfg::SK, BUFS = Cfg::BUFS;
+  __shared__ __align__(16) float sm[G][BUFS][2][SK * LD];  // [group][buffer][operand]; later the groups' partial tiles
+  static_assert(sizeof(sm) >= sizeof(float) * G * TILE * LD, "the partial tiles reuse the operand buffers");
+  const int group = threadIdx.x / T, tid = threadIdx.x % T, tx = tid % (TILE / 4), ty = tid / (TILE / 4);
   const int64_t m0 = (int64_t)blockIdx.y * TILE;
   const int64_t n0 = (int64_t)blockIdx.x * TILE;
   const int64_t kb = (int64_t)blockIdx.z * k_per_split, ke = min(kb + k_per_split, K);
   float acc[4][4] = {};
   float4 fa[NV], fb[NV];
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    fa[i] = f32_fetch<TILE, A_K>(A, lda, m0, M, kb, ke, tid + i * T, vec_a);
-    fb[i] = f32_fetch<TILE, B_K>(B, ldb, n0, N, kb, ke, tid + i * T, vec_b);
-  }
-  int buf = 0;
-  for (int64_t k0 = kb; k0 < ke; k0 += SK, buf ^= 1) {
+  auto fetch = [&](int64_t k0) {                           // this group's k-block of the round that starts at k0 (zeros from ke on)
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      f32_stage<TILE, A_K>(sm[buf][0], tid + i * T, fa[i]);
-      f32_stage<TILE, B_K>(sm[buf][1], tid + i * T, fb[i]);
+      fa[i] = f32_fetch<TILE, A_K>(A, lda, m0, M, k0 + group * SK, ke, tid + i * T, vec_a);
+      fb[i] = f32_fetch<TILE, B_K>(B, ldb, n0, N, k0 + group * SK, ke, tid + i * T, vec_b);
     }
-    __syncthreads();                 // also: everyone is done with the other buffer, which the next round fills
-    if (k0 + SK < ke) {
+  };
+  fetch(kb);
+  int buf = 0;
+  for (int64_t k0 = kb; k0 < ke; k0 += SK * G, buf ^= BUFS - 1) {
+    if (BUFS == 1 && k0 > kb) __syncthreads();             // the buffer has been read
 #pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        fa[i] = f32_fetch<TILE, A_K>(A, lda, m0, M, k0 + SK, ke, tid + i * T, vec_a);
-        fb[i] = f32_fetch<TILE, B_K>(B, ldb, n0, N, k0 + SK, ke, tid + i * T, vec_b);
-      }
+    for (int i = 0; i < NV; ++i) {
+      f32_stage<TILE, A_K>(sm[group][buf][0], tid + i * T, fa[i]);
+      f32_stage<TILE, B_K>(sm[group][buf][1], tid + i * T, fb[i]);
     }
+    __syncthreads();                 // with two buffers also: everyone is done with the other one, which the next round fills
+    if (k0 + SK * G < ke) fetch(k0 + SK * G);
 #pragma unroll
     for (int k = 0; k < SK; ++k) {
-      const float4 a4 = *reinterpret_cast<const float4*>(&sm[buf][0][k * LD + 4 * ty]);
-      const float4 b4 = *reinterpret_cast<const float4*>(&sm[buf][1][k * LD + 4 * tx]);
+      const float4 a4 = *reinterpret_cast<const float4*>(&sm[group][buf][0][k * LD + 4 * ty]);
+      const float4 b4 = *reinterpret_cast<const float4*>(&sm[group][buf][1][k * LD + 4 * tx]);
       const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
+  }
+  float* part = &sm[0][0][0][0];
+  // the groups' sum of four columns of row r of the tile
+  auto group_sum = [&](int r, int c) {
+    float4 v = *reinterpret_cast<const float4*>(part + r * LD + c);
+#pragma unroll
+    for (int g = 1; g < G; ++g) {
+      const float4 x = *reinterpret_cast<const float4*>(part + g * (TILE * LD) + r * LD + c);
+      v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+    }
+    return v;
+  };
+  constexpr int TALL = Cfg::THREADS;
+  static_assert(G == 1 || TALL * 4 == TILE * TILE, "four results per thread after the groups' sum");
+  if (G > 1) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      *reinterpret_cast<float4*>(part + group * (TILE * LD) + (4 * ty + i) * LD + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    __syncthreads();
+    const int r = threadIdx.x / (TILE / 4), c = 4 * (threadIdx.x % (TILE / 4));
+    const float4 v4 = group_sum(r, c);
+    if (gridDim.z == 1) {
+      const int64_t m = m0 + r, n = n0 + c;
+      if (m >= M || n >= N) return;
+      const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+      if (vec_e) {
+        f32_finish(e, C, m * ldc + n, v, f32_aux(e, C, m * ldc + n), f32_cols(e, (int)n), e.res_mean ? e.res_mean[m] : 0.f,
+                   e.res_mean ? e.res_rstd[m] : 1.f);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (n + j < N) epilogue_store<float, float>(e, C, ldc, m, (int)n + j, v[j]);
+      }
+      return;
+    }
+    *reinterpret_cast<float4*>(part + r * LD + c) = v4;    // only this thread reads these four places
   }
   const int splits = gridDim.z;
   if (splits == 1) {
@@ -361,14 +401,15 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
       }
     return;
   }
-  float* part = &sm[0][0][0];
-  __syncthreads();
+  if (G == 1) {
+    __syncthreads();
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-    *reinterpret_cast<float4*>(part + (4 * ty + i) * LD + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    for (int i = 0; i < 4; ++i)
+      *reinterpret_cast<float4*>(part + (4 * ty + i) * LD + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  }
   const int rows = TILE / splits, r0 = blockIdx.z * rows;          // this block's share of the tile's rows
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-  for (int idx = tid; idx < rows * (TILE / 4); idx += T) {         // four columns of a row each
+  for (int idx = threadIdx.x; idx < rows * (TILE / 4); idx += TALL) {     // four columns of a row each
     const int r = r0 + idx / (TILE / 4), c = 4 * (idx % (TILE / 4));
     const int64_t m = m0 + r, n = n0 + c;
     const uint32_t at = smem_u32(part + r * LD + c);
@@ -1681,15 +1722,16 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
   if (dtype == GRAM_F32) {
     if (!c_f32) return gram_set_error(ctx, "gemm: fp32 operands need an fp32 result"), GRAM_ERR_UNSUPPORTED;
     ProfScope prof(ctx, GRAM_K_GEMM, 2.0 * (double)M * N * (double)K, 1, st, epi.tag ? epi.tag : "gemm_f32");
-    // 64 x 64 tiles once they give every SM a block, else 32 x 32 (64 threads a block, so several blocks per SM: up to
-    // four); then the K range is halved while blocks are missing and every part keeps at least two k-blocks
+    // 64 x 64 tiles once they give every SM a block, else 32 x 32; then the K range is halved over a cluster while blocks are
+    // missing and a part has more than it should: two k-blocks of 16 with the large tiles, one round of the four groups (128 k)
+    // with the small ones.
     const int64_t b64 = ceil_div64(M, 64) * ceil_div64(N, 64), b32 = ceil_div64(M, 32) * ceil_div64(N, 32);
     const bool big = b64 >= kNumSMs;
     const int64_t blocks = big ? b64 : b32, enough = big ? kNumSMs : 4 * kNumSMs;
     int parts = 1;
     const int sk = big ? F32Cfg<64>::SK : F32Cfg<32>::SK;
     const int most = F32_MAX_SPLIT < gram_cluster_blocks(ctx) ? F32_MAX_SPLIT : gram_cluster_blocks(ctx);
-    while (parts < most && blocks * parts * 2 <= enough && K >= 64 * parts) parts *= 2;
+    while (parts < most && blocks * parts * 2 <= enough && (big ? K >= 64 * parts : K > 128 * parts)) parts *= 2;
     const int64_t per = ceil_div64(ceil_div64(K, parts), sk) * sk;
     if (ceil_div64(M, big ? 64 : 32) > 65535)
       return gram_set_error(ctx, "gemm: %lld rows are more than an fp32 product takes", (long long)M), GRAM_ERR_UNSUPPORTED;
