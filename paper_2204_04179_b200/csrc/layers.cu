@@ -1607,39 +1607,70 @@ gram_status attention_backward(gram_ctx* ctx, int dtype, const void* qkv, const 
   return GRAM_OK;
 }
 
-// fold[g][c] = sum of part[r][c] over the rows r = g, g + G, g + 2G, ... (G = gridDim.y), warps taking every
-// eighth of them and adding their sums in ascending order
-__global__ void __launch_bounds__(256) fold_partials_kernel(const float* __restrict__ part, int64_t nrows, int n,
-                                                            float* __restrict__ fold) {
+// out[c] += sum over r of part[r][c].  A cluster of blocks owns 32 columns: warp w of its block b adds the rows 8 b + w, 8 C + 8 b + w,
+// ... (eight on their way at once), and block 0 adds the warps' and then the blocks' sums in ascending order.  800 x 3072 and
+// 256 x 2304 partial rows: 6.3 us on average; as two launches, 32 folded rows and their sum, 7.5 + 3.
+__global__ void __launch_bounds__(256) colsum_partials_kernel(const float* __restrict__ part, int64_t nrows, int n, float* __restrict__ out) {
   if (!chain_begin()) return;
   __shared__ float sa[8][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __shared__ float total[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, C = gridDim.y;
   const int c = blockIdx.x * 32 + lane;
-  const int64_t G = gridDim.y;
+  const int64_t step = 8 * (int64_t)C;
   float a = 0.f;
   if (c < n) {
-    for (int64_t r = blockIdx.y + (int64_t)w * G; r < nrows; r += 8 * G) a += part[r * n + c];
+    int64_t r = 8 * (int64_t)blockIdx.y + w;
+    for (; r + 7 * step < nrows; r += 8 * step) {
+      float x[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) x[k] = part[(r + k * step) * n + c];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) a += x[k];
+    }
+    for (; r < nrows; r += step) a += part[r * n + c];
   }
   sa[w][lane] = a;
   __syncthreads();
-  if (w == 0 && c < n) {
+  if (w == 0) {
     float t = sa[0][lane];
 #pragma unroll
     for (int k = 1; k < 8; ++k) t += sa[k][lane];
-    fold[(int64_t)blockIdx.y * n + c] = t;
+    total[lane] = t;
   }
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (blockIdx.y == 0 && w == 0 && c < n) {
+    const uint32_t mine = tc::smem_u32(&total[lane]);
+    float t = 0.f;
+    for (int b = 0; b < C; ++b) {
+      uint32_t at;
+      float x;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(mine), "r"(b));
+      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(at) : "memory");
+      t += x;
+    }
+    out[c] += t;
+  }
+  // no block may leave while its total is still read
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-gram_status colsum_from_partials(gram_ctx* ctx, const float* part, int64_t nrows, int N, float* out, float* scratch,
-                                 cudaStream_t st) {
+gram_status colsum_from_partials(gram_ctx* ctx, const float* part, int64_t nrows, int N, float* out, cudaStream_t st) {
   if (nrows == 0 || N == 0) return GRAM_OK;
-  ProfScope prof(ctx, GRAM_K_COLSUM, (double)nrows * N * 4.0, 2, st, "colsum_partials");
-  int G = 32;                                             // rows of the folded matrix (fixed: the order of additions depends on it)
-  if ((size_t)G * N * sizeof(float) > kRedScratchBytes) G = (int)(kRedScratchBytes / ((size_t)N * sizeof(float)));
-  if (G < 1) return gram_set_error(ctx, "column sums: N too large for the reduction scratch"), GRAM_ERR_UNSUPPORTED;
-  launch_chain(fold_partials_kernel, dim3((unsigned)ceil_div(N, 32), (unsigned)G), 256, 0, st, part, nrows, N, scratch);
-  launch_chain(reduce_partials_kernel, ceil_div(N, 32), 256, 0, st, scratch, G, (int64_t)N, N, out, nullptr, nullptr, 1.f);
-  GRAM_LAUNCH_CHECK(ctx);
+  ProfScope prof(ctx, GRAM_K_COLSUM, (double)nrows * N * 4.0, 1, st, "colsum_partials");
+  const int C = gram_cluster_blocks(ctx) < 8 ? gram_cluster_blocks(ctx) : 8;          // fixed for a context: the order of additions depends on it
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ceil_div(N, 32), (unsigned)C);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = (unsigned)C;
+  attr[0].val.clusterDim.z = 1;
+  attr[1] = chain_attribute();
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  GRAM_CUDA(ctx, cudaLaunchKernelEx(&cfg, colsum_partials_kernel, part, nrows, N, out));
   return GRAM_OK;
 }
 

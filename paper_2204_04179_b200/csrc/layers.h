@@ -118,8 +118,7 @@ gram_status attention_backward_mma(gram_ctx* ctx, const void* qkv, const void* d
 
 // out[n] += sum_rows X[r, n]   (X operand-typed)
 // out[c] += sum over the nrows rows of part[., c] (fp32 [nrows, N]; partial column sums left by a fused producer)
-gram_status colsum_from_partials(gram_ctx* ctx, const float* part, int64_t nrows, int N, float* out, float* scratch,
-                                 cudaStream_t st);
+gram_status colsum_from_partials(gram_ctx* ctx, const float* part, int64_t nrows, int N, float* out, cudaStream_t st);
 gram_status colsum_accumulate(gram_ctx* ctx, int dtype, const void* X, int64_t rows, int N, float* out, float* scratch,
                               cudaStream_t st);
 // out[s, :] += sum_u X[u*period + s, :]  (s < period; X fp32)

@@ -443,7 +443,7 @@ gram_status layer_rest_backward(Model* m, Module& mod, const LayerOff& o, Stack&
     const bool fused_b1 = gemm_fused_colsum(m->dtype, T, f);                           // the product's epilogue also adds up its columns
     if (fused_b1) e.colsum_part = s.cpart;
     GRAM_TRY(mm_dx(m, s.dzb, W(m, mod, o.w2), s.du, false, T, d, f, e, st));           // du = (dz2 W2) * gelu'(v), the saved u
-    if (fused_b1) GRAM_TRY(colsum_from_partials(ctx, s.cpart, (T + 31) / 32, f, mod.g + o.b1, red, st));
+    if (fused_b1) GRAM_TRY(colsum_from_partials(ctx, s.cpart, (T + 31) / 32, f, mod.g + o.b1, st));
     else GRAM_TRY(colsum_accumulate(ctx, m->dtype, s.du, T, f, mod.g + o.b1, red, st));
     GRAM_TRY(mm_dw(m, s.du, a.h1, mod.g + o.w1, T, f, d, st, "dw_ffn1"));
     e = GemmEpilogue();
@@ -480,7 +480,7 @@ gram_status layer_attention_backward(Model* m, Module& mod, Stack& s, int l, con
   GRAM_TRY(attention_backward(ctx, m->dtype, a.qkv, s.dctx, a.ctx, a.lse, s.delta, s.dqkv, s.cpart,
                               (int64_t)(s.cpart_elems / ((size_t)3 * d)), &part_rows, T, n_seq, S, d, s.heads, s.causal, s.seq_len,
                               s.seq_off, s.grouped ? &s.groups : nullptr, st));
-  if (part_rows > 0) GRAM_TRY(colsum_from_partials(ctx, s.cpart, part_rows, 3 * d, mod.g + o.bqkv, m->red, st));
+  if (part_rows > 0) GRAM_TRY(colsum_from_partials(ctx, s.cpart, part_rows, 3 * d, mod.g + o.bqkv, st));
   else GRAM_TRY(colsum_accumulate(ctx, m->dtype, s.dqkv, T, 3 * d, mod.g + o.bqkv, m->red, st));
   GRAM_TRY(mm_dw(m, s.dqkv, xb_l, mod.g + o.wqkv, T, 3 * d, d, st, "dw_qkv"));
   GemmEpilogue e;
@@ -531,7 +531,7 @@ gram_status cls_attention_backward(Model* m, int32_t n, int64_t T, const int32_t
   int64_t part_rows = 0;
   GRAM_TRY(attention_cls_backward(ctx, tl.acts[0].qkv, s.acts[last].qkv, tl.dctx, tl.dqkv, s.dqkv, s.cpart,
                                   (int64_t)(s.cpart_elems / ((size_t)3 * d)), &part_rows, n, c.l_t, d, c.n_heads, seq_len, seq_off, st));
-  GRAM_TRY(colsum_from_partials(ctx, s.cpart, part_rows, 3 * d, m->ce.g + o.bqkv, m->red, st));
+  GRAM_TRY(colsum_from_partials(ctx, s.cpart, part_rows, 3 * d, m->ce.g + o.bqkv, st));
   GRAM_TRY(mm_dw(m, s.dqkv, xb, m->ce.g + o.wqkv + kv_off, T, 2 * d, d, st, "dw_kv"));
   GRAM_TRY(mm_dw(m, tl.dqkv, cls_input_rows(m), m->ce.g + o.wqkv, n, d, d, st, "dw_q"));
   GemmEpilogue e;
