@@ -316,7 +316,7 @@ def run_gemm_sites(args):
     from paper_2204_04179_b200 import binding
     dev = "cuda:0"
     peaks = measured_peaks()
-    cfg = binding.GramConfig(); cfg.n_items = 8; cfg.P_max = 8; cfg.d = 8; cfg.d_ff = 4096
+    cfg = binding.GramConfig(); cfg.n_items = 8; cfg.P_max = 8; cfg.d = 768; cfg.d_ff = 3072     # a model's workspace of partial products
     g = binding.Gram(cfg)
     T = args.rows
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
