@@ -1870,7 +1870,7 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     // the fp32 residual products with a short reduction (K <= 1024: the output projection of attention), where the epilogue's
     // memory traffic outlasts the main loop: result and residual as fp32 boxes of 32 rows x 32 columns through bulk tensor
     // copies (no bf16 copy on this path).  With longer K the register path keeps six pipeline stages instead of four and
-    // is the faster one (measured: 1279 against 1175 TFLOP/s at K = 3072).
+    // is the faster one (65 536 x 768: 209 against 244 us at K = 3072, 162 against 191 at K = 2304).
     CUtensorMap mcf, mrf;
     const bool rs_ok = m_res && !e.copy_out && K <= 1024 && res_ts_env() && M < (int64_t)1 << 31 && (uintptr_t)e.res % 16 == 0 &&
                        make_map_f32(&mcf, C, (uint64_t)N, (uint64_t)M, (uint64_t)ldc, 32, 32) &&
