@@ -209,6 +209,11 @@ gram_status gram_selftest_ring_rows(gram_ctx* ctx, int32_t rows);
  * beyond those the forms that need none; results of gram_dedup do not depend on it.  This call shows it: the context's
  * later calls use clusters of at most `blocks` (1, 2, 4, 8).  blocks <= 0: as many as can be placed (as created). */
 gram_status gram_selftest_cluster_blocks(gram_ctx* ctx, int32_t blocks);
+/* The sum behind the bias gradients whose rows a producer has already added up in part, on its own:
+ * d_out[c] += sum over r < rows of d_part[r, c], fp32 [rows, N].  For tests: within a step its error is hidden by that of
+ * the 16-bit operands. */
+gram_status gram_selftest_column_sums(gram_ctx* ctx, const float* d_part, int64_t rows, int32_t N, float* d_out,
+                                      gram_stream stream);
 
 /* Stage 3 (Section 4.3: the encoder's output h_i is handed to the task module, which completes the forward pass
  * with it; Fig. 1 draws the copies): d_E[p, :] = d_src[d_index[p], :] for p < P.  Single-step: src = H,

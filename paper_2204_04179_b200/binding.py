@@ -34,7 +34,7 @@ SYMBOLS = ["gram_create", "gram_destroy", "gram_sync", "gram_last_error", "gram_
            "gram_window_reset", "gram_get_window", "gram_gemm_bf16", "gram_profile", "gram_profile_read",
            "gram_launch_count", "gram_profile_dump", "gram_accumulate_static", "gram_optimizer_step",
            "gram_optimizer_reset", "gram_noam_rate", "gram_adam_update", "gram_state_export", "gram_state_import",
-           "gram_optimizer_export", "gram_optimizer_import", "gram_selftest_bounded_wait", "gram_selftest_ring_rows", "gram_selftest_cluster_blocks", "gram_grads_device",
+           "gram_optimizer_export", "gram_optimizer_import", "gram_selftest_bounded_wait", "gram_selftest_ring_rows", "gram_selftest_cluster_blocks", "gram_selftest_column_sums", "gram_grads_device",
            "gram_gemm_bf16_epilogue"]
 
 KINDS = ["gemm", "attention", "layernorm", "colsum", "embed_pool", "dedup", "gather", "accumulate", "task_head", "other",
@@ -221,6 +221,11 @@ class Gram:
     def selftest_cluster_blocks(self, blocks: int):
         """Later calls use clusters of at most this many thread blocks (<= 0: as many as the device places)."""
         self._ck(lib().gram_selftest_cluster_blocks(self._h, C.c_int32(blocks)))
+
+    def selftest_column_sums(self, part, out, stream=None):
+        """out[c] += the sum of column c of part (fp32 [rows, N])."""
+        self._ck(lib().gram_selftest_column_sums(self._h, _ptr(part), C.c_int64(part.shape[0]), C.c_int32(part.shape[1]), _ptr(out),
+                                                 _stream(stream)))
 
     def selftest_ring_rows(self, rows: int):
         """Later calls' row rings give up on row number `rows` of a warp (< 0: never)."""

@@ -254,6 +254,12 @@ gram_status gram_selftest_cluster_blocks(gram_ctx* ctx, int32_t blocks) {
   while (blocks > 0 && ctx->cluster_blocks > blocks) ctx->cluster_blocks /= 2;
   return GRAM_OK;
 }
+gram_status gram_selftest_column_sums(gram_ctx* ctx, const float* d_part, int64_t rows, int32_t N, float* d_out,
+                                      gram_stream stream) {
+  if (!ctx || rows < 0 || N < 0) return GRAM_ERR_ARG;
+  if (rows > 0 && N > 0 && (!d_part || !d_out)) return gram_set_error(ctx, "gram_selftest_column_sums: null buffer"), GRAM_ERR_ARG;
+  return colsum_from_partials(ctx, d_part, rows, N, d_out, S(stream));
+}
 gram_status gram_selftest_ring_rows(gram_ctx* ctx, int32_t rows) {
   if (!ctx) return GRAM_ERR_ARG;
   ctx->ring_rows = rows < 0 ? INT32_MAX : rows;

@@ -574,9 +574,6 @@ constexpr int CD_THREADS = 512;
 constexpr int CD_WARPS = CD_THREADS / 32;
 constexpr int kClusterMaxBlocks = 16;     // an opt-in above 8
 
-__device__ __forceinline__ void cd_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ uint32_t cd_remote(const void* p, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
@@ -665,7 +662,7 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
       }
       s.count[tid] = run;
     }
-    cd_cluster_sync();                                   // every block's pairs are in registers, its counts published
+    gram_cluster_sync();                                 // every block's pairs are in registers, its counts published
     int32_t total = 0, before_blocks = 0;
     if (tid < RADIX) {
       for (int b = 0; b < blocks; ++b) {
@@ -686,7 +683,7 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
         asm volatile("st.shared::cluster.v2.s32 [%0], {%1, %2};" ::"r"(at), "r"(key[r]), "r"(val[r]) : "memory");
       }
     }
-    cd_cluster_sync();                                   // all pairs are at their places
+    gram_cluster_sync();                                 // all pairs are at their places
   }
   // run lengths: thread t looks at ROUNDS consecutive places
   const int first = tid * ROUNDS;
@@ -706,7 +703,7 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
   int32_t btot;
   int32_t ex = block_exclusive_scan(tot, s.sw, &btot);
   if (tid == 0) s.heads = btot;
-  cd_cluster_sync();
+  gram_cluster_sync();
   int32_t U = 0;
   for (int b = 0; b < blocks; ++b) {
     const int32_t h = cd_load(cd_remote(&s.heads, (uint32_t)b));
@@ -729,7 +726,7 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
     *n_unique = U;
     seg_off[U] = P;
   }
-  cd_cluster_sync();                                     // nobody leaves while its counts may still be read
+  gram_cluster_sync();                                   // nobody leaves while its counts may still be read
   if (bad) {                                             // an ID out of range belongs to no item, as in inverse_kernel
 #pragma unroll
     for (int r = 0; r < ROUNDS; ++r) {

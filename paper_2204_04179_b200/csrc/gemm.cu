@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
       *reinterpret_cast<float4*>(part + (4 * ty + i) * LD + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
   }
   const int rows = TILE / splits, r0 = blockIdx.z * rows;          // this block's share of the tile's rows
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  gram_cluster_sync();
   for (int idx = threadIdx.x; idx < rows * (TILE / 4); idx += TALL) {     // four columns of a row each
     const int r = r0 + idx / (TILE / 4), c = 4 * (idx % (TILE / 4));
     const int64_t m = m0 + r, n = n0 + c;
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
     }
   }
   // no block may leave while another still reads its partial tile
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  gram_cluster_sync();
 }
 
 template <int TILE, bool A_K, bool B_K>
@@ -988,9 +988,6 @@ __device__ __forceinline__ void mbar_arrive_expect_tx_remote(uint32_t cluster_ba
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int32_t c0, int32_t c1,
                                                  uint32_t cluster_bar) {
   asm volatile(
@@ -1419,7 +1416,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();                           // both CTAs' barriers exist before anyone signals them
+  gram_cluster_sync();                           // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   if (!chain_begin()) return;              // barriers and tensor memory are set up before the wait
@@ -1582,7 +1579,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
     }
     __syncthreads();
   }
-  cluster_sync_all();                        // the peer no longer reads this CTA's memory or signals its barriers
+  gram_cluster_sync();                        // the peer no longer reads this CTA's memory or signals its barriers
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)Cfg::TMEM_COLS)

@@ -144,6 +144,13 @@ struct ProfScope {
   ~ProfScope() { if (slot >= 0) gram_prof_close(ctx, slot, st); }
 };
 
+// All threads of a cluster meet.  The instructions take whole warps (.aligned): lanes that a test or a loop of their own sent
+// different ways are brought together first.
+__device__ __forceinline__ void gram_cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // the device status word: kernels record the first error kind they meet
 __device__ __forceinline__ void gram_device_fail(int32_t* status, int32_t code) { atomicCAS(status, 0, code); }
 int32_t* gram_status_word(gram_ctx* ctx);

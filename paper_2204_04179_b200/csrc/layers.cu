@@ -1637,7 +1637,7 @@ __global__ void __launch_bounds__(256) colsum_partials_kernel(const float* __res
     for (int k = 1; k < 8; ++k) t += sa[k][lane];
     total[lane] = t;
   }
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  gram_cluster_sync();
   if (blockIdx.y == 0 && w == 0 && c < n) {
     const uint32_t mine = tc::smem_u32(&total[lane]);
     float t = 0.f;
@@ -1651,7 +1651,7 @@ __global__ void __launch_bounds__(256) colsum_partials_kernel(const float* __res
     out[c] += t;
   }
   // no block may leave while its total is still read
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  gram_cluster_sync();
 }
 
 gram_status colsum_from_partials(gram_ctx* ctx, const float* part, int64_t nrows, int N, float* out, cudaStream_t st) {
