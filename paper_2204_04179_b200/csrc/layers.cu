@@ -1607,57 +1607,61 @@ gram_status attention_backward(gram_ctx* ctx, int dtype, const void* qkv, const 
   return GRAM_OK;
 }
 
-// out[c] += sum over r of part[r][c].  A cluster of blocks owns 32 columns: warp w of its block b adds the rows 8 b + w, 8 C + 8 b + w,
-// ... (eight on their way at once), and block 0 adds the warps' and then the blocks' sums in ascending order.  800 x 3072 and
-// 256 x 2304 partial rows: 6.3 us on average; as two launches, 32 folded rows and their sum, 7.5 + 3.
+// out[c] += sum over r of part[r][c].  The rows are cut into eight parts whatever the device places: warp w adds the rows 8 p + w,
+// 8 p + w + 64, ... of part p, eight on their way at once and each into a sum of its own, so that a chain of additions is
+// nrows / 512 long.  A cluster of blocks owns 32 columns and shares the parts; block 0 adds their sums in ascending order.
+// 800 x 3072, 256 x 2304 and 4096 x 2304 partial rows: 3.9, 3.3 and 6.0 us (with one sum per lane 5.2, 3.6 and 9.0).
+constexpr int COLSUM_PARTS = 8;
 __global__ void __launch_bounds__(256) colsum_partials_kernel(const float* __restrict__ part, int64_t nrows, int n, float* __restrict__ out) {
   if (!chain_begin()) return;
-  __shared__ float sa[8][32];
-  __shared__ float total[32];
+  __shared__ float sa[COLSUM_PARTS][8][32], total[COLSUM_PARTS][32];       // this block's parts only
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, C = gridDim.y;
   const int c = blockIdx.x * 32 + lane;
-  const int64_t step = 8 * (int64_t)C;
-  float a = 0.f;
-  if (c < n) {
-    int64_t r = 8 * (int64_t)blockIdx.y + w;
-    for (; r + 7 * step < nrows; r += 8 * step) {
-      float x[8];
+  constexpr int64_t step = 8 * COLSUM_PARTS;
+  for (int p = blockIdx.y; p < COLSUM_PARTS; p += C) {
+    float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (c < n) {
+      const float* x = part + (8 * p + w) * (int64_t)n + c;
+      int64_t left = (nrows - (8 * p + w) + step - 1) / step;          // rows of this warp
+      for (; left >= 8; left -= 8, x += 8 * step * n) {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) x[k] = part[(r + k * step) * n + c];
+        for (int k = 0; k < 8; ++k) a[k] += x[k * step * n];
+      }
 #pragma unroll
-      for (int k = 0; k < 8; ++k) a += x[k];
+      for (int k = 0; k < 7; ++k)
+        if (k < left) a[k] += x[k * step * n];
     }
-    for (; r < nrows; r += step) a += part[r * n + c];
+    sa[p][w][lane] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
   }
-  sa[w][lane] = a;
   __syncthreads();
-  if (w == 0) {
-    float t = sa[0][lane];
+  if (w % C == (int)blockIdx.y) {                          // warp w: the warps' sums of part w
+    float t = sa[w][0][lane];
 #pragma unroll
-    for (int k = 1; k < 8; ++k) t += sa[k][lane];
-    total[lane] = t;
+    for (int k = 1; k < 8; ++k) t += sa[w][k][lane];
+    total[w][lane] = t;
   }
   gram_cluster_sync();
-  if (blockIdx.y == 0 && w == 0 && c < n) {
-    const uint32_t mine = tc::smem_u32(&total[lane]);
-    float t = 0.f;
-    for (int b = 0; b < C; ++b) {
+  if (blockIdx.y == 0 && w == 0) {
+    float x[COLSUM_PARTS];
+#pragma unroll
+    for (int p = 0; p < COLSUM_PARTS; ++p) {
       uint32_t at;
-      float x;
-      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(mine), "r"(b));
-      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(at) : "memory");
-      t += x;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(tc::smem_u32(&total[p][lane])), "r"(p % C));
+      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x[p]) : "r"(at) : "memory");
     }
-    out[c] += t;
+    float t = x[0];
+#pragma unroll
+    for (int p = 1; p < COLSUM_PARTS; ++p) t += x[p];
+    if (c < n) out[c] += t;
   }
-  // no block may leave while its total is still read
+  // no block may leave while its totals are still read
   gram_cluster_sync();
 }
 
 gram_status colsum_from_partials(gram_ctx* ctx, const float* part, int64_t nrows, int N, float* out, cudaStream_t st) {
   if (nrows == 0 || N == 0) return GRAM_OK;
   ProfScope prof(ctx, GRAM_K_COLSUM, (double)nrows * N * 4.0, 1, st, "colsum_partials");
-  const int C = gram_cluster_blocks(ctx) < 8 ? gram_cluster_blocks(ctx) : 8;          // fixed for a context: the order of additions depends on it
+  const int C = gram_cluster_blocks(ctx) < COLSUM_PARTS ? gram_cluster_blocks(ctx) : COLSUM_PARTS;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)ceil_div(N, 32), (unsigned)C);
   cfg.blockDim = dim3(256);

@@ -26,6 +26,26 @@ def test_column_sums(rows, N, blocks):
     assert ((out.double() - want).abs() <= (rows + 1) * 2.0 ** -24 * want).all()
 
 
+def test_column_sums_do_not_depend_on_the_clusters_and_keep_their_chains_short():
+    """64 rows far larger than the rest: an addition to them loses what a chain that does not hold them keeps."""
+    rows, N = 32_768, 72
+    part = torch.ones(rows, N, device="cuda")
+    part[:64] = 2.0 ** 24
+    part += torch.rand(rows, N, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    want, got = part.double().sum(0), []
+    for blocks in (0, 8, 4, 2, 1):
+        g = ctx()
+        g.selftest_cluster_blocks(blocks)
+        got.append(torch.zeros(N, device="cuda"))
+        g.selftest_column_sums(part, got[-1])
+        g.sync()
+        g.close()
+        assert torch.equal(got[-1], got[0])
+    # an element passes rows / 512 additions of its chain, 3 of the chains, 7 of the warps, 7 of the parts and the last one, each
+    # off by at most 2^-24 of a sum that is no larger than the whole
+    assert ((got[0].double() - want).abs() <= (rows / 512 + 18) * 2.0 ** -24 * want).all()
+
+
 @pytest.mark.parametrize("B,L", [(13, 20), (9, 60)])
 def test_feed_forward_bias_of_a_width_off_32(B, L):
     """1096 columns: the last cluster of the sum has columns that do not exist, and the product before it ends in half-width units."""
