@@ -546,7 +546,7 @@ template <int BN> struct TcCfg {
 // Epilogue variants fixed at compile time (the general one reads the EpiDev flags at run time):
 //   EPI_DG    multiply by the saved GELU derivative, bf16 out (values prefetched during the main loop)
 //   EPI_BIAS  (+ bias), bf16 or fp32 out
-//   EPI_GELU  + bias, GELU, saved derivative, both bf16
+//   EPI_GELU  + bias, GELU, saved derivative, both bf16 (pair kernel)
 //   EPI_GELU_V  the same without the derivative (passes that no backward pass follows; pair kernel)
 //   EPI_RES   (+ bias) + fp32 residual (LayerNorm on the fly when res_mean is set), fp32 out (+ bf16 copy)
 //   EPI_SUM   fp32 out (added to C on request) of a K range that is cut into several accumulator chains (pair kernel)
@@ -677,7 +677,7 @@ __device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t r
     }
     tc_fence_before();
     return true;
-  } else if constexpr (MODE == EPI_BIAS || MODE == EPI_GELU) {
+  } else if constexpr (MODE == EPI_BIAS) {
     if (!mbar_wait(tfull_addr, parity, abort_flag)) return false;
     tc_fence_after();
     const int sub = lane >> 3, slot = lane & 7;
@@ -695,39 +695,15 @@ __device__ __forceinline__ bool epilogue_tile(const TcArgs& a, CT* Cs, int64_t r
         if (a.epi.bias) ld4(a.epi.bias + n, b4);
         const int64_t o0 = (row0 + sub) * a.ldc + n;      // element offset of this lane's first row
         const int64_t step = 4 * a.ldc;
-        if constexpr (MODE == EPI_BIAS) {
-          CT* cp = Cs + o0;
+        CT* cp = Cs + o0;
 #pragma unroll
-          for (int rr = 0; rr < 8; ++rr) {
-            if (rr * 4 < rows_left) {
-              const float4 t = stage_read(stage, rr * 4 + sub, slot);
-              const float x[4] = {t.x + b4[0], t.y + b4[1], t.z + b4[2], t.w + b4[3]};
-              st4(cp, x);
-            }
-            cp += step;
+        for (int rr = 0; rr < 8; ++rr) {
+          if (rr * 4 < rows_left) {
+            const float4 t = stage_read(stage, rr * 4 + sub, slot);
+            const float x[4] = {t.x + b4[0], t.y + b4[1], t.z + b4[2], t.w + b4[3]};
+            st4(cp, x);
           }
-        } else if constexpr (MODE == EPI_GELU) {
-          CT* cp = Cs + o0;
-          bf16* pp = reinterpret_cast<bf16*>(a.epi.pre) + o0;
-#pragma unroll
-          for (int rr = 0; rr < 8; ++rr) {
-            if (rr * 4 < rows_left) {
-              const float4 t = stage_read(stage, rr * 4 + sub, slot);
-              float x[4] = {t.x + b4[0], t.y + b4[1], t.z + b4[2], t.w + b4[3]};
-              float dg[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                float c, p;
-                gelu_parts(x[i], c, p);
-                dg[i] = c + x[i] * p;
-                x[i] *= c;
-              }
-              st4(cp, x);
-              st4(pp, dg);
-            }
-            cp += step;
-            pp += step;
-          }
+          cp += step;
         }
       }
       __syncwarp();
