@@ -1781,7 +1781,7 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
       if (ceil_div(splits, per) != sp) continue;
       const int64_t total = tiles * sp;
       const double fill = (double)tiles * splits / ((double)ceil_div64(total, units) * units * per);
-      if (fill >= best - 0.02) { best_sp = sp; if (fill > best) best = fill; }
+      if (fill >= 0.98 * best) { best_sp = sp; if (fill > best) best = fill; }
     }
     args.kb_per_split = ceil_div(splits, best_sp) * args.chain;
     splits = ceil_div(args.num_kb, args.kb_per_split);

@@ -48,3 +48,17 @@ def test_chains_of_a_weight_gradient(M, N, K):
     want = A.double().T @ B.double() + 2.0
     # as in the products' own test: sums of K products of bf16 values
     assert (C.double() - want).abs().max().item() <= 1e-4 * np.sqrt(K)
+
+
+def test_parts_where_one_tile_leaves_the_chip_empty():
+    """256 x 256 over 16 k-blocks: two chains.  One after the other would halve the few units there are, so they stay two parts:
+    the product and the sum of its parts, two launches."""
+    g = base.ctx()
+    A, B = (torch.ones(1024, 256, dtype=torch.bfloat16, device=base.DEV) for _ in range(2))
+    C = torch.zeros(256, 256, device=base.DEV)
+    before = g.launch_count()
+    g.gemm_bf16(A, 0, B, 0, C, None, 1, 256, 256, 1024)
+    g.sync()
+    assert g.launch_count() - before == 2
+    g.close()
+    assert (C == 1024).all()
