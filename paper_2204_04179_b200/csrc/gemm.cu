@@ -1286,7 +1286,8 @@ __device__ __forceinline__ int64_t tc2_units(const TcArgs& a) {
 // here, the parts of the K range that go through memory need no longer be as many as the chains.  Units of one chain keep the
 // epilogues that write a block of columns as it comes out of the accumulator (2304 x 768 over 4096 rows: 26.3 us, 29.4 through
 // these registers; 768 x 3072 over 1000 rows 14.1 and 15.5).
-__device__ __forceinline__ bool epilogue_unit_sum(const TcArgs& a, float* Cs, int64_t row0, int n_first, int half, int q, int lane,
+constexpr int SUM_CHAIN_MAX = 192;       // k-blocks of a chain, whatever the tiles and the workspace: 65 536 rows in six
+__device__ __forceinline__ bool epilogue_unit_sum(const TcArgs& a, float* Cs, int64_t row0, int n_first, int n_lim, int half, int q, int lane,
                                                   float* stage, uint32_t tmem_base, int64_t it, int chains, uint32_t tfull0,
                                                   uint32_t tempty0_remote, volatile int* abort_flag) {
   float acc[4][32];
@@ -1321,7 +1322,7 @@ __device__ __forceinline__ bool epilogue_unit_sum(const TcArgs& a, float* Cs, in
     stage_write_row(stage, lane, v);
     __syncwarp();
     const int n = n_first + half * 128 + b * 32 + slot * 4;
-    if (n < a.N) {                                     // N is a multiple of 8
+    if (n < n_lim) {                                   // N is a multiple of 8
       float* cp = Cs + (row0 + sub) * a.ldc + n;
 #pragma unroll
       for (int rr = 0; rr < 8; ++rr) {
@@ -1505,7 +1506,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) gemm_tc2_kernel(const __grid_
       const int64_t row0 = (int64_t)u.tm * 2 * BM + (int64_t)rank * BM + q * 32;
       if constexpr (MODE == EPI_SUM) {
         const int chains = (u.kb1 - u.kb0 + a.chain - 1) / a.chain;
-        if (!epilogue_unit_sum(a, reinterpret_cast<float*>(C) + (int64_t)u.split * a.split_stride, row0, u.n_first, half, q, lane, stage,
+        if (!epilogue_unit_sum(a, reinterpret_cast<float*>(C) + (int64_t)u.split * a.split_stride, row0, u.n_first, n_lim, half, q, lane, stage,
                                tmem_base, it, chains, tfull_bar(0), map_to_cta(tempty_bar(0), 0), abort_flag)) {
           failed = true;
           break;
@@ -1747,25 +1748,30 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
   int splits = 1;
   // weight gradients: a plain fp32 result, added to C or not
   const bool sum_form = pair && !a_kmajor && !b_kmajor && c_f32 && !e.bias && !e.gelu && !e.dgelu_pre && !e.res && !e.copy_out && !e.pre;
-  if (allow_splitk && tiles < units && args.num_kb >= 16 && ws && ws->splitk) {
+  // parts of the K range that go through memory: where the tiles do not fill the chip, as many as the workspace takes
+  const int64_t per = (int64_t)M * N * (int64_t)sizeof(float);
+  const int64_t most = allow_splitk && tiles < units && ws && ws->splitk ? (int64_t)(ws->splitk_bytes / per) : 1;
+  int chains = 1;
+  if (allow_splitk && tiles < units && args.num_kb >= 16 && (sum_form || most > 1)) {
     // chains of additions in the accumulator: between 2 and 4 per CTA (pair), each of at least eight k-blocks; among those, the
     // count that leaves the last wave fullest.  Longer chains cost precision: the tensor core adds into its fp32 accumulator by
     // cutting off, so the error of a chain grows with its length, while the chains themselves are added with rounding
     // (65 536 rows, 3072 x 768, against 64 bits: 1.2e-5 from 6 chains, 3.8e-5 from 2).
-    const int64_t per = (int64_t)M * N * (int64_t)sizeof(float);
     int lo = (int)((2 * units + tiles - 1) / tiles), hi = (int)((4 * units + tiles - 1) / tiles);
     int cap = args.num_kb / 8;
-    if ((int64_t)cap * per > (int64_t)ws->splitk_bytes) cap = (int)(ws->splitk_bytes / per);
+    if (!sum_form && cap > most) cap = (int)most;          // each chain is a part here
     if (hi > cap) hi = cap;
     if (lo > hi) lo = hi;
     double best = -1.0;
-    for (int sp = lo; sp <= hi && sp >= 1; ++sp) {
-      const int64_t total = tiles * sp;
+    for (int ch = lo; ch <= hi && ch >= 1; ++ch) {
+      const int64_t total = tiles * ch;
       const double fill = (double)total / (double)(ceil_div64(total, units) * units);
-      if (fill > best + 1e-9) { best = fill; splits = sp; }
+      if (fill > best + 1e-9) { best = fill; chains = ch; }
     }
-    if (splits < 1) splits = 1;
   }
+  // weight gradients add their chains in registers: neither the workspace nor a chip full of tiles lets a chain grow
+  if (sum_form && chains < ceil_div(args.num_kb, SUM_CHAIN_MAX)) chains = ceil_div(args.num_kb, SUM_CHAIN_MAX);
+  splits = chains;
   args.kb_per_split = ceil_div(args.num_kb, splits);
   splits = ceil_div(args.num_kb, args.kb_per_split);
   args.chain = args.kb_per_split;
@@ -1774,13 +1780,13 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     // only as many as fill the chip: of those counts, from one unit per pair of SMs up, the one that leaves the last wave
     // fullest, the smallest of equals (within two per cent: a part costs its write, its read and a place in the sum).
     // 42 500 rows, a layer's four weight gradients on average: product 98 -> 90 us, sum of the parts 11.4 -> 7.0.
-    int best_sp = splits;
+    int best_sp = 1;
     double best = 0.0;
-    for (int sp = splits; sp >= 1; --sp) {
-      const int per = ceil_div(splits, sp);                              // chains of a part
-      if (ceil_div(splits, per) != sp) continue;
+    for (int sp = (int)(splits < most ? splits : most); sp >= 1; --sp) {
+      const int per_part = ceil_div(splits, sp);                         // chains of a part
+      if (ceil_div(splits, per_part) != sp) continue;
       const int64_t total = tiles * sp;
-      const double fill = (double)tiles * splits / ((double)ceil_div64(total, units) * units * per);
+      const double fill = (double)tiles * splits / ((double)ceil_div64(total, units) * units * per_part);
       if (fill >= 0.98 * best) { best_sp = sp; if (fill > best) best = fill; }
     }
     args.kb_per_split = ceil_div(splits, best_sp) * args.chain;
@@ -1790,7 +1796,7 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
   // The last wave's tiles as halves where twice as many still fit one wave.
   args.half_from = INT32_MAX;
   int64_t work = tiles * splits;
-  if (pair && splits == 1 && args.chain >= args.num_kb) {
+  if (pair && splits == 1) {
     const int64_t rest = tiles % units;
     if (rest > 0 && 2 * rest <= units && tiles - rest < INT32_MAX) {
       args.half_from = (int32_t)(tiles - rest);

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2204_04179_b200 import binding
 from tests import test_gpu_gemm as base
 
 pytestmark = pytest.mark.gpu
@@ -62,3 +63,34 @@ def test_parts_where_one_tile_leaves_the_chip_empty():
     assert g.launch_count() - before == 2
     g.close()
     assert (C == 1024).all()
+
+
+def _long_sum_error(M, N, K, d, d_ff):
+    """Relative error of A^T B over K rows of values of mostly one sign, in a context of width d, which sizes the workspace."""
+    cfg = binding.GramConfig()
+    cfg.n_items = cfg.P_max = 8
+    cfg.d, cfg.d_ff = d, d_ff
+    g = binding.Gram(cfg)
+    gen = torch.Generator(device=base.DEV).manual_seed(5)
+    A = (torch.randn(K, M, generator=gen, device=base.DEV) + 1).to(torch.bfloat16)
+    B = (torch.randn(K, N, generator=gen, device=base.DEV) + 1).to(torch.bfloat16)
+    C = torch.zeros(M, N, device=base.DEV)
+    g.gemm_bf16(A, 0, B, 0, C, None, 1, M, N, K)
+    g.sync()
+    g.close()
+    want = torch.zeros(M, N, dtype=torch.float64, device=base.DEV)
+    for o in range(0, K, 8192):
+        want += A[o:o + 8192].double().T @ B[o:o + 8192].double()
+    return ((C - want).norm() / want.norm()).item()
+
+
+@pytest.mark.parametrize("M,N", [(4864, 1024), (4872, 1096)])
+def test_chains_where_the_tiles_fill_the_chip(M, N):
+    """76 and 100 tiles, no parts: 65 536 rows in six chains, each of which loses at most 2^-24 per 16-term step."""
+    assert _long_sum_error(M, N, 65_536, 768, 3072) <= 65_536 / 16 / 6 * 2.0 ** -24
+
+
+def test_chains_of_a_small_workspace():
+    """As many chains as with a model's workspace, so the same losses; only the few sums of chains are put together otherwise."""
+    small, model = _long_sum_error(3072, 768, 65_536, 8, 0), _long_sum_error(3072, 768, 65_536, 768, 3072)
+    assert abs(small - model) <= 20 * 2.0 ** -24
