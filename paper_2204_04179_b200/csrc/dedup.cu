@@ -200,10 +200,17 @@ __device__ __forceinline__ int2 scan_pair(int a, int b, int32_t (*sw)[16]) {
 }
 
 // How the lanes of a round with equal digits find each other.  One vote per digit bit costs about three instructions a bit; an
-// OR of the lane's bit into the digit's word of the warp's own table costs the same for any width, but the lanes of one
-// digit follow each other, so it is for passes of MATCH_BITS bits and more.  10^7 positions of 20-bit keys, both passes:
-// 204 us with ten votes a key, 181 this way.
-constexpr int MATCH_BITS = 8;
+// OR of the lane's bit into the digit's word of the warp's own table costs the same for any width, but lanes of one digit
+// follow each other there.  So one vote finds those with the first lane's digit, which is the digit of most lanes where one ID
+// fills much of a batch, and only the others go to the table.  Whole calls over 10^7 positions, us, with a vote per bit /
+// with the table alone / this way:
+//   keys of        uniform          Zipf 1.1         Zipf 1.5         half of them one ID   one ID
+//   16 bits (2x8)  220 / 206 / 212  210 / 207 / 196  205 / 212 / 183  212 / 215 / 197       197 / 217 / 155
+//   18 bits (2x9)  269 / 257 / 261  241 / 238 / 226  231 / 236 / 210  248 / 251 / 233       223 / 246 / 181
+//   20 bits (2x10) 292 / 276 / 280  257 / 249 / 238  242 / 245 / 215  263 / 262 / 242       231 / 246 / 182
+// One pass of 7 bits: 123 with votes, 117 this way (two IDs alone, 16 lanes in line: 122 and 119); of 5 bits 115 and 107, but
+// two IDs 113 and 118, so narrower passes keep the votes.
+constexpr int MATCH_BITS = 7;
 
 template <int BINS> struct PassSmem {
   uint16_t cnt[RS_WARPS][BINS];    // keys of (warp, digit); later the warp's base inside the tile's digit run
@@ -259,9 +266,11 @@ __device__ __forceinline__ void radix_tile(PassSmem<(NBITS <= 8 ? 256 : 1024)>& 
     uint32_t peers;
     int32_t before = 0;
     if constexpr (NBITS >= MATCH_BITS) {
-      if (valid) atomicOr(&s.match[warp][dig], 1u << lane);
+      const bool with_first = dig == __shfl_sync(0xffffffffu, dig, 0);       // the valid lanes are the first ones
+      const uint32_t first_peers = __ballot_sync(0xffffffffu, valid && with_first);
+      if (valid && !with_first) atomicOr(&s.match[warp][dig], 1u << lane);
       __syncwarp();
-      peers = s.match[warp][dig];
+      peers = with_first ? first_peers : s.match[warp][dig];
     } else {
       peers = FULL ? 0xffffffffu : __ballot_sync(0xffffffffu, valid);
 #pragma unroll

@@ -40,6 +40,31 @@ def test_dedup_chain_of_launches(P, n_items):
     g.close()
 
 
+@pytest.mark.parametrize("kind", ["half", "same", "two", "runs", "uniform"])
+@pytest.mark.parametrize("n_items", [100, 40_000, 200_000, 900_000])
+def test_dedup_of_one_id_that_fills_the_batch(n_items, kind):
+    """Passes of 7 to 10 bits over rounds of 32 keys of which all, half, some or one have the first key's digit; the last
+    tile ends inside a round."""
+    P = 73_728 + 32 * 20 + 5
+    rng = np.random.default_rng(n_items)
+    ids = rng.integers(0, n_items, P).astype(np.int32)
+    if kind == "half":
+        ids[rng.random(P) < 0.5] = n_items - 1
+    elif kind == "same":
+        ids[:] = n_items // 2
+    elif kind == "two":
+        ids = np.where(ids % 2 == 0, 1, n_items - 2).astype(np.int32)
+    elif kind == "runs":
+        ids = np.repeat(ids, rng.integers(1, 60, P))[:P].copy()
+    g = index_ctx(P, n_items, 4)
+    U, *got = run_dedup(g, ids, n_items)
+    want = orc.unique_inverse(ids)
+    assert U == len(want[0])
+    for x, w in zip(got, want):
+        assert np.array_equal(x, w)
+    g.close()
+
+
 def test_dedup_of_fewer_items_than_the_context_holds():
     """A context for many items serves calls with any number of them: the widths of the passes differ from call to call."""
     P = 200_000
