@@ -66,7 +66,8 @@ constexpr int ROWS = 4;                          // row groups of a chunk: 16 ro
 constexpr int CHUNK = 4 * ROWS;
 
 // this lane's pieces of the rows j0 .. of one head's slice (zeros at and past len).  The next chunk is requested before the
-// current one is worked on, across the softmax too: a warp waits for a chunk once, not once per chunk.
+// current one is worked on, across the softmax too: a warp waits for a chunk once, not once per chunk.  That costs the forward
+// kernel registers and so blocks on an SM, which texts of a chunk or little more need: those fetch as they go (!AHEAD).
 __device__ __forceinline__ void fetch_chunk(const bf16* __restrict__ base, int64_t ld, int j0, int len, int sub, uint4 (&v)[ROWS]) {
 #pragma unroll
   for (int i = 0; i < ROWS; ++i) {
@@ -79,7 +80,8 @@ __device__ __forceinline__ void take(uint4 (&v)[ROWS], const uint4 (&next)[ROWS]
   for (int i = 0; i < ROWS; ++i) v[i] = next[i];
 }
 
-__global__ void __launch_bounds__(512) attn_cls_fwd_kernel(const bf16* __restrict__ q, const bf16* __restrict__ kv,
+template <bool AHEAD, int THREADS, int BLOCKS>
+__global__ void __launch_bounds__(THREADS, BLOCKS) attn_cls_fwd_kernel(const bf16* __restrict__ q, const bf16* __restrict__ kv,
                                                           bf16* __restrict__ ctx, int n, int l_t, int d, float c,
                                                           const int32_t* __restrict__ seq_len, const int32_t* __restrict__ seq_off) {
   if (!chain_begin()) return;
@@ -94,25 +96,16 @@ __global__ void __launch_bounds__(512) attn_cls_fwd_kernel(const bf16* __restric
     float qv[8];
     unpack8(*reinterpret_cast<const uint4*>(q + (int64_t)u * d + col), qv);
     const bf16* kb = kv + row0 * ld + col;
-    uint4 v[ROWS], next[ROWS];
-    fetch_chunk(kb, ld, 0, len, sub, v);
-    for (int j0 = 0; j0 < len; j0 += CHUNK) {
-      if (j0 + CHUNK < len) fetch_chunk(kb, ld, j0 + CHUNK, len, sub, next);
-      else fetch_chunk(kb + d, ld, 0, len, sub, next);               // the first values
+    float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    auto score = [&](int j0, const uint4 (&v)[ROWS]) {
 #pragma unroll
       for (int i = 0; i < ROWS; ++i) {
         const float s = row_sum(dot8(v[i], qv));
         const int j = j0 + 4 * i + sub;
         if (p == 0 && j < len) sc[j] = s;
       }
-      take(v, next);
-    }
-    __syncwarp();
-    const float l = softmax_scores(sc, len, c, lane);
-    __syncwarp();
-    float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int j0 = 0; j0 < len; j0 += CHUNK) {
-      if (j0 + CHUNK < len) fetch_chunk(kb + d, ld, j0 + CHUNK, len, sub, next);
+    };
+    auto add_values = [&](int j0, const uint4 (&v)[ROWS]) {
 #pragma unroll
       for (int i = 0; i < ROWS; ++i) {
         const int j = j0 + 4 * i + sub;
@@ -122,7 +115,39 @@ __global__ void __launch_bounds__(512) attn_cls_fwd_kernel(const bf16* __restric
 #pragma unroll
         for (int e = 0; e < 8; ++e) o[e] = fmaf(w, f[e], o[e]);
       }
-      take(v, next);
+    };
+    float l;
+    if constexpr (AHEAD) {
+      uint4 v[ROWS], next[ROWS];
+      fetch_chunk(kb, ld, 0, len, sub, v);
+      for (int j0 = 0; j0 < len; j0 += CHUNK) {
+        if (j0 + CHUNK < len) fetch_chunk(kb, ld, j0 + CHUNK, len, sub, next);
+        else fetch_chunk(kb + d, ld, 0, len, sub, next);             // the first values
+        score(j0, v);
+        take(v, next);
+      }
+      __syncwarp();
+      l = softmax_scores(sc, len, c, lane);
+      __syncwarp();
+      for (int j0 = 0; j0 < len; j0 += CHUNK) {
+        if (j0 + CHUNK < len) fetch_chunk(kb + d, ld, j0 + CHUNK, len, sub, next);
+        add_values(j0, v);
+        take(v, next);
+      }
+    } else {
+      for (int j0 = 0; j0 < len; j0 += CHUNK) {
+        uint4 v[ROWS];
+        fetch_chunk(kb, ld, j0, len, sub, v);
+        score(j0, v);
+      }
+      __syncwarp();
+      l = softmax_scores(sc, len, c, lane);
+      __syncwarp();
+      for (int j0 = 0; j0 < len; j0 += CHUNK) {
+        uint4 v[ROWS];
+        fetch_chunk(kb + d, ld, j0, len, sub, v);
+        add_values(j0, v);
+      }
     }
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -262,8 +287,12 @@ gram_status attention_cls_forward(gram_ctx* ctx, const void* q, const void* kv, 
   if (n == 0) return GRAM_OK;
   const size_t smem = cls_smem(n_heads, l_t, 1);
   ProfScope prof(ctx, GRAM_K_ATTENTION, 4.0 * (double)n * l_t * d, 1, st, "attn_cls_fwd");
-  if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(attn_cls_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClsSmemMost));
-  launch_chain(attn_cls_fwd_kernel, n, n_heads * 32, smem, st, (const bf16*)q, (const bf16*)kv, (bf16*)out, n, l_t, d,
+  // Short texts want blocks on the SM more than rows on their way.  32 768 rows, 12 heads, us as they go / ahead: texts of 8 tokens
+  // 41 / 46, of 2 to 16 22 / 23, of 24 30 / 31, of 32 33 / 27, of 64 29 / 25, of 100 40 / 23.  Up to 12 heads 56 registers let three
+  // blocks share an SM (with 64 registers and two: 48 tokens 31, 25 this way).
+  auto kern = l_t < 24 ? attn_cls_fwd_kernel<false, 512, 0> : (n_heads <= 12 ? attn_cls_fwd_kernel<true, 384, 3> : attn_cls_fwd_kernel<true, 512, 2>);
+  if (smem > 48 * 1024) GRAM_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClsSmemMost));
+  launch_chain(kern, n, n_heads * 32, smem, st, (const bf16*)q, (const bf16*)kv, (bf16*)out, n, l_t, d,
                                                      1.4426950408889634f / sqrtf((float)DH), seq_len, seq_off);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;

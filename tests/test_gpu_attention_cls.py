@@ -4,8 +4,11 @@ import subprocess
 import sys
 
 import pytest
+import torch
 
+from oracle import gram_oracle as orc
 from paper_2204_04179_b200 import synth
+from tests import gram_helpers as gh
 from tests.test_gpu_attention_flash import BASE, check_encoder
 
 pytestmark = pytest.mark.gpu
@@ -25,6 +28,27 @@ def test_equal_lengths(l_t, n_layers):
 def test_many_lengths(l_t):
     s = shape(l_t, 2)
     check_encoder(s, synth.item_lengths(3, s.n_items, l_t, 1))
+
+
+@pytest.mark.parametrize("heads", [4, 13])
+@pytest.mark.parametrize("l_t", [16, 23, 24, 33])
+def test_encodings_on_both_sides_of_the_forward_kernel_s_line(l_t, heads):
+    """Texts that fetch as they go and texts that fetch ahead, with the registers of up to twelve and of up to sixteen heads."""
+    s = shape(l_t, 1).replace(d=64 * heads, n_heads=heads)
+    # weights such that sums over the width vary as check_encoder's do over 128 columns at 0.1, whose bound this takes over
+    ce, tk, toks, _, _ = gh.make_inputs(s, seed=6, sigma=0.1 * (128 / s.d) ** 0.5)
+    lengths = synth.item_lengths(3, s.n_items, l_t, 1)
+    for texts, given in ((toks, None), (synth.ragged(toks, lengths), lengths)):
+        g = gh.make_ctx(s, ce, tk, toks)
+        if given is not None:
+            g.set_item_lengths(given)
+        H = torch.empty(s.n_items, s.d, device="cuda")
+        g.encode_unique(None, torch.arange(s.n_items, dtype=torch.int32, device="cuda"), s.n_items, H)
+        g.sync()
+        g.close()
+        th = orc.as_torch(ce)
+        want = torch.stack([orc.ce_forward(th, texts[i], s) for i in range(s.n_items)])
+        assert gh.rel_err(H.cpu().numpy(), want.detach().numpy()) <= 2e-2            # bf16 operands, as in check_encoder
 
 
 def test_more_items_than_blocks():
