@@ -204,14 +204,14 @@ __device__ __forceinline__ void epilogue_store4(const EpiDev& e, CT* C, int64_t 
 // workspace.  Weight gradients of the check's model (64 x 64 to 256 x 64 over about 900 rows): 130 to 185 us each with
 // one 64 x 64 block per tile and a synchronous load per k-block, 6 to 7 us now; the
 // model's whole training step 2.49 -> 0.48 ms with the chain of launches below.
-// What a k-block waits for is its loads: 32 k at a time in the small tiles, and four groups of 64 threads with a k-block each, so
-// that K = 128 takes one round of loads and no cluster; the groups' tiles are added in ascending order in shared memory (the 30
-// products of that step 204 -> 164 us, the step 0.47 -> 0.43 ms).
+// What a k-block waits for is its loads: 32 k at a time in the small tiles, and up to four groups of 64 threads with a k-block each,
+// so that K = 128 can take one round of loads and no cluster; the groups' tiles are added in ascending order in shared memory.
+// Which products get groups: f32_plan.
 constexpr int F32_MAX_SPLIT = 16;
-template <int TILE> struct F32Cfg {
+template <int TILE, int NG = 1> struct F32Cfg {
   static constexpr int SK = TILE == 32 ? 32 : 16;          // k of one k-block
   static constexpr int GROUP = TILE * TILE / 16;           // threads that hold one copy of the tile
-  static constexpr int GROUPS = TILE == 32 ? 4 : 1;        // copies, each over its own k-blocks
+  static constexpr int GROUPS = NG;                        // copies, each over its own k-blocks
   static constexpr int THREADS = GROUP * GROUPS;
   static constexpr int BUFS = GROUPS == 1 ? 2 : 1;         // operand buffers per group
   static constexpr int LD = TILE + 4;                      // keeps rows 16-byte aligned
@@ -287,13 +287,13 @@ __device__ __forceinline__ void f32_finish(const EpiDev& e, float* C, int64_t o,
   if (e.copy_out) st4(reinterpret_cast<float*>(e.copy_out) + o, v);
 }
 
-template <int TILE, bool A_K, bool B_K>
-__global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const float* __restrict__ A, int64_t lda,
-                                                                        const float* __restrict__ B, int64_t ldb, float* C,
-                                                                        int64_t ldc, int64_t M, int N, int64_t K,
-                                                                        int64_t k_per_split, int vec_a, int vec_b, int vec_e, EpiDev e) {
+template <int TILE, bool A_K, bool B_K, int NG>
+__global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(const float* __restrict__ A, int64_t lda,
+                                                                            const float* __restrict__ B, int64_t ldb, float* C,
+                                                                            int64_t ldc, int64_t M, int N, int64_t K,
+                                                                            int64_t k_per_split, int vec_a, int vec_b, int vec_e, EpiDev e) {
   if (!chain_begin()) return;
-  using Cfg = F32Cfg<TILE>;
+  using Cfg = F32Cfg<TILE, NG>;
   constexpr int LD = Cfg::LD, NV = Cfg::NV, T = Cfg::GROUP, G = Cfg::GROUPS, SK = Cfg::SK, BUFS = Cfg::BUFS;
   __shared__ __align__(16) float sm[G][BUFS][2][SK * LD];  // [group][buffer][operand]; later the groups' partial tiles
   static_assert(sizeof(sm) >= sizeof(float) * G * TILE * LD, "the partial tiles reuse the operand buffers");
@@ -321,6 +321,7 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
     }
     __syncthreads();                 // with two buffers also: everyone is done with the other one, which the next round fills
     if (k0 + SK * G < ke) fetch(k0 + SK * G);
+    if (G > 1 && k0 + group * SK >= ke) continue;          // the last round may have fewer k-blocks than groups
 #pragma unroll
     for (int k = 0; k < SK; ++k) {
       const float4 a4 = *reinterpret_cast<const float4*>(&sm[group][buf][0][k * LD + 4 * ty]);
@@ -344,18 +345,22 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
     return v;
   };
   constexpr int TALL = Cfg::THREADS;
-  static_assert(G == 1 || TALL * 4 == TILE * TILE, "four results per thread after the groups' sum");
   if (G > 1) {
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       *reinterpret_cast<float4*>(part + group * (TILE * LD) + (4 * ty + i) * LD + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
     __syncthreads();
-    const int r = threadIdx.x / (TILE / 4), c = 4 * (threadIdx.x % (TILE / 4));
-    const float4 v4 = group_sum(r, c);
-    if (gridDim.z == 1) {
+#pragma unroll
+    for (int idx = threadIdx.x; idx < TILE * TILE / 4; idx += TALL) {
+      const int r = idx / (TILE / 4), c = 4 * (idx % (TILE / 4));
+      const float4 v4 = group_sum(r, c);
+      if (gridDim.z > 1) {
+        *reinterpret_cast<float4*>(part + r * LD + c) = v4;  // only this thread reads these four places
+        continue;
+      }
       const int64_t m = m0 + r, n = n0 + c;
-      if (m >= M || n >= N) return;
+      if (m >= M || n >= N) continue;
       const float v[4] = {v4.x, v4.y, v4.z, v4.w};
       if (vec_e) {
         f32_finish(e, C, m * ldc + n, v, f32_aux(e, C, m * ldc + n), f32_cols(e, (int)n), e.res_mean ? e.res_mean[m] : 0.f,
@@ -365,9 +370,8 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
         for (int j = 0; j < 4; ++j)
           if (n + j < N) epilogue_store<float, float>(e, C, ldc, m, (int)n + j, v[j]);
       }
-      return;
     }
-    *reinterpret_cast<float4*>(part + r * LD + c) = v4;    // only this thread reads these four places
+    if (gridDim.z == 1) return;
   }
   const int splits = gridDim.z;
   if (splits == 1) {
@@ -453,17 +457,17 @@ __global__ void __launch_bounds__(F32Cfg<TILE>::THREADS) gemm_f32_kernel(const f
   gram_cluster_sync();
 }
 
-template <int TILE, bool A_K, bool B_K>
+template <int TILE, int NG, bool A_K, bool B_K>
 cudaError_t launch_f32(const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc, int64_t M, int N, int64_t K,
                        int splits, int64_t k_per_split, const EpiDev& e, cudaStream_t st) {
-  auto kern = gemm_f32_kernel<TILE, A_K, B_K>;
+  auto kern = gemm_f32_kernel<TILE, A_K, B_K, NG>;
   if (splits > 8) {                                        // clusters of more than 8 blocks are an opt-in
     const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (err != cudaSuccess) return err;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)ceil_div(N, TILE), (unsigned)ceil_div64(M, TILE), (unsigned)splits);
-  cfg.blockDim = dim3(F32Cfg<TILE>::THREADS);
+  cfg.blockDim = dim3(F32Cfg<TILE, NG>::THREADS);
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -480,13 +484,47 @@ cudaError_t launch_f32(const float* A, int64_t lda, const float* B, int64_t ldb,
                     al(e.dgelu_pre) && al(e.copy_out);
   return cudaLaunchKernelEx(&cfg, kern, A, lda, B, ldb, C, ldc, M, N, K, k_per_split, vec_a, vec_b, vec_e, e);
 }
-template <int TILE>
+template <int TILE, int NG>
 cudaError_t launch_f32_major(bool a_k, bool b_k, const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc,
                              int64_t M, int N, int64_t K, int splits, int64_t k_per_split, const EpiDev& e, cudaStream_t st) {
-  if (a_k && b_k) return launch_f32<TILE, true, true>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
-  if (a_k) return launch_f32<TILE, true, false>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
-  if (b_k) return launch_f32<TILE, false, true>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
-  return launch_f32<TILE, false, false>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
+  if (a_k && b_k) return launch_f32<TILE, NG, true, true>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
+  if (a_k) return launch_f32<TILE, NG, true, false>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
+  if (b_k) return launch_f32<TILE, NG, false, true>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
+  return launch_f32<TILE, NG, false, false>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
+}
+
+// How a product of `blocks` tiles (64 x 64 if big, else 32 x 32) is cut: parts of the K range over a cluster, and groups of a
+// block.
+//  - K of at most four k-blocks: one round of loads by that many groups, no cluster.  160 x 512 over 128: 5.5 us over a cluster, 3.6;
+//    320 x 256 over 64 5.4 and 3.9; K = 32 takes four groups too, whose threads share the tile's epilogue (160 x 128: 4.3 and 3.2).
+//    Beyond two blocks of four groups an SM (1200 x 288 over 96, 342 tiles: 7.1 us without, 7.8 with) only as many as k-blocks.
+//  - Else the K range is halved over a cluster while blocks are missing and a part keeps two k-blocks.  Groups on top where the
+//    blocks leave SMs room: 64 x 64 over 4000 (64 blocks) 10.0 and 6.6, 192 x 64 (192 blocks) 10.8 and 8.6, but 256 x 64 over 1200
+//    (256 blocks) 7.0 without, 9.8 with.
+//    Eight parts with a round of four groups instead of sixteen with two k-blocks (192 x 64 over 912: 5.6 and 4.9).
+//  - Tiles that need no parts but are no more than three an SM: four groups shorten a long K (1200 x 256 over 1024, 304 tiles: 46.8
+//    and 41.6).
+struct F32Plan {
+  int parts, groups;
+  int64_t k_per_part;
+};
+F32Plan f32_plan(int64_t blocks, int64_t K, bool big, int most_parts) {
+  F32Plan p = {1, 1, K};
+  const int sk = big ? F32Cfg<64>::SK : F32Cfg<32>::SK;
+  auto groups_of = [&](int64_t k) { return k > 2 * sk || (K <= 4 * sk && blocks <= 2 * kNumSMs) ? 4 : (k > sk ? 2 : 1); };
+  const bool one_round = !big && K <= 4 * sk && blocks * groups_of(K) <= 8 * kNumSMs;
+  if (!one_round) {
+    const int64_t enough = big ? kNumSMs : 4 * kNumSMs;
+    while (p.parts < most_parts && blocks * p.parts * 2 <= enough && K >= 64 * p.parts) {
+      if (p.parts == 8 && !big && blocks <= 16 && K > 16 * sk && K <= 32 * sk) break;
+      p.parts *= 2;
+    }
+  }
+  p.k_per_part = ceil_div64(ceil_div64(K, p.parts), sk) * sk;
+  const int groups = groups_of(p.k_per_part);
+  const int64_t all = blocks * p.parts;
+  if (!big && (one_round || (groups == 4 ? 3 * all <= 4 * kNumSMs : all <= kNumSMs) || (p.parts == 1 && all <= 3 * kNumSMs && K >= 256))) p.groups = groups;
+  return p;
 }
 
 // ============================================================================================
@@ -1698,21 +1736,15 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
   if (dtype == GRAM_F32) {
     if (!c_f32) return gram_set_error(ctx, "gemm: fp32 operands need an fp32 result"), GRAM_ERR_UNSUPPORTED;
     ProfScope prof(ctx, GRAM_K_GEMM, 2.0 * (double)M * N * (double)K, 1, st, epi.tag ? epi.tag : "gemm_f32");
-    // 64 x 64 tiles once they give every SM a block, else 32 x 32; then the K range is halved over a cluster while blocks are
-    // missing and a part has more than it should: two k-blocks of 16 with the large tiles, one round of the four groups (128 k)
-    // with the small ones.
+    // 64 x 64 tiles once they give every SM a block, else 32 x 32
     const int64_t b64 = ceil_div64(M, 64) * ceil_div64(N, 64), b32 = ceil_div64(M, 32) * ceil_div64(N, 32);
     const bool big = b64 >= kNumSMs;
-    const int64_t blocks = big ? b64 : b32, enough = big ? kNumSMs : 4 * kNumSMs;
-    int parts = 1;
-    const int sk = big ? F32Cfg<64>::SK : F32Cfg<32>::SK;
     const int most = F32_MAX_SPLIT < gram_cluster_blocks(ctx) ? F32_MAX_SPLIT : gram_cluster_blocks(ctx);
-    while (parts < most && blocks * parts * 2 <= enough && (big ? K >= 64 * parts : K > 128 * parts)) parts *= 2;
-    const int64_t per = ceil_div64(ceil_div64(K, parts), sk) * sk;
+    const F32Plan p = f32_plan(big ? b64 : b32, K, big, most);
     if (ceil_div64(M, big ? 64 : 32) > 65535)
       return gram_set_error(ctx, "gemm: %lld rows are more than an fp32 product takes", (long long)M), GRAM_ERR_UNSUPPORTED;
-    const cudaError_t ferr = big ? launch_f32_major<64>(a_kmajor, b_kmajor, (const float*)A, lda, (const float*)B, ldb, (float*)C, ldc, M, N, K, parts, per, e, st)
-                                 : launch_f32_major<32>(a_kmajor, b_kmajor, (const float*)A, lda, (const float*)B, ldb, (float*)C, ldc, M, N, K, parts, per, e, st);
+    auto launch = big ? launch_f32_major<64, 1> : (p.groups == 4 ? launch_f32_major<32, 4> : (p.groups == 2 ? launch_f32_major<32, 2> : launch_f32_major<32, 1>));
+    const cudaError_t ferr = launch(a_kmajor, b_kmajor, (const float*)A, lda, (const float*)B, ldb, (float*)C, ldc, M, N, K, p.parts, p.k_per_part, e, st);
     if (ferr != cudaSuccess) return gram_set_error(ctx, "gemm launch failed: %s", cudaGetErrorString(ferr)), GRAM_ERR_CUDA;
     return GRAM_OK;
   }

@@ -15,6 +15,13 @@ SHAPES = {
                      n_cand=3),
     # 64-wide tiles in the forward products, remainders in rows and columns
     "large_tiles": dict(d=72, n_heads=2, d_ff=264, l_t=17, n_items=420, B=40, L=20, task_heads=2, task_d_ff=136, n_layers=1),
+    # widths 32, 64 and 128 over some 900, 1600 and 1200 token rows: one round of two and of four groups, eight parts of four groups,
+    # sixteen parts of one, K ranges that leave groups of the last round without a k-block
+    "width_32": dict(d=32, n_heads=2, d_ff=128, l_t=15, n_items=60, B=8, L=20, task_heads=2, task_d_ff=128, n_layers=1),
+    "width_64": dict(d=64, n_heads=2, d_ff=256, l_t=16, n_items=100, B=30, L=20, task_heads=2, task_d_ff=256, n_layers=1),
+    "width_128": dict(d=128, n_heads=2, d_ff=512, l_t=15, n_items=80, B=8, L=20, task_heads=2, task_d_ff=512, n_layers=1),
+    # 304 tiles and K = 1024: groups without parts
+    "width_256": dict(d=256, n_heads=4, d_ff=1024, l_t=15, n_items=80, B=30, L=20, task_heads=4, task_d_ff=1024, n_layers=1),
     "one_row": dict(d=32, n_heads=2, d_ff=64, l_t=1, n_items=1, B=1, L=1, task_heads=2, task_d_ff=64),
 }
 
