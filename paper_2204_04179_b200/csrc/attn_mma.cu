@@ -331,9 +331,10 @@ __global__ void __launch_bounds__(NW * 32) attn_bwd_mma_kernel(const bf16* __res
   }
 }
 
-// Warps per block: one 16-row tile each.  Up to 32 rows that is two; with four, half of them only copied, while their registers
-// kept other blocks off the SM (42 500 rows of 32-token texts, width 768: backward 185 -> 113 us, forward 57 -> 48).
-constexpr int attn_warps(int SP) { return SP >= 96 ? 8 : SP / 16; }
+// Warps per block: one 16-row tile each.  More would only copy, while their registers keep other blocks off the SM (42 500 rows of
+// 32-token texts, width 768, two warps and four: backward 113 and 185 us, forward 48 and 57; 54 000 rows of 96-token texts, 24 heads
+// of width 32, six and eight: backward 349 and 361, forward 134 and 176).
+constexpr int attn_warps(int SP) { return SP / 16; }
 
 template <int SP, int DH>
 gram_status launch_fwd(gram_ctx* ctx, const bf16* qkv, bf16* out, int64_t n_seq, int S, int d, int n_heads, int causal,

@@ -62,3 +62,10 @@ def test_histories(L):
     for got, w in ((gce, want["grad_ce"]), (gtk, want["grad_task"])):
         err, name = gh.worst_rel_err(got, w)
         assert err <= 2e-2, name
+
+
+@pytest.mark.parametrize("l_t", [66, 80, 96])
+def test_texts_in_six_warps(l_t):
+    """Heads of width 32 and 65 to 96 rows: blocks of six warps, one 16-row tile each."""
+    check_encoder(synth.GramShape(name="s", n_items=9, l_t=l_t, B=9, L=1, **dict(BASE, n_heads=4)))
+    check_encoder(synth.GramShape(name="s", n_items=9, l_t=l_t, B=9, L=1, **dict(BASE, n_heads=4)), synth.item_lengths(2, 9, l_t, 1))
