@@ -1321,9 +1321,11 @@ __device__ __forceinline__ int64_t tc2_units(const TcArgs& a) {
 // Epilogue of EPI_SUM: the unit's K range arrives as several accumulators, each a chain of a.chain k-blocks, which the warp
 // adds up in its registers (128 columns a thread) in ascending order before it writes its 32 rows x 128 columns.  The tensor
 // core cuts off where this adds with rounding, so the length of a chain sets the precision; with the chains of one unit added
-// here, the parts of the K range that go through memory need no longer be as many as the chains.  Units of one chain keep the
-// epilogues that write a block of columns as it comes out of the accumulator (2304 x 768 over 4096 rows: 26.3 us, 29.4 through
-// these registers; 768 x 3072 over 1000 rows 14.1 and 15.5).
+// here, the parts of the K range that go through memory need no longer be as many as the chains.  A unit of one chain is handed
+// back to the MMAs sooner this way, but its first column is written later: from SUM_CHAIN_ALONE k-blocks on the former counts more,
+// below it the unit takes the epilogue that writes a block of columns as it comes out of the accumulator (2304 x 768 in eight parts,
+// us so / through these registers: chains of 8 k-blocks 26.3 / 29.4, of 16 36.1 / 36.1, of 32 57.5 / 56.3, of 128 179 / 173).
+constexpr int SUM_CHAIN_ALONE = 16;
 constexpr int SUM_CHAIN_MAX = 192;       // k-blocks of a chain, whatever the tiles and the workspace: 65 536 rows in six
 __device__ __forceinline__ bool epilogue_unit_sum(const TcArgs& a, float* Cs, int64_t row0, int n_first, int n_lim, int half, int q, int lane,
                                                   float* stage, uint32_t tmem_base, int64_t it, int chains, uint32_t tfull0,
@@ -1825,6 +1827,7 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     splits = ceil_div(args.num_kb, args.kb_per_split);
   }
   args.splits = splits;
+  const bool sum_regs = sum_form && (args.chain < args.kb_per_split || args.chain >= SUM_CHAIN_ALONE);
   // The last wave's tiles as halves where twice as many still fit one wave.
   args.half_from = INT32_MAX;
   int64_t work = tiles * splits;
@@ -1844,7 +1847,7 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     args.ldc = N;
     args.split_stride = (int64_t)M * N;
     args.epi = EpiDev{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 0};
-    if (sum_form && args.chain < args.kb_per_split) err = launch_tc2<false, false, float, EPI_SUM>(ma, mb, args, grid, st);
+    if (sum_regs) err = launch_tc2<false, false, float, EPI_SUM>(ma, mb, args, grid, st);
     else if (sum_form) err = launch_tc2<false, false, float, EPI_BIAS>(ma, mb, args, grid, st);
     else if (pair) err = launch_tc2_major<float>(a_kmajor, b_kmajor, ma, mb, args, grid, st);
     else if (BNsel == 256) err = launch_tc_major<256, float>(a_kmajor, b_kmajor, ma, mb, args, grid, st);
@@ -1900,7 +1903,7 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     else if (m_res && !b_kmajor) err = launch_tc2<true, false, float, EPI_RES>(ma, mb, args, grid, st);
     else if (m_bias && a_kmajor && b_kmajor && ts_ok) err = launch_tc2<true, true, bf16, EPI_BIAS, 8>(ma, mb, args, grid, st, pc, pp);
     else if (m_bias && a_kmajor && !b_kmajor && ts_ok) err = launch_tc2<true, false, bf16, EPI_BIAS, 8>(ma, mb, args, grid, st, pc, pp);
-    else if (sum_form && args.chain < args.num_kb) err = launch_tc2<false, false, float, EPI_SUM>(ma, mb, args, grid, st);
+    else if (sum_regs) err = launch_tc2<false, false, float, EPI_SUM>(ma, mb, args, grid, st);
     else if (m_bias && c_f32 && a_kmajor && !b_kmajor) err = launch_tc2<true, false, float, EPI_BIAS>(ma, mb, args, grid, st);
     else if (c_f32) err = launch_tc2_major<float>(a_kmajor, b_kmajor, ma, mb, args, grid, st);
     else err = launch_tc2_major<bf16>(a_kmajor, b_kmajor, ma, mb, args, grid, st);
