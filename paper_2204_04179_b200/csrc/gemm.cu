@@ -1803,8 +1803,9 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
       if (fill > best + 1e-9) { best = fill; chains = ch; }
     }
   }
-  // weight gradients add their chains in registers: neither the workspace nor a chip full of tiles lets a chain grow
-  if (sum_form && chains < ceil_div(args.num_kb, SUM_CHAIN_MAX)) chains = ceil_div(args.num_kb, SUM_CHAIN_MAX);
+  // weight gradients add their chains in registers: neither the workspace nor a chip full of tiles lets a chain grow.  Longer ones
+  // are cut evenly, so that the count still fills waves (36 tiles, 81 920 rows: 12 chains 268 us, the 7 that suffice 293).
+  if (sum_form) chains *= ceil_div(ceil_div(args.num_kb, chains), SUM_CHAIN_MAX);
   splits = chains;
   args.kb_per_split = ceil_div(args.num_kb, splits);
   splits = ceil_div(args.num_kb, args.kb_per_split);
