@@ -35,9 +35,11 @@ def test_gelu_without_its_derivative(M, N, K):
     assert (C.double().cpu() - want).abs().max().item() <= 1e-4 * np.sqrt(K) + 2.0 ** -8 * scale + 2e-6 * scale + 4e-7 * scale + 2e-6
 
 
-@pytest.mark.parametrize("M,N,K", [(768, 768, 9000), (3072, 768, 4104), (1536, 768, 2056), (2048, 2048, 136), (2304, 2304, 1104), (264, 520, 3000)])
+@pytest.mark.parametrize("M,N,K", [(768, 768, 9000), (3072, 768, 4104), (1536, 768, 2056), (2048, 2048, 136), (2304, 2304, 1104), (264, 520, 3000),
+                                   (264, 1096, 9000), (1000, 1800, 5000), (4872, 1096, 12_400)])
 def test_chains_of_a_weight_gradient(M, N, K):
-    """C += A^T B over K rows: several chains per unit and parts, one part alone, fewer k-blocks than chains would take."""
+    """C += A^T B over K rows: several chains per unit and parts, one part alone, fewer k-blocks than chains would take; narrow columns
+    (520: no pairs of SMs, no chains); ragged rows and columns with several chains, in parts and, over 100 tiles, with half-width units."""
     g = base.ctx()
     gen = torch.Generator(device=base.DEV).manual_seed(M + N + K)
     A = (torch.randn(K, M, generator=gen, device=base.DEV) * 0.5).to(torch.bfloat16)
