@@ -204,10 +204,10 @@ gram_status gram_selftest_bounded_wait(gram_ctx* ctx, gram_stream stream);
  * The calls return GRAM_OK, what the kernels add to is left without the rows' sums, and the next gram_sync returns
  * GRAM_ERR_TIMEOUT.  rows < 0: no such limit (as created). */
 gram_status gram_selftest_ring_rows(gram_ctx* ctx, int32_t rows);
-/* Small batches of gram_dedup and the fp32 matrix products use clusters of up to 16 thread blocks.  Where a process has too
- * few multiprocessors for that, a context uses the largest clusters that can be placed (found when it is created), and
- * beyond those the forms that need none; results of gram_dedup do not depend on it.  This call shows it: the context's
- * later calls use clusters of at most `blocks` (1, 2, 4, 8).  blocks <= 0: as many as can be placed (as created). */
+/* Small batches of gram_dedup and the fp32 matrix products use clusters of up to 16 thread blocks, sums of partial column sums
+ * clusters of 8.  Where a process has too few multiprocessors for that, a context uses the largest clusters that can be placed
+ * (found when it is created), and beyond those the forms that need none; results of gram_dedup and of the column sums do not
+ * depend on it.  This call shows it: the context's later calls use clusters of at most `blocks` (1, 2, 4, 8).  blocks <= 0: as many as can be placed (as created). */
 gram_status gram_selftest_cluster_blocks(gram_ctx* ctx, int32_t blocks);
 /* The sum behind the bias gradients whose rows a producer has already added up in part, on its own:
  * d_out[c] += sum over r < rows of d_part[r, c], fp32 [rows, N].  For tests: within a step its error is hidden by that of

@@ -4,7 +4,7 @@
 // dV_j = P_j dctx, dK_j = dS_j q, dq = sum_j dS_j K_j.  No products to speak of: both kernels are bound by reading K and V
 // (and writing dK and dV) once.  One block per item, one warp per head; eight lanes hold a 128-byte row, so a load
 // instruction covers four rows, and consecutive heads' warps read consecutive pieces of the same rows.
-// 1024 items of 64 tokens, width 768: 55 us forward and 90 us backward (61 and 92 with every chunk of rows requested when the
+// 1024 items of 64 tokens, width 768: 50 us forward and 90 us backward (61 and 92 with every chunk of rows requested when the
 // one before had been worked on), against 86 and 200 us with all 64 queries; the
 // products of the layer's projections shrink by a third as well (the encoder pass of two such layers 5.28 -> 4.80 ms).
 #include "layers.h"

@@ -433,12 +433,15 @@ FlashArgs flash_args(const void* qkv, int64_t rows, int S, int d, int n_heads, c
 }  // namespace
 
 // Which sequences: those whose padding to 128-row tensor-memory tiles costs more than the faster MMA of those tiles gains.
-// Per layer of about 54 000 rows of width 768, these kernels against the tcgen05 ones (attn_tc.cu), us:
-//   rows       80    100   128   147   160   176   192   224   256
-//   forward    126   151   136   152   143   175   169   181   176
-//     tcgen05  165   144    91   364   310   312   265   237   204
-//   backward   397   539   489   516   485   537   525   714   704
-//     tcgen05  314   269   221   936   874   838   773   711   650
+// One layer of about 54 000 rows of width 768, every key visible, these kernels against the tcgen05 ones (attn_tc.cu), us:
+//   rows       80    96    100   112   128   147   160   176   192   224   256
+//   forward    125   144   152   141   133   149   142   173   168   179   172
+//     tcgen05  144   121   127   117   81    342   285   292   247   218   188
+//   backward   394   407   525   492   480   505   486   531   517
+//     tcgen05  290   251   251   229   207   877   814   774   722   655   610
+// (Causal histories, forward: 120 and 142 at 80 rows, 144 and 122 at 96, 144 and 130 at 100.  The tcgen05 kernels gained since the
+// line was drawn at 96 rows; at 81 to 96 they are ahead in a layer of this size, while whole passes over 128 texts of 82, 90 and
+// 96 tokens take the same 1336, 1394 and 1442 us either way.)
 bool attention_flash_forward_supported(int S, int d, int n_heads) {
   return n_heads > 0 && d == n_heads * DH && ((S > 64 && S <= 96) || (S > 128 && S <= 256));
 }

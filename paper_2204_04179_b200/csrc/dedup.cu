@@ -234,7 +234,7 @@ static_assert(sizeof(uint32_t) * RS_WARPS * RADIX_MAX <= 2 * sizeof(int32_t) * R
 // (tile, warp, round, lane) order is position order.  The rank of a key among equal digits:
 // all earlier tiles + earlier warps of this tile + earlier rounds of this warp + earlier lanes.
 // FULL: a tile without missing keys (all but the last one): no test per key.  The pass is bound by its shared-memory accesses
-// (ten random ones per key, each some 3.5 wavefronts per warp; L1 72 % busy) and issues on 38 % of the cycles.
+// (44 wavefronts per 32 keys, random words mostly; L1 72 % busy) and issues on 39 % of the cycles.
 template <int NBITS, bool FULL>
 __device__ __forceinline__ void radix_tile(PassSmem<(NBITS <= 8 ? 256 : 1024)>& s, const int32_t* __restrict__ kin,
                                            const int32_t* __restrict__ vin, int32_t tbase, int n_valid, uint32_t n_keys, int shift,
