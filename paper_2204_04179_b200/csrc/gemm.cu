@@ -287,20 +287,36 @@ __device__ __forceinline__ void f32_finish(const EpiDev& e, float* C, int64_t o,
   if (e.copy_out) st4(reinterpret_cast<float*>(e.copy_out) + o, v);
 }
 
+struct F32Prod {
+  const float* A;
+  int64_t lda;
+  const float* B;
+  int64_t ldb;
+  float* C;
+  int64_t ldc, M, K, k_per_part;
+  int32_t N, vec_a, vec_b, vec_e;
+  float* row_sums;               // row_sums[m] += the sum of A(m, k) over k (may be null; blocks of several groups only)
+  EpiDev e;
+};
+template <int TILE, int NG> using F32Smem = float[NG][F32Cfg<TILE, NG>::BUFS][2][F32Cfg<TILE, NG>::SK * F32Cfg<TILE, NG>::LD];
+
+// One tile of a product by one block, or by `parts` blocks of a cluster whose ranks begin at rank0, this one being number `part`.
+// All threads of the blocks call it; with one part it does not touch the cluster's barrier.
 template <int TILE, bool A_K, bool B_K, int NG>
-__global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(const float* __restrict__ A, int64_t lda,
-                                                                            const float* __restrict__ B, int64_t ldb, float* C,
-                                                                            int64_t ldc, int64_t M, int N, int64_t K,
-                                                                            int64_t k_per_split, int vec_a, int vec_b, int vec_e, EpiDev e) {
-  if (!chain_begin()) return;
+__device__ __forceinline__ void f32_tile(const F32Prod& p, int64_t m0, int64_t n0, int part_no, int parts, int rank0, F32Smem<TILE, NG>& sm) {
   using Cfg = F32Cfg<TILE, NG>;
   constexpr int LD = Cfg::LD, NV = Cfg::NV, T = Cfg::GROUP, G = Cfg::GROUPS, SK = Cfg::SK, BUFS = Cfg::BUFS;
-  __shared__ __align__(16) float sm[G][BUFS][2][SK * LD];  // [group][buffer][operand]; later the groups' partial tiles
   static_assert(sizeof(sm) >= sizeof(float) * G * TILE * LD, "the partial tiles reuse the operand buffers");
+  const float* __restrict__ A = p.A;
+  const float* __restrict__ B = p.B;
+  float* C = p.C;
+  const EpiDev& e = p.e;
+  const int64_t lda = p.lda, ldb = p.ldb, ldc = p.ldc, M = p.M, K = p.K;
+  const int N = p.N, vec_a = p.vec_a, vec_b = p.vec_b, vec_e = p.vec_e;
   const int group = threadIdx.x / T, tid = threadIdx.x % T, tx = tid % (TILE / 4), ty = tid / (TILE / 4);
-  const int64_t m0 = (int64_t)blockIdx.y * TILE;
-  const int64_t n0 = (int64_t)blockIdx.x * TILE;
-  const int64_t kb = (int64_t)blockIdx.z * k_per_split, ke = min(kb + k_per_split, K);
+  const int64_t kb = (int64_t)part_no * p.k_per_part, ke = min(kb + p.k_per_part, K);
+  const bool sums = G > 1 && p.row_sums != nullptr && n0 == 0;
+  float asum[4] = {0.f, 0.f, 0.f, 0.f};        // of this thread's row of A: every fourth k
   float acc[4][4] = {};
   float4 fa[NV], fb[NV];
   auto fetch = [&](int64_t k0) {                           // this group's k-block of the round that starts at k0 (zeros from ke on)
@@ -322,6 +338,10 @@ __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(con
     __syncthreads();                 // with two buffers also: everyone is done with the other one, which the next round fills
     if (k0 + SK * G < ke) fetch(k0 + SK * G);
     if (G > 1 && k0 + group * SK >= ke) continue;          // the last round may have fewer k-blocks than groups
+    if (sums && tid < TILE) {
+#pragma unroll
+      for (int k = 0; k < SK; ++k) asum[k & 3] += sm[group][buf][0][k * LD + tid];
+    }
 #pragma unroll
     for (int k = 0; k < SK; ++k) {
       const float4 a4 = *reinterpret_cast<const float4*>(&sm[group][buf][0][k * LD + 4 * ty]);
@@ -345,17 +365,25 @@ __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(con
     return v;
   };
   constexpr int TALL = Cfg::THREADS;
-  if (G > 1) {
+  if (G > 1) {                     // a row's sum of A takes the first column of the padding
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       *reinterpret_cast<float4*>(part + group * (TILE * LD) + (4 * ty + i) * LD + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    if (sums && tid < TILE) part[group * (TILE * LD) + tid * LD + TILE] = (asum[0] + asum[1]) + (asum[2] + asum[3]);
     __syncthreads();
 #pragma unroll
     for (int idx = threadIdx.x; idx < TILE * TILE / 4; idx += TALL) {
       const int r = idx / (TILE / 4), c = 4 * (idx % (TILE / 4));
       const float4 v4 = group_sum(r, c);
-      if (gridDim.z > 1) {
+      if (sums && c == 0) {
+        float s = part[r * LD + TILE];
+#pragma unroll
+        for (int g = 1; g < G; ++g) s += part[g * (TILE * LD) + r * LD + TILE];
+        if (parts > 1) part[r * LD + TILE] = s;
+        else if (m0 + r < M) p.row_sums[m0 + r] += s;
+      }
+      if (parts > 1) {
         *reinterpret_cast<float4*>(part + r * LD + c) = v4;  // only this thread reads these four places
         continue;
       }
@@ -371,9 +399,9 @@ __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(con
           if (n + j < N) epilogue_store<float, float>(e, C, ldc, m, (int)n + j, v[j]);
       }
     }
-    if (gridDim.z == 1) return;
+    if (parts == 1) return;
   }
-  const int splits = gridDim.z;
+  const int splits = parts;
   if (splits == 1) {
     if (vec_e) {
       const int64_t n = n0 + 4 * tx;
@@ -411,7 +439,7 @@ __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(con
     for (int i = 0; i < 4; ++i)
       *reinterpret_cast<float4*>(part + (4 * ty + i) * LD + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
   }
-  const int rows = TILE / splits, r0 = blockIdx.z * rows;          // this block's share of the tile's rows
+  const int rows = TILE / splits, r0 = part_no * rows;             // this block's share of the tile's rows
   gram_cluster_sync();
   for (int idx = threadIdx.x; idx < rows * (TILE / 4); idx += TALL) {     // four columns of a row each
     const int r = r0 + idx / (TILE / 4), c = 4 * (idx % (TILE / 4));
@@ -434,7 +462,7 @@ __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(con
 #pragma unroll
       for (int s = 0; s < 8; ++s) {
         uint32_t ra;
-        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(at), "r"(min(s0 + s, splits - 1)));
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(at), "r"(rank0 + min(s0 + s, splits - 1)));
         asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
                      : "=f"(x[s].x), "=f"(x[s].y), "=f"(x[s].z), "=f"(x[s].w)
                      : "r"(ra)
@@ -443,6 +471,17 @@ __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(con
 #pragma unroll
       for (int s = 0; s < 8; ++s)
         if (s0 + s < splits) { v[0] += x[s].x; v[1] += x[s].y; v[2] += x[s].z; v[3] += x[s].w; }
+    }
+    if (sums && c == 0 && m < M) {
+      float a = 0.f;
+      for (int s = 0; s < splits; ++s) {
+        uint32_t ra;
+        float x;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(smem_u32(part + r * LD + TILE)), "r"(rank0 + s));
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(ra) : "memory");
+        a += x;
+      }
+      p.row_sums[m] += a;
     }
     if (!ok) continue;
     if (vec_e) {
@@ -457,16 +496,69 @@ __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(con
   gram_cluster_sync();
 }
 
+template <int TILE, bool A_K, bool B_K, int NG>
+__global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(const __grid_constant__ F32Prod p) {
+  if (!chain_begin()) return;
+  __shared__ __align__(16) F32Smem<TILE, NG> sm;           // [group][buffer][operand]; later the groups' partial tiles
+  f32_tile<TILE, A_K, B_K, NG>(p, (int64_t)blockIdx.y * TILE, (int64_t)blockIdx.x * TILE, blockIdx.z, gridDim.z, 0, sm);
+}
+
+// The two products that read one gradient dY [T, N]: dW [N, K] += dY^T X (product w; its row sums are the bias gradient) and
+// dX [T, K] = dY W (product x), in one launch.  Neither fills the chip in the models that run in fp32, and each is a chain of launch,
+// loads and exchange of partial sums: side by side they take little more than the longer one (64 x 256 and 256 x 64 over 900
+// rows: 9.0 us where the two took 11.3 and the bias gradient's sums, two launches more, 5).  The check's step 429 -> 386 us in 65 launches
+// instead of 87, steps of other widths and sizes 2 to 11 % less.  Clusters of gridDim.x / clusters blocks;
+// the first w_clusters work on product w, wp blocks a tile, the others on product x, xp blocks a tile.
+struct F32Pair {
+  F32Prod w, x;
+  int32_t wp, xp, w_clusters, w_tiles, x_tiles;
+};
+__global__ void __launch_bounds__(F32Cfg<32, 4>::THREADS) gemm_f32_pair_kernel(const __grid_constant__ F32Pair a) {
+  if (!chain_begin()) return;
+  __shared__ __align__(16) F32Smem<32, 4> sm;
+  uint32_t blocks, rank;
+  asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(blocks));
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  const int cluster = blockIdx.x / blocks;
+  const bool is_w = cluster < a.w_clusters;
+  const int parts = is_w ? a.wp : a.xp, item = (cluster - (is_w ? 0 : a.w_clusters)) * (int)blocks + (int)rank;
+  const int tile = item / parts, part = item % parts;
+  const F32Prod& p = is_w ? a.w : a.x;
+  const int tiles_n = (p.N + 31) / 32;
+  const int64_t m0 = (int64_t)(tile / tiles_n) * 32, n0 = (int64_t)(tile % tiles_n) * 32;
+  const bool there = tile < (is_w ? a.w_tiles : a.x_tiles);
+  if (there && is_w) f32_tile<32, false, false, 4>(a.w, m0, n0, part, parts, (int)rank - part, sm);
+  else if (there) f32_tile<32, true, false, 4>(a.x, m0, n0, part, parts, (int)rank - part, sm);
+  if (blocks > 1 && !(there && parts > 1)) {               // the cluster's barrier counts every block
+    gram_cluster_sync();
+    gram_cluster_sync();
+  }
+}
+
+F32Prod f32_prod(const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc, int64_t M, int N, int64_t K,
+                 int64_t k_per_part, const EpiDev& e) {
+  auto al = [](const void* p) { return (uintptr_t)p % 16 == 0; };
+  const int one_aux = (e.res != nullptr) + (e.dgelu_pre != nullptr) + (e.accumulate != 0) <= 1;
+  F32Prod p = {};
+  p.A = A; p.lda = lda; p.B = B; p.ldb = ldb; p.C = C; p.ldc = ldc; p.M = M; p.N = N; p.K = K;
+  p.k_per_part = k_per_part;
+  p.vec_a = lda % 4 == 0 && al(A);
+  p.vec_b = ldb % 4 == 0 && al(B);
+  p.vec_e = one_aux && N % 4 == 0 && ldc % 4 == 0 && al(C) && al(e.bias) && al(e.res) && al(e.res_gamma) && al(e.res_beta) && al(e.pre) &&
+            al(e.dgelu_pre) && al(e.copy_out);
+  p.e = e;
+  return p;
+}
+
 template <int TILE, int NG, bool A_K, bool B_K>
-cudaError_t launch_f32(const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc, int64_t M, int N, int64_t K,
-                       int splits, int64_t k_per_split, const EpiDev& e, cudaStream_t st) {
+cudaError_t launch_f32(const F32Prod& p, int splits, cudaStream_t st) {
   auto kern = gemm_f32_kernel<TILE, A_K, B_K, NG>;
   if (splits > 8) {                                        // clusters of more than 8 blocks are an opt-in
     const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (err != cudaSuccess) return err;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)ceil_div(N, TILE), (unsigned)ceil_div64(M, TILE), (unsigned)splits);
+  cfg.gridDim = dim3((unsigned)ceil_div(p.N, TILE), (unsigned)ceil_div64(p.M, TILE), (unsigned)splits);
   cfg.blockDim = dim3(F32Cfg<TILE, NG>::THREADS);
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
@@ -477,20 +569,14 @@ cudaError_t launch_f32(const float* A, int64_t lda, const float* B, int64_t ldb,
   attr[1] = chain_attribute();
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const int vec_a = (lda % 4 == 0) && ((uintptr_t)A % 16 == 0), vec_b = (ldb % 4 == 0) && ((uintptr_t)B % 16 == 0);
-  auto al = [](const void* p) { return (uintptr_t)p % 16 == 0; };
-  const int one_aux = (e.res != nullptr) + (e.dgelu_pre != nullptr) + (e.accumulate != 0) <= 1;
-  const int vec_e = one_aux && N % 4 == 0 && ldc % 4 == 0 && al(C) && al(e.bias) && al(e.res) && al(e.res_gamma) && al(e.res_beta) && al(e.pre) &&
-                    al(e.dgelu_pre) && al(e.copy_out);
-  return cudaLaunchKernelEx(&cfg, kern, A, lda, B, ldb, C, ldc, M, N, K, k_per_split, vec_a, vec_b, vec_e, e);
+  return cudaLaunchKernelEx(&cfg, kern, p);
 }
 template <int TILE, int NG>
-cudaError_t launch_f32_major(bool a_k, bool b_k, const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc,
-                             int64_t M, int N, int64_t K, int splits, int64_t k_per_split, const EpiDev& e, cudaStream_t st) {
-  if (a_k && b_k) return launch_f32<TILE, NG, true, true>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
-  if (a_k) return launch_f32<TILE, NG, true, false>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
-  if (b_k) return launch_f32<TILE, NG, false, true>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
-  return launch_f32<TILE, NG, false, false>(A, lda, B, ldb, C, ldc, M, N, K, splits, k_per_split, e, st);
+cudaError_t launch_f32_major(bool a_k, bool b_k, const F32Prod& p, int splits, cudaStream_t st) {
+  if (a_k && b_k) return launch_f32<TILE, NG, true, true>(p, splits, st);
+  if (a_k) return launch_f32<TILE, NG, true, false>(p, splits, st);
+  if (b_k) return launch_f32<TILE, NG, false, true>(p, splits, st);
+  return launch_f32<TILE, NG, false, false>(p, splits, st);
 }
 
 // How a product of `blocks` tiles (64 x 64 if big, else 32 x 32) is cut: parts of the K range over a cluster, and groups of a
@@ -1727,14 +1813,69 @@ void gemm_ws_free(GemmWorkspace* ws) {
   *ws = GemmWorkspace();
 }
 
+static EpiDev epi_dev(const GemmEpilogue& epi) {
+  return EpiDev{epi.bias, epi.res, epi.res_mean, epi.res_rstd, epi.res_gamma, epi.res_beta, epi.pre, epi.dgelu_pre, epi.copy_out,
+                epi.colsum_part, epi.gelu, epi.accumulate};
+}
+
+// Both products go together where their tiles are at most three blocks an SM: above, each fills the chip by itself (a model of
+// width 32 over some 10 000 rows: 837 us a step with the line at two blocks, which fit at once, 816 at three).  Parts of the K ranges: the
+// longer chain is halved while the blocks fit the SMs at once (a width of 128: 478 us a step, 499 with half as many blocks again)
+// and it is more than one round of four k-blocks; a dW of few tiles takes parts in any case, since its chain is over the rows.
+bool gemm_f32_grads_together(int64_t T, int N, int K) {
+  const int64_t w = (int64_t)ceil_div(N, 32) * ceil_div(K, 32), x = ceil_div64(T, 32) * ceil_div(K, 32);
+  return T > 0 && N > 0 && K > 0 && w + x <= 3 * kNumSMs;
+}
+gram_status gemm_f32_grads(gram_ctx* ctx, const float* dY, const float* X, float* dW, float* db, const float* W, float* dX, int64_t T,
+                           int N, int K, const GemmEpilogue& epi, cudaStream_t st) {
+  if (!dY || !X || !dW || !W || !dX || !gemm_f32_grads_together(T, N, K)) return gram_set_error(ctx, "gemm: bad gradient products"), GRAM_ERR_ARG;
+  ProfScope prof(ctx, GRAM_K_GEMM, 4.0 * (double)T * N * (double)K, 1, st, epi.tag ? epi.tag : "gemm_f32");
+  const int most = F32_MAX_SPLIT < gram_cluster_blocks(ctx) ? F32_MAX_SPLIT : gram_cluster_blocks(ctx);
+  constexpr int SK = F32Cfg<32, 4>::SK, ROUND = 4 * SK;
+  F32Pair a = {};
+  a.w_tiles = ceil_div(N, 32) * ceil_div(K, 32);
+  a.x_tiles = (int32_t)ceil_div64(T, 32) * ceil_div(K, 32);
+  a.wp = a.xp = 1;
+  for (;;) {
+    const int64_t wk = a.wp < most ? ceil_div64(T, a.wp) : 0, xk = a.xp < most ? ceil_div(N, a.xp) : 0;
+    const bool w_first = wk >= xk;
+    if ((w_first ? wk : xk) <= ROUND) break;
+    const int64_t w = (int64_t)a.w_tiles * a.wp, x = (int64_t)a.x_tiles * a.xp;
+    if (w + x + (w_first ? w : x) > 2 * kNumSMs && !(w_first && 2 * w <= 32)) break;
+    if (w_first) a.wp *= 2;
+    else a.xp *= 2;
+  }
+  EpiDev ew = {};
+  ew.accumulate = 1;
+  a.w = f32_prod(dY, N, X, K, dW, K, N, K, T, ceil_div64(ceil_div64(T, a.wp), SK) * SK, ew);
+  a.w.row_sums = db;
+  a.x = f32_prod(dY, N, W, K, dX, K, T, K, N, (int64_t)ceil_div(ceil_div(N, a.xp), SK) * SK, epi_dev(epi));
+  const int blocks = a.wp > a.xp ? a.wp : a.xp;
+  a.w_clusters = ceil_div(a.w_tiles * a.wp, blocks);
+  if (blocks > 8) GRAM_CUDA(ctx, cudaFuncSetAttribute(gemm_f32_pair_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(blocks * (a.w_clusters + ceil_div(a.x_tiles * a.xp, blocks))));
+  cfg.blockDim = dim3(F32Cfg<32, 4>::THREADS);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)blocks;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1] = chain_attribute();
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  GRAM_CUDA(ctx, cudaLaunchKernelEx(&cfg, gemm_f32_pair_kernel, a));
+  return GRAM_OK;
+}
+
 gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void* A, int a_kmajor, int64_t lda,
                         const void* B, int b_kmajor, int64_t ldb, void* C, int c_f32, int64_t ldc, int64_t M, int N,
                         int64_t K, const GemmEpilogue& epi, int allow_splitk, cudaStream_t st) {
   if (M < 0 || N < 0 || K < 0) return gram_set_error(ctx, "gemm: negative size"), GRAM_ERR_ARG;
   if (M == 0 || N == 0) return GRAM_OK;
   if (!A || !B || !C) return gram_set_error(ctx, "gemm: null operand"), GRAM_ERR_ARG;
-  EpiDev e{epi.bias, epi.res, epi.res_mean, epi.res_rstd, epi.res_gamma, epi.res_beta, epi.pre, epi.dgelu_pre, epi.copy_out,
-           epi.colsum_part, epi.gelu, epi.accumulate};
+  const EpiDev e = epi_dev(epi);
   if (dtype == GRAM_F32) {
     if (!c_f32) return gram_set_error(ctx, "gemm: fp32 operands need an fp32 result"), GRAM_ERR_UNSUPPORTED;
     ProfScope prof(ctx, GRAM_K_GEMM, 2.0 * (double)M * N * (double)K, 1, st, epi.tag ? epi.tag : "gemm_f32");
@@ -1746,7 +1887,7 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
     if (ceil_div64(M, big ? 64 : 32) > 65535)
       return gram_set_error(ctx, "gemm: %lld rows are more than an fp32 product takes", (long long)M), GRAM_ERR_UNSUPPORTED;
     auto launch = big ? launch_f32_major<64, 1> : (p.groups == 4 ? launch_f32_major<32, 4> : (p.groups == 2 ? launch_f32_major<32, 2> : launch_f32_major<32, 1>));
-    const cudaError_t ferr = launch(a_kmajor, b_kmajor, (const float*)A, lda, (const float*)B, ldb, (float*)C, ldc, M, N, K, p.parts, p.k_per_part, e, st);
+    const cudaError_t ferr = launch(a_kmajor, b_kmajor, f32_prod((const float*)A, lda, (const float*)B, ldb, (float*)C, ldc, M, N, K, p.k_per_part, e), p.parts, st);
     if (ferr != cudaSuccess) return gram_set_error(ctx, "gemm launch failed: %s", cudaGetErrorString(ferr)), GRAM_ERR_CUDA;
     return GRAM_OK;
   }
