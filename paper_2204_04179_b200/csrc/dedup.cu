@@ -209,8 +209,7 @@ __device__ __forceinline__ int2 scan_pair(int a, int b, int32_t (*sw)[16]) {
 //   18 bits (2x9)  269 / 257 / 261  241 / 238 / 226  231 / 236 / 210  248 / 251 / 233       223 / 246 / 181
 //   20 bits (2x10) 292 / 276 / 280  257 / 249 / 238  242 / 245 / 215  263 / 262 / 242       231 / 246 / 182
 // One pass of 7 bits: 123 with votes, 117 this way (two IDs alone, 16 lanes in line: 122 and 119); of 5 bits 115 and 107, but
-// two IDs 113 and 118, so narrower passes keep the votes.  (The one-launch form below ranks by votes at any width; the table would
-// suit it as well: 65 536 positions over 10^6 items 33.0 us and 30.8, 25 600 over 10^4 15.3 and 14.9.)
+// two IDs 113 and 118, so narrower passes keep the votes.  (The one-launch form below does the same at any width.)
 constexpr int MATCH_BITS = 7;
 
 template <int BINS> struct PassSmem {
@@ -576,10 +575,14 @@ __global__ void __launch_bounds__(256) inverse_kernel(const int32_t* __restrict_
 
 // ---- the whole dedup of a small batch in one launch -------------------------------------------
 // Up to 16 x 4096 positions the sort is a chain of launches and look-backs that move next to nothing (25 600 positions
-// over 10 000 items: 45 us, of which the traffic is 0.3; 16 us this way).  Here one cluster of up to 16 blocks holds all (ID, position)
+// over 10 000 items: 45 us, of which the traffic is 0.3; 12.5 us this way).  Here one cluster of up to 16 blocks holds all (ID, position)
 // pairs in its shared memory: block r owns the sorted places r * TILE .., a radix pass ranks a block's pairs as above,
 // the blocks read each other's digit counts, and every pair goes straight to its place in the owner's shared memory.
-// The run-length pass and `inverse` follow in the same launch.  Between phases: cluster barriers.
+// The run-length pass and `inverse` follow in the same launch.  Between phases: cluster barriers, two a pass and one for the counts of
+// items, which every block writes to all others so that none is read after it.  What bounds it is this chain of barriers and of
+// looks into other blocks' memory: with a loop over the blocks' counts, votes for equal digits and a barrier at the end 15.4 us,
+// 65 536 positions over 10^6 items 35.9 (30.5 now), 40 000 over 30 000 25.3 (21.4).  A position whose ID is out of range carries
+// the sign bit along.
 constexpr int CD_THREADS = 512;
 constexpr int CD_WARPS = CD_THREADS / 32;
 constexpr int kClusterMaxBlocks = 16;     // an opt-in above 8
@@ -595,6 +598,19 @@ __device__ __forceinline__ int32_t cd_load(uint32_t a) {
   return v;
 }
 
+// a word at the same place in every block of the cluster, all on their way together (a loop over the blocks waits some 200 cycles
+// for each of them): v[i] is that of block `rank` + i, going round, so that the blocks do not all ask the same one; 0 from `blocks` on
+__device__ __forceinline__ void cd_load_all(const void* p, int rank, int blocks, int32_t (&v)[kClusterMaxBlocks]) {
+#pragma unroll
+  for (int i = 0; i < kClusterMaxBlocks; ++i) {
+    const int b = i >= blocks ? rank : (rank + i < blocks ? rank + i : rank + i - blocks);
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.s32 p, %2, %3;\n\tmov.b32 %0, 0;\n\t@p ld.shared::cluster.s32 %0, [%1];\n\t}"
+                 : "=&r"(v[i])
+                 : "r"(cd_remote(p, (uint32_t)b)), "r"(i), "r"(blocks)
+                 : "memory");
+  }
+}
+
 template <int ROUNDS> struct ClusterSmem {
   int2 kv[CD_THREADS * ROUNDS];    // (ID, position) at this block's sorted places
   uint16_t cnt[CD_WARPS][RADIX];   // pairs of (warp, digit); later the warp's base inside the block's run of the digit
@@ -602,7 +618,8 @@ template <int ROUNDS> struct ClusterSmem {
   int32_t gbase[RADIX];            // sorted place of this block's first pair of a digit
   int32_t scan_w[2][16];
   int32_t sw[33];
-  int32_t heads;                   // items that start in this block (read by the others)
+  alignas(16) uint32_t match[CD_WARPS][RADIX];   // lanes of the current round per (warp, digit); zeros between rounds
+  int32_t heads[kClusterMaxBlocks];  // items that start in each block (written by that block)
 };
 
 template <int ROUNDS>
@@ -629,9 +646,10 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
     const int i = lbase + r * 32;
     val[r] = base + i;
     key[r] = i < n_valid ? ids[base + i] : 0;
-    if (key[r] < 0 || key[r] >= n_items) { bad = true; key[r] = 0; }
+    if (key[r] < 0 || key[r] >= n_items) { bad = true; key[r] = 0; val[r] |= INT32_MIN; }
   }
   if (bad) gram_device_fail(status, GRAM_ERR_ID_RANGE);
+  for (int i = tid; i < CD_WARPS * RADIX / 4; i += CD_THREADS) reinterpret_cast<uint4*>(&s.match[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
   for (int shift = 0; shift == 0 || shift < key_bits; shift += 8) {
     for (int i = tid; i < CD_WARPS * RADIX / 2; i += CD_THREADS) reinterpret_cast<uint32_t*>(&s.cnt[0][0])[i] = 0u;
     if (shift > 0) {
@@ -647,18 +665,19 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
     for (int r = 0; r < ROUNDS; ++r) {                   // stable rank among equal digits, as in radix_pass_kernel
       const bool valid = lbase + r * 32 < n_valid;
       const int dig = (key[r] >> shift) & 255;
-      uint32_t peers = __ballot_sync(0xffffffffu, valid);
-#pragma unroll
-      for (int b = 0; b < 8; ++b) {
-        const bool bit = (dig >> b) & 1;
-        const uint32_t vote = __ballot_sync(0xffffffffu, bit);
-        peers &= bit ? vote : ~vote;
-      }
+      const bool with_first = dig == __shfl_sync(0xffffffffu, dig, 0);
+      const uint32_t first_peers = __ballot_sync(0xffffffffu, valid && with_first);
+      if (valid && !with_first) atomicOr(&s.match[warp][dig], 1u << lane);
+      __syncwarp();
+      const uint32_t peers = with_first ? first_peers : s.match[warp][dig];
       int32_t before = 0;
       if (valid) before = my_cnt[dig];
       __syncwarp();
       pos[r] = before + __popc(peers & lt);
-      if (valid && (peers & lt) == 0u) my_cnt[dig] = (uint16_t)(before + __popc(peers));
+      if (valid && (peers & lt) == 0u) {
+        my_cnt[dig] = (uint16_t)(before + __popc(peers));
+        s.match[warp][dig] = 0u;
+      }
       __syncwarp();
     }
     __syncthreads();
@@ -675,10 +694,12 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
     gram_cluster_sync();                                 // every block's pairs are in registers, its counts published
     int32_t total = 0, before_blocks = 0;
     if (tid < RADIX) {
-      for (int b = 0; b < blocks; ++b) {
-        const int32_t c = cd_load(cd_remote(&s.count[tid], b));
-        total += c;
-        if (b < rank) before_blocks += c;
+      int32_t c[kClusterMaxBlocks];
+      cd_load_all(&s.count[tid], rank, blocks, c);
+#pragma unroll
+      for (int i = 0; i < kClusterMaxBlocks; ++i) {
+        total += c[i];
+        if (rank + i >= blocks) before_blocks += c[i];     // block rank + i - blocks; zeros past the blocks
       }
     }
     const int2 ex = scan_pair<8>(total, 0, s.scan_w);
@@ -712,13 +733,13 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
   }
   int32_t btot;
   int32_t ex = block_exclusive_scan(tot, s.sw, &btot);
-  if (tid == 0) s.heads = btot;
-  gram_cluster_sync();
+  if (tid < blocks)
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cd_remote(&s.heads[rank], (uint32_t)tid)), "r"(btot) : "memory");
+  gram_cluster_sync();                                   // the last look into another block's memory: blocks may leave after it
   int32_t U = 0;
   for (int b = 0; b < blocks; ++b) {
-    const int32_t h = cd_load(cd_remote(&s.heads, (uint32_t)b));
-    if (b < rank) ex += h;
-    U += h;
+    if (b < rank) ex += s.heads[b];
+    U += s.heads[b];
   }
 #pragma unroll
   for (int i = 0; i < ROUNDS; ++i) {
@@ -728,21 +749,14 @@ __global__ void __launch_bounds__(CD_THREADS) cluster_dedup_kernel(const int32_t
         seg_off[ex] = base + first + i;
         ++ex;
       }
-      perm[base + first + i] = val[i];
-      inverse[val[i]] = ex - 1;
+      const int32_t p = val[i] & INT32_MAX;
+      perm[base + first + i] = p;
+      inverse[p] = val[i] < 0 ? -1 : ex - 1;               // an ID out of range belongs to no item, as in inverse_kernel
     }
   }
   if (rank == 0 && tid == 0) {
     *n_unique = U;
     seg_off[U] = P;
-  }
-  gram_cluster_sync();                                   // nobody leaves while its counts may still be read
-  if (bad) {                                             // an ID out of range belongs to no item, as in inverse_kernel
-#pragma unroll
-    for (int r = 0; r < ROUNDS; ++r) {
-      const int i = lbase + r * 32;
-      if (i < n_valid && (uint32_t)ids[base + i] >= (uint32_t)n_items) inverse[base + i] = -1;
-    }
   }
 }
 
