@@ -397,73 +397,95 @@ __global__ void __launch_bounds__(32 * SEG_WARPS) segsum_ring_kernel(const float
   if (lane == 0) span[chunk] = sp;
 }
 
-// one block per (chunk, slab): if an item starts in this chunk and runs past its end, add its parts.  Warp w adds
-// the following chunks' parts number w, w+8, ... (ascending), warp 0 starts from this chunk's own part, and the
-// eight warp sums are added in ascending w: a fixed association, whatever the schedule.
+// A warp per (chunk, slab): if an item starts in this chunk and runs past its end, add its parts.  Eight runs: run w adds the
+// following chunks' parts number w, w + 8, ... (ascending), run 0 starts from this chunk's own part, and the eight sums are
+// added in ascending w: a fixed association, whatever the schedule.  With up to eight parts a run is one part, so the warp
+// simply adds them in order; an item that reaches farther is summed by the whole block, a run per warp.
+// Nearly every chunk has an item that runs into the next one, and what that takes is the chain item, parts, store: with a block of
+// eight warps for each of them 34 us at 10^6 positions of 768 columns, a twelfth of the blocks on the chip at a time; 14 this way.
+constexpr int FIX_RUNS = 8;
 template <int VPL>
-__global__ void __launch_bounds__(256) segsum_fixup_kernel(const int32_t* __restrict__ seg_off, int64_t P, int32_t U,
+__global__ void __launch_bounds__(32 * FIX_RUNS) segsum_fixup_kernel(const int32_t* __restrict__ seg_off, int64_t P, int32_t U,
                                                            int d, int64_t R, int nchunks, int nslabs,
                                                            const int32_t* __restrict__ rows, int add,
                                                            float* __restrict__ out, const float* __restrict__ partial,
                                                            const int2* __restrict__ span, const int32_t* __restrict__ d_U,
                                                            const int32_t* __restrict__ gate) {
   if (!chain_begin()) return;
-  __shared__ float4 red[8][VPL][32];
+  __shared__ float4 red[FIX_RUNS][VPL][32];
+  __shared__ int2 far[FIX_RUNS];                     // (item, last chunk) of the warps whose item takes the block, else last = -1
   if (d_U) U = *d_U;
   if (U <= 0) return;
   if (gate && *gate) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int chunk = blockIdx.x / nslabs, slab = blockIdx.x - chunk * nslabs;
+  const int chunk0 = (int)(blockIdx.x / nslabs) * FIX_RUNS, slab = (int)(blockIdx.x % nslabs);
   const int col0 = slab * (VPL * 128);
-  const int64_t c0 = (int64_t)chunk * R, c1 = min(c0 + R, P);
-  if (c0 >= c1 || c1 >= P) return;
-  const int2 sp = span[chunk];                       // left by the first launch
-  if (sp.x < 0 || sp.x >= U) return;                 // no item starts here and runs on (same for the whole block)
-  const int32_t u = sp.x;
-  const int last = min(sp.y, nchunks - 1);
-  float4 acc[VPL];
-#pragma unroll
-  for (int v = 0; v < VPL; ++v) {
-    const int c = col0 + (v * 32 + lane) * 4;
-    acc[v] = (w == 0 && c < d) ? *reinterpret_cast<const float4*>(partial + ((int64_t)chunk * 2 + 1) * d + c)
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  for (int c = chunk + 1 + w; c <= last; c += 32) {   // four parts in flight per warp
-    float4 x[4][VPL];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-#pragma unroll
-      for (int v = 0; v < VPL; ++v) {
-        const int cc = col0 + (v * 32 + lane) * 4;
-        x[k][v] = (c + 8 * k <= last && cc < d) ? *reinterpret_cast<const float4*>(partial + ((int64_t)(c + 8 * k) * 2 + 0) * d + cc)
-                                                : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (c + 8 * k <= last) {
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-          acc[v].x += x[k][v].x; acc[v].y += x[k][v].y; acc[v].z += x[k][v].z; acc[v].w += x[k][v].w;
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int v = 0; v < VPL; ++v) red[w][v][lane] = acc[v];
-  __syncthreads();
-  if (w == 0) {
+  // part of item chunk c: the own part of the chunk it starts in (which = 1), what it left in a later one (which = 0)
+  auto part = [&](int c, int which, float4 (&x)[VPL]) {
 #pragma unroll
     for (int v = 0; v < VPL; ++v) {
-      float4 t = red[0][v][lane];
-#pragma unroll
-      for (int k = 1; k < 8; ++k) {
-        const float4 y = red[k][v][lane];
-        t.x += y.x; t.y += y.y; t.z += y.z; t.w += y.w;
-      }
-      acc[v] = t;
+      const int cc = col0 + (v * 32 + lane) * 4;
+      x[v] = cc < d ? *reinterpret_cast<const float4*>(partial + ((int64_t)c * 2 + which) * d + cc) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    store_row<VPL>(out, rows ? rows[u] : u, d, col0, lane, acc, add != 0);
+  };
+  auto plus = [](float4 (&a)[VPL], const float4 (&x)[VPL]) {
+#pragma unroll
+    for (int v = 0; v < VPL; ++v) { a[v].x += x[v].x; a[v].y += x[v].y; a[v].z += x[v].z; a[v].w += x[v].w; }
+  };
+  const int chunk = chunk0 + w;
+  const int64_t c0 = (int64_t)chunk * R, c1 = min(c0 + R, P);
+  int2 sp = make_int2(-1, -1);
+  if (chunk < nchunks && c0 < c1 && c1 < P) sp = span[chunk];       // left by the first launch
+  const bool mine = sp.x >= 0 && sp.x < U;           // else no item starts here and runs on (same for the whole warp)
+  const int last = mine ? min(sp.y, nchunks - 1) : -1;
+  const bool block_wide = mine && last - chunk > FIX_RUNS;
+  if (mine && !block_wide) {
+    float4 acc[VPL];
+    part(chunk, 1, acc);
+#pragma unroll
+    for (int k0 = 0; k0 < FIX_RUNS; k0 += 4) {       // four parts on their way
+      if (chunk + 1 + k0 > last) break;
+      float4 x[4][VPL];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) part(min(chunk + 1 + k0 + k, last), 0, x[k]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (chunk + 1 + k0 + k <= last) plus(acc, x[k]);
+    }
+    store_row<VPL>(out, rows ? rows[sp.x] : sp.x, d, col0, lane, acc, add != 0);
+  }
+  if (lane == 0) far[w] = make_int2(sp.x, block_wide ? last : -1);
+  if (!__syncthreads_or(block_wide)) return;
+  for (int f = 0; f < FIX_RUNS; ++f) {
+    const int2 it = far[f];
+    if (it.y < 0) continue;
+    const int first = chunk0 + f;
+    float4 acc[VPL];
+#pragma unroll
+    for (int v = 0; v < VPL; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (w == 0) part(first, 1, acc);
+    for (int c = first + 1 + w; c <= it.y; c += 8 * FIX_RUNS) {     // eight parts on their way per warp
+      float4 x[8][VPL];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) part(min(c + FIX_RUNS * k, it.y), 0, x[k]);
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (c + FIX_RUNS * k <= it.y) plus(acc, x[k]);
+    }
+#pragma unroll
+    for (int v = 0; v < VPL; ++v) red[w][v][lane] = acc[v];
+    __syncthreads();
+    if (w == 0) {
+#pragma unroll
+      for (int k = 1; k < FIX_RUNS; ++k) {
+        float4 y[VPL];
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) y[v] = red[k][v][lane];
+        plus(acc, y);
+      }
+      store_row<VPL>(out, rows ? rows[it.x] : it.x, d, col0, lane, acc, add != 0);
+    }
+    __syncthreads();
   }
 }
 
@@ -619,7 +641,7 @@ static void segsum_run(const void* d_in, const int32_t* d_perm, const int32_t* d
   if (!ring) launch_chain(segsum_chunks_kernel<InT, VPL, 8>, blocks, 256, 0, st, (const InT*)d_in, d_perm, d_seg_off, P, U, d, R, nchunks, nslabs,
                                                             d_rows, add, d_out, partial, span, status, d_U, gate);
   if (nchunks > 1)
-    launch_chain(segsum_fixup_kernel<VPL>, (unsigned)warps, 256, 0, st, d_seg_off, P, U, d, R, nchunks, nslabs, d_rows, add, d_out, partial, span, d_U, gate);
+    launch_chain(segsum_fixup_kernel<VPL>, (unsigned)(ceil_div(nchunks, FIX_RUNS) * nslabs), 32 * FIX_RUNS, 0, st, d_seg_off, P, U, d, R, nchunks, nslabs, d_rows, add, d_out, partial, span, d_U, gate);
 }
 
 gram_status accumulate_launch(gram_ctx* ctx, IndexWorkspace* ws, const void* d_in, int in_bf16, const int32_t* d_perm,
