@@ -440,20 +440,39 @@ __device__ __forceinline__ void f32_tile(const F32Prod& p, int64_t m0, int64_t n
       *reinterpret_cast<float4*>(part + (4 * ty + i) * LD + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
   }
   const int rows = TILE / splits, r0 = part_no * rows;             // this block's share of the tile's rows
-  gram_cluster_sync();
-  for (int idx = threadIdx.x; idx < rows * (TILE / 4); idx += TALL) {     // four columns of a row each
-    const int r = r0 + idx / (TILE / 4), c = 4 * (idx % (TILE / 4));
-    const int64_t m = m0 + r, n = n0 + c;
-    const uint32_t at = smem_u32(part + r * LD + c);
-    const bool ok = m < M && n < N;
-    float4 aux = make_float4(0.f, 0.f, 0.f, 0.f);
-    F32Cols cols = {aux, aux, aux};
-    float mu = 0.f, rs = 1.f;
-    if (vec_e && ok) {
-      aux = f32_aux(e, C, m * ldc + n);
-      cols = f32_cols(e, (int)n);
-      if (e.res_mean) { mu = e.res_mean[m]; rs = e.res_rstd[m]; }
+  const int count = rows * (TILE / 4);                             // four columns of a row each
+  struct Out {
+    int r, c;
+    int64_t m, n;
+    bool ok;
+    float4 aux;
+    F32Cols cols;
+    float mu, rs, sum;
+  };
+  auto output = [&](int idx) {
+    Out o;
+    o.r = r0 + idx / (TILE / 4);
+    o.c = 4 * (idx % (TILE / 4));
+    o.m = m0 + o.r;
+    o.n = n0 + o.c;
+    o.ok = o.m < M && o.n < N;
+    o.aux = make_float4(0.f, 0.f, 0.f, 0.f);
+    o.cols = {o.aux, o.aux, o.aux};
+    o.mu = 0.f; o.rs = 1.f; o.sum = 0.f;
+    if (vec_e && o.ok) {
+      o.aux = f32_aux(e, C, o.m * ldc + o.n);
+      o.cols = f32_cols(e, (int)o.n);
+      if (e.res_mean) { o.mu = e.res_mean[o.m]; o.rs = e.res_rstd[o.m]; }
     }
+    if (sums && o.c == 0 && o.m < M) o.sum = p.row_sums[o.m];
+    return o;
+  };
+  Out o;
+  int idx = threadIdx.x;
+  if (idx < count) o = output(idx);                                // what the epilogue reads is fetched before the wait for the others
+  gram_cluster_sync();
+  while (idx < count) {
+    const uint32_t at = smem_u32(part + o.r * LD + o.c);
     float v[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int s0 = 0; s0 < F32_MAX_SPLIT; s0 += 8) {                // eight parts on their way at once, added in order
@@ -461,36 +480,44 @@ __device__ __forceinline__ void f32_tile(const F32Prod& p, int64_t m0, int64_t n
       float4 x[8];
 #pragma unroll
       for (int s = 0; s < 8; ++s) {
-        uint32_t ra;
-        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(at), "r"(rank0 + min(s0 + s, splits - 1)));
-        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                     : "=f"(x[s].x), "=f"(x[s].y), "=f"(x[s].z), "=f"(x[s].w)
-                     : "r"(ra)
+        x[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 a;\n\tsetp.lt.s32 p, %5, %6;\n\tmapa.shared::cluster.u32 a, %4, %7;\n\t"
+                     "@p ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [a];\n\t}"
+                     : "+f"(x[s].x), "+f"(x[s].y), "+f"(x[s].z), "+f"(x[s].w)
+                     : "r"(at), "r"(s0 + s), "r"(splits), "r"(rank0 + min(s0 + s, splits - 1))
                      : "memory");
       }
 #pragma unroll
       for (int s = 0; s < 8; ++s)
         if (s0 + s < splits) { v[0] += x[s].x; v[1] += x[s].y; v[2] += x[s].z; v[3] += x[s].w; }
     }
-    if (sums && c == 0 && m < M) {
-      float a = 0.f;
-      for (int s = 0; s < splits; ++s) {
-        uint32_t ra;
-        float x;
-        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(smem_u32(part + r * LD + TILE)), "r"(rank0 + s));
-        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(ra) : "memory");
-        a += x;
-      }
-      p.row_sums[m] += a;
-    }
-    if (!ok) continue;
-    if (vec_e) {
-      f32_finish(e, C, m * ldc + n, v, aux, cols, mu, rs);
-    } else {
+    if (sums && o.c == 0) {
+      const uint32_t at_sum = smem_u32(part + o.r * LD + TILE);
+      float x[F32_MAX_SPLIT], a = 0.f;
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (n + j < N) epilogue_store<float, float>(e, C, ldc, m, (int)n + j, v[j]);
+      for (int s = 0; s < F32_MAX_SPLIT; ++s) {
+        x[s] = 0.f;
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 a;\n\tsetp.lt.s32 p, %2, %3;\n\tmapa.shared::cluster.u32 a, %1, %4;\n\t"
+                     "@p ld.shared::cluster.f32 %0, [a];\n\t}"
+                     : "+f"(x[s])
+                     : "r"(at_sum), "r"(s), "r"(splits), "r"(rank0 + min(s, splits - 1))
+                     : "memory");
+      }
+#pragma unroll
+      for (int s = 0; s < F32_MAX_SPLIT; ++s) a += x[s];
+      if (o.m < M) p.row_sums[o.m] = o.sum + a;
     }
+    if (o.ok) {
+      if (vec_e) {
+        f32_finish(e, C, o.m * ldc + o.n, v, o.aux, o.cols, o.mu, o.rs);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (o.n + q < N) epilogue_store<float, float>(e, C, ldc, o.m, (int)o.n + q, v[q]);
+      }
+    }
+    idx += TALL;
+    if (idx < count) o = output(idx);
   }
   // no block may leave while another still reads its partial tile
   gram_cluster_sync();
@@ -584,6 +611,8 @@ cudaError_t launch_f32_major(bool a_k, bool b_k, const F32Prod& p, int splits, c
 //  - K of at most four k-blocks: one round of loads by that many groups, no cluster.  160 x 512 over 128: 5.5 us over a cluster, 3.6;
 //    320 x 256 over 64 5.4 and 3.9; K = 32 takes four groups too, whose threads share the tile's epilogue (160 x 128: 4.3 and 3.2).
 //    Beyond two blocks of four groups an SM (1200 x 288 over 96, 342 tiles: 7.1 us without, 7.8 with) only as many as k-blocks.
+//  - A K range that fills one round of four groups in each of its parts, while those blocks fit at once (912 x 64 over 256: 6.6 us with
+//    eight parts of one k-block, two parts now; the check's step 390 -> 387).
 //  - Else the K range is halved over a cluster while blocks are missing and a part keeps two k-blocks.  Groups on top where the
 //    blocks leave SMs room: 64 x 64 over 4000 (64 blocks) 10.0 and 6.6, 192 x 64 (192 blocks) 10.8 and 8.6, but 256 x 64 over 1200
 //    (256 blocks) 7.0 without, 9.8 with.
@@ -599,6 +628,11 @@ F32Plan f32_plan(int64_t blocks, int64_t K, bool big, int most_parts) {
   const int sk = big ? F32Cfg<64>::SK : F32Cfg<32>::SK;
   auto groups_of = [&](int64_t k) { return k > 2 * sk || (K <= 4 * sk && blocks <= 2 * kNumSMs) ? 4 : (k > sk ? 2 : 1); };
   const bool one_round = !big && K <= 4 * sk && blocks * groups_of(K) <= 8 * kNumSMs;
+  if (!one_round && !big) {
+    int parts = 1;
+    while (parts < most_parts && K > 4 * sk * parts) parts *= 2;
+    if (K <= 4 * sk * parts && blocks * parts <= 2 * kNumSMs) { p.parts = parts; p.k_per_part = ceil_div64(ceil_div64(K, parts), sk) * sk; p.groups = 4; return p; }
+  }
   if (!one_round) {
     const int64_t enough = big ? kNumSMs : 4 * kNumSMs;
     while (p.parts < most_parts && blocks * p.parts * 2 <= enough && K >= 64 * p.parts) {
