@@ -97,9 +97,8 @@ const gram_config* gram_cfg(const gram_ctx* ctx) { return &ctx->cfg; }
 
 static cudaStream_t S(gram_stream s) { return reinterpret_cast<cudaStream_t>(s); }
 
-static gram_status check_device_status(gram_ctx* ctx) {
-  int32_t h = 0;
-  GRAM_CUDA(ctx, cudaMemcpy(&h, ctx->d_status, sizeof(h), cudaMemcpyDeviceToHost));
+// what the status word held: an error is cleared and named
+static gram_status report_device_status(gram_ctx* ctx, int32_t h) {
   if (h != 0) {
     GRAM_CUDA(ctx, cudaMemset(ctx->d_status, 0, sizeof(int32_t)));
     gram_set_error(ctx, h == GRAM_ERR_ID_RANGE ? "an ID outside its range was met on the device"
@@ -107,6 +106,11 @@ static gram_status check_device_status(gram_ctx* ctx) {
     return (gram_status)h;
   }
   return GRAM_OK;
+}
+static gram_status check_device_status(gram_ctx* ctx) {
+  int32_t h = 0;
+  GRAM_CUDA(ctx, cudaMemcpy(&h, ctx->d_status, sizeof(h), cudaMemcpyDeviceToHost));
+  return report_device_status(ctx, h);
 }
 
 extern "C" {
@@ -377,14 +381,16 @@ gram_status gram_encoder_backward(gram_ctx* ctx, const float* d_G, const int32_t
 gram_status gram_step(gram_ctx* ctx, const int32_t* d_ids, const int32_t* d_labels, int32_t B,
                       gram_step_report* report, gram_stream stream) {
   NEED_MODEL("gram_step");
-  GRAM_TRY(model_step(ctx->model, d_ids, d_labels, B, 0, report, S(stream)));
-  return check_device_status(ctx);
+  int32_t at_end = 0;
+  GRAM_TRY(model_step(ctx->model, d_ids, d_labels, B, 0, report, &at_end, S(stream)));
+  return report_device_status(ctx, at_end);
 }
 gram_status gram_step_host(gram_ctx* ctx, const int32_t* h_ids, const int32_t* h_labels, int32_t B,
                            gram_step_report* report, gram_stream stream) {
   NEED_MODEL("gram_step_host");
-  GRAM_TRY(model_step(ctx->model, h_ids, h_labels, B, 1, report, S(stream)));
-  return check_device_status(ctx);
+  int32_t at_end = 0;
+  GRAM_TRY(model_step(ctx->model, h_ids, h_labels, B, 1, report, &at_end, S(stream)));
+  return report_device_status(ctx, at_end);
 }
 gram_status gram_cache_fill(gram_ctx* ctx, gram_stream stream) {
   NEED_MODEL("gram_cache_fill");

@@ -1188,15 +1188,26 @@ static gram_status device_error(Model* m, int32_t code, cudaStream_t st) {
   return (gram_status)code;
 }
 
+// the step's last wait: the loss, and the status word as the step leaves it
+static gram_status read_loss(Model* m, int32_t* status, cudaStream_t st) {
+  GRAM_CUDA(m->ctx, cudaMemcpyAsync(m->h_pinned + 12, m->loss, 4, cudaMemcpyDeviceToHost, st));
+  GRAM_CUDA(m->ctx, cudaMemcpyAsync(m->h_pinned + 13, gram_status_word(m->ctx), 4, cudaMemcpyDeviceToHost, st));
+  GRAM_CUDA(m->ctx, cudaStreamSynchronize(st));
+  *status = m->h_pinned[13];
+  return GRAM_OK;
+}
+
 // Host synchronisation points: Single-step waits once after the dedup (it needs U to size the encoder pass, and reads the
 // status word in the same wait, so a batch with an ID out of range is rejected before anything else runs) and once at the
-// end.  A Multi-step step without encoder pass waits once, at the end: U stays on the device, and every kernel that
+// end, where *at_end receives the status word in the same wait as the loss (a copy of its own after that wait cost a step of
+// 390 us another round trip).  A Multi-step step without encoder pass waits once, at the end: U stays on the device, and every kernel that
 // changes state that outlives the step (table, touched bits, task parameters) is gated on the status word, so a rejected
 // batch still changes nothing.  The K-th step of a window waits once more to read the number of touched items.
 gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in, int32_t B, int on_host,
-                       gram_step_report* rep, cudaStream_t st) {
+                       gram_step_report* rep, int32_t* at_end, cudaStream_t st) {
   const gram_config& c = m->cfg;
   gram_ctx* ctx = m->ctx;
+  *at_end = 0;
   if (c.n_layers <= 0 || c.task == GRAM_TASK_NONE) return gram_set_error(ctx, "gram_step needs both modules"), GRAM_ERR_ARG;
   if (B <= 0 || B > c.B_max) return gram_set_error(ctx, "gram_step: B=%d outside 1..B_max=%d", B, c.B_max), GRAM_ERR_WORKSPACE;
   if (!ids_in || !labels_in) return gram_set_error(ctx, "gram_step: null buffer"), GRAM_ERR_ARG;
@@ -1326,8 +1337,7 @@ gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in
       n_encoded = n_touched;
       encoder_ran = 1;
       GRAM_CUDA(ctx, cudaEventRecord(ev[6], st));
-      GRAM_CUDA(ctx, cudaMemcpyAsync(m->h_pinned + 12, m->loss, 4, cudaMemcpyDeviceToHost, st));
-      GRAM_CUDA(ctx, cudaStreamSynchronize(st));
+      GRAM_TRY(read_loss(m, at_end, st));
     } else {
       GRAM_CUDA(ctx, cudaEventRecord(ev[6], st));
       GRAM_CUDA(ctx, cudaMemcpyAsync(m->h_pinned + 12, m->loss, 4, cudaMemcpyDeviceToHost, st));
@@ -1346,8 +1356,7 @@ gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in
   }
   if (!multi) {
     GRAM_CUDA(ctx, cudaEventRecord(ev[6], st));
-    GRAM_CUDA(ctx, cudaMemcpyAsync(m->h_pinned + 12, m->loss, 4, cudaMemcpyDeviceToHost, st));
-    GRAM_CUDA(ctx, cudaStreamSynchronize(st));
+    GRAM_TRY(read_loss(m, at_end, st));
   }
   if (rep) {
     memset(rep, 0, sizeof(*rep));

@@ -25,7 +25,7 @@ gram_status model_task(Model* m, const float* d_E, const int32_t* d_labels, int3
                        cudaStream_t st);
 gram_status model_encoder_backward(Model* m, const float* d_G, const int32_t* d_items, int32_t U, cudaStream_t st);
 gram_status model_step(Model* m, const int32_t* ids, const int32_t* labels, int32_t B, int on_host,
-                       gram_step_report* report, cudaStream_t st);
+                       gram_step_report* report, int32_t* at_end, cudaStream_t st);   // *at_end: the status word after a step that went through
 gram_status model_cache_fill(Model* m, cudaStream_t st);
 gram_status model_window_reset(Model* m, cudaStream_t st);
 gram_status model_get_window(Model* m, float* h_table, uint32_t* h_touched, float* h_cache);
