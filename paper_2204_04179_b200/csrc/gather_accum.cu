@@ -201,11 +201,62 @@ __device__ __forceinline__ void store_row(float* __restrict__ out, int64_t row, 
   }
 }
 
-template <typename InT, int VPL, int UNROLL>
+// The items of a chunk in ascending order: where each ends and the output row it goes to.
+// AHEAD, for sums that are added to rows picked by `rows`: lane l holds those of item `base` + l, the next 32 are on their way, so an
+// item costs shuffles.  With loads of its own, one after the other (its row, the row's old values, the end of the next item), a chunk of
+// short items waited for each: 10^6 positions over 10^5 items into a table of 768 columns 882 us, 636 with the old values fetched when
+// the item begins; 25 600 over 10^4 58 and 35.  Plain sums have the one load of the next end, and keep it: there the shuffles cost
+// more (10^6 x 128 over 3 10^5 items 158 us, 174 ahead).  All lanes of a warp call.
+template <bool AHEAD> struct SegItems {
+  const int32_t* seg_off;
+  const int32_t* rows;
+  int32_t U, base, u, off, row, off_next, row_next;      // u: the current item
+  int lane;
+  __device__ __forceinline__ void fetch(int32_t first, int32_t& o, int32_t& r) const {
+    const int32_t i = first + lane;
+    o = i < U ? seg_off[i + 1] : INT32_MAX;
+    r = i < U ? (rows ? rows[i] : i) : 0;
+  }
+  __device__ __forceinline__ SegItems(const int32_t* so, const int32_t* rw, int32_t n, int32_t first, int l)
+      : seg_off(so), rows(rw), U(n), base(first), u(first), lane(l) {
+    if (AHEAD) {
+      fetch(first, off, row);
+      fetch(first + 32, off_next, row_next);
+    }
+  }
+  __device__ __forceinline__ void advance() {
+    ++u;
+    if (AHEAD && u - base == 32) {
+      base = u;
+      off = off_next;
+      row = row_next;
+      fetch(base + 32, off_next, row_next);
+    }
+  }
+  __device__ __forceinline__ int32_t end() const { return AHEAD ? __shfl_sync(0xffffffffu, off, u - base) : seg_off[u + 1]; }
+  __device__ __forceinline__ int32_t out_row() const { return AHEAD ? __shfl_sync(0xffffffffu, row, u - base) : (rows ? rows[u] : u); }
+};
+// what a row of sums is added to, fetched when its item begins
+template <int VPL>
+__device__ __forceinline__ void load_old(const float* __restrict__ out, int64_t row, int d, int col0, int lane, float4 (&old)[VPL]) {
+#pragma unroll
+  for (int v = 0; v < VPL; ++v) {
+    const int c = col0 + (v * 32 + lane) * 4;
+    old[v] = c < d ? *reinterpret_cast<const float4*>(out + row * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+template <int VPL>
+__device__ __forceinline__ void add_old(float4 (&acc)[VPL], const float4 (&old)[VPL]) {
+#pragma unroll
+  for (int v = 0; v < VPL; ++v) { acc[v].x += old[v].x; acc[v].y += old[v].y; acc[v].z += old[v].z; acc[v].w += old[v].w; }
+}
+
+// ADD: out[row] += the sum
+template <typename InT, int VPL, int UNROLL, bool ADD>
 __global__ void __launch_bounds__(256) segsum_chunks_kernel(const InT* __restrict__ in, const int32_t* __restrict__ perm,
                                                             const int32_t* __restrict__ seg_off, int64_t P, int32_t U,
                                                             int d, int64_t R, int nchunks, int nslabs,
-                                                            const int32_t* __restrict__ rows, int add,
+                                                            const int32_t* __restrict__ rows,
                                                             float* __restrict__ out, float* __restrict__ partial,
                                                             int2* __restrict__ span, int32_t* status,
                                                             const int32_t* __restrict__ d_U,
@@ -222,11 +273,12 @@ __global__ void __launch_bounds__(256) segsum_chunks_kernel(const InT* __restric
   const int64_t c0 = (int64_t)chunk * R, c1 = min(c0 + R, P);
   if (c0 >= c1) return;
 
-  int32_t u = find_segment(seg_off, U, c0, lane);
-  int64_t seg_begin = seg_off[u], seg_end = seg_off[u + 1];
-  float4 acc[VPL];
+  SegItems<ADD> it(seg_off, rows, U, find_segment(seg_off, U, c0, lane), lane);
+  int32_t seg_begin = seg_off[it.u], seg_end = it.end();
+  float4 acc[VPL], old[ADD ? VPL : 1];
 #pragma unroll
   for (int v = 0; v < VPL; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if constexpr (ADD) load_old<VPL>(out, it.out_row(), d, col0, lane, old);
 
   for (int64_t j0 = c0; j0 < c1; j0 += 32) {
     const int nrow = (int)min((int64_t)32, c1 - j0);
@@ -251,14 +303,17 @@ __global__ void __launch_bounds__(256) segsum_chunks_kernel(const InT* __restric
       for (int r = 0; r < UNROLL; ++r) {
         const int64_t j = j0 + b + r;
         if (j < c1) {
-          while (j == seg_end && u + 1 < U) {   // item u is complete (its end lies inside this chunk)
-            if (seg_begin >= c0) store_row<VPL>(out, rows ? rows[u] : u, d, col0, lane, acc, add != 0);
-            else store_row<VPL>(partial, (int64_t)chunk * 2 + 0, d, col0, lane, acc, false);
-            ++u;
+          while (j == seg_end && it.u + 1 < U) {   // the item is complete (its end lies inside this chunk)
+            if (seg_begin >= c0) {
+              if constexpr (ADD) add_old<VPL>(acc, old);
+              store_row<VPL>(out, it.out_row(), d, col0, lane, acc, false);
+            } else store_row<VPL>(partial, (int64_t)chunk * 2 + 0, d, col0, lane, acc, false);
+            it.advance();
             seg_begin = seg_end;
-            seg_end = seg_off[u + 1];
+            seg_end = it.end();
 #pragma unroll
             for (int v = 0; v < VPL; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (ADD) load_old<VPL>(out, it.out_row(), d, col0, lane, old);
           }
 #pragma unroll
           for (int v = 0; v < VPL; ++v) {
@@ -271,11 +326,13 @@ __global__ void __launch_bounds__(256) segsum_chunks_kernel(const InT* __restric
   // the item still open at the end of the chunk
   int2 sp = make_int2(-1, 0);
   if (seg_end <= c1) {             // it ends exactly at the chunk end
-    if (seg_begin >= c0) store_row<VPL>(out, rows ? rows[u] : u, d, col0, lane, acc, add != 0);
-    else store_row<VPL>(partial, (int64_t)chunk * 2 + 0, d, col0, lane, acc, false);
+    if (seg_begin >= c0) {
+      if constexpr (ADD) add_old<VPL>(acc, old);
+      store_row<VPL>(out, it.out_row(), d, col0, lane, acc, false);
+    } else store_row<VPL>(partial, (int64_t)chunk * 2 + 0, d, col0, lane, acc, false);
   } else {                         // it continues to the right
     store_row<VPL>(partial, (int64_t)chunk * 2 + (seg_begin >= c0 ? 1 : 0), d, col0, lane, acc, false);
-    if (seg_begin >= c0) sp = make_int2(u, (int)((seg_end - 1) / R));      // it starts here: the fix-up adds its parts
+    if (seg_begin >= c0) sp = make_int2(it.u, (int)((seg_end - 1) / R));      // it starts here: the fix-up adds its parts
   }
   if (slab == 0 && lane == 0) span[chunk] = sp;   // (item, last chunk it reaches), or -1: nothing to fix up from here
 }
@@ -290,12 +347,12 @@ constexpr int SEG_WARPS = 8, SEG_STAGES_MAX = 8;
 constexpr int kSegRingMin = 512;                 // columns, more than
 constexpr int64_t kSegRingRows = 20000;          // positions, at least
 constexpr int64_t kSegRingBytes = 110 * 1024;    // shared memory of a block: two per SM
-template <int NQ>
-__global__ void __launch_bounds__(32 * SEG_WARPS) segsum_ring_kernel(const float* __restrict__ in, const int32_t* __restrict__ perm,
+template <int NQ, bool ADD>
+__global__ void __launch_bounds__(32 * SEG_WARPS, 2) segsum_ring_kernel(const float* __restrict__ in, const int32_t* __restrict__ perm,
                                                                     const int32_t* __restrict__ seg_off, int64_t P, int32_t U, int d,
                                                                     int64_t R, int nchunks, int stages, int32_t ring_rows,
                                                                     const int32_t* __restrict__ rows,
-                                                                    int add, float* __restrict__ out, float* __restrict__ partial,
+                                                                    float* __restrict__ out, float* __restrict__ partial,
                                                                     int2* __restrict__ span, int32_t* status,
                                                                     const int32_t* __restrict__ d_U, const int32_t* __restrict__ gate) {
   if (!chain_begin()) return;
@@ -337,11 +394,12 @@ __global__ void __launch_bounds__(32 * SEG_WARPS) segsum_ring_kernel(const float
     const int32_t p = __shfl_sync(0xffffffffu, cur, k);
     if (lane == 0 && c0 + k < c1) request(p, k);
   }
-  int32_t u = find_segment(seg_off, U, c0, lane);
-  int64_t seg_begin = seg_off[u], seg_end = seg_off[u + 1];
-  float4 acc[NQ];
+  SegItems<ADD> it(seg_off, rows, U, find_segment(seg_off, U, c0, lane), lane);
+  int32_t seg_begin = seg_off[it.u], seg_end = it.end();
+  float4 acc[NQ], old[ADD ? NQ : 1];
 #pragma unroll
   for (int v = 0; v < NQ; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if constexpr (ADD) load_old<NQ>(out, it.out_row(), d, 0, lane, old);
   int s = 0;
   uint32_t parity = 0;
   bool failed = false;
@@ -363,14 +421,17 @@ __global__ void __launch_bounds__(32 * SEG_WARPS) segsum_ring_kernel(const float
       nxt = fetch_perm(j + 33);
     }
     if (++s == stages) { s = 0; parity ^= 1u; }
-    while (j == seg_end && u + 1 < U) {                        // item u is complete (its end lies inside this chunk)
-      if (seg_begin >= c0) store_row<NQ>(out, rows ? rows[u] : u, d, 0, lane, acc, add != 0);
-      else store_row<NQ>(partial, (int64_t)chunk * 2 + 0, d, 0, lane, acc, false);
-      ++u;
+    while (j == seg_end && it.u + 1 < U) {                     // the item is complete (its end lies inside this chunk)
+      if (seg_begin >= c0) {
+        if constexpr (ADD) add_old<NQ>(acc, old);
+        store_row<NQ>(out, it.out_row(), d, 0, lane, acc, false);
+      } else store_row<NQ>(partial, (int64_t)chunk * 2 + 0, d, 0, lane, acc, false);
+      it.advance();
       seg_begin = seg_end;
-      seg_end = seg_off[u + 1];
+      seg_end = it.end();
 #pragma unroll
       for (int v = 0; v < NQ; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if constexpr (ADD) load_old<NQ>(out, it.out_row(), d, 0, lane, old);
     }
 #pragma unroll
     for (int v = 0; v < NQ; ++v) { acc[v].x += x[v].x; acc[v].y += x[v].y; acc[v].z += x[v].z; acc[v].w += x[v].w; }
@@ -388,11 +449,13 @@ __global__ void __launch_bounds__(32 * SEG_WARPS) segsum_ring_kernel(const float
   }
   int2 sp = make_int2(-1, 0);
   if (seg_end <= c1) {             // the item still open ends exactly at the chunk end
-    if (seg_begin >= c0) store_row<NQ>(out, rows ? rows[u] : u, d, 0, lane, acc, add != 0);
-    else store_row<NQ>(partial, (int64_t)chunk * 2 + 0, d, 0, lane, acc, false);
+    if (seg_begin >= c0) {
+      if constexpr (ADD) add_old<NQ>(acc, old);
+      store_row<NQ>(out, it.out_row(), d, 0, lane, acc, false);
+    } else store_row<NQ>(partial, (int64_t)chunk * 2 + 0, d, 0, lane, acc, false);
   } else {                         // it continues to the right
     store_row<NQ>(partial, (int64_t)chunk * 2 + (seg_begin >= c0 ? 1 : 0), d, 0, lane, acc, false);
-    if (seg_begin >= c0) sp = make_int2(u, (int)((seg_end - 1) / R));
+    if (seg_begin >= c0) sp = make_int2(it.u, (int)((seg_end - 1) / R));
   }
   if (lane == 0) span[chunk] = sp;
 }
@@ -630,16 +693,16 @@ static void segsum_run(const void* d_in, const int32_t* d_perm, const int32_t* d
   if constexpr (sizeof(InT) == 4) {
     if (d > kSegRingMin && d <= 1024 && P >= kSegRingRows) {
       ring = true;
-      auto kern = d <= 768 ? segsum_ring_kernel<6> : segsum_ring_kernel<8>;
+      auto kern = d <= 768 ? (add ? segsum_ring_kernel<6, true> : segsum_ring_kernel<6, false>) : (add ? segsum_ring_kernel<8, true> : segsum_ring_kernel<8, false>);
       int stages = (int)(kSegRingBytes / ((int64_t)SEG_WARPS * d * 4));
       if (stages > SEG_STAGES_MAX) stages = SEG_STAGES_MAX;
       (void)cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegRingBytes);
       launch_chain(kern, ceil_div(nchunks, SEG_WARPS), 32 * SEG_WARPS, (size_t)SEG_WARPS * stages * d * 4, st, (const float*)d_in, d_perm,
-                   d_seg_off, P, U, d, R, nchunks, stages, ring_rows, d_rows, add, d_out, partial, span, status, d_U, gate);
+                   d_seg_off, P, U, d, R, nchunks, stages, ring_rows, d_rows, d_out, partial, span, status, d_U, gate);
     }
   }
-  if (!ring) launch_chain(segsum_chunks_kernel<InT, VPL, 8>, blocks, 256, 0, st, (const InT*)d_in, d_perm, d_seg_off, P, U, d, R, nchunks, nslabs,
-                                                            d_rows, add, d_out, partial, span, status, d_U, gate);
+  if (!ring) launch_chain(add ? segsum_chunks_kernel<InT, VPL, 8, true> : segsum_chunks_kernel<InT, VPL, 8, false>, blocks, 256, 0, st, (const InT*)d_in, d_perm, d_seg_off, P, U, d, R, nchunks, nslabs,
+                                                            d_rows, d_out, partial, span, status, d_U, gate);
   if (nchunks > 1)
     launch_chain(segsum_fixup_kernel<VPL>, (unsigned)(ceil_div(nchunks, FIX_RUNS) * nslabs), 32 * FIX_RUNS, 0, st, d_seg_off, P, U, d, R, nchunks, nslabs, d_rows, add, d_out, partial, span, d_U, gate);
 }
