@@ -865,6 +865,25 @@ __global__ void __launch_bounds__(128) kt_input_bwd_vec_kernel(const float* __re
   }
 }
 
+// Predictions of a batch that are not padding.  Up to kHeadCounts positions every block of the head counts them for itself (16 labels
+// a thread) and block 0 leaves the count for the reduction: the launch that counts and the clearing before it, some 6 us of the
+// check's step of 377, only pay above.
+constexpr int64_t kHeadCounts = 4096;
+__device__ __forceinline__ int32_t head_count(const int32_t* __restrict__ labels, int64_t P, int32_t* n_real) {
+  if (P > kHeadCounts) return *n_real;
+  int32_t c = 0, total = 0;
+#pragma unroll 4
+  for (int p = threadIdx.x; p < (int)P; p += 256) c += labels[p] >= 0;
+  __shared__ int32_t sw[8];
+  c = __reduce_add_sync(0xffffffffu, c);
+  if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = c;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) total += sw[k];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *n_real = total;
+  return total;
+}
+
 // warp per position; per-block partials: [d] for dw, then loss and db.  A warp keeps the sums of its own rows in
 // registers (d <= 1024); the warps' sums are added in warp order at the end, so the order of additions is fixed.
 template <typename T>
@@ -872,11 +891,11 @@ __global__ void __launch_bounds__(256) kt_head_kernel(StreamRef y, const float* 
                                                       const float* __restrict__ bias, const int32_t* __restrict__ labels,
                                                       float* __restrict__ dy, T* __restrict__ dy_b,
                                                       float* __restrict__ part, int64_t P, int d, int64_t pstride,
-                                                      const int32_t* __restrict__ n_real) {
+                                                      int32_t* n_real) {
   if (!chain_begin()) return;
   extern __shared__ float sacc[];            // [warps][d + 2]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
-  const float b0 = bias[0], invP = 1.f / (float)max(*n_real, 1);   // the mean runs over the real predictions
+  const float b0 = bias[0], invP = 1.f / (float)max(head_count(labels, P, n_real), 1);   // the mean runs over the real predictions
   // rows are dealt to blocks in contiguous ranges, and inside a block to warps round-robin
   const int64_t per = (P + gridDim.x - 1) / gridDim.x;
   const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(r0 + per, P);
@@ -939,7 +958,7 @@ template <typename T, int NQ>
 __global__ void __launch_bounds__(256) kt_head_vec_kernel(StreamRef y, const float* __restrict__ w, const float* __restrict__ bias,
                                                          const int32_t* __restrict__ labels, float* __restrict__ dy,
                                                          T* __restrict__ dy_b, float* __restrict__ part, int64_t P, int d,
-                                                         int64_t pstride, const int32_t* __restrict__ n_real) {
+                                                         int64_t pstride, int32_t* n_real) {
   if (!chain_begin()) return;
   extern __shared__ __align__(16) float sacc[];  // w, gain, shift [3][d]; later the warps' sums [8][d + 4]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
@@ -950,7 +969,7 @@ __global__ void __launch_bounds__(256) kt_head_vec_kernel(StreamRef y, const flo
     sacc[2 * d + i] = ln ? y.beta[i] : 0.f;
   }
   __syncthreads();
-  const float b0 = bias[0], invP = 1.f / (float)max(*n_real, 1);   // the mean runs over the real predictions
+  const float b0 = bias[0], invP = 1.f / (float)max(head_count(labels, P, n_real), 1);   // the mean runs over the real predictions
   const int64_t per = (P + gridDim.x - 1) / gridDim.x;
   const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(r0 + per, P);
   float4 aw[NQ];
@@ -1774,9 +1793,11 @@ gram_status kt_head(gram_ctx* ctx, int dtype, const StreamRef& y, const float* w
   const int64_t pstride = d + 2;
   if (d > 1024) return gram_set_error(ctx, "kt head: d must be at most 1024"), GRAM_ERR_UNSUPPORTED;
   const size_t smem = (size_t)8 * (d + 2) * sizeof(float);
-  ProfScope prof(ctx, GRAM_K_TASK_HEAD, 12.0 * (double)P * d, 3, st);
-  GRAM_CUDA(ctx, cudaMemsetAsync(n_real, 0, sizeof(int32_t), st));
-  launch_chain(count_real_kernel, grid_for(P, 256, kNumSMs), 256, 0, st, labels, P, n_real);
+  ProfScope prof(ctx, GRAM_K_TASK_HEAD, 12.0 * (double)P * d, P > kHeadCounts ? 3 : 2, st);
+  if (P > kHeadCounts) {
+    GRAM_CUDA(ctx, cudaMemsetAsync(n_real, 0, sizeof(int32_t), st));
+    launch_chain(count_real_kernel, grid_for(P, 256, kNumSMs), 256, 0, st, labels, P, n_real);
+  }
   const size_t smem_vec = (size_t)8 * (d + 4) * sizeof(float);
   if (d % 4 == 0 && rows_aligned({y.z, dy, dy_b})) {
     DISPATCH_T(dtype, DISPATCH_NQ(d, launch_chain(kt_head_vec_kernel<T, NQ>, blocks, 256, smem_vec, st, y, w, b, labels, dy, (T*)dy_b, scratch, P, d,

@@ -1,0 +1,34 @@
+"""The mean over the predictions that are not padding, where every block of the task head counts them for itself and where a launch of
+its own does (4096 positions and one more), for rows that allow 16-byte accesses and rows that do not."""
+import pytest
+import torch
+
+from paper_2204_04179_b200 import binding, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d", [32, 18])
+@pytest.mark.parametrize("B,L", [(1, 1), (5, 51), (32, 128), (241, 17)])
+def test_mean_over_real_predictions(B, L, d):
+    shape = synth.GramShape(name="h", dtype="f32", n_items=1, l_t=1, vocab=1, d=d, n_heads=1, d_ff=4, n_layers=0, task="kt", task_layers=0,
+                            task_heads=1, task_d_ff=4, task_attn_only=False, B=B, L=L)
+    g = binding.Gram(binding.config_from_shape(shape))
+    params = synth.task_params(shape, 3, sigma=0.1, plain=False)
+    g.set_params(binding.GRAM_MODULE_TASK, synth.flatten(params))
+    gen = torch.Generator().manual_seed(B * L)
+    E = torch.randn(B, L, d, generator=gen)
+    lab = torch.randint(0, 2, (B, L), generator=gen, dtype=torch.int32)
+    n = torch.randint(1, L + 1, (B,), generator=gen)
+    real = torch.arange(L)[None] < n[:, None]
+    lab[~real] = -1
+    dE, loss = torch.empty(B * L, d, device="cuda"), torch.empty(1, device="cuda")
+    g.task(E.cuda(), lab.cuda(), B, dE, loss)
+    g.sync()
+    g.close()
+    p = {k: torch.from_numpy(v).double() for k, v in params.items()}
+    prev = torch.cat([torch.full((B, 1), 2), lab[:, :-1].clamp(min=0).long()], 1)
+    z = (E.double() + p["pos"].view(L, d) + p["resp"].view(3, d)[prev]) @ p["head_w"].view(d) + p["head_b"]
+    want = torch.nn.functional.binary_cross_entropy_with_logits(z[real], lab[real].double())
+    # a mean of terms of about 0.7 in 32 bits: some hundred roundings of 2^-24 each
+    assert abs(float(loss) - float(want)) <= 1e-5 * float(want)
