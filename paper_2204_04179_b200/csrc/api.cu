@@ -36,7 +36,7 @@ struct gram_ctx {
   ProfTag prof_tags[kProfTags] = {};
   int prof_ntags = 0;
   char err[512];
-  int32_t* d_status = nullptr;      // device status word (first device-side error)
+  int32_t* d_status = nullptr;      // kStepWords device words, the first of them the status (first device-side error)
   int32_t ring_rows = INT32_MAX;    // gram_selftest_ring_rows
   int32_t cluster_blocks = 1;       // what the device can place, or gram_selftest_cluster_blocks
   IndexWorkspace iws;
@@ -138,7 +138,7 @@ gram_status gram_create(const gram_config* cfg, gram_ctx** out) {
   ctx->cfg.d_max = d_max;
   gram_status s = GRAM_OK;
   do {
-    if (cudaMalloc(&ctx->d_status, sizeof(int32_t)) != cudaSuccess || cudaMemset(ctx->d_status, 0, sizeof(int32_t)) != cudaSuccess) {
+    if (cudaMalloc(&ctx->d_status, kStepWords * sizeof(int32_t)) != cudaSuccess || cudaMemset(ctx->d_status, 0, kStepWords * sizeof(int32_t)) != cudaSuccess) {
       s = GRAM_ERR_CUDA;
       break;
     }

@@ -154,5 +154,8 @@ __device__ __forceinline__ void gram_cluster_sync() {
 // the device status word: kernels record the first error kind they meet
 __device__ __forceinline__ void gram_device_fail(int32_t* status, int32_t code) { atomicCAS(status, 0, code); }
 int32_t* gram_status_word(gram_ctx* ctx);
+// the words that a step's host side reads lie together, the status word first: the number of unique items, the loss (fp32 bits), the
+// number of touched items of the window
+constexpr int STEP_STATUS = 0, STEP_UNIQUE = 1, STEP_LOSS = 2, STEP_TOUCHED = 3, kStepWords = 4;
 int32_t gram_cluster_blocks(const gram_ctx* ctx);   // blocks of the largest cluster that can be placed: 16, 8, 4, 2 or 1
 int32_t gram_ring_rows(const gram_ctx* ctx);   // rows a warp may take from a ring of bulk copies before it gives up; see gram_selftest_ring_rows

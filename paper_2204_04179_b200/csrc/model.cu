@@ -261,14 +261,12 @@ void layout_buffers(Model* m, Arena& a) {
   m->inverse = (int32_t*)a.take((size_t)P * 4);
   m->perm = (int32_t*)a.take((size_t)P * 4);
   m->seg_off = (int32_t*)a.take(((size_t)m->u_cap + 1) * 4);
-  m->n_unique = (int32_t*)a.take(4);
   const size_t hrows = (size_t)(m->u_cap > m->mb ? m->u_cap : m->mb);
   m->H = (float*)a.take(hrows * d * 4);
   m->G = (float*)a.take(hrows * d * 4);
   m->E = (float*)a.take((size_t)P * d * 4);
   m->Eb = a.take((size_t)P * d * esz);
   m->dE = (float*)a.take((size_t)P * d * 4);
-  m->loss = (float*)a.take(4);
   m->n_real = (int32_t*)a.take(4);
   m->red = (float*)a.take(kRedScratchBytes);
   if (c.K > 1) {
@@ -276,7 +274,6 @@ void layout_buffers(Model* m, Arena& a) {
     m->touched = (uint32_t*)a.take((size_t)((c.n_items + 31) / 32) * 4);
     m->cache = a.take((size_t)c.n_items * d * (m->cache_dtype == GRAM_BF16 ? 2 : 4));
     m->tlist = (int32_t*)a.take((size_t)c.n_items * 4);
-    m->tcount = (int32_t*)a.take(4);
   }
 }
 
@@ -944,6 +941,10 @@ gram_status model_create(gram_ctx* ctx, const gram_config* cfg, Model** out) {
     m->tail.cap = m->mb;
     m->tail.off.assign(1, m->enc.off.back());
   }
+  int32_t* words = gram_status_word(ctx);            // kStepWords: what the host reads comes back in one copy
+  m->n_unique = words + STEP_UNIQUE;
+  m->loss = reinterpret_cast<float*>(words + STEP_LOSS);
+  m->tcount = words + STEP_TOUCHED;
   Arena dry;
   layout_buffers(m, dry);
   m->arena_bytes = dry.off + 256;
@@ -1170,12 +1171,11 @@ gram_status model_optimizer_import(Model* m, int module, const float* h_m, const
   return GRAM_OK;
 }
 
-// reads a few device words with one wait: out[k] = *d_ptr[k]
-static gram_status read_words(Model* m, const int32_t* const* d_ptr, int n, int32_t* out, cudaStream_t st) {
-  for (int k = 0; k < n; ++k)
-    GRAM_CUDA(m->ctx, cudaMemcpyAsync(m->h_pinned + k, d_ptr[k], 4, cudaMemcpyDeviceToHost, st));
+// the step's words as the stream leaves them, with one copy and one wait (a copy for each word took 3 us each, 7 of the check's 366)
+static gram_status read_words(Model* m, int32_t (&out)[kStepWords], cudaStream_t st) {
+  GRAM_CUDA(m->ctx, cudaMemcpyAsync(m->h_pinned, gram_status_word(m->ctx), sizeof(out), cudaMemcpyDeviceToHost, st));
   GRAM_CUDA(m->ctx, cudaStreamSynchronize(st));
-  for (int k = 0; k < n; ++k) out[k] = m->h_pinned[k];
+  for (int k = 0; k < kStepWords; ++k) out[k] = m->h_pinned[k];
   return GRAM_OK;
 }
 
@@ -1186,15 +1186,6 @@ static gram_status device_error(Model* m, int32_t code, cudaStream_t st) {
   gram_set_error(m->ctx, code == GRAM_ERR_ID_RANGE ? "gram_step: an ID outside its range was met on the device; the step changed no state"
                                                    : (code == GRAM_ERR_TIMEOUT ? "gram_step: a bounded device-side wait ran out" : "gram_step: device-side error"));
   return (gram_status)code;
-}
-
-// the step's last wait: the loss, and the status word as the step leaves it
-static gram_status read_loss(Model* m, int32_t* status, cudaStream_t st) {
-  GRAM_CUDA(m->ctx, cudaMemcpyAsync(m->h_pinned + 12, m->loss, 4, cudaMemcpyDeviceToHost, st));
-  GRAM_CUDA(m->ctx, cudaMemcpyAsync(m->h_pinned + 13, gram_status_word(m->ctx), 4, cudaMemcpyDeviceToHost, st));
-  GRAM_CUDA(m->ctx, cudaStreamSynchronize(st));
-  *status = m->h_pinned[13];
-  return GRAM_OK;
 }
 
 // Host synchronisation points: Single-step waits once after the dedup (it needs U to size the encoder pass, and reads the
@@ -1215,7 +1206,6 @@ gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in
   const bool multi = c.K > 1;
   const bool kt = c.task == GRAM_TASK_KT;
   cudaEvent_t* ev = m->ev;
-  int32_t* status = gram_status_word(ctx);
   GRAM_CUDA(ctx, cudaEventRecord(ev[0], st));
   const int32_t* ids = ids_in;
   const int32_t* labels = labels_in;
@@ -1229,13 +1219,12 @@ gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in
   IndexWorkspace* iws = gram_index_ws(ctx);
   GRAM_TRY(dedup_launch(ctx, iws, ids, P, c.n_items, m->unique, m->inverse, m->perm, m->seg_off, m->n_unique, st));
   int32_t U = 0, n_encoded = 0, n_touched = 0, encoder_ran = 0;
+  int32_t got[kStepWords] = {};
   const float* dE_at = nullptr;
   if (!multi) {
-    const int32_t* words[2] = {m->n_unique, status};
-    int32_t got[2] = {0, 0};
-    GRAM_TRY(read_words(m, words, 2, got, st));
-    if (got[1] != 0) return device_error(m, got[1], st);
-    U = got[0];
+    GRAM_TRY(read_words(m, got, st));
+    if (got[STEP_STATUS] != 0) return device_error(m, got[STEP_STATUS], st);
+    U = got[STEP_UNIQUE];
     if (U <= 0 || U > m->u_cap) return gram_set_error(ctx, "gram_step: dedup returned U=%d", U), GRAM_ERR_ID_RANGE;
     GRAM_CUDA(ctx, cudaEventRecord(ev[1], st));
     // stage 2: one encoding per unique item (Eq. 4)
@@ -1305,16 +1294,14 @@ gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in
     if (m->step_in_window + 1 >= c.K) {
       // last step of the window: the list of touched items and its length are needed on the host now
       GRAM_TRY(touched_list_launch(ctx, m->touched, c.n_items, m->tlist, m->tcount, st));
-      const int32_t* words[3] = {m->tcount, m->n_unique, status};
-      int32_t got[3] = {0, 0, 0};
-      GRAM_TRY(read_words(m, words, 3, got, st));
-      if (got[2] != 0) {
+      GRAM_TRY(read_words(m, got, st));
+      if (got[STEP_STATUS] != 0) {
         m->task.updates = task_updates;
         m->task.wb_stale = true;
-        return device_error(m, got[2], st);
+        return device_error(m, got[STEP_STATUS], st);
       }
-      n_touched = got[0];
-      U = got[1];
+      n_touched = got[STEP_TOUCHED];
+      U = got[STEP_UNIQUE];
       GRAM_CUDA(ctx, cudaMemsetAsync(m->ce.g, 0, m->ce.n * 4, st));
       GRAM_TRY(encoder_pass(m, m->tlist, n_touched, true,
                             [&](int32_t u0, int32_t n, const float** G) {
@@ -1337,30 +1324,29 @@ gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in
       n_encoded = n_touched;
       encoder_ran = 1;
       GRAM_CUDA(ctx, cudaEventRecord(ev[6], st));
-      GRAM_TRY(read_loss(m, at_end, st));
+      GRAM_TRY(read_words(m, got, st));
+      *at_end = got[STEP_STATUS];
     } else {
       GRAM_CUDA(ctx, cudaEventRecord(ev[6], st));
-      GRAM_CUDA(ctx, cudaMemcpyAsync(m->h_pinned + 12, m->loss, 4, cudaMemcpyDeviceToHost, st));
-      const int32_t* words[3] = {m->tcount, m->n_unique, status};
-      int32_t got[3] = {0, 0, 0};
-      GRAM_TRY(read_words(m, words, 3, got, st));           // the step's only wait
-      if (got[2] != 0) {
+      GRAM_TRY(read_words(m, got, st));                     // the step's only wait
+      if (got[STEP_STATUS] != 0) {
         m->task.updates = task_updates;
         m->task.wb_stale = true;
-        return device_error(m, got[2], st);
+        return device_error(m, got[STEP_STATUS], st);
       }
-      n_touched = got[0];
-      U = got[1];
+      n_touched = got[STEP_TOUCHED];
+      U = got[STEP_UNIQUE];
       ++m->step_in_window;
     }
   }
   if (!multi) {
     GRAM_CUDA(ctx, cudaEventRecord(ev[6], st));
-    GRAM_TRY(read_loss(m, at_end, st));
+    GRAM_TRY(read_words(m, got, st));
+    *at_end = got[STEP_STATUS];
   }
   if (rep) {
     memset(rep, 0, sizeof(*rep));
-    memcpy(&rep->loss, m->h_pinned + 12, 4);
+    memcpy(&rep->loss, &got[STEP_LOSS], 4);
     rep->n_positions = (int32_t)P;
     rep->n_unique = U;
     rep->boost_ratio = U > 0 ? (float)P / (float)U : 0.f;
