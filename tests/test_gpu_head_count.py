@@ -1,5 +1,6 @@
 """The mean over the predictions that are not padding, where every block of the task head counts them for itself and where a launch of
-its own does (4096 positions and one more), for rows that allow 16-byte accesses and rows that do not."""
+its own does (4096 positions and one more), a row a warp and several (1184 positions and one more, 9472 and some more), for rows that
+allow 16-byte accesses and rows that do not."""
 import pytest
 import torch
 
@@ -9,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d", [32, 18])
-@pytest.mark.parametrize("B,L", [(1, 1), (5, 51), (32, 128), (241, 17)])
+@pytest.mark.parametrize("B,L", [(1, 1), (5, 51), (16, 74), (15, 79), (32, 128), (241, 17), (102, 93)])
 def test_mean_over_real_predictions(B, L, d):
     shape = synth.GramShape(name="h", dtype="f32", n_items=1, l_t=1, vocab=1, d=d, n_heads=1, d_ff=4, n_layers=0, task="kt", task_layers=0,
                             task_heads=1, task_d_ff=4, task_attn_only=False, B=B, L=L)
