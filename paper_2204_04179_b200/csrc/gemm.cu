@@ -295,14 +295,17 @@ struct F32Prod {
   float* C;
   int64_t ldc, M, K, k_per_part;
   int32_t N, vec_a, vec_b, vec_e;
-  float* row_sums;               // row_sums[m] += the sum of A(m, k) over k (may be null; blocks of several groups only)
+  float* row_sums;               // row_sums[m] += the sum of A(m, k) over k (may be null; FOLD only)
+  int32_t fold;                  // FOLD: k-blocks of a group that are added up in one chain
   EpiDev e;
 };
 template <int TILE, int NG> using F32Smem = float[NG][F32Cfg<TILE, NG>::BUFS][2][F32Cfg<TILE, NG>::SK * F32Cfg<TILE, NG>::LD];
 
 // One tile of a product by one block, or by `parts` blocks of a cluster whose ranks begin at rank0, this one being number `part`.
 // All threads of the blocks call it; with one part it does not touch the cluster's barrier.
-template <int TILE, bool A_K, bool B_K, int NG>
+// FOLD: after every `fold` k-blocks of a group their sum goes to the sum of those before, so that few parts of a long K are no longer
+// a chain of additions than many.
+template <int TILE, bool A_K, bool B_K, int NG, bool FOLD>
 __device__ __forceinline__ void f32_tile(const F32Prod& p, int64_t m0, int64_t n0, int part_no, int parts, int rank0, F32Smem<TILE, NG>& sm) {
   using Cfg = F32Cfg<TILE, NG>;
   constexpr int LD = Cfg::LD, NV = Cfg::NV, T = Cfg::GROUP, G = Cfg::GROUPS, SK = Cfg::SK, BUFS = Cfg::BUFS;
@@ -315,9 +318,11 @@ __device__ __forceinline__ void f32_tile(const F32Prod& p, int64_t m0, int64_t n
   const int N = p.N, vec_a = p.vec_a, vec_b = p.vec_b, vec_e = p.vec_e;
   const int group = threadIdx.x / T, tid = threadIdx.x % T, tx = tid % (TILE / 4), ty = tid / (TILE / 4);
   const int64_t kb = (int64_t)part_no * p.k_per_part, ke = min(kb + p.k_per_part, K);
-  const bool sums = G > 1 && p.row_sums != nullptr && n0 == 0;
-  float asum[4] = {0.f, 0.f, 0.f, 0.f};        // of this thread's row of A: every fourth k
-  float acc[4][4] = {};
+  static_assert(!FOLD || G > 1, "the row sums go through the groups' partial tiles");
+  const bool sums = FOLD && p.row_sums != nullptr && n0 == 0;
+  float asum = 0.f;                                        // of this thread's row of A
+  float acc[4][4] = {}, folded[FOLD ? 4 : 1][4] = {};
+  int chain = p.fold;
   float4 fa[NV], fb[NV];
   auto fetch = [&](int64_t k0) {                           // this group's k-block of the round that starts at k0 (zeros from ke on)
 #pragma unroll
@@ -339,8 +344,10 @@ __device__ __forceinline__ void f32_tile(const F32Prod& p, int64_t m0, int64_t n
     if (k0 + SK * G < ke) fetch(k0 + SK * G);
     if (G > 1 && k0 + group * SK >= ke) continue;          // the last round may have fewer k-blocks than groups
     if (sums && tid < TILE) {
+      float a[4] = {};                                     // every fourth k
 #pragma unroll
-      for (int k = 0; k < SK; ++k) asum[k & 3] += sm[group][buf][0][k * LD + tid];
+      for (int k = 0; k < SK; ++k) a[k & 3] += sm[group][buf][0][k * LD + tid];
+      asum += (a[0] + a[1]) + (a[2] + a[3]);
     }
 #pragma unroll
     for (int k = 0; k < SK; ++k) {
@@ -352,6 +359,21 @@ __device__ __forceinline__ void f32_tile(const F32Prod& p, int64_t m0, int64_t n
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
+    if constexpr (FOLD) {
+      if (--chain == 0) {
+        chain = p.fold;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) { folded[i][j] += acc[i][j]; acc[i][j] = 0.f; }
+      }
+    }
+  }
+  if constexpr (FOLD) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] += folded[i][j];
   }
   float* part = &sm[0][0][0][0];
   // the groups' sum of four columns of row r of the tile
@@ -370,7 +392,7 @@ __device__ __forceinline__ void f32_tile(const F32Prod& p, int64_t m0, int64_t n
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       *reinterpret_cast<float4*>(part + group * (TILE * LD) + (4 * ty + i) * LD + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-    if (sums && tid < TILE) part[group * (TILE * LD) + tid * LD + TILE] = (asum[0] + asum[1]) + (asum[2] + asum[3]);
+    if (sums && tid < TILE) part[group * (TILE * LD) + tid * LD + TILE] = asum;
     __syncthreads();
 #pragma unroll
     for (int idx = threadIdx.x; idx < TILE * TILE / 4; idx += TALL) {
@@ -527,7 +549,7 @@ template <int TILE, bool A_K, bool B_K, int NG>
 __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(const __grid_constant__ F32Prod p) {
   if (!chain_begin()) return;
   __shared__ __align__(16) F32Smem<TILE, NG> sm;           // [group][buffer][operand]; later the groups' partial tiles
-  f32_tile<TILE, A_K, B_K, NG>(p, (int64_t)blockIdx.y * TILE, (int64_t)blockIdx.x * TILE, blockIdx.z, gridDim.z, 0, sm);
+  f32_tile<TILE, A_K, B_K, NG, false>(p, (int64_t)blockIdx.y * TILE, (int64_t)blockIdx.x * TILE, blockIdx.z, gridDim.z, 0, sm);
 }
 
 // The two products that read one gradient dY [T, N]: dW [N, K] += dY^T X (product w; its row sums are the bias gradient) and
@@ -554,8 +576,8 @@ __global__ void __launch_bounds__(F32Cfg<32, 4>::THREADS) gemm_f32_pair_kernel(c
   const int tiles_n = (p.N + 31) / 32;
   const int64_t m0 = (int64_t)(tile / tiles_n) * 32, n0 = (int64_t)(tile % tiles_n) * 32;
   const bool there = tile < (is_w ? a.w_tiles : a.x_tiles);
-  if (there && is_w) f32_tile<32, false, false, 4>(a.w, m0, n0, part, parts, (int)rank - part, sm);
-  else if (there) f32_tile<32, true, false, 4>(a.x, m0, n0, part, parts, (int)rank - part, sm);
+  if (there && is_w) f32_tile<32, false, false, 4, true>(a.w, m0, n0, part, parts, (int)rank - part, sm);
+  else if (there) f32_tile<32, true, false, 4, true>(a.x, m0, n0, part, parts, (int)rank - part, sm);
   if (blocks > 1 && !(there && parts > 1)) {               // the cluster's barrier counts every block
     gram_cluster_sync();
     gram_cluster_sync();
@@ -1852,10 +1874,16 @@ static EpiDev epi_dev(const GemmEpilogue& epi) {
                 epi.colsum_part, epi.gelu, epi.accumulate};
 }
 
-// Both products go together where their tiles are at most three blocks an SM: above, each fills the chip by itself (a model of
-// width 32 over some 10 000 rows: 837 us a step with the line at two blocks, which fit at once, 816 at three).  Parts of the K ranges: the
-// longer chain is halved while the blocks fit the SMs at once (a width of 128: 478 us a step, 499 with half as many blocks again)
-// and it is more than one round of four k-blocks; a dW of few tiles takes parts in any case, since its chain is over the rows.
+// Both products go together where their tiles are at most three blocks an SM: above, each fills the chip by itself.  Together against
+// apart with the bias gradient's two launches, widths 16 to 128 over 100 to 14 000 rows: 0.59 of the time up to 148 tiles, 0.74 up to
+// 370, 0.81 (0.98 at worst) up to 444, 0.96 (1.57 at worst) on from there to 900.
+// Parts of the K ranges: the longer chain is halved while the blocks fit the SMs at once (a width of 128: 478 us a step, 499 with half
+// as many blocks again) and it is more than one round of four k-blocks.  dW's chain runs over the rows, and dX's blocks, which are as
+// many as the rows are, would leave it no parts: while it is longer than four rounds it is halved up to a block an SM whatever dX takes.
+// us with the SMs shared out and this way: 192 x 64 over 4096 rows 32.6 and 16.6 (apart 21.0), over 6400 47.3 and 23.7, 288 x 96 over 2952
+// 44.8 and 22.8, 384 x 128 48.3 and 32.0, 96 x 32 over 10 000 22.2 and 15.4; a line at two rounds or eight loses up to a fifth at single sizes.
+// What a group adds up in one chain is no longer than in the product alone (`fold`; error against 64 bits of 192 x 64 over 6400 4.9e-7 -> 2.0e-7, which is
+// the product alone): folding costs 3 to 5 % of a launch of many rounds.
 bool gemm_f32_grads_together(int64_t T, int N, int K) {
   const int64_t w = (int64_t)ceil_div(N, 32) * ceil_div(K, 32), x = ceil_div64(T, 32) * ceil_div(K, 32);
   return T > 0 && N > 0 && K > 0 && w + x <= 3 * kNumSMs;
@@ -1875,7 +1903,7 @@ gram_status gemm_f32_grads(gram_ctx* ctx, const float* dY, const float* X, float
     const bool w_first = wk >= xk;
     if ((w_first ? wk : xk) <= ROUND) break;
     const int64_t w = (int64_t)a.w_tiles * a.wp, x = (int64_t)a.x_tiles * a.xp;
-    if (w + x + (w_first ? w : x) > 2 * kNumSMs && !(w_first && 2 * w <= 32)) break;
+    if (w + x + (w_first ? w : x) > 2 * kNumSMs && !(w_first && wk > 4 * ROUND && 2 * w <= kNumSMs)) break;
     if (w_first) a.wp *= 2;
     else a.xp *= 2;
   }
@@ -1883,7 +1911,13 @@ gram_status gemm_f32_grads(gram_ctx* ctx, const float* dY, const float* X, float
   ew.accumulate = 1;
   a.w = f32_prod(dY, N, X, K, dW, K, N, K, T, ceil_div64(ceil_div64(T, a.wp), SK) * SK, ew);
   a.w.row_sums = db;
+  auto fold_of = [&](int64_t tiles, int64_t k) {
+    const F32Plan alone = f32_plan(tiles, k, false, most);
+    return (int32_t)ceil_div64(alone.k_per_part, SK * alone.groups);
+  };
+  a.w.fold = fold_of(a.w_tiles, T);
   a.x = f32_prod(dY, N, W, K, dX, K, T, K, N, (int64_t)ceil_div(ceil_div(N, a.xp), SK) * SK, epi_dev(epi));
+  a.x.fold = fold_of(a.x_tiles, N);
   const int blocks = a.wp > a.xp ? a.wp : a.xp;
   a.w_clusters = ceil_div(a.w_tiles * a.wp, blocks);
   if (blocks > 8) GRAM_CUDA(ctx, cudaFuncSetAttribute(gemm_f32_pair_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
