@@ -11,7 +11,7 @@
 constexpr int kProfSlots = 16384;
 struct ProfRec {
   int kind;
-  const char* tag;
+  const char *tag, *tag2;
   double work;
   int launches;
 };
@@ -56,13 +56,13 @@ int32_t* gram_status_word(gram_ctx* ctx) { return ctx->d_status; }
 int32_t gram_cluster_blocks(const gram_ctx* ctx) { return ctx->cluster_blocks; }
 int32_t gram_ring_rows(const gram_ctx* ctx) { return ctx->ring_rows; }
 
-void gram_prof_open(gram_ctx* ctx, int kind, const char* tag, double work, int launches, cudaStream_t st, int* slot) {
+void gram_prof_open(gram_ctx* ctx, int kind, const char* tag, const char* tag2, double work, int launches, cudaStream_t st, int* slot) {
   *slot = -1;
   if (!ctx) return;
   ctx->launch_count += launches;
   if (!ctx->prof_on || ctx->prof_used >= kProfSlots) return;
   const int k = ctx->prof_used++;
-  ctx->prof_rec[k] = ProfRec{kind, tag, work, launches};
+  ctx->prof_rec[k] = ProfRec{kind, tag, tag2, work, launches};
   cudaEventRecord(ctx->prof_ev[2 * k], st);
   *slot = k;
 }
@@ -77,13 +77,15 @@ static void prof_fold(gram_ctx* ctx) {
       ctx->prof_ms[r.kind] += ms;
       ctx->prof_work[r.kind] += r.work;
       ctx->prof_launches[r.kind] += r.launches;
-      if (r.tag) {
+      const double share = r.tag2 ? 0.5 : 1.0;
+      for (const char* tag : {r.tag, r.tag2}) {
+        if (!tag) continue;
         int t = 0;
-        while (t < ctx->prof_ntags && ctx->prof_tags[t].tag != r.tag && strcmp(ctx->prof_tags[t].tag, r.tag) != 0) ++t;
-        if (t == ctx->prof_ntags && t < kProfTags) ctx->prof_tags[ctx->prof_ntags++] = ProfTag{r.tag, r.kind, 0, 0, 0};
+        while (t < ctx->prof_ntags && ctx->prof_tags[t].tag != tag && strcmp(ctx->prof_tags[t].tag, tag) != 0) ++t;
+        if (t == ctx->prof_ntags && t < kProfTags) ctx->prof_tags[ctx->prof_ntags++] = ProfTag{tag, r.kind, 0, 0, 0};
         if (t < kProfTags) {
-          ctx->prof_tags[t].ms += ms;
-          ctx->prof_tags[t].work += r.work;
+          ctx->prof_tags[t].ms += share * ms;
+          ctx->prof_tags[t].work += share * r.work;
           ctx->prof_tags[t].launches += r.launches;
         }
       }

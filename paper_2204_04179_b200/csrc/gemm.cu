@@ -1888,10 +1888,10 @@ bool gemm_f32_grads_together(int64_t T, int N, int K) {
   const int64_t w = (int64_t)ceil_div(N, 32) * ceil_div(K, 32), x = ceil_div64(T, 32) * ceil_div(K, 32);
   return T > 0 && N > 0 && K > 0 && w + x <= 3 * kNumSMs;
 }
-gram_status gemm_f32_grads(gram_ctx* ctx, const float* dY, const float* X, float* dW, float* db, const float* W, float* dX, int64_t T,
-                           int N, int K, const GemmEpilogue& epi, cudaStream_t st) {
+gram_status gemm_f32_grads(gram_ctx* ctx, const float* dY, const float* X, float* dW, const char* dw_tag, float* db, const float* W, float* dX,
+                           int64_t T, int N, int K, const GemmEpilogue& epi, cudaStream_t st) {
   if (!dY || !X || !dW || !W || !dX || !gemm_f32_grads_together(T, N, K)) return gram_set_error(ctx, "gemm: bad gradient products"), GRAM_ERR_ARG;
-  ProfScope prof(ctx, GRAM_K_GEMM, 4.0 * (double)T * N * (double)K, 1, st, epi.tag ? epi.tag : "gemm_f32");
+  ProfScope prof(ctx, GRAM_K_GEMM, 4.0 * (double)T * N * (double)K, 1, st, dw_tag ? dw_tag : "gemm_f32", epi.tag ? epi.tag : "gemm_f32");
   const int most = F32_MAX_SPLIT < gram_cluster_blocks(ctx) ? F32_MAX_SPLIT : gram_cluster_blocks(ctx);
   constexpr int SK = F32Cfg<32, 4>::SK, ROUND = 4 * SK;
   F32Pair a = {};

@@ -50,10 +50,10 @@ gram_status gemm_launch(gram_ctx* ctx, GemmWorkspace* ws, int dtype, const void*
                         int64_t K, const GemmEpilogue& epi, int allow_splitk, cudaStream_t st);
 
 // fp32: dW [N, K] += dY^T X, db [N] += the column sums of dY (db may be null) and dX [T, K] = dY W with its epilogue, in one
-// launch; dY [T, N], X [T, K], W [N, K].  Offered for the sizes that ..._together names.
+// launch; dY [T, N], X [T, K], W [N, K].  Offered for the sizes that ..._together names.  dw_tag, epi.tag: the call sites of the two
 bool gemm_f32_grads_together(int64_t T, int N, int K);
-gram_status gemm_f32_grads(gram_ctx* ctx, const float* dY, const float* X, float* dW, float* db, const float* W, float* dX, int64_t T,
-                           int N, int K, const GemmEpilogue& epi, cudaStream_t st);
+gram_status gemm_f32_grads(gram_ctx* ctx, const float* dY, const float* X, float* dW, const char* dw_tag, float* db, const float* W, float* dX,
+                           int64_t T, int N, int K, const GemmEpilogue& epi, cudaStream_t st);
 
 // true when gemm_launch(dtype, ..., M, N, ...) with dgelu_pre set runs the variant that can fill colsum_part
 bool gemm_fused_colsum(int dtype, int64_t M, int N);

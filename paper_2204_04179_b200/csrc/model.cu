@@ -336,7 +336,7 @@ bool bias_in_products(const Model* m, int64_t T, int N, int K) { return m->dtype
 gram_status mm_dw_dx(Model* m, const void* dY, const void* X, float* dW, const char* dw_tag, float* db, const void* Wt, void* dX, bool x_f32,
                      int64_t T, int N, int K, const GemmEpilogue& e, cudaStream_t st) {
   if (bias_in_products(m, T, N, K))
-    return gemm_f32_grads(m->ctx, (const float*)dY, (const float*)X, dW, db, (const float*)Wt, (float*)dX, T, N, K, e, st);
+    return gemm_f32_grads(m->ctx, (const float*)dY, (const float*)X, dW, dw_tag, db, (const float*)Wt, (float*)dX, T, N, K, e, st);
   GRAM_TRY(mm_dw(m, dY, X, dW, T, N, K, st, dw_tag));
   return mm_dx(m, dY, Wt, dX, x_f32, T, N, K, e, st);
 }
