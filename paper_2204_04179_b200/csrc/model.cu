@@ -330,13 +330,13 @@ gram_status mm_dw(Model* m, const void* dY, const void* X, float* dW, int64_t T,
   return gemm_launch(m->ctx, gram_gemm_ws(m->ctx), m->dtype, dY, 0, N, X, 0, K, dW, 1, K, N, K, T, e, 1, st);
 }
 
-// the products that read one gradient dY [T, N]: dW [N, K] += dY^T X and dX [T, K] = dY W (+ epilogue); db: the bias gradient, or null
-// where the caller has it already (bias_in_products: it need not)
-bool bias_in_products(const Model* m, int64_t T, int N, int K) { return m->dtype == GRAM_F32 && gemm_f32_grads_together(T, N, K); }
+// what reads one gradient dY [T, N]: dW [N, K] += dY^T X, dX [T, K] = dY W (+ epilogue) and db [N] += the column sums of dY (null where
+// the producer of dY left them already)
 gram_status mm_dw_dx(Model* m, const void* dY, const void* X, float* dW, const char* dw_tag, float* db, const void* Wt, void* dX, bool x_f32,
                      int64_t T, int N, int K, const GemmEpilogue& e, cudaStream_t st) {
-  if (bias_in_products(m, T, N, K))
+  if (m->dtype == GRAM_F32 && gemm_f32_grads_together(T, N, K))
     return gemm_f32_grads(m->ctx, (const float*)dY, (const float*)X, dW, dw_tag, db, (const float*)Wt, (float*)dX, T, N, K, e, st);
+  if (db) GRAM_TRY(colsum_accumulate(m->ctx, m->dtype, dY, T, N, db, m->red, st));
   GRAM_TRY(mm_dw(m, dY, X, dW, T, N, K, st, dw_tag));
   return mm_dx(m, dY, Wt, dX, x_f32, T, N, K, e, st);
 }
@@ -439,7 +439,6 @@ gram_status layer_rest_backward(Model* m, Module& mod, const LayerOff& o, Stack&
   float* red = m->red;
   float* cur = *cur_io;
   float* oth = *oth_io;
-  float* bo = nullptr;                 // where the products at the end are to add the output projection's bias gradient
   GemmEpilogue e;
   if (!s.attn_only) {
     // out = LN2(z2), z2 = h1 + W2 gelu(u) + b2, u = W1 h1 + b1, h1 = LN1(z1), z1 = x + Wo ctx + bo
@@ -451,23 +450,19 @@ gram_status layer_rest_backward(Model* m, Module& mod, const LayerOff& o, Stack&
     const bool fused_b1 = gemm_fused_colsum(m->dtype, T, f);                           // the product's epilogue also adds up its columns
     if (fused_b1) e.colsum_part = s.cpart;
     GRAM_TRY(mm_dw_dx(m, s.dzb, a.g, mod.g + o.w2, "dw_ffn2", nullptr, W(m, mod, o.w2), s.du, false, T, d, f, e, st));   // du = (dz2 W2) * gelu'(v), the saved u
-    const bool b1_later = bias_in_products(m, T, f, d);
     if (fused_b1) GRAM_TRY(colsum_from_partials(ctx, s.cpart, (T + 31) / 32, f, mod.g + o.b1, st));
-    else if (!b1_later) GRAM_TRY(colsum_accumulate(ctx, m->dtype, s.du, T, f, mod.g + o.b1, red, st));
     e = GemmEpilogue();
     e.res = oth;
     e.tag = "dx_ffn1";
-    GRAM_TRY(mm_dw_dx(m, s.du, a.h1, mod.g + o.w1, "dw_ffn1", b1_later ? mod.g + o.b1 : nullptr, W(m, mod, o.w1), cur, true, T, f, d, e, st));   // cur = dh1 = du W1 + dz2
+    GRAM_TRY(mm_dw_dx(m, s.du, a.h1, mod.g + o.w1, "dw_ffn1", fused_b1 ? nullptr : mod.g + o.b1, W(m, mod, o.w1), cur, true, T, f, d, e, st));   // cur = dh1 = du W1 + dz2
     GRAM_TRY(layernorm_backward(ctx, m->dtype, cur, a.z1, a.mean1, a.rstd1, mod.w + o.ln1g, oth, s.dzb, mod.g + o.ln1g,
                                 mod.g + o.ln1b, mod.g + o.bo, red, T, d, st));         // oth, dzb = dz1; dbo += its column sums
   } else {
     float* t = cur; cur = oth; oth = t;                                                // oth = d(out), dzb its copy
-    if (bias_in_products(m, T, d, d)) bo = mod.g + o.bo;
-    else GRAM_TRY(colsum_accumulate(ctx, m->dtype, s.dzb, T, d, mod.g + o.bo, red, st));
   }
   e = GemmEpilogue();
   e.tag = "dx_attn_out";
-  GRAM_TRY(mm_dw_dx(m, s.dzb, a.ctx, mod.g + o.wo, "dw_attn_out", bo, W(m, mod, o.wo), s.dctx, false, T, d, d, e, st));
+  GRAM_TRY(mm_dw_dx(m, s.dzb, a.ctx, mod.g + o.wo, "dw_attn_out", s.attn_only ? mod.g + o.bo : nullptr, W(m, mod, o.wo), s.dctx, false, T, d, d, e, st));
   *cur_io = cur;
   *oth_io = oth;
   return GRAM_OK;
@@ -488,14 +483,12 @@ gram_status layer_attention_backward(Model* m, Module& mod, Stack& s, int l, con
   GRAM_TRY(attention_backward(ctx, m->dtype, a.qkv, s.dctx, a.ctx, a.lse, s.delta, s.dqkv, s.cpart,
                               (int64_t)(s.cpart_elems / ((size_t)3 * d)), &part_rows, T, n_seq, S, d, s.heads, s.causal, s.seq_len,
                               s.seq_off, s.grouped ? &s.groups : nullptr, st));
-  const bool bias_later = bias_in_products(m, T, 3 * d, d);
   if (part_rows > 0) GRAM_TRY(colsum_from_partials(ctx, s.cpart, part_rows, 3 * d, mod.g + o.bqkv, st));
-  else if (!bias_later) GRAM_TRY(colsum_accumulate(ctx, m->dtype, s.dqkv, T, 3 * d, mod.g + o.bqkv, m->red, st));
   GemmEpilogue e;
   e.res = oth;
   e.tag = "dx_qkv";
   if (copy_b) e.copy_out = s.dzb;
-  return mm_dw_dx(m, s.dqkv, xb_l, mod.g + o.wqkv, "dw_qkv", bias_later ? mod.g + o.bqkv : nullptr, W(m, mod, o.wqkv), cur, true, T, 3 * d, d, e,
+  return mm_dw_dx(m, s.dqkv, xb_l, mod.g + o.wqkv, "dw_qkv", part_rows > 0 ? nullptr : mod.g + o.bqkv, W(m, mod, o.wqkv), cur, true, T, 3 * d, d, e,
                   st);                                                               // cur = dx = dqkv Wqkv + dz1
 }
 
