@@ -281,7 +281,7 @@ gram_status gram_gather(gram_ctx* ctx, const void* d_src, int64_t n_src_rows, co
 gram_status gram_accumulate(gram_ctx* ctx, const float* d_dE, const int32_t* d_perm, const int32_t* d_seg_off,
                             int64_t P, int32_t U, int32_t d, float* d_G, gram_stream stream) {
   if (!ctx) return GRAM_ERR_ARG;
-  return accumulate_launch(ctx, &ctx->iws, d_dE, 0, d_perm, d_seg_off, P, U, nullptr, d, nullptr, 0, d_G, S(stream));
+  return accumulate_launch(ctx, &ctx->iws, d_dE, d_perm, d_seg_off, P, U, nullptr, d, nullptr, 0, d_G, S(stream));
 }
 
 gram_status gram_accumulate_multistep(gram_ctx* ctx, const float* d_dE, const int32_t* d_perm,
@@ -296,7 +296,7 @@ gram_status gram_accumulate_multistep(gram_ctx* ctx, const float* d_dE, const in
     if (!d_table) d_table = model_table(ctx->model);
     if (!d_touched_bits) d_touched_bits = model_touched(ctx->model);
   }
-  GRAM_TRY(accumulate_launch(ctx, &ctx->iws, d_dE, 0, d_perm, d_seg_off, P, U, nullptr, d, d_unique, 1, d_table, S(stream)));
+  GRAM_TRY(accumulate_launch(ctx, &ctx->iws, d_dE, d_perm, d_seg_off, P, U, nullptr, d, d_unique, 1, d_table, S(stream)));
   return touched_mark_launch(ctx, d_unique, U, nullptr, n_items, d_touched_bits, nullptr, 0, S(stream));
 }
 

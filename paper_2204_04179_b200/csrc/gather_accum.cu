@@ -152,21 +152,6 @@ __global__ void __launch_bounds__(256) gather_diff_kernel(const float* __restric
 // on (P, U, seg_off), never on scheduling: repeated runs are bit-identical.
 // Algorithmic bytes: 4*P*d read + 4*U*d written + 4P (perm) + 4(U+1) (seg_off).
 // ---------------------------------------------------------------------------
-template <typename InT> struct Row4;
-template <> struct Row4<float> {
-  typedef float4 vec;
-  static __device__ __forceinline__ float4 load(const float* p) { return __ldcs(reinterpret_cast<const float4*>(p)); }
-};
-template <> struct Row4<bf16> {
-  typedef uint2 vec;
-  static __device__ __forceinline__ float4 load(const bf16* p) {
-    uint2 u = __ldcs(reinterpret_cast<const uint2*>(p));
-    __nv_bfloat162 a = *reinterpret_cast<__nv_bfloat162*>(&u.x), b = *reinterpret_cast<__nv_bfloat162*>(&u.y);
-    float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
-    return make_float4(fa.x, fa.y, fb.x, fb.y);
-  }
-};
-
 // largest u in [0, U) with seg_off[u] <= j, found by the whole warp: every lane probes one of 32 evenly spaced
 // entries per round, so U = 10^6 takes four dependent loads instead of twenty.  All 32 lanes must call it.
 __device__ __forceinline__ int32_t find_segment(const int32_t* __restrict__ seg_off, int32_t U, int64_t j, int lane) {
@@ -252,8 +237,8 @@ __device__ __forceinline__ void add_old(float4 (&acc)[VPL], const float4 (&old)[
 }
 
 // ADD: out[row] += the sum
-template <typename InT, int VPL, int UNROLL, bool ADD>
-__global__ void __launch_bounds__(256) segsum_chunks_kernel(const InT* __restrict__ in, const int32_t* __restrict__ perm,
+template <int VPL, int UNROLL, bool ADD>
+__global__ void __launch_bounds__(256) segsum_chunks_kernel(const float* __restrict__ in, const int32_t* __restrict__ perm,
                                                             const int32_t* __restrict__ seg_off, int64_t P, int32_t U,
                                                             int d, int64_t R, int nchunks, int nslabs,
                                                             const int32_t* __restrict__ rows,
@@ -296,7 +281,7 @@ __global__ void __launch_bounds__(256) segsum_chunks_kernel(const InT* __restric
 #pragma unroll
         for (int v = 0; v < VPL; ++v) {
           int c = col0 + (v * 32 + lane) * 4;
-          x[r][v] = (live && c < d) ? Row4<InT>::load(in + (int64_t)p * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+          x[r][v] = (live && c < d) ? __ldcs(reinterpret_cast<const float4*>(in + (int64_t)p * d + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
       }
 #pragma unroll
@@ -682,38 +667,35 @@ gram_status gather_diff_launch(gram_ctx* ctx, const float* d_a, const float* d_b
   return GRAM_OK;
 }
 
-template <typename InT, int VPL>
-static void segsum_run(const void* d_in, const int32_t* d_perm, const int32_t* d_seg_off, int64_t P, int32_t U, int32_t d,
+template <int VPL>
+static void segsum_run(const float* d_in, const int32_t* d_perm, const int32_t* d_seg_off, int64_t P, int32_t U, int32_t d,
                        int64_t R, int nchunks, const int32_t* d_rows, int add, float* d_out, float* partial, int2* span,
                        int32_t* status, const int32_t* d_U, cudaStream_t st, const int32_t* gate, int32_t ring_rows) {
   const int nslabs = ceil_div(d, VPL * 128);
   const int64_t warps = (int64_t)nchunks * nslabs;
   const int blocks = (int)ceil_div64(warps, 8);
-  bool ring = false;
-  if constexpr (sizeof(InT) == 4) {
-    if (d > kSegRingMin && d <= 1024 && P >= kSegRingRows) {
-      ring = true;
-      auto kern = d <= 768 ? (add ? segsum_ring_kernel<6, true> : segsum_ring_kernel<6, false>) : (add ? segsum_ring_kernel<8, true> : segsum_ring_kernel<8, false>);
-      int stages = (int)(kSegRingBytes / ((int64_t)SEG_WARPS * d * 4));
-      if (stages > SEG_STAGES_MAX) stages = SEG_STAGES_MAX;
-      (void)cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegRingBytes);
-      launch_chain(kern, ceil_div(nchunks, SEG_WARPS), 32 * SEG_WARPS, (size_t)SEG_WARPS * stages * d * 4, st, (const float*)d_in, d_perm,
-                   d_seg_off, P, U, d, R, nchunks, stages, ring_rows, d_rows, d_out, partial, span, status, d_U, gate);
-    }
+  if (d > kSegRingMin && d <= 1024 && P >= kSegRingRows) {
+    auto kern = d <= 768 ? (add ? segsum_ring_kernel<6, true> : segsum_ring_kernel<6, false>) : (add ? segsum_ring_kernel<8, true> : segsum_ring_kernel<8, false>);
+    int stages = (int)(kSegRingBytes / ((int64_t)SEG_WARPS * d * 4));
+    if (stages > SEG_STAGES_MAX) stages = SEG_STAGES_MAX;
+    (void)cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegRingBytes);
+    launch_chain(kern, ceil_div(nchunks, SEG_WARPS), 32 * SEG_WARPS, (size_t)SEG_WARPS * stages * d * 4, st, d_in, d_perm,
+                 d_seg_off, P, U, d, R, nchunks, stages, ring_rows, d_rows, d_out, partial, span, status, d_U, gate);
+  } else {
+    launch_chain(add ? segsum_chunks_kernel<VPL, 8, true> : segsum_chunks_kernel<VPL, 8, false>, blocks, 256, 0, st, d_in, d_perm, d_seg_off, P, U, d, R,
+                 nchunks, nslabs, d_rows, d_out, partial, span, status, d_U, gate);
   }
-  if (!ring) launch_chain(add ? segsum_chunks_kernel<InT, VPL, 8, true> : segsum_chunks_kernel<InT, VPL, 8, false>, blocks, 256, 0, st, (const InT*)d_in, d_perm, d_seg_off, P, U, d, R, nchunks, nslabs,
-                                                            d_rows, d_out, partial, span, status, d_U, gate);
   if (nchunks > 1)
     launch_chain(segsum_fixup_kernel<VPL>, (unsigned)(ceil_div(nchunks, FIX_RUNS) * nslabs), 32 * FIX_RUNS, 0, st, d_seg_off, P, U, d, R, nchunks, nslabs, d_rows, add, d_out, partial, span, d_U, gate);
 }
 
-gram_status accumulate_launch(gram_ctx* ctx, IndexWorkspace* ws, const void* d_in, int in_bf16, const int32_t* d_perm,
+gram_status accumulate_launch(gram_ctx* ctx, IndexWorkspace* ws, const float* d_in, const int32_t* d_perm,
                               const int32_t* d_seg_off, int64_t P, int32_t U, const int32_t* d_U, int32_t d,
                               const int32_t* d_rows, int add, float* d_out, cudaStream_t st, int gated) {
   if (P < 0 || U < 0 || d <= 0 || U > P) return gram_set_error(ctx, "gram_accumulate: bad argument"), GRAM_ERR_ARG;
   if (P == 0 || (U == 0 && !d_U)) return GRAM_OK;
   if (!d_in || !d_perm || !d_seg_off || !d_out) return gram_set_error(ctx, "gram_accumulate: null buffer"), GRAM_ERR_ARG;
-  if (d % 4 != 0 || ((uintptr_t)d_in % (in_bf16 ? 8 : 16)) || ((uintptr_t)d_out % 16))
+  if (d % 4 != 0 || ((uintptr_t)d_in % 16) || ((uintptr_t)d_out % 16))
     return gram_set_error(ctx, "gram_accumulate: d must be a multiple of 4 and buffers 16-byte aligned"), GRAM_ERR_UNSUPPORTED;
   if (d > ws->d_max) return gram_set_error(ctx, "gram_accumulate: d=%d exceeds the context's d_max=%d", d, ws->d_max), GRAM_ERR_WORKSPACE;
   // chunks: at least 16 rows each, at most kAccMaxChunks
@@ -722,18 +704,13 @@ gram_status accumulate_launch(gram_ctx* ctx, IndexWorkspace* ws, const void* d_i
   const int64_t R = ceil_div64(P, nchunks);
   nchunks = ceil_div64(P, R);
   int2* span = reinterpret_cast<int2*>(ws->partial + (size_t)kAccMaxChunks * 2 * (ws->d_max > 0 ? ws->d_max : 1));   // after the partial sums
-  ProfScope prof(ctx, GRAM_K_ACCUMULATE, (in_bf16 ? 2.0 : 4.0) * (double)P * d + 4.0 * (double)U * d + 4.0 * P + 4.0 * (U + 1),
+  ProfScope prof(ctx, GRAM_K_ACCUMULATE, 4.0 * (double)P * d + 4.0 * (double)U * d + 4.0 * P + 4.0 * (U + 1),
                  nchunks > 1 ? 2 : 1, st);
   int32_t* sw = gram_status_word(ctx);
   const int32_t* gate = gated ? sw : nullptr;
   const int32_t ring_rows = gram_ring_rows(ctx);
-  if (d >= 256) {
-    if (in_bf16) segsum_run<bf16, 2>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate, ring_rows);
-    else segsum_run<float, 2>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate, ring_rows);
-  } else {
-    if (in_bf16) segsum_run<bf16, 1>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate, ring_rows);
-    else segsum_run<float, 1>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate, ring_rows);
-  }
+  if (d >= 256) segsum_run<2>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate, ring_rows);
+  else segsum_run<1>(d_in, d_perm, d_seg_off, P, U, d, R, (int)nchunks, d_rows, add, d_out, ws->partial, span, sw, d_U, st, gate, ring_rows);
   GRAM_LAUNCH_CHECK(ctx);
   return GRAM_OK;
 }
@@ -818,8 +795,8 @@ extern "C" gram_status gram_accumulate_static(const float* d_dE, const int32_t* 
   if (nchunks > kStaticChunks) nchunks = kStaticChunks;
   const int64_t R = ceil_div64(P, nchunks);
   nchunks = ceil_div64(P, R);
-  if (d >= 256) segsum_run<float, 2>(d_dE, d_perm, d_seg_off, P, U, d, R, (int)nchunks, nullptr, 0, d_G, partial, span, status, nullptr, st, nullptr, INT32_MAX);
-  else segsum_run<float, 1>(d_dE, d_perm, d_seg_off, P, U, d, R, (int)nchunks, nullptr, 0, d_G, partial, span, status, nullptr, st, nullptr, INT32_MAX);
+  if (d >= 256) segsum_run<2>(d_dE, d_perm, d_seg_off, P, U, d, R, (int)nchunks, nullptr, 0, d_G, partial, span, status, nullptr, st, nullptr, INT32_MAX);
+  else segsum_run<1>(d_dE, d_perm, d_seg_off, P, U, d, R, (int)nchunks, nullptr, 0, d_G, partial, span, status, nullptr, st, nullptr, INT32_MAX);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     if (h_err && err_len) snprintf(h_err, err_len, "gram_accumulate_static: launch failed: %s", cudaGetErrorString(e));

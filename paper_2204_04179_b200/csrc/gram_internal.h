@@ -111,11 +111,10 @@ gram_status gather_diff_launch(gram_ctx* ctx, const float* d_a, const float* d_b
 gram_status gather_widen_launch(gram_ctx* ctx, const void* d_src_bf16, int64_t n_src_rows, const int32_t* d_index, int64_t P,
                                 int32_t d, float* d_E, cudaStream_t st);
 
-// in_bf16: rows of d_in are bf16 instead of fp32.  d_U (may be NULL): the number of segments is read
-// from the device instead of U.  d_rows (may be NULL): output row of segment u is d_rows[u] instead
-// of u.  add != 0: out[row] += sum instead of out[row] = sum.  gated != 0: the kernels leave d_out alone
+// d_U (may be NULL): the number of segments is read from the device instead of U.
+// d_rows (may be NULL): output row of segment u is d_rows[u] instead of u.  add != 0: out[row] += sum instead of out[row] = sum.  gated != 0: the kernels leave d_out alone
 // when the context's status word already holds an error (a step that must not change state after a bad input).
-gram_status accumulate_launch(gram_ctx* ctx, IndexWorkspace* ws, const void* d_in, int in_bf16, const int32_t* d_perm,
+gram_status accumulate_launch(gram_ctx* ctx, IndexWorkspace* ws, const float* d_in, const int32_t* d_perm,
                               const int32_t* d_seg_off, int64_t P, int32_t U, const int32_t* d_U, int32_t d,
                               const int32_t* d_rows, int add, float* d_out, cudaStream_t st, int gated = 0);
 

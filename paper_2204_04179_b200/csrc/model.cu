@@ -685,7 +685,7 @@ gram_status encoder_backward_chunk(Model* m, const float* G, int32_t n, cudaStre
   // token-embedding gradient: sum dz0 over the occurrences of each token (same index kernels as stage 1 / 4)
   IndexWorkspace* iws = gram_index_ws(ctx);
   GRAM_TRY(dedup_launch(ctx, iws, m->tok_ids, T, c.vocab, m->tok_unique, m->tok_inverse, m->tok_perm, m->tok_seg, m->tok_nu, st));
-  GRAM_TRY(accumulate_launch(ctx, iws, dz0, 0, m->tok_perm, m->tok_seg, T, 0, m->tok_nu, c.d, m->tok_unique, 1,
+  GRAM_TRY(accumulate_launch(ctx, iws, dz0, m->tok_perm, m->tok_seg, T, 0, m->tok_nu, c.d, m->tok_unique, 1,
                              m->ce.g + m->o_tok, st));
   return GRAM_OK;
 }
@@ -1239,7 +1239,7 @@ gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in
     GRAM_TRY(task_forward_backward(m, src, labels, B, kt ? nullptr : m->dE, m->loss, &dE_at, st));
     GRAM_CUDA(ctx, cudaEventRecord(ev[4], st));
     // stage 4 (Eq. 6)
-    GRAM_TRY(accumulate_launch(ctx, iws, dE_at, 0, m->perm, m->seg_off, P, U, nullptr, c.d, nullptr, 0, m->G, st));
+    GRAM_TRY(accumulate_launch(ctx, iws, dE_at, m->perm, m->seg_off, P, U, nullptr, c.d, nullptr, 0, m->G, st));
     GRAM_CUDA(ctx, cudaEventRecord(ev[5], st));
     // stage 5 (Eq. 7)
     GRAM_CUDA(ctx, cudaMemsetAsync(m->ce.g, 0, m->ce.n * 4, st));
@@ -1279,7 +1279,7 @@ gram_status model_step(Model* m, const int32_t* ids_in, const int32_t* labels_in
     GRAM_TRY(task_forward_backward(m, src, labels, B, kt ? nullptr : m->dE, m->loss, &dE_at, st));
     GRAM_CUDA(ctx, cudaEventRecord(ev[4], st));
     // stage 4 (Eq. 6) into the table; U is read on the device
-    GRAM_TRY(accumulate_launch(ctx, iws, dE_at, 0, m->perm, m->seg_off, P, 0, m->n_unique, c.d, m->unique, 1, m->table, st, 1));
+    GRAM_TRY(accumulate_launch(ctx, iws, dE_at, m->perm, m->seg_off, P, 0, m->n_unique, c.d, m->unique, 1, m->table, st, 1));
     GRAM_TRY(touched_mark_launch(ctx, m->unique, 0, m->n_unique, c.n_items, m->touched, m->tcount, 1, st));
     GRAM_CUDA(ctx, cudaEventRecord(ev[5], st));
     const int64_t task_updates = m->task.updates;
