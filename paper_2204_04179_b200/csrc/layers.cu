@@ -866,8 +866,9 @@ __global__ void __launch_bounds__(128) kt_input_bwd_vec_kernel(const float* __re
 }
 
 // Predictions of a batch that are not padding.  Up to kHeadCounts positions every block of the head counts them for itself (16 labels
-// a thread) and block 0 leaves the count for the reduction: the launch that counts and the clearing before it, some 6 us of the
-// check's step of 377, only pay above.
+// a thread) and block 0 leaves the count for the reduction.  The head with its reduction this way and with a launch that counts and
+// the clearing before it, us: 160 x 64 4.4 and 8.4, 4096 x 64 8.1 and 12.4, 4096 x 768 11.4 and 16.1.  Above, what the blocks count for
+// themselves grows with the rows: 9472 x 768 still 16.6 and 20.5, but 16 384 30.4 and 28.9, 25 600 55 and 48.
 constexpr int64_t kHeadCounts = 4096;
 __device__ __forceinline__ int32_t head_count(const int32_t* __restrict__ labels, int64_t P, int32_t* n_real) {
   if (P > kHeadCounts) return *n_real;
@@ -1788,8 +1789,10 @@ gram_status kt_head(gram_ctx* ctx, int dtype, const StreamRef& y, const float* w
                     float* dy, void* dy_b, float* dw, float* db, float* loss, float* scratch, int32_t* n_real, int64_t P,
                     int d, cudaStream_t st) {
   if (P == 0) return GRAM_OK;
-  // eight rows a warp, one where eight would leave SMs without a block: a warp's rows are a chain (160 rows: 7.2 us with eight each,
-  // 3.5 with one)
+  // A warp's rows are a chain (160 rows: 7.2 us with eight each, 3.5 with one): one row a warp while those blocks are at most one an SM,
+  // then two to eight in a block an SM, and eight from 9472 rows on, in up to four blocks an SM.  One row a warp in up to four blocks an
+  // SM also above: 1185 x 64 6.3 us for 6.7, but 2400 8.2 for 7.6, 4096 11.0 for 8.1 (768 columns: 8.3 for 8.9, 13.1 for 10.3, 16.0 for
+  // 11.4): every block counts, reads the weights and leaves a partial row.
   int blocks = (int)ceil_div64(P, P <= 8 * kNumSMs ? 8 : 64);
   if (P > 8 * kNumSMs && blocks < kNumSMs) blocks = kNumSMs;
   if (blocks > kRedBlocks) blocks = kRedBlocks;
