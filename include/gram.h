@@ -80,6 +80,11 @@ enum { GRAM_MULTI_TABLE = 0, GRAM_MULTI_PSEUDO_TARGET = 1 };
  * Texts and histories longer than 128 rows need dtype = GRAM_BF16 with heads of
  * width 64 (d / n_heads, d / task_heads); other contexts return
  * GRAM_ERR_UNSUPPORTED from the attention of such a sequence.
+ * LayerNorm (the encoder; task layers with a feed-forward part) reads rows and
+ * parameters 16 bytes at a time: d a multiple of 4 and at most 1024, and in fp32
+ * contexts d_ff (task_d_ff) a multiple of 4, since another width moves the
+ * parameters behind it.  Other contexts can be created; a pass through such a
+ * layer returns GRAM_ERR_UNSUPPORTED.
  * dtype = GRAM_BF16: matrix products and attention take bf16 operands with fp32
  * accumulation; the residual stream, LayerNorm statistics, encodings,
  * parameters and their gradients stay fp32.  GRAM_F32: everything fp32. */

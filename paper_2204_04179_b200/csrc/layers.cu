@@ -1488,7 +1488,7 @@ gram_status layernorm_forward(gram_ctx* ctx, int dtype, const float* z, const fl
                               float* mean, float* rstd, int64_t rows, int d, cudaStream_t st) {
   if (rows == 0) return GRAM_OK;
   if (d > 1024 || (d & 3)) return gram_set_error(ctx, "LayerNorm: d must be a multiple of 4 and at most 1024"), GRAM_ERR_UNSUPPORTED;
-  if (!rows_aligned({z, gamma, beta, y}))          // in fp32 contexts an odd width elsewhere moves the parameters behind it
+  if (!rows_aligned({z, gamma, beta, y}))          // in fp32 contexts an odd feed-forward width moves the parameters behind it
     return gram_set_error(ctx, "LayerNorm: rows and parameters must start on 16 bytes (feed-forward widths that are multiples of 4)"), GRAM_ERR_UNSUPPORTED;
   const int blocks = grid_for(rows * 32, 256, kNumSMs * 8);
   ProfScope prof(ctx, GRAM_K_LAYERNORM, (double)rows * d * (4.0 + (dtype == GRAM_BF16 ? 2.0 : 4.0)), 1, st, "ln_fwd");
