@@ -633,14 +633,18 @@ cudaError_t launch_f32_major(bool a_k, bool b_k, const F32Prod& p, int splits, c
 //  - K of at most four k-blocks: one round of loads by that many groups, no cluster.  160 x 512 over 128: 5.5 us over a cluster, 3.6;
 //    320 x 256 over 64 5.4 and 3.9; K = 32 takes four groups too, whose threads share the tile's epilogue (160 x 128: 4.3 and 3.2).
 //    Beyond two blocks of four groups an SM (1200 x 288 over 96, 342 tiles: 7.1 us without, 7.8 with) only as many as k-blocks.
-//  - A K range that fills one round of four groups in each of its parts, while those blocks fit at once (912 x 64 over 256: 6.6 us with
-//    eight parts of one k-block, two parts now; the check's step 390 -> 387).
 //  - Else the K range is halved over a cluster while blocks are missing and a part keeps two k-blocks.  Groups on top where the
 //    blocks leave SMs room: 64 x 64 over 4000 (64 blocks) 10.0 and 6.6, 192 x 64 (192 blocks) 10.8 and 8.6, but 256 x 64 over 1200
 //    (256 blocks) 7.0 without, 9.8 with.
 //    Eight parts with a round of four groups instead of sixteen with two k-blocks (192 x 64 over 912: 5.6 and 4.9).
 //  - Tiles that need no parts but are no more than three an SM: four groups shorten a long K (1200 x 256 over 1024, 304 tiles: 46.8
 //    and 41.6).
+//  - Instead of all that, as few parts as let each take its K in one round of four groups: where the blocks above are more than 2.75
+//    an SM, or take more than one round while these are at most one an SM, and these fit at once.  (Clusters of four and more do not
+//    reach every SM: 258 blocks of the 296.)  With those parts and with the ones above, us: 160 x 256 over 160 4.7 and 5.4, 480 x 64 over 384
+//    4.8 and 5.4, 64 x 512 over 768 6.5 and 7.9, 912 x 64 over 256 5.1 and 5.2, 912 x 128 over 192 6.3 and 7.0.  Everywhere that
+//    they fit they would lose: 64 x 64 over 256 4.8 and 3.9 (eight parts of a k-block are one round too), 320 x 128 over 384 6.4 and 5.9,
+//    576 x 128 over 512 (288 blocks) 1.4 times the time.
 struct F32Plan {
   int parts, groups;
   int64_t k_per_part;
@@ -650,11 +654,6 @@ F32Plan f32_plan(int64_t blocks, int64_t K, bool big, int most_parts) {
   const int sk = big ? F32Cfg<64>::SK : F32Cfg<32>::SK;
   auto groups_of = [&](int64_t k) { return k > 2 * sk || (K <= 4 * sk && blocks <= 2 * kNumSMs) ? 4 : (k > sk ? 2 : 1); };
   const bool one_round = !big && K <= 4 * sk && blocks * groups_of(K) <= 8 * kNumSMs;
-  if (!one_round && !big) {
-    int parts = 1;
-    while (parts < most_parts && K > 4 * sk * parts) parts *= 2;
-    if (K <= 4 * sk * parts && blocks * parts <= 2 * kNumSMs) { p.parts = parts; p.k_per_part = ceil_div64(ceil_div64(K, parts), sk) * sk; p.groups = 4; return p; }
-  }
   if (!one_round) {
     const int64_t enough = big ? kNumSMs : 4 * kNumSMs;
     while (p.parts < most_parts && blocks * p.parts * 2 <= enough && K >= 64 * p.parts) {
@@ -666,6 +665,14 @@ F32Plan f32_plan(int64_t blocks, int64_t K, bool big, int most_parts) {
   const int groups = groups_of(p.k_per_part);
   const int64_t all = blocks * p.parts;
   if (!big && (one_round || (groups == 4 ? 3 * all <= 4 * kNumSMs : all <= kNumSMs) || (p.parts == 1 && all <= 3 * kNumSMs && K >= 256))) p.groups = groups;
+  if (!one_round && !big) {
+    int parts = 1;
+    while (parts < most_parts && K > 4 * sk * parts) parts *= 2;
+    const int sms = parts > 2 ? kNumSMs * 7 / 8 : kNumSMs;
+    const bool fits = K <= 4 * sk * parts && blocks * parts <= 2 * sms;
+    if (fits && (4 * all > 11 * kNumSMs || (p.k_per_part > sk * p.groups && blocks * parts <= sms)))
+      p = {parts, 4, ceil_div64(ceil_div64(K, parts), sk) * sk};
+  }
   return p;
 }
 
