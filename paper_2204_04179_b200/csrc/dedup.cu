@@ -896,8 +896,8 @@ gram_status dedup_launch(gram_ctx* ctx, IndexWorkspace* ws, const int32_t* d_ids
   const DigitPlan plan = digit_plan(key_bits);
   const int passes = plan.passes;
   // Up to 65 536 positions: the single launch, with the fewest positions per block.  Against the chain of launches, 10 000
-  // items: 16 against 30 us at 25 600 positions, 25 / 33 at 65 536; with twice the positions per block it took 42 us at
-  // 131 072 where the chain takes 35: 16 SMs are then too few.  Where only smaller clusters can be placed, the line is lower.
+  // items: 13 against 32 us at 25 600 positions, 21 / 32 at 65 536 (over 10^6 items 30 / 40); with twice the positions per block it took
+  // 42 us at 131 072 where the chain takes 35: 16 SMs are then too few.  Where only smaller clusters can be placed, the line is lower.
   int form = 0;
   while (form < kClusterForms && P > (int64_t)gram_cluster_blocks(ctx) * cluster_dedup_form(form).tile) ++form;
   if (form < kClusterForms) {

@@ -203,7 +203,8 @@ __device__ __forceinline__ void epilogue_store4(const EpiDev& e, CT* C, int64_t 
 // (the order depends on the sizes alone), each block finishing its share of the tile's rows.  One launch, no
 // workspace.  Weight gradients of the check's model (64 x 64 to 256 x 64 over about 900 rows): 130 to 185 us each with
 // one 64 x 64 block per tile and a synchronous load per k-block, 6 to 7 us now; the
-// model's whole training step 2.49 -> 0.48 ms with the chain of launches below, 0.36 with gradients' products in pairs (gemm_f32_pair_kernel).
+// model's whole training step 2.49 -> 0.48 ms with the chain of launches below, 0.43 -> 0.39 with gradients' products in pairs
+// (gemm_f32_pair_kernel).
 // What a k-block waits for is its loads: 32 k at a time in the small tiles, and up to four groups of 64 threads with a k-block each,
 // so that K = 128 can take one round of loads and no cluster; the groups' tiles are added in ascending order in shared memory.
 // Which products get groups: f32_plan.
@@ -555,8 +556,8 @@ __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(con
 // The two products that read one gradient dY [T, N]: dW [N, K] += dY^T X (product w; its row sums are the bias gradient) and
 // dX [T, K] = dY W (product x), in one launch.  Neither fills the chip in the models that run in fp32, and each is a chain of launch,
 // loads and exchange of partial sums: side by side they take little more than the longer one (64 x 256 and 256 x 64 over 900
-// rows: 9.0 us where the two took 11.3 and the bias gradient's sums, two launches more, 5).  The check's step 429 -> 386 us in 65 launches
-// instead of 87, steps of other widths and sizes 2 to 11 % less.  Clusters of gridDim.x / clusters blocks;
+// rows: 9.0 us where the two took 11.3 and the bias gradient's sums, two launches more, 5).  By this alone the check's step went from 429 to
+// 386 us, 87 launches to 65, steps of other widths and sizes 2 to 11 % less.  Clusters of gridDim.x / clusters blocks;
 // the first w_clusters work on product w, wp blocks a tile, the others on product x, xp blocks a tile.
 struct F32Pair {
   F32Prod w, x;
