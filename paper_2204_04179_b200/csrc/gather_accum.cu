@@ -4,6 +4,8 @@
 #include "gram_internal.h"
 #include "tc_common.cuh"
 
+#include <type_traits>
+
 namespace {
 
 // ---------------------------------------------------------------------------
@@ -258,8 +260,11 @@ __global__ void __launch_bounds__(256) segsum_chunks_kernel(const float* __restr
   const int64_t c0 = (int64_t)chunk * R, c1 = min(c0 + R, P);
   if (c0 >= c1) return;
 
+  // the current item's ends, in the width that the row loop is faster with: 300 000 x 256 65.8 us with 32 bits and 61.2 with 64, 1600 x 768 7.3
+  // and 6.6; with half the columns a warp 300 000 x 64 42.0 and 43.2, 3200 x 64 6.4 and 6.6
+  typedef typename std::conditional<VPL == 2, int64_t, int32_t>::type Bound;
   SegItems<ADD> it(seg_off, rows, U, find_segment(seg_off, U, c0, lane), lane);
-  int32_t seg_begin = seg_off[it.u], seg_end = it.end();
+  Bound seg_begin = seg_off[it.u], seg_end = it.end();
   float4 acc[VPL], old[ADD ? VPL : 1];
 #pragma unroll
   for (int v = 0; v < VPL; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -451,8 +456,12 @@ __global__ void __launch_bounds__(32 * SEG_WARPS, 2) segsum_ring_kernel(const fl
 // simply adds them in order; an item that reaches farther is summed by the whole block, a run per warp.
 // Nearly every chunk has an item that runs into the next one, and what that takes is the chain item, parts, store: with a block of
 // eight warps for each of them 34 us at 10^6 positions of 768 columns, a twelfth of the blocks on the chip at a time; 14 this way.
+// While a block for each of them fits the chip at once (eight blocks an SM) it has one all the same (PER = 1): an item over more than nine
+// parts then waits for no others.  us with a block each and with eight to a block: 1600 positions of 768 columns 2.7 and 3.6, 3200 x 64 2.7
+// and 3.1, 4200 x 768 3.2 and 3.9, 6400 x 768 (1200 pairs) 3.8 and 3.8, 9000 x 768 4.5 and 4.2, 25 600 x 128 5.4 and 4.8.
 constexpr int FIX_RUNS = 8;
-template <int VPL>
+constexpr int64_t kFixAlone = 8 * kNumSMs;
+template <int VPL, int PER>
 __global__ void __launch_bounds__(32 * FIX_RUNS) segsum_fixup_kernel(const int32_t* __restrict__ seg_off, int64_t P, int32_t U,
                                                            int d, int64_t R, int nchunks, int nslabs,
                                                            const int32_t* __restrict__ rows, int add,
@@ -466,7 +475,7 @@ __global__ void __launch_bounds__(32 * FIX_RUNS) segsum_fixup_kernel(const int32
   if (U <= 0) return;
   if (gate && *gate) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int chunk0 = (int)(blockIdx.x / nslabs) * FIX_RUNS, slab = (int)(blockIdx.x % nslabs);
+  const int chunk0 = (int)(blockIdx.x / nslabs) * PER, slab = (int)(blockIdx.x % nslabs);
   const int col0 = slab * (VPL * 128);
   // part of item chunk c: the own part of the chunk it starts in (which = 1), what it left in a later one (which = 0)
   auto part = [&](int c, int which, float4 (&x)[VPL]) {
@@ -480,14 +489,15 @@ __global__ void __launch_bounds__(32 * FIX_RUNS) segsum_fixup_kernel(const int32
 #pragma unroll
     for (int v = 0; v < VPL; ++v) { a[v].x += x[v].x; a[v].y += x[v].y; a[v].z += x[v].z; a[v].w += x[v].w; }
   };
-  const int chunk = chunk0 + w;
+  constexpr bool alone = PER == 1;                   // all warps look at the same chunk
+  const int chunk = chunk0 + (alone ? 0 : w);
   const int64_t c0 = (int64_t)chunk * R, c1 = min(c0 + R, P);
   int2 sp = make_int2(-1, -1);
   if (chunk < nchunks && c0 < c1 && c1 < P) sp = span[chunk];       // left by the first launch
   const bool mine = sp.x >= 0 && sp.x < U;           // else no item starts here and runs on (same for the whole warp)
   const int last = mine ? min(sp.y, nchunks - 1) : -1;
   const bool block_wide = mine && last - chunk > FIX_RUNS;
-  if (mine && !block_wide) {
+  if (mine && !block_wide && (!alone || w == 0)) {
     float4 acc[VPL];
     part(chunk, 1, acc);
 #pragma unroll
@@ -502,11 +512,13 @@ __global__ void __launch_bounds__(32 * FIX_RUNS) segsum_fixup_kernel(const int32
     }
     store_row<VPL>(out, rows ? rows[sp.x] : sp.x, d, col0, lane, acc, add != 0);
   }
-  if (lane == 0) far[w] = make_int2(sp.x, block_wide ? last : -1);
-  if (!__syncthreads_or(block_wide)) return;
-  for (int f = 0; f < FIX_RUNS; ++f) {
-    const int2 it = far[f];
-    if (it.y < 0) continue;
+  if (!alone) {
+    if (lane == 0) far[w] = make_int2(sp.x, block_wide ? last : -1);
+    if (!__syncthreads_or(block_wide)) return;
+  }
+  for (int f = 0; f < PER; ++f) {
+    const int2 it = alone ? make_int2(sp.x, block_wide ? last : -1) : far[f];
+    if (it.y < 0) continue;                          // the same for the whole block
     const int first = chunk0 + f;
     float4 acc[VPL];
 #pragma unroll
@@ -685,8 +697,10 @@ static void segsum_run(const float* d_in, const int32_t* d_perm, const int32_t* 
     launch_chain(add ? segsum_chunks_kernel<VPL, 8, true> : segsum_chunks_kernel<VPL, 8, false>, blocks, 256, 0, st, d_in, d_perm, d_seg_off, P, U, d, R,
                  nchunks, nslabs, d_rows, d_out, partial, span, status, d_U, gate);
   }
+  const int per_block = warps <= kFixAlone ? 1 : FIX_RUNS;
   if (nchunks > 1)
-    launch_chain(segsum_fixup_kernel<VPL>, (unsigned)(ceil_div(nchunks, FIX_RUNS) * nslabs), 32 * FIX_RUNS, 0, st, d_seg_off, P, U, d, R, nchunks, nslabs, d_rows, add, d_out, partial, span, d_U, gate);
+    launch_chain(per_block == 1 ? segsum_fixup_kernel<VPL, 1> : segsum_fixup_kernel<VPL, FIX_RUNS>, (unsigned)(ceil_div(nchunks, per_block) * nslabs),
+                 32 * FIX_RUNS, 0, st, d_seg_off, P, U, d, R, nchunks, nslabs, d_rows, add, d_out, partial, span, d_U, gate);
 }
 
 gram_status accumulate_launch(gram_ctx* ctx, IndexWorkspace* ws, const float* d_in, const int32_t* d_perm,
