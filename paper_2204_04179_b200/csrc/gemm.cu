@@ -552,6 +552,15 @@ __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(con
   __shared__ __align__(16) F32Smem<TILE, NG> sm;           // [group][buffer][operand]; later the groups' partial tiles
   f32_tile<TILE, A_K, B_K, NG, false>(p, (int64_t)blockIdx.y * TILE, (int64_t)blockIdx.x * TILE, blockIdx.z, gridDim.z, 0, sm);
 }
+// Tiles of 64 x 64 with room for PER_SM blocks an SM: two have the registers to keep their loads apart, three take half as long again
+// for a round of blocks, so three go where that makes fewer rounds by more than that.  256 columns over 768: 188 blocks 53.8 us
+// with two and 59.0 with three, 440 blocks 107 and 82.
+template <bool A_K, bool B_K, int PER_SM>
+__global__ void __launch_bounds__(F32Cfg<64>::THREADS, PER_SM) gemm_f32_wide_kernel(const __grid_constant__ F32Prod p) {
+  if (!chain_begin()) return;
+  __shared__ __align__(16) F32Smem<64, 1> sm;
+  f32_tile<64, A_K, B_K, 1, false>(p, (int64_t)blockIdx.y * 64, (int64_t)blockIdx.x * 64, blockIdx.z, gridDim.z, 0, sm);
+}
 
 // The two products that read one gradient dY [T, N]: dW [N, K] += dY^T X (product w; its row sums are the bias gradient) and
 // dX [T, K] = dY W (product x), in one launch.  Neither fills the chip in the models that run in fp32, and each is a chain of launch,
@@ -602,7 +611,12 @@ F32Prod f32_prod(const float* A, int64_t lda, const float* B, int64_t ldb, float
 
 template <int TILE, int NG, bool A_K, bool B_K>
 cudaError_t launch_f32(const F32Prod& p, int splits, cudaStream_t st) {
-  auto kern = gemm_f32_kernel<TILE, A_K, B_K, NG>;
+  const int64_t blocks = ceil_div64(p.M, TILE) * ceil_div(p.N, TILE) * splits;
+  void (*kern)(F32Prod);
+  if constexpr (TILE == 64)
+    kern = 3 * ceil_div64(blocks, 3 * kNumSMs) < 2 * ceil_div64(blocks, 2 * kNumSMs) ? gemm_f32_wide_kernel<A_K, B_K, 3> : gemm_f32_wide_kernel<A_K, B_K, 2>;
+  else
+    kern = gemm_f32_kernel<TILE, A_K, B_K, NG>;
   if (splits > 8) {                                        // clusters of more than 8 blocks are an opt-in
     const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (err != cudaSuccess) return err;
