@@ -456,9 +456,10 @@ __global__ void __launch_bounds__(32 * SEG_WARPS, 2) segsum_ring_kernel(const fl
 // simply adds them in order; an item that reaches farther is summed by the whole block, a run per warp.
 // Nearly every chunk has an item that runs into the next one, and what that takes is the chain item, parts, store: with a block of
 // eight warps for each of them 34 us at 10^6 positions of 768 columns, a twelfth of the blocks on the chip at a time; 14 this way.
-// While a block for each of them fits the chip at once (eight blocks an SM) it has one all the same (PER = 1): an item over more than nine
-// parts then waits for no others.  us with a block each and with eight to a block: 1600 positions of 768 columns 2.7 and 3.6, 3200 x 64 2.7
-// and 3.1, 4200 x 768 3.2 and 3.9, 6400 x 768 (1200 pairs) 3.8 and 3.8, 9000 x 768 4.5 and 4.2, 25 600 x 128 5.4 and 4.8.
+// While a block for each of them fits the chip at once (eight blocks an SM) it has one all the same (PER = 1), and all eight warps take
+// the item: one over more than nine parts then waits for no others.  us with a block each and with eight to a block: 912 positions of 64
+// columns 2.28 and 2.85 (Zipf 1.1; 2.23 and 2.11 at 0.8, where no item is that long), 3200 x 64 2.50 and 3.10, 1600 x 768 3.06 and 3.51,
+// 12 800 x 128 (800 pairs) 3.46 and 3.66, into a table 3.73 and 4.19; 6400 x 768 (1200 pairs) 4.13 and 3.81, 9000 x 768 4.98 and 4.11.
 constexpr int FIX_RUNS = 8;
 constexpr int64_t kFixAlone = 8 * kNumSMs;
 template <int VPL, int PER>
@@ -496,8 +497,8 @@ __global__ void __launch_bounds__(32 * FIX_RUNS) segsum_fixup_kernel(const int32
   if (chunk < nchunks && c0 < c1 && c1 < P) sp = span[chunk];       // left by the first launch
   const bool mine = sp.x >= 0 && sp.x < U;           // else no item starts here and runs on (same for the whole warp)
   const int last = mine ? min(sp.y, nchunks - 1) : -1;
-  const bool block_wide = mine && last - chunk > FIX_RUNS;
-  if (mine && !block_wide && (!alone || w == 0)) {
+  const bool block_wide = mine && (alone || last - chunk > FIX_RUNS);
+  if (!alone && mine && !block_wide) {
     float4 acc[VPL];
     part(chunk, 1, acc);
 #pragma unroll
@@ -524,12 +525,13 @@ __global__ void __launch_bounds__(32 * FIX_RUNS) segsum_fixup_kernel(const int32
 #pragma unroll
     for (int v = 0; v < VPL; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (w == 0) part(first, 1, acc);
-    for (int c = first + 1 + w; c <= it.y; c += 8 * FIX_RUNS) {     // eight parts on their way per warp
-      float4 x[8][VPL];
+    constexpr int AHEAD = alone ? 4 : 8;             // parts on their way per warp
+    for (int c = first + 1 + w; c <= it.y; c += AHEAD * FIX_RUNS) {
+      float4 x[AHEAD][VPL];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) part(min(c + FIX_RUNS * k, it.y), 0, x[k]);
+      for (int k = 0; k < AHEAD; ++k) part(min(c + FIX_RUNS * k, it.y), 0, x[k]);
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
+      for (int k = 0; k < AHEAD; ++k)
         if (c + FIX_RUNS * k <= it.y) plus(acc, x[k]);
     }
 #pragma unroll
