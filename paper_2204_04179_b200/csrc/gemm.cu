@@ -296,7 +296,7 @@ struct F32Prod {
   float* C;
   int64_t ldc, M, K, k_per_part;
   int32_t N, vec_a, vec_b, vec_e;
-  float* row_sums;               // row_sums[m] += the sum of A(m, k) over k (may be null; FOLD only)
+  float* row_sums;               // row_sums[m] += the sum of A(m, k) over k (may be null; SUMS only)
   int32_t fold;                  // FOLD: k-blocks of a group that are added up in one chain
   EpiDev e;
 };
@@ -305,8 +305,8 @@ template <int TILE, int NG> using F32Smem = float[NG][F32Cfg<TILE, NG>::BUFS][2]
 // One tile of a product by one block, or by `parts` blocks of a cluster whose ranks begin at rank0, this one being number `part`.
 // All threads of the blocks call it; with one part it does not touch the cluster's barrier.
 // FOLD: after every `fold` k-blocks of a group their sum goes to the sum of those before, so that few parts of a long K are no longer
-// a chain of additions than many.
-template <int TILE, bool A_K, bool B_K, int NG, bool FOLD>
+// a chain of additions than many.  SUMS: row_sums may be asked for.
+template <int TILE, bool A_K, bool B_K, int NG, bool FOLD, bool SUMS>
 __device__ __forceinline__ void f32_tile(const F32Prod& p, int64_t m0, int64_t n0, int part_no, int parts, int rank0, F32Smem<TILE, NG>& sm) {
   using Cfg = F32Cfg<TILE, NG>;
   constexpr int LD = Cfg::LD, NV = Cfg::NV, T = Cfg::GROUP, G = Cfg::GROUPS, SK = Cfg::SK, BUFS = Cfg::BUFS;
@@ -319,8 +319,8 @@ __device__ __forceinline__ void f32_tile(const F32Prod& p, int64_t m0, int64_t n
   const int N = p.N, vec_a = p.vec_a, vec_b = p.vec_b, vec_e = p.vec_e;
   const int group = threadIdx.x / T, tid = threadIdx.x % T, tx = tid % (TILE / 4), ty = tid / (TILE / 4);
   const int64_t kb = (int64_t)part_no * p.k_per_part, ke = min(kb + p.k_per_part, K);
-  static_assert(!FOLD || G > 1, "the row sums go through the groups' partial tiles");
-  const bool sums = FOLD && p.row_sums != nullptr && n0 == 0;
+  static_assert(!SUMS || G > 1, "the row sums go through the groups' partial tiles");
+  const bool sums = SUMS && p.row_sums != nullptr && n0 == 0;
   float asum = 0.f;                                        // of this thread's row of A
   float acc[4][4] = {}, folded[FOLD ? 4 : 1][4] = {};
   int chain = p.fold;
@@ -550,7 +550,7 @@ template <int TILE, bool A_K, bool B_K, int NG>
 __global__ void __launch_bounds__(F32Cfg<TILE, NG>::THREADS) gemm_f32_kernel(const __grid_constant__ F32Prod p) {
   if (!chain_begin()) return;
   __shared__ __align__(16) F32Smem<TILE, NG> sm;           // [group][buffer][operand]; later the groups' partial tiles
-  f32_tile<TILE, A_K, B_K, NG, false>(p, (int64_t)blockIdx.y * TILE, (int64_t)blockIdx.x * TILE, blockIdx.z, gridDim.z, 0, sm);
+  f32_tile<TILE, A_K, B_K, NG, false, false>(p, (int64_t)blockIdx.y * TILE, (int64_t)blockIdx.x * TILE, blockIdx.z, gridDim.z, 0, sm);
 }
 // Tiles of 64 x 64 with room for PER_SM blocks an SM: two have the registers to keep their loads apart, three take half as long again
 // for a round of blocks, so three go where that makes fewer rounds by more than that.  256 columns over 768: 188 blocks 53.8 us
@@ -559,7 +559,7 @@ template <bool A_K, bool B_K, int PER_SM>
 __global__ void __launch_bounds__(F32Cfg<64>::THREADS, PER_SM) gemm_f32_wide_kernel(const __grid_constant__ F32Prod p) {
   if (!chain_begin()) return;
   __shared__ __align__(16) F32Smem<64, 1> sm;
-  f32_tile<64, A_K, B_K, 1, false>(p, (int64_t)blockIdx.y * 64, (int64_t)blockIdx.x * 64, blockIdx.z, gridDim.z, 0, sm);
+  f32_tile<64, A_K, B_K, 1, false, false>(p, (int64_t)blockIdx.y * 64, (int64_t)blockIdx.x * 64, blockIdx.z, gridDim.z, 0, sm);
 }
 
 // The two products that read one gradient dY [T, N]: dW [N, K] += dY^T X (product w; its row sums are the bias gradient) and
@@ -572,7 +572,8 @@ struct F32Pair {
   F32Prod w, x;
   int32_t wp, xp, w_clusters, w_tiles, x_tiles;
 };
-__global__ void __launch_bounds__(F32Cfg<32, 4>::THREADS) gemm_f32_pair_kernel(const __grid_constant__ F32Pair a) {
+template <bool FOLD>
+__global__ void __launch_bounds__(F32Cfg<32, 4>::THREADS, 2) gemm_f32_pair_kernel(const __grid_constant__ F32Pair a) {
   if (!chain_begin()) return;
   __shared__ __align__(16) F32Smem<32, 4> sm;
   uint32_t blocks, rank;
@@ -586,8 +587,8 @@ __global__ void __launch_bounds__(F32Cfg<32, 4>::THREADS) gemm_f32_pair_kernel(c
   const int tiles_n = (p.N + 31) / 32;
   const int64_t m0 = (int64_t)(tile / tiles_n) * 32, n0 = (int64_t)(tile % tiles_n) * 32;
   const bool there = tile < (is_w ? a.w_tiles : a.x_tiles);
-  if (there && is_w) f32_tile<32, false, false, 4, true>(a.w, m0, n0, part, parts, (int)rank - part, sm);
-  else if (there) f32_tile<32, true, false, 4, true>(a.x, m0, n0, part, parts, (int)rank - part, sm);
+  if (there && is_w) f32_tile<32, false, false, 4, FOLD, true>(a.w, m0, n0, part, parts, (int)rank - part, sm);
+  else if (there) f32_tile<32, true, false, 4, FOLD, false>(a.x, m0, n0, part, parts, (int)rank - part, sm);
   if (blocks > 1 && !(there && parts > 1)) {               // the cluster's barrier counts every block
     gram_cluster_sync();
     gram_cluster_sync();
@@ -1905,7 +1906,8 @@ static EpiDev epi_dev(const GemmEpilogue& epi) {
 // us with the SMs shared out and this way: 192 x 64 over 4096 rows 32.6 and 16.6 (apart 21.0), over 6400 47.3 and 23.7, 288 x 96 over 2952
 // 44.8 and 22.8, 384 x 128 48.3 and 32.0, 96 x 32 over 10 000 22.2 and 15.4; a line at two rounds or eight loses up to a fifth at single sizes.
 // What a group adds up in one chain is no longer than in the product alone (`fold`; error against 64 bits of 192 x 64 over 6400 4.9e-7 -> 2.0e-7, which is
-// the product alone): folding costs 3 to 5 % of a launch of many rounds.
+// the product alone): folding costs 3 to 5 % of a launch of many rounds, and launches that need none have a kernel of
+// their own (steps of the check's size take up to 1 % less than with folding in all of them).  Both keep to the registers of two blocks an SM.
 bool gemm_f32_grads_together(int64_t T, int N, int K) {
   const int64_t w = (int64_t)ceil_div(N, 32) * ceil_div(K, 32), x = ceil_div64(T, 32) * ceil_div(K, 32);
   return T > 0 && N > 0 && K > 0 && w + x <= 3 * kNumSMs;
@@ -1942,7 +1944,9 @@ gram_status gemm_f32_grads(gram_ctx* ctx, const float* dY, const float* X, float
   a.x.fold = fold_of(a.x_tiles, N);
   const int blocks = a.wp > a.xp ? a.wp : a.xp;
   a.w_clusters = ceil_div(a.w_tiles * a.wp, blocks);
-  if (blocks > 8) GRAM_CUDA(ctx, cudaFuncSetAttribute(gemm_f32_pair_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  auto folds = [](const F32Prod& p) { return p.k_per_part > (int64_t)p.fold * ROUND; };
+  auto kern = folds(a.w) || folds(a.x) ? gemm_f32_pair_kernel<true> : gemm_f32_pair_kernel<false>;
+  if (blocks > 8) GRAM_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(blocks * (a.w_clusters + ceil_div(a.x_tiles * a.xp, blocks))));
   cfg.blockDim = dim3(F32Cfg<32, 4>::THREADS);
@@ -1955,7 +1959,7 @@ gram_status gemm_f32_grads(gram_ctx* ctx, const float* dY, const float* X, float
   attr[1] = chain_attribute();
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  GRAM_CUDA(ctx, cudaLaunchKernelEx(&cfg, gemm_f32_pair_kernel, a));
+  GRAM_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, a));
   return GRAM_OK;
 }
 
